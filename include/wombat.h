@@ -318,7 +318,7 @@ int wb_pool_free_bytes(wb_batch* b, size_t* largest, size_t* total);
 int wb_batch_steps_left(wb_batch* b, int* out);
 
 /* Self-test of the library's FP64 reciprocal and reciprocal-square-root
- * helpers (PTX approximations refined by a third-order correction) against
+ * helpers (fixed-point arithmetic on the integer pipes) against
  * the CUDA library division and rsqrt on n inputs spread over [1e-300, 1e300]:
  * worst[0] = max |rcp(x) x - 1|, worst[1] = max |rsqrt_ours / rsqrt_cuda - 1|.
  * Uses the grid's reduction words; synchronises the grid's stream. */

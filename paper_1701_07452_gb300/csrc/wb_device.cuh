@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "wb_soft.cuh"
+
 #define WB_NG 5  // boundary zones per patch (Sec. "MHD in Two Dimensions")
 
 // zone-centred state fields
@@ -141,32 +143,6 @@ __device__ __forceinline__ double wb_minmod(double a, double b) {
   long long ia = __double_as_longlong(a), ib = __double_as_longlong(b);
   double r = wb_abs_less(a, b) ? a : b;
   return ((ia ^ ib) >= 0) ? r : 0.0;
-}
-
-// Reciprocal and reciprocal square root for FP64 without the library
-// division/sqrt sequences: the PTX approximations rcp.approx.ftz.f64 and
-// rsqrt.approx.ftz.f64 (relative error ~1e-6, measured) refined by one
-// third-order correction from the series of (1-e)^-1 and (1-e)^-1/2:
-//   1/x:       e = 1 - x y,    y <- y (1 + e + e^2)
-//   1/sqrt(x): e = 1 - x y^2,  y <- y (1 + e/2 + 3 e^2 / 8)
-// The truncation error is O(e^3) ~ 1e-18, below one ulp.  Inputs must be
-// positive, finite and normal: the approximations flush subnormal inputs to
-// zero (callers test with wb_normal_pos or know the range).
-__device__ __forceinline__ double wb_rcp(double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  double e = __fma_rn(-x, y, 1.0);
-  double p = __fma_rn(e, e, e);
-  return __fma_rn(y, p, y);
-}
-
-__device__ __forceinline__ double wb_rsqrt(double x) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  double h = __dmul_rn(x, y);
-  double e = __fma_rn(-h, y, 1.0);
-  double p = __fma_rn(0.375, e, 0.5);
-  return __fma_rn(__dmul_rn(y, e), p, y);
 }
 
 // Comparisons on the IEEE bit patterns (integer pipe; the FP64 pipe is the

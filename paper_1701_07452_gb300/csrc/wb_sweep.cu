@@ -24,7 +24,7 @@
 // time drops their Q-branch arithmetic.
 //
 // FP64 is the scarce unit on this GPU, so the arithmetic avoids the library
-// divide and square-root sequences (wb_rcp / wb_rsqrt), and gamma_k = dg/alpha
+// divide and square-root sequences (wb_rcp / wb_roots run on the integer pipes), and gamma_k = dg/alpha
 // is never formed: Q(nu + gamma) alpha = |nu alpha + dg| sign(alpha) when
 // |nu alpha + dg| >= 2 eps |alpha|, else (nu alpha + dg)^2 / (4 eps alpha) +
 // eps alpha, which is the same quantity with one reciprocal, needed only for

@@ -32,7 +32,7 @@ constexpr int kBlock = 64;
 constexpr int kEpsZeroLD = (1 << 1) | (1 << 3) | (1 << 5);
 
 struct Cell {
-  double rho, ir, sr, isr;        // rho, 1/rho, sqrt(rho), 1/sqrt(rho)
+  double rho, ir, sr;             // rho, 1/rho, sqrt(rho)
   double vn, vt1, vt2;
   double bt1, bt2;
   double eref;                    // E - bn^2/2 (energy referred to the face field)
@@ -66,9 +66,9 @@ __device__ __forceinline__ void load_cell(const double* const* q, long long off,
   const double bn = ld<NC>(q[F_BX + D] + off);
   c.bt1 = ld<NC>(q[F_BX + T1] + off);
   c.bt2 = ld<NC>(q[F_BX + T2] + off);
-  c.isr = wb_rsqrt(c.rho);
-  c.ir = __dmul_rn(c.isr, c.isr);
-  c.sr = __dmul_rn(c.rho, c.isr);
+  const WbRoots rr = wb_roots(c.rho);
+  c.sr = rr.sq;
+  c.ir = rr.rcp;
   c.vn = __dmul_rn(c.mn, c.ir);
   c.vt1 = __dmul_rn(c.mt1, c.ir);
   c.vt2 = __dmul_rn(c.mt2, c.ir);
@@ -222,7 +222,9 @@ __device__ __forceinline__ int face_system(const Cell& L, const Cell& R, double 
   const double iD = wb_rcp(WB_ADD(L.sr, R.sr));
   const double wL = WB_MUL(L.sr, iD), wR = WB_MUL(R.sr, iD);
   const double rho = WB_MUL(L.sr, R.sr);
-  const double irho = WB_MUL(L.isr, R.isr);
+  const WbRoots rroe = wb_roots(rho);
+  const double irho = rroe.rcp;
+  const double isrho = rroe.rsq, srho = rroe.sq;
   const double vn = WB_FMA(wL, L.vn, WB_MUL(wR, R.vn));
   const double vt1 = WB_FMA(wL, L.vt1, WB_MUL(wR, R.vt1));
   const double vt2 = WB_FMA(wL, L.vt2, WB_MUL(wR, R.vt2));
@@ -237,30 +239,25 @@ __device__ __forceinline__ int face_system(const Cell& L, const Cell& R, double 
   const double bt2s = WB_FMA(bt1, bt1, WB_MUL(bt2, bt2));
   const double a2 = WB_FMA(P.gm1, WB_FMA(-WB_ADD(b2, bt2s), irho, WB_SUB(H, hv2)), -gX);
   if (!wb_normal_pos(a2)) return 2;
-  const double isrho = wb_rsqrt(rho);
-  const double srho = WB_MUL(rho, isrho);
   const double ca2 = WB_MUL(b2, irho), ct2 = WB_MUL(bt2s, irho);
   const double dac = WB_SUB(a2, ca2);
   const double disc = WB_FMA(dac, dac, WB_MUL(ct2, WB_FMA(2.0, WB_ADD(a2, ca2), ct2)));
   const double sum = WB_ADD(WB_ADD(a2, ca2), ct2);
-  double rsd = 0.0, sd = 0.0;
-  if (wb_normal_pos(disc)) {  // a subnormal discriminant is degenerate (sd ~ 0)
-    rsd = wb_rsqrt(disc);
-    sd = WB_MUL(disc, rsd);
-  }
+  // a subnormal discriminant is degenerate (sd ~ 0)
+  const double sd = wb_normal_pos(disc) ? wb_sqrt(disc) : 0.0;
   const double cf2 = wb_half(WB_ADD(sum, sd));
-  const double icf = wb_rsqrt(cf2);
-  const double ia = wb_rsqrt(a2);
-  const double a = WB_MUL(a2, ia);
+  const WbRoots rcf = wb_roots(cf2), ra_ = wb_roots(a2);
+  const double icf = rcf.rsq, ia = ra_.rsq;
+  const double cf = rcf.sq, a = ra_.sq;
   const double ca = WB_MUL(wb_fabs(b), isrho);
-  const double cf = WB_MUL(cf2, icf);
   const double cs = WB_MUL(WB_MUL(a, ca), icf);  // c_f c_s = a c_a
   // 1/|B_t| and c_t = |B_t| / sqrt(rho_); a transverse field whose square is
   // not a normal double (underflowing noise ahead of a front) counts as 0
   double ib = 0.0, ct = 0.0, btm = 0.0;  // btm = |B_t|
   if (wb_normal_pos(bt2s)) {
-    ib = wb_rsqrt(bt2s);
-    btm = WB_MUL(bt2s, ib);
+    const WbRoots rb = wb_roots(bt2s);
+    ib = rb.rsq;
+    btm = rb.sq;
     ct = WB_MUL(btm, isrho);
   }
   double af, as;
@@ -311,7 +308,7 @@ __device__ __forceinline__ int face_system(const Cell& L, const Cell& R, double 
   const double dvp = WB_FMA(-b2n, dvt1, WB_MUL(b1n, dvt2));
   const double dbb = WB_FMA(b1n, dbt1, WB_MUL(b2n, dbt2));
   const double dbpS = wb_xsgn(WB_FMA(-b2n, dbt1, WB_MUL(b1n, dbt2)), S);
-  const double ia2 = WB_MUL(ia, ia);
+  const double ia2 = ra_.rcp;
   const double hir = wb_half(irho), hisr = wb_half(isrho);
   const double i2ra = WB_MUL(hisr, ia);   // 1 / (2 sqrt(rho) a)
   const double ri2a2 = WB_MUL(hir, ia2);  // 1 / (2 rho a^2)
@@ -830,7 +827,7 @@ __device__ __forceinline__ void eref_half(const WbView& v, long long qo, long lo
 
 // sqrt for the CFL rate; inputs below the normal range (or not > 0) give 0
 __device__ __forceinline__ double wb_sqrt_fast(double x) {
-  return wb_normal_pos(x) ? __dmul_rn(x, wb_rsqrt(x)) : 0.0;
+  return wb_normal_pos(x) ? wb_sqrt(x) : 0.0;
 }
 
 // CFL signal rate sum_d (|v_d| + c_f,d)/dx_d of one zone (Sec. 3 fast speed)
