@@ -62,16 +62,17 @@ ALG_FLOPS_PER_FACE = 879.0
 ALG_FLOPS_PER_CELL_UPDATE = 5871.0
 # FP64 flops (DFMA = 2, DMUL = DADD = 1) the kernels execute, from the ncu
 # FP64 instruction counters of one step of the 96^3 box: per interface system
-# of k_sweep (the mean of the six sweeps), and per zone of the other stage
+# of k_sweep (the mean over a step), and per zone of the other stage
 # kernels of the step together (profiles/k_sweep_96cube_ncu_full.md,
 # profiles/stages_96cube_fp64_counts.md).  Counted per face of the box the
 # figure leaves out the ~2 % of overlap systems a 256^3 launch adds.
 EXEC_FLOPS_PER_FACE = 450.8
 EXEC_STAGE_FLOPS_PER_ZONE = 431.8
 # DRAM bytes (read + write) of one k_sweep launch at the 256^3 workload, the
-# mean of the six sweeps of a step from one ncu capture
+# mean of the launches of a step from one ncu capture
 # (profiles/k_sweep_256cube_dram.md), valid only for the kernel sources it was
-# taken on (their SHA-256 over csrc/wb_sweep.cu, wb_units.cuh, wb_device.cuh);
+# taken on (their SHA-256 over csrc/wb_sweep.cu, wb_units.cuh, wb_soft.cuh,
+# wb_device.cuh);
 # the algorithmic figure is 128 B per face.
 SWEEP_DRAM_CAPTURE = {"n": 256, "bytes": 3.6763e9,
                       "src_sha256": "68f8615198707e20999cb9332cdfca1bc16d4505845845c06e39a34523ecfa46"}
@@ -87,7 +88,7 @@ FP64_FLOPS_PER_CLK_PER_SM = 4.0
 def sweep_src_sha256():
     """SHA-256 over the sweep kernel's sources (the DRAM capture's stamp)."""
     h = hashlib.sha256()
-    for name in ("wb_sweep.cu", "wb_units.cuh", "wb_device.cuh"):
+    for name in ("wb_sweep.cu", "wb_units.cuh", "wb_soft.cuh", "wb_device.cuh"):
         with open(os.path.join(ROOT, "paper_1701_07452_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()
@@ -117,8 +118,8 @@ def cpu_model():
 
 
 def step_launches(desc):
-    """Kernels one wb_advance step launches: the dt kernel, 14 per pass over a
-    batch of patches (6 sweeps, reference EMF, corner EMFs, half CT,
+    """Kernels one wb_advance step launches: the dt kernel, 10 per pass over a
+    batch of patches (2 sweeps of all axes, reference EMF, corner EMFs, half CT,
     transverse states, half-step reference EMF, corner EMFs, final CT, update)
     and the ghost fill; a grid periodic on every axis with all patches in one
     pass adds the 7 periodic-image fills of its interior-only stages."""
@@ -127,7 +128,7 @@ def step_launches(desc):
     passes = -(-npatch // per_pass)
     flat = desc.n[2] == 1 and desc.patches[2] == 1 and desc.bc[2] == 0
     images = passes == 1 and not flat and all(desc.bc[a] == 0 for a in range(3))
-    return 2 + (21 if images else 14) * passes
+    return 2 + (17 if images else 10) * passes
 
 
 def workload_name(n):
@@ -668,7 +669,7 @@ def main():
 
     if rank == 0:
         per_launch_ms = sweep_ms / max(sweep_launches, 1)
-        faces_per_launch = sweep_faces_per_step(n) / 6.0
+        faces_per_launch = sweep_faces_per_step(n) / 2.0  # three axes a launch, two launches a step
         achieved = ALG_FLOPS_PER_FACE * faces_per_launch / (per_launch_ms * 1e-3) / 1e12
         achieved_exec = EXEC_FLOPS_PER_FACE * faces_per_launch / (per_launch_ms * 1e-3) / 1e12
         clk_summary = clk.summary()

@@ -184,7 +184,8 @@ const char* wb_last_error(const wb_grid* g);
  * doubles); *written = doubles written. */
 int wb_debug_stage(wb_grid* g, int which, double* out, long long cap, long long* written);
 
-/* Kernel timing of the MHDTVD sweep launches (Steps 1, 6, 7): enable != 0
+/* Kernel timing of the MHDTVD sweep launches (Step 1; Steps 6 and 7; each
+ * launch takes the three axes): enable != 0
  * starts recording CUDA events around every sweep launch on the grid's stream
  * (at most 8192 launches; later ones are not recorded); enable == 0 stops.
  * wb_profile_read synchronises the stream and returns the summed duration in
@@ -231,7 +232,7 @@ const char* wb_noalloc_last_error(void);
  * box must share gamma, cfl, eps, sweby and floors).  One wb_batch_advance
  * launches one persistent kernel that advances every box with steps left by
  * up to nsteps CTU+CT steps, each box with its own CFL dt: thread blocks take
- * chunks of work items (pencil segments, zones, faces, edges) of all boxes
+ * chunks of work items (sweep tiles, zones, faces, edges) of all boxes
  * from a device work counter, and a bounded grid-wide barrier separates the
  * stages of a step.  The state of all boxes stays resident; the step's
  * intermediates are shared by workspace groups of boxes whose combined
@@ -248,10 +249,11 @@ const char* wb_noalloc_last_error(void);
  * wb_batch_advance: one persistent launch of nsteps steps; use_graph != 0
  * replays it from a captured CUDA graph (captured on first use per nsteps).
  * Synchronises the stream; returns WB_ERR_TIMEOUT if a barrier wait ran out.
- * wb_batch_autotune: times trial_steps real steps per candidate segment
- * length and blocks per SM in each form (below), keeps the fastest (cached
- * per box-size mix).
- * wb_batch_config: set them explicitly (0 = keep); barrier_budget_cycles is
+ * wb_batch_autotune: times trial_steps real steps per candidate number of
+ * blocks per SM in each form (below), keeps the fastest (cached per box-size
+ * mix).
+ * wb_batch_config: set them explicitly (0 = keep; seg_len is accepted and
+ * reported, but the sweeps have no segments); barrier_budget_cycles is
  * the per-barrier wait limit in SM clock cycles (default 20 s worth).
  * wb_batch_stage_timer: on != 0 zeroes and starts the per-stage timer (one
  * block stamps the GPU global timer at the barrier closing every stage), 0

@@ -7,7 +7,7 @@
 // in Three Dimensions", Steps 1-11), each box with its own CFL dt.  Inside the
 // launch the stages of a step run one after another over all boxes of a
 // workspace group; within a stage, thread blocks take chunks of work items
-// (pencil segments, zones, faces, edges of some box) from an atomic counter,
+// (sweep tiles, zones, faces, edges of some box) from an atomic counter,
 // and a grid-wide barrier separates stages.  The barrier waits are bounded:
 // a block that waits longer than the budget sets an error word and every
 // block returns, so a stalled launch ends with WB_ERR_TIMEOUT instead of a
@@ -123,41 +123,35 @@ __host__ __device__ inline long long box_cnt(const WbBox& b) {
   return (long long)(b.hi[0] - b.lo[0] + 1) * (b.hi[1] - b.lo[1] + 1) * (b.hi[2] - b.lo[2] + 1);
 }
 
-// sweep items: pencils x segments.  seg_len is the longest segment wanted;
-// a pencil is cut into nseg segments of nearly equal length (*len_out each,
-// the last one shorter by less than nseg faces) so that no item is left far
-// shorter than the others.
-__host__ __device__ inline void sweep_shape(const WbBox& b, int d, int seg_len, long long* npen,
-                                            int* nseg, int* len_out = nullptr) {
+// the pencils of a sweep along d, and their thread layout
+__host__ __device__ inline long long sweep_pencils(const WbBox& b, int d) {
   const int U = (d == 0) ? 1 : 0, W = (d == 2) ? 1 : 2;
-  *npen = (long long)(b.hi[U] - b.lo[U] + 1) * (b.hi[W] - b.lo[W] + 1);
-  const int len = b.hi[d] - b.lo[d] + 1;
-  *nseg = (len + seg_len - 1) / seg_len;
-  if (len_out) *len_out = (len + *nseg - 1) / *nseg;
+  return (long long)(b.hi[U] - b.lo[U] + 1) * (b.hi[W] - b.lo[W] + 1);
 }
 
-__host__ __device__ inline long long stage_items(int s, int d, const WbGeo& g, bool wrap, int seg_len) {
+__host__ __device__ inline long long stage_items(int s, int d, const WbGeo& g, bool wrap) {
   if (s == BS_DT) return 1;
   if (stage_is_wrap(s)) return wrap ? wbu::shell_count(g, s == BS_W_QH ? 2 : 1) : 0;
   if (s == BS_HALO) return wbu::shell_count(g, WB_NG);
   WbBox b = stage_box(s, d, g.n, wrap);
   if (stage_is_sweep(s)) {
-    long long np;
-    int ns;
-    sweep_shape(b, d, seg_len, &np, &ns);
-    return np * ns;
+    const int len = b.hi[d] - b.lo[d] + 1;
+    return wbu::sweep_tiles(sweep_pencils(b, d), len, wbu::sweep_ring(len, wrap));
   }
   return box_cnt(b);
 }
 
 __host__ __device__ inline int items_per_chunk(int s) {
-  return (stage_is_sweep(s) || s == BS_DT) ? kB : kB * kItemsPerThread;
+  return stage_is_sweep(s) ? 1 : (s == BS_DT ? kB : kB * kItemsPerThread);
 }
 
 struct BoxInfo {
   WbView v;
   int bc[3];
   int wrap;  // periodic on every axis: interior-only stages + periodic images
+  // the sweeps' fields, [corrector][axis]: read where they are needed rather
+  // than held in registers through a sweep
+  wbu::SweepFrame sw[2][3];
 };
 
 // Axes whose high boundary face is an outflow copy of the last owned face
@@ -181,7 +175,6 @@ struct BatchParams {
   WbPhys phys;
   double cfl;
   int dt_lag;                 // dt from the previous step's start state
-  int seg_len;
   long long budget;           // barrier wait budget in SM clock cycles
 };
 
@@ -232,44 +225,23 @@ __device__ __forceinline__ void warp_max_atomic(double w, unsigned long long* ds
   warp_max_key(wb_rate_bits(w), dst);
 }
 
-template <int D, int EZ, bool PROT>
-__device__ __forceinline__ int sweep_item(const BoxInfo& bi, bool corr, const WbBox& b, long long item,
-                                          int seg_len, double dt, const WbPhys& P,
-                                          const wbu::Rec rec[2]) {
-  constexpr int U = (D == 0) ? 1 : 0, W = (D == 2) ? 1 : 2;
-  long long npen;
-  int nseg, slen;
-  sweep_shape(b, D, seg_len, &npen, &nseg, &slen);
-  const int seg = (int)(item / npen);
-  const long long pen = item - seg * npen;
-  const int nu = b.hi[U] - b.lo[U] + 1;
-  const int fa = b.lo[D] + seg * slen;
-  int fb = fa + slen - 1;
-  if (fb > b.hi[D]) fb = b.hi[D];
+// One tile of a sweep of one box (every thread of the block).
+template <int EZ, bool PROT>
+__device__ __forceinline__ int box_sweep_tile(const BoxInfo& bi, bool corr, int d, long long tile, double dt,
+                                              const WbPhys& P, wbu::LaneEdge& X) {
   const WbView& v = bi.v;
-  const double* const* q = corr ? v.qh[D] : v.q;
-  const double* bn = corr ? v.bh[D] : v.b[D];
-  double* const* F = corr ? v.Fc[D] : v.Fp[D];
-  return wbu::sweep_segment<D, false, EZ, PROT>(v.geo, q, bn, F, 0, 0, b.lo[U] + (int)(pen % nu), b.lo[W] + (int)(pen / nu),
-                               fa, fb, dt, P, rec);
+  const bool wrap = bi.wrap != 0;
+  const WbBox b = stage_box(corr ? BS_CORR : BS_PRED, d, v.geo.n, wrap);
+  return wbu::sweep_tile<EZ, PROT, false>(v.geo, b, d, bi.sw[corr ? 1 : 0][d], tile,
+                                          wbu::sweep_ring(b.hi[d] - b.lo[d] + 1, wrap), 1, 0, 0,
+                                          dt, P, X);
 }
 
-template <int EZ, bool PROT>
-__device__ __forceinline__ void unit_item(const BatchParams& B, int s, int d, int box,
-                                          const BoxInfo& bi, long long item, double dt,
-                                          const wbu::Rec rec[2], unsigned long long* wkey, int* hits, int* bad,
-                                          int* hll) {
+__device__ __forceinline__ void unit_item(const BatchParams& B, int s, int d, const BoxInfo& bi, long long item,
+                                          double dt, unsigned long long* wkey, int* hits, int* bad) {
   const WbView& v = bi.v;
   const int* n = v.geo.n;
   const bool wrap = bi.wrap != 0;
-  if (stage_is_sweep(s)) {
-    const WbBox b = stage_box(s, d, n, wrap);
-    const bool corr = s == BS_CORR;
-    if (d == 0) *hll += sweep_item<0, EZ, PROT>(bi, corr, b, item, B.seg_len, dt, B.phys, rec);
-    else if (d == 1) *hll += sweep_item<1, EZ, PROT>(bi, corr, b, item, B.seg_len, dt, B.phys, rec);
-    else *hll += sweep_item<2, EZ, PROT>(bi, corr, b, item, B.seg_len, dt, B.phys, rec);
-    return;
-  }
   // the remaining stages (transverse states, half-step EMF, update); the
   // cheap ones go through unit_pair
   const WbBox b = stage_box(s, d, n, wrap);
@@ -295,7 +267,6 @@ __device__ __forceinline__ void unit_item(const BatchParams& B, int s, int d, in
     }
     default: break;
   }
-  (void)box;
 }
 
 // Stages whose items are cheap and mostly waiting on memory: a thread takes
@@ -522,10 +493,9 @@ __device__ __forceinline__ void stage_stamp(const BatchParams& B, int s, unsigne
 }
 
 template <int EZ, bool PROT>
-__global__ void __launch_bounds__(wbu::kBlock, 4) k_batch(BatchParams B, int nsteps) {
-  __shared__ double srec[2][wbu::R_WORDS][wbu::kBlock];
+__global__ void __launch_bounds__(kB, wbu::kSweepBlocks) k_batch(BatchParams B, int nsteps) {
+  __shared__ wbu::LaneEdge X;
   __shared__ long long s_chunk;
-  const wbu::Rec rec[2] = {{&srec[0][0][threadIdx.x]}, {&srec[1][0][threadIdx.x]}};
   const unsigned nblocks = gridDim.x;
   unsigned stage_seq = 0;
   // stage timer: block 0 stamps the end of every stage (after its barrier)
@@ -565,18 +535,20 @@ __global__ void __launch_bounds__(wbu::kBlock, 4) k_batch(BatchParams B, int nst
           const double dt = *(volatile const double*)&B.scal[box].dt;
           if (!wb_pos(dt)) continue;
           const BoxInfo& bi = B.boxes[box];
-          const long long nitems = stage_items(s, sub, bi.v.geo, bi.wrap != 0, B.seg_len);
+          const long long nitems = stage_items(s, sub, bi.v.geo, bi.wrap != 0);
           const long long i0 = (c - pre[lo]) * ipc;
           long long i1 = i0 + ipc;
           if (i1 > nitems) i1 = nitems;
           unsigned long long wkey = 0ULL;
           int hits = 0, bad = 0, hll = 0;
-          if (stage_pairs(s)) {
+          if (stage_is_sweep(s)) {
+            hll = box_sweep_tile<EZ, PROT>(bi, s == BS_CORR, sub, i0, dt, B.phys, X);
+          } else if (stage_pairs(s)) {
             for (long long it = i0 + threadIdx.x; it < i1; it += 2 * kB)
               unit_pair(s, sub, bi, it, it + kB < i1 ? it + kB : -1, dt);
           } else {
             for (long long it = i0 + threadIdx.x; it < i1; it += kB)
-              unit_item<EZ, PROT>(B, s, sub, box, bi, it, dt, rec, &wkey, &hits, &bad, &hll);
+              unit_item(B, s, sub, bi, it, dt, &wkey, &hits, &bad);
           }
           if (s == BS_FINAL) warp_max_key(wkey, &B.scal[box].wmax_next);
           if (hits) atomicAdd((unsigned long long*)&B.scal[box].floor_hits, (unsigned long long)hits);
@@ -655,24 +627,14 @@ __device__ __forceinline__ void drain_stage(const BatchParams& B, int grp, int s
 // (the flux arithmetic is explicitly rounded, so the bits do not depend on
 // which kernel runs it).
 template <int EZ, bool PROT>
-__global__ void __launch_bounds__(kB, 4) k_bstage_sweep(BatchParams B, int grp, int s, unsigned seq) {
-  __shared__ double srec[2][wbu::R_WORDS][kB];
-  const wbu::Rec rec[2] = {{&srec[0][0][threadIdx.x]}, {&srec[1][0][threadIdx.x]}};
+__global__ void __launch_bounds__(kB, wbu::kSweepBlocks) k_bstage_sweep(BatchParams B, int grp, int s, unsigned seq) {
+  __shared__ wbu::LaneEdge X;
   unsigned* ctr = stage_counter(B, seq);
-  const bool corr = s == BS_CORR;
   drain_stage(B, grp, s, ctr, [&](int box, int d, long long cc) {
     const double dt = B.scal[box].dt;
     if (!wb_pos(dt)) return;
-    const BoxInfo& bi = B.boxes[box];
-    const long long nitems = stage_items(s, d, bi.v.geo, bi.wrap != 0, B.seg_len);
-    const long long it = cc * kB + threadIdx.x;
-    if (it >= nitems) return;
-    const WbBox b = stage_box(s, d, bi.v.geo.n, bi.wrap != 0);
-    int hll;
-    if (d == 0) hll = sweep_item<0, EZ, PROT>(bi, corr, b, it, B.seg_len, dt, B.phys, rec);
-    else if (d == 1) hll = sweep_item<1, EZ, PROT>(bi, corr, b, it, B.seg_len, dt, B.phys, rec);
-    else hll = sweep_item<2, EZ, PROT>(bi, corr, b, it, B.seg_len, dt, B.phys, rec);
-    if (hll) atomicAdd((unsigned long long*)&B.scal[box].hll_faces, (unsigned long long)hll);
+    const int hll = box_sweep_tile<EZ, PROT>(B.boxes[box], s == BS_CORR, d, cc, dt, B.phys, X);
+    if (hll) atomicAdd((unsigned long long*)&B.scal[box].hll_faces, 1ULL);
   });
   stage_stamp(B, s, seq);
 }
@@ -691,7 +653,7 @@ __global__ void __launch_bounds__(kNtZone, zone_min_blocks(CLS))
     const double dt = B.scal[box].dt;
     if (!wb_pos(dt)) return;
     const BoxInfo& bi = B.boxes[box];
-    const long long nitems = stage_items(s, d, bi.v.geo, bi.wrap != 0, B.seg_len);
+    const long long nitems = stage_items(s, d, bi.v.geo, bi.wrap != 0);
     const long long i0 = cc * ipc;
     const long long i1 = i0 + ipc < nitems ? i0 + ipc : nitems;
     if (CLS == SC_COPY) {
@@ -757,7 +719,7 @@ struct TuneKey {
 };
 std::mutex g_tune_mu;
 struct TuneVal {
-  int seg_len, blocks_per_sm, form;
+  int blocks_per_sm, form;
 };
 std::map<TuneKey, TuneVal> g_tune_cache;
 
@@ -810,7 +772,7 @@ struct wb_batch {
   int form = WB_BATCH_PERSISTENT;
   int zone_blocks[SC_COUNT];  // resident blocks per SM of each zone-stage kernel (staged form)
   int sweep_blocks = 1;       // resident blocks per SM of the staged form's sweep kernel
-  int seg_len;
+  int seg_len;  // accepted and reported for callers; the sweeps have no segments
   int blocks_per_sm;
   int max_blocks_per_sm;
   int sms;
@@ -890,7 +852,7 @@ PoolSizes pool_sizes(size_t state_bytes, size_t work_bytes, int cap, int max_n) 
   return P;
 }
 
-// chunk prefix tables for the current groups and seg_len
+// chunk prefix tables for the current groups
 void build_prefix(const wb_batch* b, std::vector<long long>& pre, std::vector<long long>& off) {
   const int ngroups = (int)b->gfirst.size() - 1;
   pre.clear();
@@ -904,7 +866,7 @@ void build_prefix(const wb_batch* b, std::vector<long long>& pre, std::vector<lo
         const int box = b->gbox[e];
         for (int sub = 0; sub < nsub; ++sub) {
           pre.push_back(acc);
-          const long long items = stage_items(s, sub, b->geo[box], b->info[box].wrap != 0, b->seg_len);
+          const long long items = stage_items(s, sub, b->geo[box], b->info[box].wrap != 0);
           acc += (items + items_per_chunk(s) - 1) / items_per_chunk(s);
         }
       }
@@ -934,8 +896,8 @@ int rebuild(wb_batch* b) {
   double* work = b->work_base;
   b->nbox = 0;
   // boxes in decreasing size: within a stage the work list then starts with
-  // the longest items (the big boxes' pencil segments) and ends with the
-  // shortest, so the blocks that finish last leave little idle time
+  // the big boxes' items and ends with the smallest boxes', so the blocks that
+  // finish last leave little idle time
   std::vector<int> order;
   std::vector<char> want(b->cap);
   const bool any = any_granted(b);
@@ -967,6 +929,12 @@ int rebuild(wb_batch* b) {
     for (int dd = 0; dd < 3; ++dd) bi.v.bh[dd] = base + (size_t)g.V * k++;
     for (int dd = 0; dd < 3; ++dd)
       for (int c = 0; c < 8; ++c) bi.v.qh[dd][c] = base + (size_t)g.V * k++;
+    for (int corr = 0; corr < 2; ++corr) {
+      const WbView& v = bi.v;
+      wbu::sweep_frame<0>(corr ? v.qh[0] : v.q, corr ? v.bh[0] : v.b[0], corr ? v.Fc[0] : v.Fp[0], bi.sw[corr][0]);
+      wbu::sweep_frame<1>(corr ? v.qh[1] : v.q, corr ? v.bh[1] : v.b[1], corr ? v.Fc[1] : v.Fp[1], bi.sw[corr][1]);
+      wbu::sweep_frame<2>(corr ? v.qh[2] : v.q, corr ? v.bh[2] : v.b[2], corr ? v.Fc[2] : v.Fp[2], bi.sw[corr][2]);
+    }
     cur += w;
     b->gbox.push_back(i);
   }
@@ -1017,7 +985,6 @@ BatchParams params(const wb_batch* b) {
   p.phys = b->phys;
   p.cfl = b->cfl;
   p.dt_lag = b->dt_lag;
-  p.seg_len = b->seg_len;
   p.budget = b->budget;
   return p;
 }
@@ -1133,7 +1100,6 @@ void apply_tune_cache(wb_batch* b) {
   std::sort(key.sizes.begin(), key.sizes.end());
   auto it = g_tune_cache.find(key);
   if (it != g_tune_cache.end()) {
-    b->seg_len = it->second.seg_len;
     b->blocks_per_sm = std::min(it->second.blocks_per_sm, b->max_blocks_per_sm);
     b->form = it->second.form;
   }
@@ -1605,20 +1571,19 @@ int wb_batch_get_config(wb_batch* b, int* seg_len, int* blocks_per_sm, int* grou
   return WB_OK;
 }
 
-// Online autotuner: time trial_steps steps under each candidate segment
-// length, then each block count, keep the fastest.  The candidates change
-// only the work decomposition, so the trial steps are ordinary steps of the
-// simulation (results do not depend on the configuration).
+// Online autotuner: time trial_steps steps of each form under each block count,
+// keep the fastest.  The candidates change only the work decomposition, so the
+// trial steps are ordinary steps of the simulation (results do not depend on
+// the configuration).
 int wb_batch_autotune(wb_batch* b, int trial_steps, double* best_ms) {
   if (!b || trial_steps < 1) return bfail(b, WB_ERR_INVALID, "bad argument");
   int brc = ensure_built(b);
   if (brc) return brc;
-  const int segs[] = {16, 24, 32, 48, 64, 96, 136};
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
-  auto trial = [&](int seg, int bps, float* ms) -> int {
-    int rc = wb_batch_config(b, seg, bps, 0);
+  auto trial = [&](int bps, float* ms) -> int {
+    int rc = wb_batch_config(b, 0, bps, 0);
     if (rc) return rc;
     cudaEventRecord(e0, b->stream);
     cudaError_t e = enqueue_advance(b, trial_steps);
@@ -1629,30 +1594,22 @@ int wb_batch_autotune(wb_batch* b, int trial_steps, double* best_ms) {
     cudaEventElapsedTime(ms, e0, e1);
     return WB_OK;
   };
-  int best_seg = b->seg_len, best_b = b->max_blocks_per_sm, best_form = b->form;
+  int best_b = b->max_blocks_per_sm, best_form = b->form;
   float best = 1e30f, ms = 0.f;
   int rc = WB_OK;
   for (int form = WB_BATCH_PERSISTENT; rc == WB_OK && form <= WB_BATCH_STAGED; ++form) {
     b->form = form;
-    int fseg = b->seg_len, fb = b->max_blocks_per_sm;
-    float fbest = 1e30f;
-    for (int seg : segs) {
-      rc = trial(seg, b->max_blocks_per_sm, &ms);
+    for (int bps = b->max_blocks_per_sm; bps >= 1; --bps) {
+      rc = trial(bps, &ms);
       if (rc) break;
-      if (ms < fbest) { fbest = ms; fseg = seg; }
+      if (ms < best) { best = ms; best_b = bps; best_form = form; }
     }
-    for (int bps = 1; rc == WB_OK && bps < b->max_blocks_per_sm; ++bps) {
-      rc = trial(fseg, bps, &ms);
-      if (rc) break;
-      if (ms < fbest) { fbest = ms; fb = bps; }
-    }
-    if (rc == WB_OK && fbest < best) { best = fbest; best_seg = fseg; best_b = fb; best_form = form; }
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   b->form = best_form;
   if (rc) return rc;
-  rc = wb_batch_config(b, best_seg, best_b, 0);
+  rc = wb_batch_config(b, 0, best_b, 0);
   if (rc) return rc;
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
@@ -1660,7 +1617,7 @@ int wb_batch_autotune(wb_batch* b, int trial_steps, double* best_ms) {
     for (int i = 0; i < b->cap; ++i)
       if (b->alive[i]) key.sizes.push_back(b->d[i].n[0] * 1000000 + b->d[i].n[1] * 1000 + b->d[i].n[2]);
     std::sort(key.sizes.begin(), key.sizes.end());
-    g_tune_cache[key] = {best_seg, best_b, best_form};
+    g_tune_cache[key] = {best_b, best_form};
   }
   if (best_ms) *best_ms = best;
   return WB_OK;

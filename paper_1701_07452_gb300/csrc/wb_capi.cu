@@ -260,28 +260,33 @@ StageArgs stage_args(wb_grid* g, long long p0, int nslots) {
   return a;
 }
 
-SweepArgs sweep_args(wb_grid* g, const StageArgs& s, int dir, bool corr, const WbBox& bx) {
+SweepArgs sweep_args(wb_grid* g, const StageArgs& s, bool corr, const WbBox (&bx)[3], int nslots) {
   SweepArgs a;
   std::memset(&a, 0, sizeof(a));
-  for (int c = 0; c < 8; ++c) a.q[c] = corr ? s.v.qh[dir][c] : s.v.q[c];
-  a.bn = corr ? s.v.bh[dir] : s.v.b[dir];
-  for (int c = 0; c < 8; ++c) a.F[c] = corr ? s.v.Fc[dir][c] : s.v.Fp[dir][c];
+  const WbView& v = s.v;
+  wbu::sweep_frame<0>(corr ? v.qh[0] : v.q, corr ? v.bh[0] : v.b[0], corr ? v.Fc[0] : v.Fp[0], a.s[0]);
+  wbu::sweep_frame<1>(corr ? v.qh[1] : v.q, corr ? v.bh[1] : v.b[1], corr ? v.Fc[1] : v.Fp[1], a.s[1]);
+  wbu::sweep_frame<2>(corr ? v.qh[2] : v.q, corr ? v.bh[2] : v.b[2], corr ? v.Fc[2] : v.Fp[2], a.s[2]);
   a.slot_in = corr ? s.slot_w : s.slot_q;
   a.slot_out = s.slot_w;
   a.geo = g->geo;
-  a.box = bx;
+  for (int d = 0; d < 3; ++d) a.box[d] = bx[d];
   a.dt = &g->scal->dt;
   a.phys = g->phys;
   a.scal = g->scal;
+  a.nslots = nslots;
   return a;
 }
 
 const size_t kMaxProfiled = 8192;
 
-void sweep(wb_grid* g, int dir, const SweepArgs& a, int nslots) {
+void sweeps(wb_grid* g, const SweepArgs& a) {
   bool rec = g->prof && g->ev_used + 2 <= g->ev.size();
   if (rec) cudaEventRecord(g->ev[g->ev_used], g->stream);
-  wb_launch_sweep(dir, a, nslots, g->stream);
+  int closed = 0;  // an axis of one patch, its images in place
+  for (int d = 0; d < 3; ++d)
+    if (g->wrap && g->map.np[d] == 1) closed |= 1 << d;
+  wb_launch_sweeps(a, closed, g->stream);
   if (rec) {
     cudaEventRecord(g->ev[g->ev_used + 1], g->stream);
     g->ev_used += 2;
@@ -313,7 +318,7 @@ void enqueue_pass_wrap(wb_grid* g) {
   const WbBox in = box(0, N0 - 1, 0, N1 - 1, 0, N2 - 1);
   const WbBox in3[3] = {in, in, in};
   // Step 1: predictor fluxes on the interior faces (face N_d is face 0)
-  for (int d = 0; d < 3; ++d) sweep(g, d, sweep_args(g, A, d, false, in), ns);
+  sweeps(g, sweep_args(g, A, false, in3, ns));
   // Step 2: reference EMF; then the images of both
   wb_launch_eref(A, in, s);
   wb_launch_wrap(wrap_list({g->Fp[0][0], g->Fp[0][1], g->Fp[0][2], g->Fp[0][3], g->Fp[0][4], g->Fp[0][6],
@@ -336,7 +341,7 @@ void enqueue_pass_wrap(wb_grid* g) {
     wb_launch_wrap(L, G, g->map, 2, s);
   }
   // Steps 6, 7: corrector fluxes
-  for (int d = 0; d < 3; ++d) sweep(g, d, sweep_args(g, A, d, true, in), ns);
+  sweeps(g, sweep_args(g, A, true, in3, ns));
   wb_launch_wrap(wrap_list({g->Fc[0][0], g->Fc[0][1], g->Fc[0][2], g->Fc[0][3], g->Fc[0][4], g->Fc[0][6],
                             g->Fc[0][7], g->Fc[1][0], g->Fc[1][1], g->Fc[1][2], g->Fc[1][3], g->Fc[1][4],
                             g->Fc[1][5], g->Fc[1][7], g->Fc[2][0], g->Fc[2][1], g->Fc[2][2], g->Fc[2][3],
@@ -371,9 +376,11 @@ void enqueue_pass(wb_grid* g, long long p0, int nslots) {
     return flat ? ::box(l0, h0, l1, h1, 0, 0) : ::box(l0, h0, l1, h1, l2, h2);
   };
   // Step 1: predictor fluxes from q^n
-  sweep(g, 0, sweep_args(g, A, 0, false, box(-3, N0 + 3, -4, N1 + 3, -4, N2 + 3)), nslots);
-  sweep(g, 1, sweep_args(g, A, 1, false, box(-4, N0 + 3, -3, N1 + 3, -4, N2 + 3)), nslots);
-  sweep(g, 2, sweep_args(g, A, 2, false, box(-4, N0 + 3, -4, N1 + 3, -3, N2 + 3)), nslots);
+  {
+    const WbBox pb[3] = {box(-3, N0 + 3, -4, N1 + 3, -4, N2 + 3), box(-4, N0 + 3, -3, N1 + 3, -4, N2 + 3),
+                         box(-4, N0 + 3, -4, N1 + 3, -3, N2 + 3)};
+    sweeps(g, sweep_args(g, A, false, pb, nslots));
+  }
   // Step 2: reference EMF; Step 3: corner EMFs
   wb_launch_eref(A, box(-4, N0 + 3, -4, N1 + 3, -4, N2 + 3), s);
   {
@@ -394,9 +401,11 @@ void enqueue_pass(wb_grid* g, long long p0, int nslots) {
     wb_launch_transverse(A, tb, s);
   }
   // Steps 6, 7: corrector fluxes
-  sweep(g, 0, sweep_args(g, A, 0, true, box(-1, N0 + 1, -1, N1, -1, N2)), nslots);
-  sweep(g, 1, sweep_args(g, A, 1, true, box(-1, N0, -1, N1 + 1, -1, N2)), nslots);
-  sweep(g, 2, sweep_args(g, A, 2, true, box(-1, N0, -1, N1, -1, N2 + 1)), nslots);
+  {
+    const WbBox cb[3] = {box(-1, N0 + 1, -1, N1, -1, N2), box(-1, N0, -1, N1 + 1, -1, N2),
+                         box(-1, N0, -1, N1, -1, N2 + 1)};
+    sweeps(g, sweep_args(g, A, true, cb, nslots));
+  }
   // Step 8: half-step reference EMF; Step 9: corner EMFs
   wb_launch_eref_half(A, box(-1, N0, -1, N1, -1, N2), s);
   {

@@ -15,7 +15,8 @@ struct WbPhys {
   double gamma, gm1, gm2, g_over_gm1, inv_gm1, gm2_over_gm1, cfl;
   float gamma_f;  // gamma for the FP32 screen of the signal rate
   double hgm2;  // (gamma - 2) / 2
-  double eps[7], two_eps[7], four_eps[7], inv16eps[7];
+  double eps[7], two_eps[7], inv16eps[7];
+  double four_eps[7];
   double inv4eps_m1[7];  // 1/(4 eps_k) - 1: Q_k(nu) - nu^2 = nu^2 (1/(4 eps) - 1) + eps
   int eps_zero;  // bit k set when eps_k == 0
   double sweby;
@@ -192,6 +193,18 @@ __device__ __forceinline__ bool wb_zero(double x) {
 // a <= b for a, b >= 0 (non-negative, non-NaN operands)
 __device__ __forceinline__ bool wb_le_nonneg(double a, double b) {
   return __double_as_longlong(a) <= __double_as_longlong(b);
+}
+// x 2^n in the order of high words (x >= 0): a quick comparison by magnitude
+__device__ __forceinline__ unsigned wb_hi_scaled(double x, int n) { return wb_hi32(x) + ((unsigned)n << 20); }
+// x <= 2^-77 max(a, b) is possible (x, a, b >= 0): a cheap test ahead of
+// x <= 1e-24 (a + b + x), whose right side is below 2^-78 max(a, b) (1 + 2^-20)
+__device__ __forceinline__ bool wb_maybe_small(double x, double a, double b) {
+  return wb_hi_scaled(x, 77) <= max(wb_hi32(a), wb_hi32(b));
+}
+// x <= f s for x, s >= 0.  Not inlined: the multiply would be issued by every
+// warp, its lanes predicated off, where a quick test has ruled the case out.
+static __device__ __noinline__ bool wb_at_most(double x, double f, double s) {
+  return __double_as_longlong(x) <= __double_as_longlong(__dmul_rn(f, s));
 }
 // 2 x, exact: the exponent field raised by one on the integer pipe for a
 // normal x whose double is normal; zero, subnormals, the top binade, inf and

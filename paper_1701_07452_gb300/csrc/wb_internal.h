@@ -9,20 +9,18 @@ struct wb_desc;
 // Physics constants of a descriptor (gamma, CFL, eps_k, limiter, floors).
 WbPhys wb_phys_of(const struct wb_desc* d);
 
+// The sweeps along the three axes of one pass.
 struct SweepArgs {
-  const double* q[8];      // input zone fields (slot 0)
-  const double* bn;        // normal face field (slot 0)
-  double* F[8];            // output flux fields (slot 0); F[F_BX + dir] unused
+  wbu::SweepFrame s[3];    // fields (slot 0)
   long long slot_in, slot_out;
   WbGeo geo;
-  WbBox box;               // faces along the sweep axis, zones across it
+  WbBox box[3];            // faces along the sweep axis, zones across it
   const double* dt;
   WbPhys phys;
   WbScalars* scal;
-  int nseg;                // segments per pencil (0: chosen at launch)
-  int seg_len;             // faces per segment (set at launch)
-  int balanced;            // 1: equal runs of (slot, 32-pencil group, face) units per warp
-  int nslots;              // slots of the pass (balanced launches take them all in one row)
+  int nslots;
+  int ring[3];             // thread layout (wbu::sweep_ring; set at launch)
+  long long tile0[4];      // first tile of each axis (set at launch)
 };
 
 // Pointers of one pipeline pass over a batch of patches: the view holds the
@@ -49,7 +47,9 @@ struct GridMap {
   long long npatch;
 };
 
-void wb_launch_sweep(int dir, const SweepArgs& a, int nslots, cudaStream_t s);
+// closed: bit d set when the pencils along axis d are whole and periodic (the
+// last zone is the first one's neighbour)
+void wb_launch_sweeps(SweepArgs a, int closed, cudaStream_t s);
 
 void wb_launch_eref(const StageArgs& a, const WbBox& box, cudaStream_t s);
 void wb_launch_edges(const StageArgs& a, bool corrector, const WbBox box[3], cudaStream_t s);

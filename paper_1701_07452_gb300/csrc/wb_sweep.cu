@@ -3,13 +3,11 @@
 // for the predictor fluxes of Step 1 and the corrector fluxes of Steps 6-7 of
 // the 3D CTU+CT integrator (Sec. "MHD in Three Dimensions").
 //
-// One thread marches along one segment of a pencil of faces.  For each face it
-// builds the Roe-averaged interface state (a Cargo-Gallice type average,
-// App. A), the characteristic amplitudes alpha_k, nu_k = (dt/dx) a_k and
-// g-tilde_k; the flux of face f is emitted once g-tilde of face f+1 is known,
-// so every eigen-system is computed once per segment (segments overlap by the
-// two faces whose g-tilde the limiter needs).  The per-face eigen-data wait
-// for one iteration in a double-buffered shared-memory record.
+// One launch takes the three axes, one thread one face: it builds the
+// Roe-averaged interface state (a Cargo-Gallice type average, App. A), the
+// characteristic amplitudes alpha_k, nu_k = (dt/dx) a_k and g-tilde_k, trades
+// g-tilde and limited slopes with its neighbours along the pencil and emits the
+// flux (wbu::sweep_tile).
 //
 // Eigen-structure (derived for this implementation): the linearisation
 // dF = A dU with rho_ = sL sR, s-weighted v and H, opposite-weighted B_t and
@@ -34,174 +32,42 @@
 
 namespace {
 
-// threads per block and resident blocks per SM the sweep is compiled for
-// (registers per thread follow from their product; the face records take
-// 2 x 38 doubles per thread of shared memory)
-#ifndef WB_SWEEP_BLOCK
-#define WB_SWEEP_BLOCK 64
-#endif
-// equal runs per warp once a launch has at least this many units per
-// resident warp (measured: 128^3 sweeps 7 % faster than the one-segment-per-
-// thread form at 54 units a warp, 64^3 2 % at 14)
-#ifndef WB_BAL_MIN
-#define WB_BAL_MIN 4
-#endif
-#ifndef WB_SWEEP_MIN_BLOCKS
-#define WB_SWEEP_MIN_BLOCKS 4
-#endif
-constexpr int kBlock = WB_SWEEP_BLOCK;
-using SRec = wbu::RecT<kBlock>;
-
 using wbu::kEpsZeroLD;
 
-template <int D, int EZ, bool PROT>
-__global__ void __launch_bounds__(kBlock, WB_SWEEP_MIN_BLOCKS) k_sweep(SweepArgs A) {
-  constexpr int U = (D == 0) ? 1 : 0;  // fastest transverse axis of the thread map
-  constexpr int W = (D == 2) ? 1 : 2;
-  __shared__ double srec[2][wbu::R_WORDS][kBlock];
+template <int EZ, bool PROT>
+__global__ void __launch_bounds__(wbu::kBlock, wbu::kSweepBlocks) k_sweep(SweepArgs A) {
+  __shared__ wbu::LaneEdge X;
   const double dt = *A.dt;
   if (!wb_pos(dt)) return;
-  const int nu_ = A.box.hi[U] - A.box.lo[U] + 1;
-  const int nw_ = A.box.hi[W] - A.box.lo[W] + 1;
-  const long long npen = (long long)nu_ * nw_;
-  const int len = A.box.hi[D] - A.box.lo[D] + 1;
-  long long slot = blockIdx.y;
-  const SRec rec[2] = {{&srec[0][0][threadIdx.x]}, {&srec[1][0][threadIdx.x]}};
-  // Balanced: the work is the list of units (slot, group of 32 adjacent
-  // pencils, face), slot- then group-major, over every slot of the pass; warp
-  // w takes units [w U / C, (w+1) U / C) of the C warps of the launch (one
-  // grid row) and marches one segment per group it touches, its 32 lanes on
-  // the 32 pencils of the group (adjacent pencils: coalesced rows).
-  // Otherwise one segment per thread: item = segment x pencils + pencil, one
-  // grid row per slot.
-  const long long ngroups = (npen + 31) / 32;
-  const long long units = ngroups * len * (A.balanced ? A.nslots : 1);
-  const long long C = (long long)gridDim.x * (kBlock / 32);
-  const long long wid = ((long long)blockIdx.x * kBlock + threadIdx.x) / 32;
-  const int lane = threadIdx.x % 32;
-  long long u = wid * units / C;
-  const long long u1 = (wid + 1) * units / C;
-  const long long item = blockIdx.x * (long long)kBlock + threadIdx.x;
-  bool once = !A.balanced;
-  int nhll = 0;
-  for (;;) {
-    long long pen;
-    int fa, fb;
-    bool ok;
-    if (A.balanced) {
-      if (u >= u1) break;
-      const long long sg = u / len;          // slot x ngroups + group
-      slot = sg / ngroups;
-      const long long grp = sg - slot * ngroups;
-      const int off = (int)(u - sg * len);
-      const int take = (int)((len - off) < (u1 - u) ? (len - off) : (u1 - u));
-      pen = grp * 32 + lane;
-      fa = A.box.lo[D] + off;
-      fb = fa + take - 1;
-      ok = pen < npen;
-      u += take;
-    } else {
-      if (!once) break;
-      once = false;
-      const int seg = (int)(item / npen);
-      pen = item - seg * npen;
-      fa = A.box.lo[D] + seg * A.seg_len;
-      fb = fa + A.seg_len - 1;
-      if (fb > A.box.hi[D]) fb = A.box.hi[D];
-      ok = item < npen * A.nseg && fa <= fb;
-    }
-    if (ok)
-      nhll += wbu::sweep_segment<D, true, EZ, PROT>(A.geo, A.q, A.bn, A.F, slot * A.slot_in, slot * A.slot_out,
-                                                    A.box.lo[U] + (int)(pen % nu_), A.box.lo[W] + (int)(pen / nu_),
-                                                    fa, fb, dt, A.phys, rec);
-  }
-  if (nhll) atomicAdd((unsigned long long*)&A.scal->hll_faces, (unsigned long long)nhll);
-}
-
-template <int D, int EZ, bool PROT>
-int blocks_per_sm() {
-  static int cached = -1;
-  if (cached < 0) {
-    int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_sweep<D, EZ, PROT>, kBlock, 0) != cudaSuccess ||
-        nb < 1)
-      nb = 1;
-    cached = nb;
-  }
-  return cached;
-}
-
-int sm_count() {
-  static int cached = -1;
-  if (cached < 0) {
-    int dev = 0, n = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) n = 1;
-    cached = n;
-  }
-  return cached;
-}
-
-// Segments per pencil: balance waves of resident threads against the two
-// extra interfaces each segment recomputes.
-int choose_segments(long long pencils, int len, int resident) {
-  int best = 1;
-  double best_cost = 1e300;
-  for (int s = 1; s <= 16; ++s) {
-    int seg_len = (len + s - 1) / s;
-    if (seg_len < 4 && s > 1) break;
-    long long items = pencils * s;
-    long long waves = (items + resident - 1) / resident;
-    double cost = (double)waves * (seg_len + 2);
-    if (cost < best_cost * 0.999) { best_cost = cost; best = s; }
-  }
-  return best;
+  const long long t = blockIdx.x;
+  const int d = t >= A.tile0[2] ? 2 : (t >= A.tile0[1] ? 1 : 0);
+  const int hll = wbu::sweep_tile<EZ, PROT, true>(A.geo, A.box[d], d, A.s[d], t - A.tile0[d], A.ring[d] != 0, A.nslots,
+                                                  A.slot_in, A.slot_out, dt, A.phys, X);
+  if (hll) atomicAdd((unsigned long long*)&A.scal->hll_faces, 1ULL);
 }
 
 }  // namespace
 
-template <int D, int EZ, bool PROT>
-static void launch_sweep(SweepArgs a, int nslots, cudaStream_t s) {
-  constexpr int U = (D == 0) ? 1 : 0;
-  constexpr int W = (D == 2) ? 1 : 2;
-  long long npen = (long long)(a.box.hi[U] - a.box.lo[U] + 1) * (a.box.hi[W] - a.box.lo[W] + 1);
-  int len = a.box.hi[D] - a.box.lo[D] + 1;
-  int resident = blocks_per_sm<D, EZ, PROT>() * sm_count() * kBlock;
-  // big launches: equal runs of units per resident warp over every slot of
-  // the pass, so every warp finishes with the others (no partial last wave)
-  const long long units = (npen + 31) / 32 * (long long)len * nslots;
-  const long long warps = resident / 32;
-  if (a.nseg == 0 && units >= WB_BAL_MIN * warps) {
-    a.balanced = 1;
-    a.nslots = nslots;
-    k_sweep<D, EZ, PROT><<<dim3((unsigned)(resident / kBlock), 1), kBlock, 0, s>>>(a);
-    return;
-  }
-  a.balanced = 0;
-  int nseg = a.nseg > 0 ? a.nseg : choose_segments(npen * nslots, len, resident);
-  a.nseg = nseg;
-  a.seg_len = (len + nseg - 1) / nseg;
-  dim3 grid((unsigned)((npen * nseg + kBlock - 1) / kBlock), (unsigned)nslots);
-  k_sweep<D, EZ, PROT><<<grid, kBlock, 0, s>>>(a);
-}
-
-template <int EZ, bool PROT>
-static void launch_sweep_dir(int dir, const SweepArgs& a, int nslots, cudaStream_t s) {
-  if (dir == 0) launch_sweep<0, EZ, PROT>(a, nslots, s);
-  else if (dir == 1) launch_sweep<1, EZ, PROT>(a, nslots, s);
-  else launch_sweep<2, EZ, PROT>(a, nslots, s);
-}
-
 // Kernel variants: eps_k = 0 on the linearly degenerate waves (the default)
 // or general eps; protection floors off (the default) or on.
-void wb_launch_sweep(int dir, const SweepArgs& a, int nslots, cudaStream_t s) {
+void wb_launch_sweeps(SweepArgs a, int closed, cudaStream_t s) {
+  a.tile0[0] = 0;
+  for (int d = 0; d < 3; ++d) {
+    const int U = d == 0 ? 1 : 0, W = d == 2 ? 1 : 2;
+    const WbBox& b = a.box[d];
+    const int len = b.hi[d] - b.lo[d] + 1;
+    a.ring[d] = wbu::sweep_ring(len, (closed >> d) & 1);
+    a.tile0[d + 1] = a.tile0[d] + wbu::sweep_tiles((long long)(b.hi[U] - b.lo[U] + 1) * (b.hi[W] - b.lo[W] + 1) * a.nslots,
+                                                   len, a.ring[d] != 0);
+  }
+  const dim3 grid((unsigned)a.tile0[3]);
   const bool ez = (a.phys.eps_zero & kEpsZeroLD) == kEpsZeroLD;
   if (a.phys.prot) {
-    if (ez) launch_sweep_dir<kEpsZeroLD, true>(dir, a, nslots, s);
-    else launch_sweep_dir<0, true>(dir, a, nslots, s);
+    if (ez) k_sweep<kEpsZeroLD, true><<<grid, wbu::kBlock, 0, s>>>(a);
+    else k_sweep<0, true><<<grid, wbu::kBlock, 0, s>>>(a);
   } else {
-    if (ez) launch_sweep_dir<kEpsZeroLD, false>(dir, a, nslots, s);
-    else launch_sweep_dir<0, false>(dir, a, nslots, s);
+    if (ez) k_sweep<kEpsZeroLD, false><<<grid, wbu::kBlock, 0, s>>>(a);
+    else k_sweep<0, false><<<grid, wbu::kBlock, 0, s>>>(a);
   }
 }
 

@@ -25,7 +25,12 @@ struct WbView {
 namespace wbu {
 
 // ---------------------------------------------------------------- sweep ----
-constexpr int kBlock = 64;
+constexpr int kWarps = 4;             // warps of a sweep block
+constexpr int kBlock = 32 * kWarps;
+constexpr int kTile = kBlock - 3;     // faces a block emits from its kBlock zones
+// resident blocks per SM the sweep kernels are compiled for: 168 registers a
+// thread, 12 warps per SM
+constexpr int kSweepBlocks = 3;
 
 // waves 2, 4, 6 (Alfven, entropy, Alfven) have eps = 0 (the default eps_k):
 // the mask of the sweep specialisation that drops their Q-branch arithmetic
@@ -54,27 +59,27 @@ __device__ __forceinline__ double ld(const double* p) {
 // (no contraction left to the compiler): a zone is loaded both before and
 // inside the march over a segment, and the two inlined copies must round
 // identically, or a face's flux would depend on where a segment starts.
-template <int D, bool NC>
-__device__ __forceinline__ void load_cell(const double* const* q, long long off, const WbPhys& P,
-                                          Cell& c) {
-  constexpr int T1 = (D + 1) % 3, T2 = (D + 2) % 3;
-  c.rho = ld<NC>(q[F_RHO] + off);
-  c.mn = ld<NC>(q[F_MX + D] + off);
-  c.mt1 = ld<NC>(q[F_MX + T1] + off);
-  c.mt2 = ld<NC>(q[F_MX + T2] + off);
-  const double e = ld<NC>(q[F_EN] + off);
-  const double bn = ld<NC>(q[F_BX + D] + off);
-  c.bt1 = ld<NC>(q[F_BX + T1] + off);
-  c.bt2 = ld<NC>(q[F_BX + T2] + off);
+// q: the fields in the sweep's frame (rho, Mn, Mt1, Mt2, E, Bn, Bt1, Bt2).
+template <bool NC>
+__device__ __forceinline__ void load_cell(const double* const (&q)[8], long long off, const WbPhys& P,
+                                                Cell& c) {
+  c.rho = ld<NC>(q[0] + off);
+  c.mn = ld<NC>(q[1] + off);
+  c.mt1 = ld<NC>(q[2] + off);
+  c.mt2 = ld<NC>(q[3] + off);
+  const double e = ld<NC>(q[4] + off);
+  const double bn = ld<NC>(q[5] + off);
+  c.bt1 = ld<NC>(q[6] + off);
+  c.bt2 = ld<NC>(q[7] + off);
   const WbRoots rr = wb_roots(c.rho);
   c.sr = rr.sq;
   c.ir = rr.rcp;
-  c.vn = __dmul_rn(c.mn, c.ir);
-  c.vt1 = __dmul_rn(c.mt1, c.ir);
-  c.vt2 = __dmul_rn(c.mt2, c.ir);
-  const double ke = wb_half(__fma_rn(c.mt2, c.vt2, __fma_rn(c.mt1, c.vt1, __dmul_rn(c.mn, c.vn))));
-  const double bt2 = __fma_rn(c.bt2, c.bt2, __dmul_rn(c.bt1, c.bt1));
-  const double bn2 = __dmul_rn(bn, bn);
+  c.vn = wb_smul(c.mn, c.ir);
+  c.vt1 = wb_smul(c.mt1, c.ir);
+  c.vt2 = wb_smul(c.mt2, c.ir);
+  const double hbn = wb_half(bn), bn2 = wb_smul(bn, bn);
+  const double ke = wb_half(__fma_rn(c.mt2, c.vt2, __fma_rn(c.mt1, c.vt1, wb_smul(c.mn, c.vn))));
+  const double bt2 = __fma_rn(c.bt2, c.bt2, wb_smul(c.bt1, c.bt1));
   const double me = wb_half(__dadd_rn(bn2, bt2));
   const double p = __dmul_rn(P.gm1, __dsub_rn(__dsub_rn(e, ke), me));
   const double pstar = __dadd_rn(p, me);
@@ -83,34 +88,31 @@ __device__ __forceinline__ void load_cell(const double* const* q, long long off,
   // rho h = gamma/(gamma-1) P + rho v^2/2 + |B_t|^2 = (E + P*) - B_n^2
   c.hr = __dmul_rn(__dsub_rn(ep, bn2), c.ir);
   // half fluxes: the face needs (F_L + F_R) / 2
-  const double hmn = wb_half(c.mn), hvn = wb_half(c.vn), hbn = wb_half(bn);
+  const double hmn = wb_half(c.mn), hvn = wb_half(c.vn);
   c.F[0] = hmn;
   c.F[1] = __fma_rn(hmn, c.vn, wb_half(__dsub_rn(pstar, bn2)));
-  c.F[2] = __fma_rn(hmn, c.vt1, __dmul_rn(-hbn, c.bt1));
-  c.F[3] = __fma_rn(hmn, c.vt2, __dmul_rn(-hbn, c.bt2));
-  c.F[4] = __fma_rn(c.bt1, hvn, __dmul_rn(-hbn, c.vt1));
-  c.F[5] = __fma_rn(c.bt2, hvn, __dmul_rn(-hbn, c.vt2));
-  const double bv = __fma_rn(c.bt2, c.vt2, __fma_rn(c.bt1, c.vt1, __dmul_rn(bn, c.vn)));
+  c.F[2] = __fma_rn(hmn, c.vt1, -wb_smul(c.bt1, hbn));
+  c.F[3] = __fma_rn(hmn, c.vt2, -wb_smul(c.bt2, hbn));
+  c.F[4] = __fma_rn(c.bt1, hvn, -wb_smul(c.vt1, hbn));
+  c.F[5] = __fma_rn(c.bt2, hvn, -wb_smul(c.vt2, hbn));
+  const double bv = __fma_rn(c.bt2, c.vt2, __fma_rn(c.bt1, c.vt1, wb_smul(bn, c.vn)));
   c.F[6] = __fma_rn(ep, hvn, __dmul_rn(-hbn, bv));
 }
 
-// Per-face record (shared memory, structure of arrays over the block).
+// Per-face record.
 // R_PG = rho a^2 / (gamma-1); R_KX = (gamma-2)/(gamma-1) X - v^2/2 (= K - v^2 for the
 // K = v^2/2 + (gamma-2)/(gamma-1) X of the energy row);
 // R_AFCF = alpha_f c_f, R_ASCS = alpha_s c_s.
 enum {
-  R_AL = 0, R_NU = 7, R_RHO = 14, R_SRHO, R_A, R_PG, R_CF, R_ASCS, R_AFCF, R_AF, R_AS, R_B1, R_B2, R_S,
+  R_AL = 0, R_NU = 7, R_RHO = 14, R_SRHO, R_A, R_PG, R_CF, R_ASCS, R_AFCF, R_AF, R_AS, R_B1, R_B2,
   R_VN, R_VT1, R_VT2, R_BTM, R_KX, R_FAVG, R_WORDS = R_FAVG + 7
 };
 
-// One thread's face record in shared memory, word w at p[w * BS] (the block's
-// records interleaved, BS = threads per block).
-template <int BS>
-struct RecT {
-  double* p;
-  __device__ __forceinline__ double& operator[](int w) const { return p[w * BS]; }
+// A face record in registers (every index a constant after unrolling).
+struct RegRec {
+  mutable double w[R_WORDS];
+  __device__ __forceinline__ double& operator[](int i) const { return w[i]; }
 };
-using Rec = RecT<kBlock>;
 
 // The flux arithmetic below is written with explicit rounding: every product
 // that feeds a sum is one fused multiply-add (__fma_rn), every other operation
@@ -132,7 +134,7 @@ __device__ __forceinline__ double Qk_m_nu2(double nu, int k, const WbPhys& P) {
   // one FMA of operands chosen on the integer pipe, FMA(x, nu, y) with (x, y) = (-nu, |nu|)
   // or (nu (1/(4 eps) - 1), eps), so that no warp issues both forms
   const bool band = wb_abs_less(nu, P.two_eps[k]);
-  const double x = band ? WB_MUL(nu, P.inv4eps_m1[k]) : wb_flip(nu);
+  const double x = band ? wb_smul(nu, P.inv4eps_m1[k]) : wb_flip(nu);
   return WB_FMA(x, nu, band ? P.eps[k] : wb_fabs(nu));
 }
 
@@ -220,26 +222,25 @@ template <int EZ, bool PROT, class Rc>
 __device__ __forceinline__ int face_system(const Cell& L, const Cell& R, double b, double dtdx,
                                            const WbPhys& P, const Rc& f, double gt[7]) {
   const double iD = wb_rcp(WB_ADD(L.sr, R.sr));
-  const double wL = WB_MUL(L.sr, iD), wR = WB_MUL(R.sr, iD);
-  const double rho = WB_MUL(L.sr, R.sr);
+  const double wL = wb_smul(L.sr, iD), wR = wb_smul(R.sr, iD);
+  const double rho = wb_smul(L.sr, R.sr);
   const WbRoots rroe = wb_roots(rho);
-  const double irho = rroe.rcp;
-  const double isrho = rroe.rsq, srho = rroe.sq;
-  const double vn = WB_FMA(wL, L.vn, WB_MUL(wR, R.vn));
-  const double vt1 = WB_FMA(wL, L.vt1, WB_MUL(wR, R.vt1));
-  const double vt2 = WB_FMA(wL, L.vt2, WB_MUL(wR, R.vt2));
-  const double bt1 = WB_FMA(wR, L.bt1, WB_MUL(wL, R.bt1));
-  const double bt2 = WB_FMA(wR, L.bt2, WB_MUL(wL, R.bt2));
-  const double b2 = WB_MUL(b, b);
+  const double irho = rroe.rcp, isrho = rroe.rsq, srho = rroe.sq;
+  const double vn = WB_FMA(wL, L.vn, wb_smul(R.vn, wR));
+  const double vt1 = WB_FMA(wL, L.vt1, wb_smul(R.vt1, wR));
+  const double vt2 = WB_FMA(wL, L.vt2, wb_smul(R.vt2, wR));
+  const double bt1 = WB_FMA(wR, L.bt1, wb_smul(R.bt1, wL));
+  const double bt2 = WB_FMA(wR, L.bt2, wb_smul(R.bt2, wL));
+  const double b2 = wb_smul(b, b);
   // H = wL (h_L + b^2)/rho_L + wR (h_R + b^2)/rho_R, with wL/rho_L + wR/rho_R = 1/rho_
-  const double H = WB_FMA(b2, irho, WB_FMA(wL, L.hr, WB_MUL(wR, R.hr)));
+  const double H = WB_FMA(b2, irho, WB_FMA(wL, L.hr, wb_smul(R.hr, wR)));
   const double dbt1 = WB_SUB(R.bt1, L.bt1), dbt2 = WB_SUB(R.bt2, L.bt2);
-  const double gX = WB_MUL(P.hgm2, WB_MUL(WB_FMA(dbt1, dbt1, WB_MUL(dbt2, dbt2)), WB_MUL(iD, iD)));  // (gamma-2) X
-  const double hv2 = wb_half(WB_FMA(vn, vn, WB_FMA(vt1, vt1, WB_MUL(vt2, vt2))));
-  const double bt2s = WB_FMA(bt1, bt1, WB_MUL(bt2, bt2));
+  const double gX = WB_MUL(P.hgm2, WB_MUL(WB_FMA(dbt1, dbt1, wb_smul(dbt2, dbt2)), wb_smul(iD, iD)));  // (gamma-2) X
+  const double hv2 = wb_half(WB_FMA(vn, vn, WB_FMA(vt1, vt1, wb_smul(vt2, vt2))));
+  const double bt2s = WB_FMA(bt1, bt1, wb_smul(bt2, bt2));
   const double a2 = WB_FMA(P.gm1, WB_FMA(-WB_ADD(b2, bt2s), irho, WB_SUB(H, hv2)), -gX);
   if (!wb_normal_pos(a2)) return 2;
-  const double ca2 = WB_MUL(b2, irho), ct2 = WB_MUL(bt2s, irho);
+  const double ca2 = wb_smul(b2, irho), ct2 = wb_smul(bt2s, irho);
   const double dac = WB_SUB(a2, ca2);
   const double disc = WB_FMA(dac, dac, WB_MUL(ct2, WB_FMA(2.0, WB_ADD(a2, ca2), ct2)));
   const double sum = WB_ADD(WB_ADD(a2, ca2), ct2);
@@ -247,50 +248,43 @@ __device__ __forceinline__ int face_system(const Cell& L, const Cell& R, double 
   const double sd = wb_normal_pos(disc) ? wb_sqrt(disc) : 0.0;
   const double cf2 = wb_half(WB_ADD(sum, sd));
   const WbRoots rcf = wb_roots(cf2), ra_ = wb_roots(a2);
-  const double icf = rcf.rsq, ia = ra_.rsq;
+  const double icf = rcf.rsq, ia = ra_.rsq, ia2 = ra_.rcp;
   const double cf = rcf.sq, a = ra_.sq;
-  const double ca = WB_MUL(wb_fabs(b), isrho);
-  const double cs = WB_MUL(WB_MUL(a, ca), icf);  // c_f c_s = a c_a
+  const double ca = wb_smul(wb_fabs(b), isrho);
+  const double cs = wb_smul(wb_smul(a, ca), icf);  // c_f c_s = a c_a
   // 1/|B_t| and c_t = |B_t| / sqrt(rho_); a transverse field whose square is
   // not a normal double (underflowing noise ahead of a front) counts as 0
-  double ib = 0.0, ct = 0.0, btm = 0.0;  // btm = |B_t|
+  double ib = 0.0, btm = 0.0;  // btm = |B_t|
   if (wb_normal_pos(bt2s)) {
     const WbRoots rb = wb_roots(bt2s);
     ib = rb.rsq;
     btm = rb.sq;
-    ct = WB_MUL(btm, isrho);
   }
-  double af, as;
-  if (wb_le_nonneg(sd, WB_MUL(1e-12, sum))) {
+  // With t1 = ca^2 + ct^2 - a^2: alpha_f^2 = (sd - t1) / (2 sd) and
+  // alpha_s^2 = (sd + t1) / (2 sd) (cf^2 + cs^2 = a^2 + ca^2 + ct^2,
+  // cf^2 - cs^2 = sd), and (sd - t1)(sd + t1) = disc - t1^2 = 4 a^2 ct^2,
+  // so alpha_f alpha_s = a ct / sd.  The larger of the two is sqrt(m / (2 sd))
+  // with m = sd + |t1| (no cancellation), = m r for r = 1/sqrt(2 sd m), and
+  // the smaller a ct / (sd m r) = 2 a ct r: one reciprocal square root.
+  // t1 takes the difference ca^2 - a^2 first: it is exact where the two
+  // nearly cancel (the degenerate neighbourhood, where sd is small).
+  const double t1 = WB_ADD(WB_SUB(ca2, a2), ct2);
+  const bool slow_major = !wb_neg(t1);
+  const double m = WB_ADD(sd, slow_major ? t1 : wb_flip(t1));
+  const double r = wb_rsqrt(wb_twice(wb_smul(sd, m)));
+  const double major = wb_smul(m, r);
+  const double minor = WB_MUL(wb_smul(a, wb_smul(btm, isrho)), wb_twice(r));
+  double af = slow_major ? minor : major;
+  double as = slow_major ? major : minor;
+  if (wb_hi_scaled(sd, 39) <= wb_hi32(sum) && wb_at_most(sd, 1e-12, sum)) {
     const bool fast = wb_le_nonneg(ca2, a2);
     af = fast ? 1.0 : 0.0;
     as = fast ? 0.0 : 1.0;
-  } else {
-    // With t1 = ca^2 + ct^2 - a^2: alpha_f^2 = (sd - t1) / (2 sd) and
-    // alpha_s^2 = (sd + t1) / (2 sd) (cf^2 + cs^2 = a^2 + ca^2 + ct^2,
-    // cf^2 - cs^2 = sd), and (sd - t1)(sd + t1) = disc - t1^2 = 4 a^2 ct^2,
-    // so alpha_f alpha_s = a ct / sd.  The larger of the two is sqrt(m / (2 sd))
-    // with m = sd + |t1| (no cancellation), = m r for r = 1/sqrt(2 sd m), and
-    // the smaller a ct / (sd m r) = 2 a ct r: one reciprocal square root.
-    // t1 takes the difference ca^2 - a^2 first: it is exact where the two
-    // nearly cancel (the degenerate neighbourhood, where sd is small).
-    const double t1 = WB_ADD(WB_SUB(ca2, a2), ct2);
-    const bool slow_major = !wb_neg(t1);
-    const double m = WB_ADD(sd, slow_major ? t1 : wb_flip(t1));
-    const double r = wb_rsqrt(wb_twice(WB_MUL(sd, m)));
-    const double major = WB_MUL(m, r);
-    const double minor = WB_MUL(WB_MUL(a, ct), wb_twice(r));
-    af = slow_major ? minor : major;
-    as = slow_major ? major : minor;
   }
-  const double ra2 = WB_MUL(rho, a2);
-  double b1n, b2n;
-  if (wb_le_nonneg(bt2s, WB_MUL(1e-24, WB_ADD(WB_ADD(ra2, b2), bt2s)))) {
+  const double ra2 = wb_smul(rho, a2);
+  double b1n = wb_smul(bt1, ib), b2n = wb_smul(bt2, ib);
+  if (wb_maybe_small(bt2s, ra2, b2) && wb_at_most(bt2s, 1e-24, WB_ADD(WB_ADD(ra2, b2), bt2s)))
     b1n = b2n = 0.70710678118654752440;
-  } else {
-    b1n = WB_MUL(bt1, ib);
-    b2n = WB_MUL(bt2, ib);
-  }
   const double S = wb_sgn(b);
   // primitive differences of the 7-variable system; the velocity differences
   // are kept times rho_ (dv' = rho_ dv), the 1/rho_ goes into the coefficients
@@ -300,28 +294,27 @@ __device__ __forceinline__ int face_system(const Cell& L, const Cell& R, double 
   const double dvn = WB_FMA(-vn, drho, dmn);
   const double dvt1 = WB_FMA(-vt1, drho, dmt1);
   const double dvt2 = WB_FMA(-vt2, drho, dmt2);
-  const double vdm = WB_FMA(vn, dmn, WB_FMA(vt1, dmt1, WB_MUL(vt2, dmt2)));
-  const double bdb = WB_FMA(bt1, dbt1, WB_MUL(bt2, dbt2));
+  const double vdm = WB_FMA(vn, dmn, WB_FMA(vt1, dmt1, wb_smul(vt2, dmt2)));
+  const double bdb = WB_FMA(bt1, dbt1, wb_smul(bt2, dbt2));
   const double dp = WB_FMA(-gX, drho, WB_MUL(P.gm1, WB_SUB(WB_FMA(hv2, drho, WB_SUB(de, vdm)), bdb)));
   // projections on the transverse field direction beta and its normal; S = sign(b)
-  const double dvbS = wb_xsgn(WB_FMA(b1n, dvt1, WB_MUL(b2n, dvt2)), S);
-  const double dvp = WB_FMA(-b2n, dvt1, WB_MUL(b1n, dvt2));
-  const double dbb = WB_FMA(b1n, dbt1, WB_MUL(b2n, dbt2));
-  const double dbpS = wb_xsgn(WB_FMA(-b2n, dbt1, WB_MUL(b1n, dbt2)), S);
-  const double ia2 = ra_.rcp;
+  const double dvbS = wb_xsgn(WB_FMA(b1n, dvt1, wb_smul(dvt2, b2n)), S);
+  const double dvp = WB_FMA(-b2n, dvt1, wb_smul(dvt2, b1n));
+  const double dbb = WB_FMA(b1n, dbt1, wb_smul(dbt2, b2n));
+  const double dbpS = wb_xsgn(WB_FMA(-b2n, dbt1, wb_smul(dbt2, b1n)), S);
   const double hir = wb_half(irho), hisr = wb_half(isrho);
-  const double i2ra = WB_MUL(hisr, ia);   // 1 / (2 sqrt(rho) a)
-  const double ri2a2 = WB_MUL(hir, ia2);  // 1 / (2 rho a^2)
-  const double dpr = WB_MUL(dp, ri2a2);
-  const double afcf = WB_MUL(af, cf), ascs = WB_MUL(as, cs);
-  const double dbbi = WB_MUL(dbb, i2ra);
+  const double i2ra = wb_smul(hisr, ia);   // 1 / (2 sqrt(rho) a)
+  const double ri2a2 = wb_smul(hir, ia2);  // 1 / (2 rho a^2)
+  const double dpr = wb_smul(dp, ri2a2);
+  const double afcf = wb_smul(af, cf), ascs = wb_smul(as, cs);
+  const double dbbi = wb_smul(dbb, i2ra);
   // alpha_{1,7} = Cf -+ Xf / (2 rho a^2), alpha_{3,5} = Cs -+ Xs / (2 rho a^2): the factor
   // goes into the FMAs that form them
-  const double Xf = WB_FMA(afcf, dvn, -WB_MUL(ascs, dvbS));
-  const double Cf = WB_FMA(as, dbbi, WB_MUL(af, dpr));
-  const double Xs = WB_FMA(ascs, dvn, WB_MUL(afcf, dvbS));
-  const double Cs = WB_FMA(-af, dbbi, WB_MUL(as, dpr));
-  const double hAa = WB_MUL(hisr, dbpS);
+  const double Xf = WB_FMA(afcf, dvn, -wb_smul(dvbS, ascs));
+  const double Cf = WB_FMA(as, dbbi, wb_smul(af, dpr));
+  const double Xs = WB_FMA(ascs, dvn, wb_smul(dvbS, afcf));
+  const double Cs = WB_FMA(-af, dbbi, wb_smul(as, dpr));
+  const double hAa = wb_smul(hisr, dbpS);
   double al[7];
   al[0] = WB_FMA(-ri2a2, Xf, Cf);
   al[6] = WB_FMA(ri2a2, Xf, Cf);
@@ -331,7 +324,7 @@ __device__ __forceinline__ int face_system(const Cell& L, const Cell& R, double 
   al[5] = WB_FMA(hir, dvp, -hAa);
   al[3] = WB_FMA(-dp, ia2, drho);
   // nu_k = (dt/dx) a_k for the eigenvalues a_1..a_7 (Sec. 3)
-  const double tvn = WB_MUL(dtdx, vn);
+  const double tvn = wb_smul(vn, dtdx);
   const double nuk[7] = {WB_FMA(-dtdx, cf, tvn), WB_FMA(-dtdx, ca, tvn), WB_FMA(-dtdx, cs, tvn), tvn,
                          WB_FMA(dtdx, cs, tvn),  WB_FMA(dtdx, ca, tvn),  WB_FMA(dtdx, cf, tvn)};
 #pragma unroll
@@ -339,10 +332,10 @@ __device__ __forceinline__ int face_system(const Cell& L, const Cell& R, double 
     const double nu = nuk[k];
     f[R_AL + k] = al[k];
     f[R_NU + k] = nu;
-    gt[k] = WB_MUL(Qk_m_nu2<EZ>(nu, k, P), al[k]);  // 2 g-tilde
+    gt[k] = wb_smul(Qk_m_nu2<EZ>(nu, k, P), al[k]);  // 2 g-tilde
   }
-  f[R_RHO] = rho; f[R_SRHO] = srho; f[R_A] = a; f[R_PG] = WB_MUL(ra2, P.inv_gm1); f[R_CF] = cf;
-  f[R_ASCS] = ascs; f[R_AFCF] = afcf; f[R_AF] = af; f[R_AS] = as; f[R_B1] = b1n; f[R_B2] = b2n; f[R_S] = S;
+  f[R_RHO] = rho; f[R_SRHO] = wb_xsgn(srho, S); f[R_A] = a; f[R_PG] = wb_smul(ra2, P.inv_gm1); f[R_CF] = cf;
+  f[R_ASCS] = ascs; f[R_AFCF] = afcf; f[R_AF] = af; f[R_AS] = as; f[R_B1] = b1n; f[R_B2] = b2n;
   f[R_VN] = vn; f[R_VT1] = vt1; f[R_VT2] = vt2; f[R_BTM] = btm;
   f[R_KX] = WB_FMA(gX, P.inv_gm1, -hv2);  // K - v^2 (the energy row of face_flux)
 #pragma unroll
@@ -370,7 +363,7 @@ __device__ __forceinline__ double beta_k(double al, double nu, double Gi, double
     return (wb_order_less(b1, b2) != wb_neg(al)) ? b2 : b1;
   }
   const double d = WB_FMA(wb_twice(nu), al, WB_SUB(Gi1, Gi));  // 2 w
-  if (!wb_abs_less(d, WB_MUL(P.four_eps[k], al))) {
+  if (!wb_abs_less(d, wb_smul(al, P.four_eps[k]))) {
     const bool same = (__double_as_longlong(d) ^ __double_as_longlong(al)) >= 0;
     return WB_FMA(same ? nu : wb_flip(nu), al, -(same ? Gi : Gi1));
   }
@@ -388,26 +381,25 @@ __device__ __forceinline__ void face_flux(const Rc& f, const double gi[7], const
 #pragma unroll
   for (int k = 0; k < 7; ++k) be[k] = beta_k<EZ>(f[R_AL + k], f[R_NU + k], gi[k], gi1[k], k, P);
   const double rho = f[R_RHO], af = f[R_AF], as = f[R_AS];
-  const double S = f[R_S], b1 = f[R_B1], b2 = f[R_B2];
+  const double S = f[R_SRHO], b1 = f[R_B1], b2 = f[R_B2];  // S: sign(b) sqrt(rho_)
   // sum_k beta_k r_k in w = (rho, vn, vt, Bt, p)
   const double sf = WB_ADD(be[0], be[6]), df = WB_SUB(be[6], be[0]);
   const double ss = WB_ADD(be[2], be[4]), ds = WB_SUB(be[4], be[2]);
-  const double tfs = WB_FMA(af, sf, WB_MUL(as, ss));
-  const double wr = WB_FMA(rho, tfs, be[3]);
-  const double afcf = f[R_AFCF], ascs = f[R_ASCS];
-  const double wvn = WB_FMA(afcf, df, WB_MUL(ascs, ds));
-  const double vb = wb_xsgn(WB_FMA(afcf, ds, -WB_MUL(ascs, df)), S);  // along beta
+  const double afcf = f[R_AFCF], ascs = f[R_ASCS], srho = wb_fabs(S);
   const double vp = WB_ADD(be[1], be[5]);                             // along beta-perp
-  const double ra = WB_MUL(f[R_SRHO], f[R_A]);
-  const double bb = WB_MUL(ra, WB_FMA(as, sf, -WB_MUL(af, ss)));
-  const double bp = wb_xsgn(WB_MUL(f[R_SRHO], WB_SUB(be[1], be[5])), S);
-  const double wvt1 = WB_FMA(b1, vb, -WB_MUL(b2, vp)), wvt2 = WB_FMA(b2, vb, WB_MUL(b1, vp));
-  const double wbt1 = WB_FMA(b1, bb, -WB_MUL(b2, bp)), wbt2 = WB_FMA(b2, bb, WB_MUL(b1, bp));
+  const double tfs = WB_FMA(af, sf, wb_smul(ss, as));
+  const double wr = WB_FMA(rho, tfs, be[3]);
+  const double wvn = WB_FMA(afcf, df, wb_smul(ds, ascs));
+  const double vb = wb_xsgn(WB_FMA(afcf, ds, -wb_smul(df, ascs)), S);  // along beta
+  const double bb = wb_smul(WB_FMA(as, sf, -wb_smul(ss, af)), wb_smul(f[R_A], srho));
+  const double bp = wb_xsgn(wb_smul(WB_SUB(be[1], be[5]), srho), S);
+  const double wvt1 = WB_FMA(b1, vb, -wb_smul(vp, b2)), wvt2 = WB_FMA(b2, vb, wb_smul(vp, b1));
+  const double wbt1 = WB_FMA(b1, bb, -wb_smul(bp, b2)), wbt2 = WB_FMA(b2, bb, wb_smul(bp, b1));
   // to conserved variables (the pressure row enters the energy as p/(gamma-1))
   const double vn = f[R_VN], vt1 = f[R_VT1], vt2 = f[R_VT2];
-  const double u1 = WB_FMA(vn, wr, WB_MUL(rho, wvn));
-  const double u2 = WB_FMA(vt1, wr, WB_MUL(rho, wvt1));
-  const double u3 = WB_FMA(vt2, wr, WB_MUL(rho, wvt2));
+  const double u1 = WB_FMA(vn, wr, wb_smul(wvn, rho));
+  const double u2 = WB_FMA(vt1, wr, wb_smul(wvt1, rho));
+  const double u3 = WB_FMA(vt2, wr, wb_smul(wvt2, rho));
   // energy: B_t . w_Bt + p/(gamma-1) row + K w_rho + rho v . w_v, with
   // rho v . w_v = v . u - v^2 w_rho and the record holding K - v^2, and
   // B_t . w_Bt = |B_t| w_beta: beta is B_t / |B_t|, so the beta-perpendicular
@@ -425,93 +417,207 @@ __device__ __forceinline__ void face_flux(const Rc& f, const double gi[7], const
   out[6] = WB_FMA(-dx_2dt, u6, f[R_FAVG + 6]);
 }
 
-// One pencil segment of an MHDTVD sweep along D: fluxes of faces [fa, fb]
-// at transverse position (pos[U], pos[W]) of the input fields q (zone B),
-// normal face field bn; outputs F.  qo / wo: slot offsets of the input and
-// output arrays.  rec: two shared-memory face records of this thread.
-// Faces without a Roe state or below the protection floor take the HLL flux
-// and give g-tilde = 0 to the limiters of their neighbours.  Returns the
-// number of HLL faces among [fa, fb] that are interior faces of the box.
-template <int D, bool NC, int EZ = 0, bool PROT = true, class Rc = Rec>
-__device__ __forceinline__ int sweep_segment(const WbGeo& g, const double* const* q,
-                                             const double* bn, double* const* F, long long qo,
-                                             long long wo, int pu, int pw, int fa, int fb,
-                                             double dt, const WbPhys& P, const Rc rec[2]) {
+// What a face needs of its left zone, word by word.
+constexpr int kCellWords = 19;
+__device__ __forceinline__ double& cell_word(Cell& c, int i) {
+  switch (i) {
+    case 0: return c.rho;
+    case 1: return c.sr;
+    case 2: return c.vn;
+    case 3: return c.vt1;
+    case 4: return c.vt2;
+    case 5: return c.bt1;
+    case 6: return c.bt2;
+    case 7: return c.eref;
+    case 8: return c.hr;
+    case 9: return c.mn;
+    case 10: return c.mt1;
+    case 11: return c.mt2;
+    default: return c.F[i - 12];
+  }
+}
+
+// The words that cross from one warp of a block to the next.
+struct LaneEdge {
+  double cell[kWarps][kCellWords];                // zone of lane 31
+  double gt0[kWarps][7], gz31[kWarps][7];         // g-tilde of lane 0, limited slope of lane 31
+};
+
+// A sweep along one axis: fields in the sweep's frame (q: rho, Mn, Mt1, Mt2,
+// E, Bn, Bt1, Bt2; F: rho, Mn, Mt1, Mt2, Bt1, Bt2, E), faces of `box` along
+// axis d, zones of it across.
+struct SweepFrame {
+  const double* q[8];
+  const double* bn;
+  double* F[7];
+};
+template <int D>
+__host__ __device__ __forceinline__ void sweep_frame(const double* const* q, const double* bn, double* const* F,
+                                                     SweepFrame& f) {
   constexpr int T1 = (D + 1) % 3, T2 = (D + 2) % 3;
-  constexpr int U = (D == 0) ? 1 : 0;
-  constexpr int W = (D == 2) ? 1 : 2;
+  f.q[0] = q[F_RHO];
+  f.q[1] = q[F_MX + D];
+  f.q[2] = q[F_MX + T1];
+  f.q[3] = q[F_MX + T2];
+  f.q[4] = q[F_EN];
+  f.q[5] = q[F_BX + D];
+  f.q[6] = q[F_BX + T1];
+  f.q[7] = q[F_BX + T2];
+  f.bn = bn;
+  f.F[0] = F[F_RHO];
+  f.F[1] = F[F_MX + D];
+  f.F[2] = F[F_MX + T1];
+  f.F[3] = F[F_MX + T2];
+  f.F[4] = F[F_BX + T1];
+  f.F[5] = F[F_BX + T2];
+  f.F[6] = F[F_EN];
+}
+
+// How the faces of a sweep are laid out over threads.  In the open layout
+// every pencil of len faces is a run of len + 3 zones (two before its first
+// face's right zone, one after its last), the runs follow one another, and a
+// block takes kBlock zones of them, emits the faces that find both neighbours'
+// slopes in the block and advances by kTile: kTile / kBlock x len / (len + 3)
+// of the threads emit a face.  A closed pencil (periodic, its first and last
+// zone neighbours) of at most 32 zones can sit in a warp as a ring instead:
+// floor(32 / len) len of the 32 lanes emit.  The better of the two is taken
+// (16 and 32 zones: all lanes against 82 and 89 %; 24: 75 against 87 %).
+__host__ __device__ __forceinline__ bool sweep_ring(int len, bool closed) {
+  return closed && len <= 32 && (32 / len) * len * (len + 3) * kBlock >= 32 * len * kTile;
+}
+// tiles (blocks' worth of work) of npen pencils
+__host__ __device__ __forceinline__ long long sweep_tiles(long long npen, int len, bool ring) {
+  const long long per = ring ? (long long)(32 / len) * kWarps : kTile;
+  const long long n = ring ? npen : npen * (len + 3) - 3;
+  return (n + per - 1) / per;
+}
+
+// One tile of a sweep, one face per thread: the thread holds a zone and its low
+// face; its neighbours along the pencil hand over zone state, g-tilde and
+// limited slopes by shuffles and, at the ends of a warp, through shared memory
+// (X).  Every thread of the block calls this.  Faces without a Roe state or
+// below the protection floor take the HLL flux and give g-tilde = 0 to the
+// limiters of their neighbours.  Returns 1 when the thread's stored flux is an
+// HLL flux of an interior face of the box (ghost rings, which depend on how a
+// box is split, are not counted).
+//
+// What bounds it: the FP64 pipe (one warp instruction per 19 cycles and SM) and
+// beside it the latency of the integer work that takes FP64 work over (wb_soft).
+// A thread that marched along a pencil kept two zones, two slopes and a face
+// record in 226 to 255 registers and 40 KB of shared memory a block, which left
+// 2 warps per scheduler; one face per thread needs 168, 3 warps.
+template <int EZ, bool PROT, bool NC>
+__device__ __forceinline__ int sweep_tile(const WbGeo& g, const WbBox& box, int d, const SweepFrame& s, long long tile,
+                                          bool ring, int nslots, long long slot_in, long long slot_out, double dt,
+                                          const WbPhys& P, LaneEdge& X) {
+  const int U = d == 0 ? 1 : 0, W = d == 2 ? 1 : 2;
+  const int nu = box.hi[U] - box.lo[U] + 1, nw = box.hi[W] - box.lo[W] + 1;
+  const int len = box.hi[d] - box.lo[d] + 1;
+  const long long npen = (long long)nu * nw * nslots;
+  const int t = threadIdx.x, lane = t % 32, wp = t / 32;
+  long long pen;
+  int idx, left, right;  // zone along the pencil; neighbour lanes
+  bool has_left, emit;
+  if (ring) {
+    const int per = 32 / len, seg = lane / len;
+    idx = lane - seg * len;
+    pen = (tile * kWarps + wp) * per + seg;
+    emit = seg < per && pen < npen;
+    if (pen >= npen) pen = npen - 1;
+    has_left = true;
+    left = idx > 0 ? lane - 1 : lane + len - 1;
+    right = idx < len - 1 ? lane + 1 : lane - len + 1;
+    if (seg >= per) left = right = lane;
+  } else {
+    const long long total = npen * (len + 3);
+    long long z = tile * kTile + t;
+    emit = z < total;
+    if (z >= total) z = total - 1;
+    pen = z / (len + 3);
+    idx = (int)(z - pen * (len + 3)) - 2;
+    has_left = idx > -2 && t > 0;
+    emit = emit && idx >= 0 && idx < len && t >= 2 && t <= kBlock - 2;
+    left = (lane + 31) % 32;
+    right = (lane + 1) % 32;
+  }
+  const long long slot = pen / ((long long)nu * nw);
+  const int r = (int)(pen - slot * nu * nw);
   int pos[3];
-  pos[U] = pu;
-  pos[W] = pw;
-  pos[D] = fa - 2;
-  const long long st = wb_stride<D>(g);
-  const long long base = wb_at(g, pos[0], pos[1], pos[2]);
-  {
-    int last[3] = {pos[0], pos[1], pos[2]};
-    last[D] = fb + 1;  // the segment reads zones fa-2 .. fb+1
-    WB_CHECK_ZONE(g, last[0], last[1], last[2]);
-    (void)last;
-  }
-  const long long off_in = qo + base;
-  const long long off_out = wo + base;
-  const double dtdx = WB_MUL(dt, g.idx[D]);
-  const double dx_2dt = WB_MUL(wb_half(g.dx[D]), wb_rcp(dt));
-  Cell cL, cR;
-  load_cell<D, NC>(q, off_in, P, cL);
-  double gt_p[7], g_p[7];  // 2 g-tilde of face f-1; 2 g of zone f-2
-  int nhll = 0;
-  // HLL faces are counted on interior faces only (distinct faces, whatever
-  // part of the ghost rings the region covers)
-  const bool across = pu >= 0 && pu < g.n[U] && pw >= 0 && pw < g.n[W];
-  int cur = 0;
-  // faces f = fa-1 .. fb+1; face f lies between zones f-1 and f
-  for (int f = fa - 1; f <= fb + 1; ++f) {
-    const int c = f - (fa - 2);  // zone f relative to the first zone
-    load_cell<D, NC>(q, off_in + c * st, P, cR);
-    const double b = ld<NC>(bn + off_in + c * st);
-    double gt[7];
-    const int code = face_system<EZ, PROT>(cL, cR, b, dtdx, P, rec[cur], gt);
-    if (code) {
-      const double bnL = ld<NC>(q[F_BX + D] + off_in + (c - 1) * st);
-      const double bnR = ld<NC>(q[F_BX + D] + off_in + c * st);
-      hll_face(cL, cR, bnL, bnR, code == 1, P, rec[cur]);
+  pos[U] = box.lo[U] + r % nu;
+  pos[W] = box.lo[W] + r / nu;
+  pos[d] = box.lo[d] + idx;
+  const long long at = wb_at(g, pos[0], pos[1], pos[2]);
+  const long long off = slot * slot_in + at;
+  Cell R;
+  load_cell<NC>(s.q, off, P, R);
+  const double b = ld<NC>(s.bn + off);
+  Cell L;
+  L.ir = 0.0;  // not used across a face
+  if (!ring) {
+    if (lane == 31) {
 #pragma unroll
-      for (int k = 0; k < 7; ++k) gt[k] = 0.0;
+      for (int i = 0; i < kCellWords; ++i) X.cell[wp][i] = cell_word(R, i);
     }
-    if (f >= fa) {
-      // 2 g of zone f-1 from 2 g-tilde of faces f (i+1/2) and f-1 (i-1/2)
-      double gz[7];
+    __syncthreads();
+  }
 #pragma unroll
-      for (int k = 0; k < 7; ++k) gz[k] = wb_sweby(gt[k], gt_p[k], P.sweby, P.minmod);
-      if (f >= fa + 1) {
-        // flux of face f-1 (zones f-2, f-1): g_{i} = g_p (zone f-2), g_{i+1} = gz
-        double out[7];
-        const Rc& fr = rec[cur ^ 1];
-        if (wb_neg(fr[R_RHO])) {
+  for (int i = 0; i < kCellWords; ++i) cell_word(L, i) = __shfl_sync(0xffffffffu, cell_word(R, i), left);
+  if (!ring && lane == 0 && wp > 0) {
 #pragma unroll
-          for (int m = 0; m < 7; ++m) out[m] = fr[R_FAVG + m];
-          if (across && f - 1 >= 0 && f - 1 < g.n[D]) ++nhll;
-        } else {
-          face_flux<EZ>(fr, g_p, gz, dx_2dt, P, out);
-        }
-        const long long o = off_out + (c - 1) * st;
-        F[F_RHO][o] = out[0];
-        F[F_MX + D][o] = out[1];
-        F[F_MX + T1][o] = out[2];
-        F[F_MX + T2][o] = out[3];
-        F[F_EN][o] = out[6];
-        F[F_BX + T1][o] = out[4];
-        F[F_BX + T2][o] = out[5];
-      }
-#pragma unroll
-      for (int k = 0; k < 7; ++k) g_p[k] = gz[k];
+    for (int i = 0; i < kCellWords; ++i) cell_word(L, i) = X.cell[wp - 1][i];
+  }
+  RegRec f;
+  double gt[7];
+  const int code = face_system<EZ, PROT>(L, R, b, __dmul_rn(dt, g.idx[d]), P, f, gt);
+  bool hll = false;
+  if (code) {
+    if (has_left) {
+      const long long st = d == 0 ? 1LL : (d == 1 ? g.sy : g.sz);
+      hll_face(L, R, ld<NC>(s.q[5] + off - st), ld<NC>(s.q[5] + off), code == 1, P, f);
+      hll = true;
     }
 #pragma unroll
-    for (int k = 0; k < 7; ++k) gt_p[k] = gt[k];
-    cur ^= 1;
-    cL = cR;
+    for (int k = 0; k < 7; ++k) gt[k] = 0.0;
   }
-  return nhll;
+  __syncwarp();
+  if (!ring) {
+    if (lane == 0) {
+#pragma unroll
+      for (int k = 0; k < 7; ++k) X.gt0[wp][k] = gt[k];
+    }
+    __syncthreads();
+  }
+  double gz[7], gl[7];  // 2 g of this zone, of the left zone
+#pragma unroll
+  for (int k = 0; k < 7; ++k) {
+    double gr = __shfl_sync(0xffffffffu, gt[k], right);
+    if (!ring && lane == 31 && wp < kWarps - 1) gr = X.gt0[wp + 1][k];
+    gz[k] = wb_sweby(gr, gt[k], P.sweby, P.minmod);
+  }
+  if (!ring) {
+    if (lane == 31) {
+#pragma unroll
+      for (int k = 0; k < 7; ++k) X.gz31[wp][k] = gz[k];
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int k = 0; k < 7; ++k) {
+    gl[k] = __shfl_sync(0xffffffffu, gz[k], left);
+    if (!ring && lane == 0 && wp > 0) gl[k] = X.gz31[wp - 1][k];
+  }
+  if (!emit) return 0;
+  double out[7];
+  if (hll) {
+#pragma unroll
+    for (int m = 0; m < 7; ++m) out[m] = f[R_FAVG + m];
+  } else {
+    face_flux<EZ>(f, gl, gz, __dmul_rn(wb_half(g.dx[d]), wb_rcp(dt)), P, out);
+  }
+  const long long o = slot * slot_out + at;
+#pragma unroll
+  for (int m = 0; m < 7; ++m) s.F[m][o] = out[m];
+  return hll && pos[0] >= 0 && pos[0] < g.n[0] && pos[1] >= 0 && pos[1] < g.n[1] && pos[2] >= 0 && pos[2] < g.n[2];
 }
 
 // ---------------------------------------------------------------- stages ---

@@ -20,6 +20,9 @@ extern "C" void soft_roots(int n, const double* x, double* rsq, double* sq, doub
     rsq[i] = r.rsq; sq[i] = r.sq; rc[i] = r.rcp; rcp[i] = wb_rcp(x[i]);
   }
 }
+extern "C" void soft_mul(int n, const double* x, const double* y, double* p) {
+  for (int i = 0; i < n; ++i) p[i] = wb_smul(x[i], y[i]);
+}
 """
 
 
@@ -99,3 +102,43 @@ def test_reciprocal_sign_and_bad_inputs(soft):
         assert np.all(np.isnan(o)), o
     assert out[3][0] == 1 / -3.0 and out[3][1] == -1.0 and out[3][2] == 1 / -1e300
     assert np.all(np.isnan(out[3][3:]))
+
+
+@pytest.mark.parametrize("lo,hi", [(1003, 1043), (400, 1600), (1, 2046)])
+def test_products_have_the_bits_of_the_fp64_multiply(soft, lo, hi):
+    """Random and short significands (ties and exact products among them), both
+    signs, zeros: the bits of the FP64 product wherever its magnitude is zero or
+    in [2^-1021, 2^1023); zero below the normal range, NaN above it."""
+    x = np.concatenate([samples(20000, lo, hi, s) for s in range(5)])
+    rng = np.random.default_rng(lo)
+    y = rng.permutation(x) * rng.choice([-1.0, 1.0], x.size)
+    keep = (np.uint64(0xFFFFFFFFFFFFFFFF) << rng.integers(0, 53, x.size).astype(np.uint64))
+    x = (x.view(np.uint64) & np.where(rng.random(x.size) < 0.5, keep, ~np.uint64(0))).view(np.float64)
+    y[::501], x[1::501], y[3::501] = 0.0, -0.0, 1.0
+    p = np.empty_like(x)
+    call(soft.soft_mul, x.size, x, y, p)
+    with np.errstate(over="ignore", under="ignore"):
+        want = x * y
+    mag = np.abs(want)
+    low, high = mag < 2.0 ** -1021, mag >= 2.0 ** 1023
+    mid = ~low & ~high
+    assert np.array_equal(p[mid].view(np.uint64), want[mid].view(np.uint64))
+    # at the ends of the range the exponents' sum decides: flushed (NaN) or exact
+    flushed = p[low].view(np.uint64) == np.copysign(0.0, want[low]).view(np.uint64)
+    assert np.all(flushed | ((p[low] == want[low]) & (mag[low] >= 2.0 ** -1022)))
+    assert np.all(np.isnan(p[high]) | (p[high] == want[high]))
+    if (lo, hi) == (1003, 1043):
+        assert np.all(mid | (want == 0.0))
+
+
+def test_products_of_bad_factors_are_nan(soft):
+    """Infinities and NaN give NaN with any factor but a subnormal or zero one,
+    where NaN too; subnormal factors count as zero."""
+    bad = np.array([np.inf, -np.inf, np.nan])
+    for other in (1.0, -3e-200, 2e200, 0.0, 5e-324, np.inf):
+        p = np.empty(3)
+        call(soft.soft_mul, 3, bad, np.full(3, other), p)
+        assert np.all(np.isnan(p)), other
+    p = np.empty(2)
+    call(soft.soft_mul, 2, np.array([5e-324, -2e-308]), np.array([1e300, 1e300]), p)
+    assert p[0] == 0.0 and p[1] == 0.0 and np.signbit(p[1])
