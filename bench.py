@@ -118,17 +118,22 @@ def cpu_model():
 
 
 def step_launches(desc):
-    """Kernels one wb_advance step launches: the dt kernel, 10 per pass over a
-    batch of patches (2 sweeps of all axes, reference EMF, corner EMFs, half CT,
-    transverse states, half-step reference EMF, corner EMFs, final CT, update)
-    and the ghost fill; a grid periodic on every axis with all patches in one
-    pass adds the 7 periodic-image fills of its interior-only stages."""
+    """Kernels one wb_advance step launches: 9 per pass over a batch of patches
+    (2 sweeps of all axes, the first with the reference EMF, corner EMFs, half
+    CT, transverse states, half-step reference EMF, corner EMFs, final CT and
+    the update, which also prepares the next dt) and the ghost fill, which a
+    single patch periodic on every axis does without; several patches of such a
+    grid in one pass add the 7 image fills of its interior-only stages.  (The dt
+    kernel of a call's first step is not counted.)"""
     npatch = desc.patches[0] * desc.patches[1] * desc.patches[2]
     per_pass = desc.batch_patches if desc.batch_patches > 0 else npatch
     passes = -(-npatch // per_pass)
+    periodic = all(desc.bc[a] == 0 for a in range(3))
+    if periodic and npatch == 1:
+        return 9
     flat = desc.n[2] == 1 and desc.patches[2] == 1 and desc.bc[2] == 0
-    images = passes == 1 and not flat and all(desc.bc[a] == 0 for a in range(3))
-    return 2 + (17 if images else 10) * passes
+    images = passes == 1 and not flat and periodic
+    return 1 + (16 if images else 9) * passes
 
 
 def workload_name(n):

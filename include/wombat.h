@@ -263,9 +263,10 @@ const char* wb_noalloc_last_error(void);
  * images, half CT (4), its images, transverse states (5, 7), their images,
  * corrector sweeps (6, 7), their images, half-step EMF (8), its images,
  * corner EMFs (9), their images, final CT (11), update (10), ghost fill;
- * *count = the number of stages (19).  The image stages copy periodic
- * images of intermediates for boxes periodic on every axis, whose other
- * stages then cover the interior only.  It synchronises the stream.
+ * *count = the number of stages (19).  The image stages (and the ghost fill,
+ * for boxes periodic on every axis) have no work and read 0: the stages of
+ * such a box cover its interior and read across its ends.  It synchronises
+ * the stream.
  * wb_batch_set_form: how wb_batch_advance runs the stages.
  * WB_BATCH_PERSISTENT (the default): the one persistent cooperative launch
  * above.  WB_BATCH_STAGED: one ordinary launch per stage of each step over

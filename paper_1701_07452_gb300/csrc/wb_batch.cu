@@ -37,9 +37,11 @@
 
 namespace {
 
-// Stages of a step.  BS_W* fill the periodic images of intermediates for
-// boxes periodic on every axis, whose other stages then run on the interior
-// only (the grid path's enqueue_pass_wrap); they have no work for other boxes.
+// Stages of a step.  Boxes periodic on every axis (wrap) run every stage on
+// their interior and read across their own ends, as a single-patch grid does
+// (enqueue_pass_interior): they need no ghost fill.  BS_W* (once the images of
+// their intermediates) have no work and are not launched; they keep their
+// places in the stage times.
 enum {
   BS_DT = 0, BS_PRED, BS_EREF, BS_W_FP, BS_EDGE_P, BS_W_EE, BS_CT_H, BS_W_BH, BS_TRANS, BS_W_QH,
   BS_CORR, BS_W_FC, BS_EREF_H, BS_W_ERH, BS_EDGE_C, BS_W_EEH, BS_CT_F, BS_FINAL, BS_HALO, BS_COUNT
@@ -70,7 +72,7 @@ __host__ __device__ inline bool stage_is_sweep(int s) { return s == BS_PRED || s
 // wrap: the box is periodic on every axis (interior-only regions).
 __host__ __device__ inline WbBox stage_box(int s, int d, const int* n, bool wrap) {
   const int N0 = n[0], N1 = n[1], N2 = n[2];
-  if (wrap && s != BS_CT_F && s != BS_HALO) return bxx(0, N0 - 1, 0, N1 - 1, 0, N2 - 1);
+  if (wrap && s != BS_HALO) return bxx(0, N0 - 1, 0, N1 - 1, 0, N2 - 1);
   switch (s) {
     case BS_PRED:
       if (d == 0) return bxx(-3, N0 + 3, -4, N1 + 3, -4, N2 + 3);
@@ -131,8 +133,8 @@ __host__ __device__ inline long long sweep_pencils(const WbBox& b, int d) {
 
 __host__ __device__ inline long long stage_items(int s, int d, const WbGeo& g, bool wrap) {
   if (s == BS_DT) return 1;
-  if (stage_is_wrap(s)) return wrap ? wbu::shell_count(g, s == BS_W_QH ? 2 : 1) : 0;
-  if (s == BS_HALO) return wbu::shell_count(g, WB_NG);
+  if (stage_is_wrap(s)) return 0;
+  if (s == BS_HALO) return wrap ? 0 : wbu::shell_count(g, WB_NG);
   WbBox b = stage_box(s, d, g.n, wrap);
   if (stage_is_sweep(s)) {
     const int len = b.hi[d] - b.lo[d] + 1;
@@ -148,7 +150,7 @@ __host__ __device__ inline int items_per_chunk(int s) {
 struct BoxInfo {
   WbView v;
   int bc[3];
-  int wrap;  // periodic on every axis: interior-only stages + periodic images
+  int wrap;  // periodic on every axis: interior-only stages that read across the ends
   // the sweeps' fields, [corrector][axis]: read where they are needed rather
   // than held in registers through a sweep
   wbu::SweepFrame sw[2][3];
@@ -232,7 +234,7 @@ __device__ __forceinline__ int box_sweep_tile(const BoxInfo& bi, bool corr, int 
   const WbView& v = bi.v;
   const bool wrap = bi.wrap != 0;
   const WbBox b = stage_box(corr ? BS_CORR : BS_PRED, d, v.geo.n, wrap);
-  return wbu::sweep_tile<EZ, PROT, false>(v.geo, b, d, bi.sw[corr ? 1 : 0][d], tile,
+  return wbu::sweep_tile<EZ, PROT, false>(v.geo, b, d, bi.sw[corr ? 1 : 0][d], tile, wrap,
                                           wbu::sweep_ring(b.hi[d] - b.lo[d] + 1, wrap), 1, 0, 0,
                                           dt, P, X);
 }
@@ -250,16 +252,17 @@ __device__ __forceinline__ void unit_item(const BatchParams& B, int s, int d, co
   const long long r = item / nx;
   const int j = b.lo[1] + (int)(r % ny);
   const int k = b.lo[2] + (int)(r / ny);
+  const wbu::Nbr nb = wbu::neighbours(v.geo, i, j, k, wrap ? 7 : 0);
   switch (s) {
     case BS_TRANS: {
       const int mask = trans_mask(n, i, j, k);
-      if (mask == 7) wbu::transverse_set(v, 0, 0, dt, 7, i, j, k);  // constant mask: see k_transverse
-      else if (mask) wbu::transverse_set(v, 0, 0, dt, mask, i, j, k);
+      if (mask == 7) wbu::transverse_set(v, 0, 0, dt, 7, i, j, k, nb);  // constant mask: see k_transverse
+      else if (mask) wbu::transverse_set(v, 0, 0, dt, mask, i, j, k, nb);
       break;
     }
-    case BS_EREF_H: wbu::eref_half(v, 0, 0, dt, i, j, k); break;
+    case BS_EREF_H: wbu::eref_half(v, 0, 0, dt, i, j, k, nb); break;
     case BS_FINAL: {
-      const double w = wbu::final_update(v, 0, 0, dt, B.phys, i, j, k, outflow_mask(bi), hits, bad);
+      const double w = wbu::final_update(v, 0, 0, dt, B.phys, i, j, k, nb, outflow_mask(bi), hits, bad);
       // running max of the rate keys: integer compares, and a NaN stays
       const unsigned long long kw = wb_rate_bits(w);
       if (kw > *wkey) *wkey = kw;
@@ -274,7 +277,7 @@ __device__ __forceinline__ void unit_item(const BatchParams& B, int s, int d, co
 // per-stage kernels hide that latency with many resident warps instead).
 __host__ __device__ inline bool stage_pairs(int s) {
   return s == BS_EREF || s == BS_EDGE_P || s == BS_EDGE_C || s == BS_CT_H || s == BS_CT_F ||
-         s == BS_HALO || stage_is_wrap(s);
+         s == BS_HALO;
 }
 
 __device__ __forceinline__ void item_ijk(const WbBox& b, long long item, int* i, int* j, int* k) {
@@ -295,60 +298,17 @@ __device__ __forceinline__ void copy2(double* a, long long d0, long long s0, lon
   if (two) a[d1] = x1;
 }
 
-// The arrays of a copy stage (state for the ghost fill, intermediates for
-// the periodic-image stages), moved for two shell points at a time.
-__device__ __forceinline__ void copy_stage(const WbView& v, int s, long long d0, long long s0, long long d1,
-                                           long long s1, bool two) {
-  switch (s) {
-    case BS_HALO:
-#pragma unroll
-      for (int c = 0; c < 8; ++c) copy2(v.q[c], d0, s0, d1, s1, two);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) copy2(v.b[c], d0, s0, d1, s1, two);
-      return;
-    case BS_W_FP:
-    case BS_W_FC: {
-      double* const(*F)[8] = s == BS_W_FP ? v.Fp : v.Fc;
-#pragma unroll
-      for (int e = 0; e < 3; ++e)
-#pragma unroll
-        for (int c = 0; c < 8; ++c)
-          if (c != F_BX + e) copy2(F[e][c], d0, s0, d1, s1, two);
-      if (s == BS_W_FP) {
-#pragma unroll
-        for (int e = 0; e < 3; ++e) copy2(v.Eref[e], d0, s0, d1, s1, two);
-      }
-      return;
-    }
-    case BS_W_QH:
-#pragma unroll
-      for (int e = 0; e < 3; ++e)
-#pragma unroll
-        for (int c = 0; c < 8; ++c) copy2(v.qh[e][c], d0, s0, d1, s1, two);
-      return;
-    default: {
-      double* const* a3 = s == BS_W_EE ? v.Eedge : (s == BS_W_BH ? v.bh : (s == BS_W_ERH ? v.Erefh : v.Eedgeh));
-#pragma unroll
-      for (int e = 0; e < 3; ++e) copy2(a3[e], d0, s0, d1, s1, two);
-    }
-  }
-}
-
-// Items it0 and it1 (it1 < 0: none) of a copy stage (ghost fill, periodic
-// images) for one box.
-__device__ __forceinline__ void unit_pair_copy(int s, const BoxInfo& bi, long long it0, long long it1) {
+// Items it0 and it1 (it1 < 0: none) of the ghost fill of one box.
+__device__ __forceinline__ void unit_pair_halo(const BoxInfo& bi, long long it0, long long it1) {
   const WbView& v = bi.v;
   const bool two = it1 >= 0;
   long long d0, s0, d1 = 0, s1 = 0;
-  if (s == BS_HALO) {
-    wbu::halo_self_offsets(v.geo, bi.bc, it0, &d0, &s0);
-    if (two) wbu::halo_self_offsets(v.geo, bi.bc, it1, &d1, &s1);
-  } else {
-    const int depth = s == BS_W_QH ? 2 : 1;
-    wbu::wrap_shell_point(v.geo, depth, it0, &d0, &s0);
-    if (two) wbu::wrap_shell_point(v.geo, depth, it1, &d1, &s1);
-  }
-  copy_stage(v, s, d0, s0, d1, s1, two);
+  wbu::halo_self_offsets(v.geo, bi.bc, it0, &d0, &s0);
+  if (two) wbu::halo_self_offsets(v.geo, bi.bc, it1, &d1, &s1);
+#pragma unroll
+  for (int c = 0; c < 8; ++c) copy2(v.q[c], d0, s0, d1, s1, two);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) copy2(v.b[c], d0, s0, d1, s1, two);
 }
 
 // Items it0 and it1 (it1 < 0: none) of the reference EMF, corner EMF or CT
@@ -361,13 +321,15 @@ __device__ __forceinline__ void unit_pair_emf(int s, int d, const BoxInfo& bi, l
   int i0, j0, k0, i1 = 0, j1 = 0, k1 = 0;
   item_ijk(b, it0, &i0, &j0, &k0);
   if (two) item_ijk(b, it1, &i1, &j1, &k1);
+  const int closed = bi.wrap ? 7 : 0;
+  const wbu::Nbr n0 = wbu::neighbours(v.geo, i0, j0, k0, closed), n1 = wbu::neighbours(v.geo, i1, j1, k1, closed);
   switch (s) {
     case BS_EREF: {
       wbu::ErefIn a0, a1;
       wbu::eref_load(v, 0, 0, i0, j0, k0, a0);
       if (two) wbu::eref_load(v, 0, 0, i1, j1, k1, a1);
-      wbu::eref_finish(v, a0);
-      if (two) wbu::eref_finish(v, a1);
+      wbu::eref_finish(v.Eref, a0);
+      if (two) wbu::eref_finish(v.Eref, a1);
       return;
     }
     case BS_EDGE_P:
@@ -375,8 +337,8 @@ __device__ __forceinline__ void unit_pair_emf(int s, int d, const BoxInfo& bi, l
       const bool corr = s == BS_EDGE_C;
       wbu::EdgeIn a0, a1;
 #define WB_EDGE_PAIR(C)                                             \
-  wbu::edge_load<C>(v, 0, corr, i0, j0, k0, a0);                    \
-  if (two) wbu::edge_load<C>(v, 0, corr, i1, j1, k1, a1);           \
+  wbu::edge_load<C>(v, 0, corr, i0, j0, k0, n0, a0);                \
+  if (two) wbu::edge_load<C>(v, 0, corr, i1, j1, k1, n1, a1);       \
   wbu::edge_finish<C>(v, corr, a0);                                 \
   if (two) wbu::edge_finish<C>(v, corr, a1);
       if (d == 0) { WB_EDGE_PAIR(0) } else if (d == 1) { WB_EDGE_PAIR(1) } else { WB_EDGE_PAIR(2) }
@@ -387,8 +349,8 @@ __device__ __forceinline__ void unit_pair_emf(int s, int d, const BoxInfo& bi, l
       const bool fin = s == BS_CT_F;
       wbu::CtIn a0, a1;
 #define WB_CT_PAIR(D)                                               \
-  wbu::ct_load<D>(v, 0, 0, fin, i0, j0, k0, a0);                    \
-  if (two) wbu::ct_load<D>(v, 0, 0, fin, i1, j1, k1, a1);           \
+  wbu::ct_load<D>(v, 0, 0, fin, i0, j0, k0, n0, a0);                \
+  if (two) wbu::ct_load<D>(v, 0, 0, fin, i1, j1, k1, n1, a1);       \
   wbu::ct_finish<D>(v, fin, dt, a0);                                \
   if (two) wbu::ct_finish<D>(v, fin, dt, a1);
       if (d == 0) { WB_CT_PAIR(0) } else if (d == 1) { WB_CT_PAIR(1) } else { WB_CT_PAIR(2) }
@@ -405,25 +367,26 @@ __device__ __forceinline__ void unit_emf(int s, int d, const BoxInfo& bi, long l
   const WbBox b = stage_box(s, d, v.geo.n, bi.wrap != 0);
   int i, j, k;
   item_ijk(b, it, &i, &j, &k);
+  const wbu::Nbr nb = wbu::neighbours(v.geo, i, j, k, bi.wrap ? 7 : 0);
   if (s == BS_EREF) {
     wbu::eref(v, 0, 0, i, j, k);
   } else if (s == BS_EDGE_P || s == BS_EDGE_C) {
     const bool corr = s == BS_EDGE_C;
-    if (d == 0) wbu::edge<0>(v, 0, corr, i, j, k);
-    else if (d == 1) wbu::edge<1>(v, 0, corr, i, j, k);
-    else wbu::edge<2>(v, 0, corr, i, j, k);
+    if (d == 0) wbu::edge<0>(v, 0, corr, i, j, k, nb);
+    else if (d == 1) wbu::edge<1>(v, 0, corr, i, j, k, nb);
+    else wbu::edge<2>(v, 0, corr, i, j, k, nb);
   } else {
     const bool fin = s == BS_CT_F;
-    if (d == 0) wbu::ct<0>(v, 0, 0, fin, dt, i, j, k);
-    else if (d == 1) wbu::ct<1>(v, 0, 0, fin, dt, i, j, k);
-    else wbu::ct<2>(v, 0, 0, fin, dt, i, j, k);
+    if (d == 0) wbu::ct<0>(v, 0, 0, fin, dt, i, j, k, nb);
+    else if (d == 1) wbu::ct<1>(v, 0, 0, fin, dt, i, j, k, nb);
+    else wbu::ct<2>(v, 0, 0, fin, dt, i, j, k, nb);
   }
 }
 
 // Items it0 and it1 (it1 < 0: none) of a pairing stage for one box.
 __device__ __forceinline__ void unit_pair(int s, int d, const BoxInfo& bi, long long it0, long long it1,
                                           double dt) {
-  if (s == BS_HALO || stage_is_wrap(s)) unit_pair_copy(s, bi, it0, it1);
+  if (s == BS_HALO) unit_pair_halo(bi, it0, it1);
   else unit_pair_emf(s, d, bi, it0, it1, dt);
 }
 
@@ -505,14 +468,16 @@ __global__ void __launch_bounds__(kB, wbu::kSweepBlocks) k_batch(BatchParams B, 
     for (int grp = 0; grp < B.ngroups; ++grp) {
       const int gb0 = B.gfirst[grp];
       const int nbox = B.gfirst[grp + 1] - gb0;
-      for (int s = 0; s < BS_COUNT; ++s, ++stage_seq) {
+      for (int s = 0; s < BS_COUNT; ++s) {
+        const int nsub = stage_nsub(s);
+        const int nent = nbox * nsub;
+        const long long* pre = B.pre + B.pre_off[grp * BS_COUNT + s];
+        const long long nchunks = pre[nent];
+        if (nchunks == 0) continue;  // the same for every block
         unsigned* ctr = B.sync + 3 + (stage_seq & 1u);
         // the other counter is idle during this stage: block 0 clears it
         if (blockIdx.x == 0 && threadIdx.x == 0) atomicExch(B.sync + 3 + ((stage_seq + 1) & 1u), 0u);
-        const long long* pre = B.pre + B.pre_off[grp * BS_COUNT + s];
-        const int nsub = stage_nsub(s);
-        const int nent = nbox * nsub;
-        const long long nchunks = pre[nent];
+        ++stage_seq;
         const int ipc = items_per_chunk(s);
         for (;;) {
           if (threadIdx.x == 0) s_chunk = (long long)atomicAdd(ctr, 1u);
@@ -579,7 +544,7 @@ enum { SC_SWEEP = 0, SC_COPY, SC_EMF, SC_TRANS, SC_EREF_H, SC_FINAL, SC_DT, SC_C
 
 __host__ __device__ inline int stage_class(int s) {
   if (stage_is_sweep(s)) return SC_SWEEP;
-  if (s == BS_HALO || stage_is_wrap(s)) return SC_COPY;  // copies of up to 24 arrays
+  if (s == BS_HALO) return SC_COPY;
   if (stage_pairs(s)) return SC_EMF;                    // reference EMF, corner EMFs, CT (one item a thread)
   if (s == BS_TRANS) return SC_TRANS;
   if (s == BS_EREF_H) return SC_EREF_H;
@@ -658,7 +623,7 @@ __global__ void __launch_bounds__(kNtZone, zone_min_blocks(CLS))
     const long long i1 = i0 + ipc < nitems ? i0 + ipc : nitems;
     if (CLS == SC_COPY) {
       for (long long it = i0 + threadIdx.x; it < i1; it += 2 * NT)
-        unit_pair_copy(s, bi, it, it + NT < i1 ? it + NT : -1);
+        unit_pair_halo(bi, it, it + NT < i1 ? it + NT : -1);
       return;
     }
     if (CLS == SC_EMF) {
@@ -672,14 +637,15 @@ __global__ void __launch_bounds__(kNtZone, zone_min_blocks(CLS))
     for (long long it = i0 + threadIdx.x; it < i1; it += NT) {
       int i, j, k;
       item_ijk(b, it, &i, &j, &k);
+      const wbu::Nbr nb = wbu::neighbours(v.geo, i, j, k, bi.wrap ? 7 : 0);
       if (CLS == SC_TRANS) {
         const int mask = trans_mask(v.geo.n, i, j, k);
-        if (mask == 7) wbu::transverse_set(v, 0, 0, dt, 7, i, j, k);  // constant mask: see k_transverse
-        else if (mask) wbu::transverse_set(v, 0, 0, dt, mask, i, j, k);
+        if (mask == 7) wbu::transverse_set(v, 0, 0, dt, 7, i, j, k, nb);  // constant mask: see k_transverse
+        else if (mask) wbu::transverse_set(v, 0, 0, dt, mask, i, j, k, nb);
       } else if (CLS == SC_EREF_H) {
-        wbu::eref_half(v, 0, 0, dt, i, j, k);
+        wbu::eref_half(v, 0, 0, dt, i, j, k, nb);
       } else {
-        const double w = wbu::final_update(v, 0, 0, dt, B.phys, i, j, k, outflow_mask(bi), &hits, &bad);
+        const double w = wbu::final_update(v, 0, 0, dt, B.phys, i, j, k, nb, outflow_mask(bi), &hits, &bad);
         const unsigned long long kw = wb_rate_bits(w);
         if (kw > wkey) wkey = kw;
       }
@@ -754,6 +720,7 @@ struct wb_batch {
   double* state_base;
   double* work_base;
   std::vector<int> gbox, gfirst;
+  std::vector<long long> stage_chunks;  // chunks of each (group, stage)
   bool dirty;
   // device tables
   BoxInfo* d_info;
@@ -853,10 +820,11 @@ PoolSizes pool_sizes(size_t state_bytes, size_t work_bytes, int cap, int max_n) 
 }
 
 // chunk prefix tables for the current groups
-void build_prefix(const wb_batch* b, std::vector<long long>& pre, std::vector<long long>& off) {
+void build_prefix(wb_batch* b, std::vector<long long>& pre, std::vector<long long>& off) {
   const int ngroups = (int)b->gfirst.size() - 1;
   pre.clear();
   off.assign((size_t)ngroups * BS_COUNT, 0);
+  b->stage_chunks.assign((size_t)ngroups * BS_COUNT, 0);
   for (int gi = 0; gi < ngroups; ++gi)
     for (int s = 0; s < BS_COUNT; ++s) {
       off[gi * BS_COUNT + s] = (long long)pre.size();
@@ -871,6 +839,7 @@ void build_prefix(const wb_batch* b, std::vector<long long>& pre, std::vector<lo
         }
       }
       pre.push_back(acc);
+      b->stage_chunks[gi * BS_COUNT + s] = acc;
     }
 }
 
@@ -1024,7 +993,8 @@ cudaError_t enqueue_staged(wb_batch* b, int nsteps) {
   unsigned seq = 0;
   for (int step = 0; step < nsteps; ++step)
     for (int grp = 0; grp < p.ngroups; ++grp)
-      for (int s = 0; s < BS_COUNT; ++s, ++seq) {
+      for (int s = 0; s < BS_COUNT; ++s) {
+        if (!b->stage_chunks[(size_t)grp * BS_COUNT + s]) continue;
         const int cls = stage_class(s);
         const void* fn;
         unsigned nt, nblocks;
@@ -1040,6 +1010,7 @@ cudaError_t enqueue_staged(wb_batch* b, int nsteps) {
         void* args[] = {&p, &grp, &s, &seq};
         e = cudaLaunchKernel(fn, dim3(nblocks), dim3(nt), args, 0, b->stream);
         if (e != cudaSuccess) return e;
+        ++seq;
       }
   return cudaSuccess;
 }
@@ -1389,7 +1360,7 @@ int wb_batch_load(wb_batch* b, int box, const double* U, const double* bx, const
   for (int c = 0; c < 8; ++c) q[c] = bi.v.q[c];
   for (int c = 0; c < 3; ++c) bb[c] = bi.v.b[c];
   wb_launch_halo(q, bb, g, m, s);
-  wb_launch_ccb(q, bb, g, 1, s);
+  wb_launch_ccb(q, bb, g, 1, 0, s);
   if (primitive) wb_launch_prim_to_cons(q, g, 1, b->phys, s);
   wb_launch_halo(q, bb, g, m, s);
   cudaError_t e = cudaMemsetAsync(b->d_scal + box, 0, sizeof(WbScalars), s);

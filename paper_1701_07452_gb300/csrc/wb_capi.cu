@@ -43,8 +43,11 @@ struct wb_grid {
   unsigned long long* red;
   std::string err;
   bool loaded;
-  // interior-only stages with periodic images of the intermediates: periodic
-  // on every axis, 3D storage, every patch in one pass
+  // interior-only stages, for a grid periodic on every axis whose patches all
+  // sit in one pass: closed (7: one patch, whose stages read across its ends,
+  // so that no ghost of it is ever read; else 0), or wrap (several patches:
+  // images of the intermediates between the stages)
+  int closed = 0;
   bool wrap = false;
   // sweep timing (wb_profile_sweeps)
   bool prof;
@@ -251,6 +254,7 @@ StageArgs stage_args(wb_grid* g, long long p0, int nslots) {
   v.scal = g->scal;
   a.phys = g->phys;
   a.nslots = nslots;
+  a.closed = g->closed;
   a.p0 = p0;
   a.ohi_bc = 0;
   for (int d = 0; d < 3; ++d) {
@@ -260,7 +264,8 @@ StageArgs stage_args(wb_grid* g, long long p0, int nslots) {
   return a;
 }
 
-SweepArgs sweep_args(wb_grid* g, const StageArgs& s, bool corr, const WbBox (&bx)[3], int nslots) {
+// ebox: the zones of the reference EMF (Step 2) that the predictor's launch takes along
+SweepArgs sweep_args(wb_grid* g, const StageArgs& s, bool corr, const WbBox (&bx)[3], int nslots, const WbBox& ebox) {
   SweepArgs a;
   std::memset(&a, 0, sizeof(a));
   const WbView& v = s.v;
@@ -275,6 +280,12 @@ SweepArgs sweep_args(wb_grid* g, const StageArgs& s, bool corr, const WbBox (&bx
   a.phys = g->phys;
   a.scal = g->scal;
   a.nslots = nslots;
+  for (int d = 0; d < 3; ++d)  // whole periodic pencils: one patch along the axis
+    if ((g->closed || g->wrap) && g->map.np[d] == 1) a.closed |= 1 << d;
+  if (!corr) {
+    for (int d = 0; d < 3; ++d) a.Eref[d] = v.Eref[d];
+    a.ebox = ebox;
+  }
   return a;
 }
 
@@ -283,10 +294,7 @@ const size_t kMaxProfiled = 8192;
 void sweeps(wb_grid* g, const SweepArgs& a) {
   bool rec = g->prof && g->ev_used + 2 <= g->ev.size();
   if (rec) cudaEventRecord(g->ev[g->ev_used], g->stream);
-  int closed = 0;  // an axis of one patch, its images in place
-  for (int d = 0; d < 3; ++d)
-    if (g->wrap && g->map.np[d] == 1) closed |= 1 << d;
-  wb_launch_sweeps(a, closed, g->stream);
+  wb_launch_sweeps(a, g->stream);
   if (rec) {
     cudaEventRecord(g->ev[g->ev_used + 1], g->stream);
     g->ev_used += 2;
@@ -303,13 +311,13 @@ WrapList wrap_list(std::initializer_list<double*> arrays) {
 
 // One step of a grid periodic on every axis whose patches all sit in one
 // pass (a single patch, or every patch resident: slot = patch).  Every stage
-// runs on the interior index range of each patch only; between stages the
-// ghost points a later stage reads (1 deep, 2 for the preconditioned states
-// the corrector sweeps read) are filled with periodic images, from the
-// neighbouring patch where there is one.  On one GPU the copies cost a small
-// fraction of recomputing the ghost rings, which the 5-zone scheme (one
-// exchange per step) otherwise does at every stage.
-void enqueue_pass_wrap(wb_grid* g) {
+// runs on the interior index range of each patch only.  A single patch reads
+// across its own ends (closed).  With several, the ghost points a later stage
+// reads (1 deep, 2 for the preconditioned states the corrector sweeps read)
+// are filled between the stages from the neighbouring patch; on one GPU the
+// copies cost a small fraction of recomputing the ghost rings, which the
+// 5-zone scheme (one exchange per step) otherwise does at every stage.
+void enqueue_pass_interior(wb_grid* g, const StepControl& c) {
   cudaStream_t s = g->stream;
   const int ns = (int)g->npatch;
   StageArgs A = stage_args(g, 0, ns);
@@ -317,54 +325,45 @@ void enqueue_pass_wrap(wb_grid* g) {
   const int N0 = G.n[0], N1 = G.n[1], N2 = G.n[2];
   const WbBox in = box(0, N0 - 1, 0, N1 - 1, 0, N2 - 1);
   const WbBox in3[3] = {in, in, in};
-  // Step 1: predictor fluxes on the interior faces (face N_d is face 0)
-  sweeps(g, sweep_args(g, A, false, in3, ns));
-  // Step 2: reference EMF; then the images of both
-  wb_launch_eref(A, in, s);
-  wb_launch_wrap(wrap_list({g->Fp[0][0], g->Fp[0][1], g->Fp[0][2], g->Fp[0][3], g->Fp[0][4], g->Fp[0][6],
-                            g->Fp[0][7], g->Fp[1][0], g->Fp[1][1], g->Fp[1][2], g->Fp[1][3], g->Fp[1][4],
-                            g->Fp[1][5], g->Fp[1][7], g->Fp[2][0], g->Fp[2][1], g->Fp[2][2], g->Fp[2][3],
-                            g->Fp[2][4], g->Fp[2][5], g->Fp[2][6], g->Eref[0], g->Eref[1], g->Eref[2]}),
-                 G, g->map, 1, s);
+  auto images = [&](std::initializer_list<double*> arrays, int depth) {
+    if (!g->closed) wb_launch_wrap(wrap_list(arrays), G, g->map, depth, s);
+  };
+  // Step 1: predictor fluxes on the interior faces (face N_d is face 0); Step 2: reference EMF
+  sweeps(g, sweep_args(g, A, false, in3, ns, in));
+  images({g->Fp[0][0], g->Fp[0][1], g->Fp[0][2], g->Fp[0][3], g->Fp[0][4], g->Fp[0][6], g->Fp[0][7], g->Fp[1][0],
+          g->Fp[1][1], g->Fp[1][2], g->Fp[1][3], g->Fp[1][4], g->Fp[1][5], g->Fp[1][7], g->Fp[2][0], g->Fp[2][1],
+          g->Fp[2][2], g->Fp[2][3], g->Fp[2][4], g->Fp[2][5], g->Fp[2][6], g->Eref[0], g->Eref[1], g->Eref[2]}, 1);
   // Step 3: corner EMFs; Step 4: b^{n+1/2}
   wb_launch_edges(A, false, in3, s);
-  wb_launch_wrap(wrap_list({g->Eedge[0], g->Eedge[1], g->Eedge[2]}), G, g->map, 1, s);
+  images({g->Eedge[0], g->Eedge[1], g->Eedge[2]}, 1);
   wb_launch_ct(A, false, in3, s);
-  wb_launch_wrap(wrap_list({g->bh[0], g->bh[1], g->bh[2]}), G, g->map, 1, s);
+  images({g->bh[0], g->bh[1], g->bh[2]}, 1);
   // Steps 5, 7: preconditioned states (the corrector sweeps read 2 zones out)
   wb_launch_transverse(A, in3, s);
-  {
-    WrapList L = wrap_list({});
-    for (int d = 0; d < 3; ++d)
-      for (int c = 0; c < 8; ++c)
-        if (g->qh[d][c]) L.a[L.n++] = g->qh[d][c];
-    wb_launch_wrap(L, G, g->map, 2, s);
-  }
+  images({g->qh[0][0], g->qh[0][1], g->qh[0][2], g->qh[0][3], g->qh[0][4], g->qh[0][5], g->qh[0][6], g->qh[0][7],
+          g->qh[1][0], g->qh[1][1], g->qh[1][2], g->qh[1][3], g->qh[1][4], g->qh[1][5], g->qh[1][6], g->qh[1][7],
+          g->qh[2][0], g->qh[2][1], g->qh[2][2], g->qh[2][3], g->qh[2][4], g->qh[2][5], g->qh[2][6], g->qh[2][7]}, 2);
   // Steps 6, 7: corrector fluxes
-  sweeps(g, sweep_args(g, A, true, in3, ns));
-  wb_launch_wrap(wrap_list({g->Fc[0][0], g->Fc[0][1], g->Fc[0][2], g->Fc[0][3], g->Fc[0][4], g->Fc[0][6],
-                            g->Fc[0][7], g->Fc[1][0], g->Fc[1][1], g->Fc[1][2], g->Fc[1][3], g->Fc[1][4],
-                            g->Fc[1][5], g->Fc[1][7], g->Fc[2][0], g->Fc[2][1], g->Fc[2][2], g->Fc[2][3],
-                            g->Fc[2][4], g->Fc[2][5], g->Fc[2][6]}),
-                 G, g->map, 1, s);
+  sweeps(g, sweep_args(g, A, true, in3, ns, in));
+  images({g->Fc[0][0], g->Fc[0][1], g->Fc[0][2], g->Fc[0][3], g->Fc[0][4], g->Fc[0][6], g->Fc[0][7], g->Fc[1][0],
+          g->Fc[1][1], g->Fc[1][2], g->Fc[1][3], g->Fc[1][4], g->Fc[1][5], g->Fc[1][7], g->Fc[2][0], g->Fc[2][1],
+          g->Fc[2][2], g->Fc[2][3], g->Fc[2][4], g->Fc[2][5], g->Fc[2][6]}, 1);
   // Step 8: half-step reference EMF; Step 9: corner EMFs
   wb_launch_eref_half(A, in, s);
-  wb_launch_wrap(wrap_list({g->Erefh[0], g->Erefh[1], g->Erefh[2]}), G, g->map, 1, s);
+  images({g->Erefh[0], g->Erefh[1], g->Erefh[2]}, 1);
   wb_launch_edges(A, true, in3, s);
-  wb_launch_wrap(wrap_list({g->Eedgeh[0], g->Eedgeh[1], g->Eedgeh[2]}), G, g->map, 1, s);
-  // Step 11 (faces, the high boundary face included), then Step 10
-  {
-    WbBox bb[3] = {box(0, N0, 0, N1 - 1, 0, N2 - 1), box(0, N0 - 1, 0, N1, 0, N2 - 1),
-                   box(0, N0 - 1, 0, N1 - 1, 0, N2)};
-    wb_launch_ct(A, true, bb, s);
-  }
-  wb_launch_final(A, s);
+  images({g->Eedgeh[0], g->Eedgeh[1], g->Eedgeh[2]}, 1);
+  // Step 11 (faces, with several patches the high boundary face included), then Step 10
+  const WbBox bb[3] = {box(0, N0, 0, N1 - 1, 0, N2 - 1), box(0, N0 - 1, 0, N1, 0, N2 - 1),
+                       box(0, N0 - 1, 0, N1 - 1, 0, N2)};
+  wb_launch_ct(A, true, g->closed ? in3 : bb, s);
+  wb_launch_final(A, c, s);
 }
 
 // One pipeline pass (Steps 1-11) over patches [p0, p0 + nslots).
-void enqueue_pass(wb_grid* g, long long p0, int nslots) {
-  if (g->wrap) {
-    enqueue_pass_wrap(g);
+void enqueue_pass(wb_grid* g, long long p0, int nslots, const StepControl& c) {
+  if (g->wrap || g->closed) {
+    enqueue_pass_interior(g, c);
     return;
   }
   cudaStream_t s = g->stream;
@@ -375,14 +374,13 @@ void enqueue_pass(wb_grid* g, long long p0, int nslots) {
   auto box = [flat](int l0, int h0, int l1, int h1, int l2, int h2) {
     return flat ? ::box(l0, h0, l1, h1, 0, 0) : ::box(l0, h0, l1, h1, l2, h2);
   };
-  // Step 1: predictor fluxes from q^n
+  // Step 1: predictor fluxes from q^n; Step 2: reference EMF
   {
     const WbBox pb[3] = {box(-3, N0 + 3, -4, N1 + 3, -4, N2 + 3), box(-4, N0 + 3, -3, N1 + 3, -4, N2 + 3),
                          box(-4, N0 + 3, -4, N1 + 3, -3, N2 + 3)};
-    sweeps(g, sweep_args(g, A, false, pb, nslots));
+    sweeps(g, sweep_args(g, A, false, pb, nslots, box(-4, N0 + 3, -4, N1 + 3, -4, N2 + 3)));
   }
-  // Step 2: reference EMF; Step 3: corner EMFs
-  wb_launch_eref(A, box(-4, N0 + 3, -4, N1 + 3, -4, N2 + 3), s);
+  // Step 3: corner EMFs
   {
     WbBox eb[3] = {box(-1, N0, -3, N1 + 3, -3, N2 + 3), box(-3, N0 + 3, -1, N1, -3, N2 + 3),
                    box(-3, N0 + 3, -3, N1 + 3, -1, N2)};
@@ -404,7 +402,7 @@ void enqueue_pass(wb_grid* g, long long p0, int nslots) {
   {
     const WbBox cb[3] = {box(-1, N0 + 1, -1, N1, -1, N2), box(-1, N0, -1, N1 + 1, -1, N2),
                          box(-1, N0, -1, N1, -1, N2 + 1)};
-    sweeps(g, sweep_args(g, A, true, cb, nslots));
+    sweeps(g, sweep_args(g, A, true, cb, nslots, cb[0]));
   }
   // Step 8: half-step reference EMF; Step 9: corner EMFs
   wb_launch_eref_half(A, box(-1, N0, -1, N1, -1, N2), s);
@@ -419,7 +417,16 @@ void enqueue_pass(wb_grid* g, long long p0, int nslots) {
                    box(0, N0 - 1, 0, N1 - 1, 0, N2)};
     wb_launch_ct(A, true, bb, s);
   }
-  wb_launch_final(A, s);
+  wb_launch_final(A, c, s);
+}
+
+// How the grid covers its ghosts (see wb_grid): from d, map and npatch.
+void set_interior(wb_grid* g) {
+  const wb_desc& d = g->d;
+  const bool periodic = d.bc[0] == WB_BC_PERIODIC && d.bc[1] == WB_BC_PERIODIC && d.bc[2] == WB_BC_PERIODIC;
+  const bool one_pass = d.batch_patches == 0 || d.batch_patches >= g->npatch;
+  g->closed = periodic && g->npatch == 1 ? 7 : 0;
+  g->wrap = periodic && g->npatch > 1 && one_pass && !flat_z(&d);
 }
 
 int sync(wb_grid* g, const char* where) {
@@ -473,10 +480,10 @@ int load_common(wb_grid* g, const double* U, const double* bx, const double* by,
       if (rc) return rc;
     }
   }
-  wb_launch_halo(g->q, g->b, g->geo, g->map, s);
-  wb_launch_ccb(g->q, g->b, g->geo, g->npatch, s);
+  if (!g->closed) wb_launch_halo(g->q, g->b, g->geo, g->map, s);
+  wb_launch_ccb(g->q, g->b, g->geo, g->npatch, g->closed, s);
   if (primitive) wb_launch_prim_to_cons(g->q, g->geo, g->npatch, g->phys, s);
-  wb_launch_halo(g->q, g->b, g->geo, g->map, s);
+  if (!g->closed) wb_launch_halo(g->q, g->b, g->geo, g->map, s);
   WbScalars z;
   std::memset(&z, 0, sizeof(z));
   cudaError_t e = cudaMemcpyAsync(g->scal, &z, sizeof(z), cudaMemcpyHostToDevice, s);
@@ -534,8 +541,7 @@ int wb_grid_create(const wb_desc* d, void* dev_mem, size_t bytes, void* stream, 
   }
   g->map.npatch = L.npatch;
   g->npatch = L.npatch;
-  g->wrap = L.S == L.npatch && !flat_z(d) && d->bc[0] == WB_BC_PERIODIC && d->bc[1] == WB_BC_PERIODIC &&
-            d->bc[2] == WB_BC_PERIODIC;
+  set_interior(g);
   g->S = L.S;
   g->phys = wb_phys_of(d);
   g->stream = reinterpret_cast<cudaStream_t>(stream);
@@ -642,6 +648,7 @@ int wb_advance(wb_grid* g, int nsteps, double t_end, double* t_out) {
   // With a time limit, the device clock is read back every kStepsPerCheck
   // steps and the remaining steps (which would do nothing) are not launched.
   constexpr int kStepsPerCheck = 64;
+  bool chained = false;
   for (int st = 0; st < nsteps; ++st) {
     if (t_end > 0.0 && st > 0 && st % kStepsPerCheck == 0) {
       double t_now = 0.0;
@@ -650,12 +657,18 @@ int wb_advance(wb_grid* g, int nsteps, double t_end, double* t_out) {
       if (e != cudaSuccess) return check_cuda(g, e, "advance");
       if (t_now >= t_end) break;
     }
-    wb_launch_dt_step(g->scal, g->d.cfl, t_end, g->d.dt_lag, s);
+    // the previous step's update has prepared this step's dt, unless the clock
+    // was read between the two (it must not count a step that may not come)
+    const bool check_next = t_end > 0.0 && (st + 1) % kStepsPerCheck == 0;
+    StepControl c = {g->d.cfl, t_end, g->d.dt_lag, 0};
+    if (!chained) wb_launch_dt_step(g->scal, c, s);
+    chained = st + 1 < nsteps && !check_next;
     for (long long p0 = 0; p0 < g->npatch; p0 += g->S) {
       int ns = (int)std::min<long long>(g->S, g->npatch - p0);
-      enqueue_pass(g, p0, ns);
+      c.chain = chained && p0 + g->S >= g->npatch;  // in the step's last launch of the update
+      enqueue_pass(g, p0, ns, c);
     }
-    wb_launch_halo(g->q, g->b, g->geo, g->map, s);
+    if (!g->closed) wb_launch_halo(g->q, g->b, g->geo, g->map, s);
   }
   e = cudaGetLastError();
   if (e != cudaSuccess) return check_cuda(g, e, "advance launch");
@@ -729,7 +742,7 @@ int wb_divb_max(wb_grid* g, double* divb) {
   cudaStream_t s = g->stream;
   cudaError_t e = cudaMemsetAsync(g->red, 0, sizeof(unsigned long long), s);
   if (e != cudaSuccess) return check_cuda(g, e, "divb");
-  wb_launch_divb(g->b, g->geo, g->npatch, g->red, s);
+  wb_launch_divb(g->b, g->geo, g->npatch, g->closed, g->red, s);
   unsigned long long bits = 0;
   e = cudaMemcpyAsync(&bits, g->red, sizeof(bits), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -784,6 +797,12 @@ int wb_debug_stage(wb_grid* g, int which, double* out, long long cap, long long*
   long long need = per * (long long)arrays.size();
   if (cap < need) return fail(g, WB_ERR_INVALID, "output too small");
   const double nanv = std::nan("");
+  if (g->closed) {  // the stages leave the high boundary faces to their images
+    WrapList L = wrap_list({});
+    for (const double* a : arrays)
+      if (a) L.a[L.n++] = const_cast<double*>(a);
+    wb_launch_wrap(L, g->geo, g->map, 1, g->stream);
+  }
   for (size_t a = 0; a < arrays.size(); ++a) {
     if (!arrays[a]) {
       for (long long i = 0; i < per; ++i) out[a * per + i] = (which < 6) ? 0.0 : nanv;
@@ -958,13 +977,14 @@ int wb_step_noalloc(const wb_desc* d, const double* U, const double* bx, const d
     double* dst = comp < 5 ? g.q[comp] : g.b[comp - 5];
     wb_launch_scatter(src, dst, comp, g.geo, g.map, s);
   }
-  wb_launch_halo(g.q, g.b, g.geo, g.map, s);
-  wb_launch_ccb(g.q, g.b, g.geo, 1, s);
-  wb_launch_halo(g.q, g.b, g.geo, g.map, s);
+  set_interior(&g);
+  if (!g.closed) wb_launch_halo(g.q, g.b, g.geo, g.map, s);
+  wb_launch_ccb(g.q, g.b, g.geo, 1, g.closed, s);
+  if (!g.closed) wb_launch_halo(g.q, g.b, g.geo, g.map, s);
   wb_launch_dt_init(g.q, g.geo, 1, g.phys, g.scal, s);
-  wb_launch_dt_step(g.scal, one.cfl, 0.0, 0, s);
-  enqueue_pass(&g, 0, 1);
-  wb_launch_halo(g.q, g.b, g.geo, g.map, s);
+  const StepControl c = {one.cfl, 0.0, 0, 0};
+  wb_launch_dt_step(g.scal, c, s);
+  enqueue_pass(&g, 0, 1, c);
   double* outs[3] = {bx_out, by_out, bz_out};
   for (int comp = 0; comp < 8; ++comp) {
     const double* src = comp < 5 ? g.q[comp] : g.b[comp - 5];

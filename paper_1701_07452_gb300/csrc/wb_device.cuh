@@ -101,7 +101,7 @@ struct WbScalars {
   unsigned long long wmax_lag;   // lagged dt: signal rate of the previous step's start state (0: none)
   unsigned long long wmax_next;  // accumulated by the final update for the next step
   unsigned int rate_screen;      // running max of the FP32 screen of the signal rate (float bits)
-  unsigned int pad_;
+  unsigned int blocks_done;      // blocks of the current final update that have finished
   long long steps;
   long long floor_hits;
   long long unphysical;

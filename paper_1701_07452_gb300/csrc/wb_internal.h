@@ -19,8 +19,11 @@ struct SweepArgs {
   WbPhys phys;
   WbScalars* scal;
   int nslots;
+  int closed;              // bit d: the pencils along axis d are periodic and whole
   int ring[3];             // thread layout (wbu::sweep_ring; set at launch)
   long long tile0[4];      // first tile of each axis (set at launch)
+  double* Eref[3];         // predictor: the reference EMF of the zones of ebox too
+  WbBox ebox;              // (Eref[0] null: none)
 };
 
 // Pointers of one pipeline pass over a batch of patches: the view holds the
@@ -31,6 +34,7 @@ struct StageArgs {
   long long slot_q, slot_w;
   WbPhys phys;
   int nslots;
+  int closed;  // axes whose neighbours wrap inside the patch (wbu::neighbours)
   // the final update's view of the domain boundary: slot s holds patch
   // p0 + s of a grid with np[] patches per axis; bit a of ohi_bc is set when
   // axis a is outflow (its high boundary face is a copy of the last owned one)
@@ -47,16 +51,19 @@ struct GridMap {
   long long npatch;
 };
 
-// closed: bit d set when the pencils along axis d are whole and periodic (the
-// last zone is the first one's neighbour)
-void wb_launch_sweeps(SweepArgs a, int closed, cudaStream_t s);
+void wb_launch_sweeps(SweepArgs a, cudaStream_t s);
 
-void wb_launch_eref(const StageArgs& a, const WbBox& box, cudaStream_t s);
 void wb_launch_edges(const StageArgs& a, bool corrector, const WbBox box[3], cudaStream_t s);
 void wb_launch_ct(const StageArgs& a, bool final_step, const WbBox box[3], cudaStream_t s);
 void wb_launch_transverse(const StageArgs& a, const WbBox box[3], cudaStream_t s);
 void wb_launch_eref_half(const StageArgs& a, const WbBox& box, cudaStream_t s);
-void wb_launch_final(const StageArgs& a, cudaStream_t s);
+// The time-step control of a grid (wb_launch_dt_step); chain: another step
+// follows, and the final update's last block prepares its dt.
+struct StepControl {
+  double cfl, t_end;
+  int lag, chain;
+};
+void wb_launch_final(const StageArgs& a, const StepControl& c, cudaStream_t s);
 
 void wb_launch_halo(double* const q[8], double* const b[3], const WbGeo& geo, const GridMap& m,
                     cudaStream_t s);
@@ -72,8 +79,8 @@ struct WrapList {
 void wb_launch_wrap(const WrapList& L, const WbGeo& geo, const GridMap& m, int depth, cudaStream_t s);
 void wb_launch_dt_init(double* const q[8], const WbGeo& geo, long long npatch, const WbPhys& ph,
                        WbScalars* scal, cudaStream_t s);
-void wb_launch_dt_step(WbScalars* scal, double cfl, double t_end, int lag, cudaStream_t s);
-void wb_launch_ccb(double* const q[8], double* const b[3], const WbGeo& geo, long long npatch,
+void wb_launch_dt_step(WbScalars* scal, const StepControl& c, cudaStream_t s);
+void wb_launch_ccb(double* const q[8], double* const b[3], const WbGeo& geo, long long npatch, int closed,
                    cudaStream_t s);
 void wb_launch_prim_to_cons(double* const q[8], const WbGeo& geo, long long npatch,
                             const WbPhys& ph, cudaStream_t s);
@@ -86,7 +93,7 @@ void wb_launch_gather(const double* src_field, double* dst, int comp, const WbGe
 // totals x vol in out (device memory).
 void wb_launch_totals(double* const q[8], double* const b[3], const WbGeo& geo, long long npatch, double vol,
                       double* part, int nblocks, double* out, cudaStream_t s);
-void wb_launch_divb(double* const b[3], const WbGeo& geo, long long npatch,
+void wb_launch_divb(double* const b[3], const WbGeo& geo, long long npatch, int closed,
                     unsigned long long* out_bits, cudaStream_t s);
 void wb_launch_copy_box(const double* src, long long slot, const WbGeo& geo, const WbBox& box,
                         double* dst, cudaStream_t s);

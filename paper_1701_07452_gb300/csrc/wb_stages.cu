@@ -27,14 +27,6 @@ inline dim3 grid_for(long long n, int nslots, int bs) {
   return dim3((unsigned)((n + bs - 1) / bs), (unsigned)nslots);
 }
 
-// Step 2: zone-centred reference EMF from q^n.
-__global__ void k_eref(StageArgs A, WbBox box) {
-  if (!wb_pos(A.v.scal->dt)) return;
-  int i, j, k;
-  if (!box_index(box, blockIdx.x * (long long)blockDim.x + threadIdx.x, i, j, k)) return;
-  wbu::eref(A.v, blockIdx.y * A.slot_q, blockIdx.y * A.slot_w, i, j, k);
-}
-
 inline WbBox box_union(const WbBox b[3]) {
   WbBox u = b[0];
   for (int n = 1; n < 3; ++n)
@@ -57,9 +49,10 @@ __global__ void k_edges(StageArgs A, bool corr, Boxes3 B) {
   int i, j, k;
   if (!box_index(B.u, blockIdx.x * (long long)blockDim.x + threadIdx.x, i, j, k)) return;
   const long long wo = blockIdx.y * A.slot_w;
-  if (wbu::in_box(B.b[0], i, j, k)) wbu::edge<0>(A.v, wo, corr, i, j, k);
-  if (wbu::in_box(B.b[1], i, j, k)) wbu::edge<1>(A.v, wo, corr, i, j, k);
-  if (wbu::in_box(B.b[2], i, j, k)) wbu::edge<2>(A.v, wo, corr, i, j, k);
+  const wbu::Nbr nb = wbu::neighbours(A.v.geo, i, j, k, A.closed);
+  if (wbu::in_box(B.b[0], i, j, k)) wbu::edge<0>(A.v, wo, corr, i, j, k, nb);
+  if (wbu::in_box(B.b[1], i, j, k)) wbu::edge<1>(A.v, wo, corr, i, j, k, nb);
+  if (wbu::in_box(B.b[2], i, j, k)) wbu::edge<2>(A.v, wo, corr, i, j, k, nb);
 }
 
 // Steps 4 and 11: constrained transport of the three face components.
@@ -69,9 +62,10 @@ __global__ void k_ct(StageArgs A, bool fin, Boxes3 B) {
   int i, j, k;
   if (!box_index(B.u, blockIdx.x * (long long)blockDim.x + threadIdx.x, i, j, k)) return;
   const long long qo = blockIdx.y * A.slot_q, wo = blockIdx.y * A.slot_w;
-  if (wbu::in_box(B.b[0], i, j, k)) wbu::ct<0>(A.v, qo, wo, fin, dt, i, j, k);
-  if (wbu::in_box(B.b[1], i, j, k)) wbu::ct<1>(A.v, qo, wo, fin, dt, i, j, k);
-  if (wbu::in_box(B.b[2], i, j, k)) wbu::ct<2>(A.v, qo, wo, fin, dt, i, j, k);
+  const wbu::Nbr nb = wbu::neighbours(A.v.geo, i, j, k, A.closed);
+  if (wbu::in_box(B.b[0], i, j, k)) wbu::ct<0>(A.v, qo, wo, fin, dt, i, j, k, nb);
+  if (wbu::in_box(B.b[1], i, j, k)) wbu::ct<1>(A.v, qo, wo, fin, dt, i, j, k, nb);
+  if (wbu::in_box(B.b[2], i, j, k)) wbu::ct<2>(A.v, qo, wo, fin, dt, i, j, k, nb);
 }
 
 // Steps 5 and 7: the three transverse-flux preconditioned states, all
@@ -85,8 +79,9 @@ __global__ void k_transverse(StageArgs A, Boxes3 B) {
                    (wbu::in_box(B.b[2], i, j, k) ? 4 : 0);
   // zones that need every direction take the mask as a constant: with a run-time
   // mask the compiler recomputes shared zone terms (13 FP64 instructions a zone)
-  if (mask == 7) wbu::transverse_set(A.v, blockIdx.y * A.slot_q, blockIdx.y * A.slot_w, dt, 7, i, j, k);
-  else if (mask) wbu::transverse_set(A.v, blockIdx.y * A.slot_q, blockIdx.y * A.slot_w, dt, mask, i, j, k);
+  const wbu::Nbr nb = wbu::neighbours(A.v.geo, i, j, k, A.closed);
+  if (mask == 7) wbu::transverse_set(A.v, blockIdx.y * A.slot_q, blockIdx.y * A.slot_w, dt, 7, i, j, k, nb);
+  else if (mask) wbu::transverse_set(A.v, blockIdx.y * A.slot_q, blockIdx.y * A.slot_w, dt, mask, i, j, k, nb);
 }
 
 // Step 8: half-step reference EMF.
@@ -95,11 +90,13 @@ __global__ void k_eref_half(StageArgs A, WbBox box) {
   if (!wb_pos(dt)) return;
   int i, j, k;
   if (!box_index(box, blockIdx.x * (long long)blockDim.x + threadIdx.x, i, j, k)) return;
-  wbu::eref_half(A.v, blockIdx.y * A.slot_q, blockIdx.y * A.slot_w, dt, i, j, k);
+  wbu::eref_half(A.v, blockIdx.y * A.slot_q, blockIdx.y * A.slot_w, dt, i, j, k,
+                 wbu::neighbours(A.v.geo, i, j, k, A.closed));
 }
 
 // Periodic images of intermediate arrays of a single-patch box that is
-// periodic on every axis: each ghost point within `depth` zones of the
+// periodic on every axis (its stages read across the ends themselves; stage
+// dumps want the high boundary faces): each ghost point within `depth` zones of the
 // interior takes the value computed at the interior point it is an image of
 // (the same function of the same inputs, so the copy equals a recomputation
 // bit for bit).  One thread per shell point.
@@ -154,14 +151,54 @@ __device__ __forceinline__ void block_max_atomic(double w, unsigned long long* d
   if ((threadIdx.x & 31) == 0 && bits) atomicMax(dst, bits);
 }
 
+// dt of the next step from the signal rate of its start state (reading R3),
+// or with lag from the rate of the previous step's start state (the paper
+// delays the dt reduction by one step to overlap it with work; the first two
+// steps both use the loaded state's rate)
+__device__ void dt_step(volatile WbScalars* s, const StepControl& c) {
+  const double w_now = __longlong_as_double((long long)s->wmax_next);
+  const double t_end = c.t_end;
+  double w = w_now;
+  if (c.lag) {
+    const double wl = __longlong_as_double((long long)s->wmax_lag);
+    if (wl > 0.0) w = wl;
+  }
+  double dt = c.cfl / w;
+  bool ok = (w > 0.0) && isfinite(w) && isfinite(dt) && dt > 0.0 && (w_now > 0.0) && isfinite(w_now);
+  bool last = false;
+  if (t_end > 0.0) {
+    double rem = t_end - s->t;
+    if (!(rem > 0.0)) { s->dt = 0.0; return; }  // past t_end: skip, keep the rate
+    // the step that reaches t_end lands on it exactly and leaves no sliver
+    // below 1e-10 of a step (a near-zero dt still carries the eps_k
+    // dissipation of Q_k and dx/(2 dt) overflows the flux scale)
+    if (ok && dt >= rem * (1.0 - 1e-10)) { dt = rem; last = true; }
+  }
+  if (!ok) {
+    s->dt = 0.0;
+    s->unphysical += 1;
+    return;
+  }
+  s->dt = dt;
+  s->t = last ? t_end : s->t + dt;
+  if (c.lag) s->wmax_lag = s->wmax_next;
+  s->steps += 1;
+  s->wmax_next = 0ULL;
+  s->rate_screen = 0u;
+}
+
 // Step 10 (+ zone field of Step 11, floors, next signal rate) on interior zones.
-__global__ void k_final(StageArgs A) {
+// With a step to follow (c.chain) the last block to finish prepares its dt; a
+// launch that has nothing to do (dt = 0) still does that, as a launch of
+// k_dt_step would.
+__global__ void k_final(StageArgs A, StepControl c) {
   const double dt = A.v.scal->dt;
-  if (!wb_pos(dt)) return;
+  const bool run = wb_pos(dt);
+  if (!run && !c.chain) return;
   const WbGeo& g = A.v.geo;
   WbBox box = {{0, 0, 0}, {g.n[0] - 1, g.n[1] - 1, g.n[2] - 1}};
   int i, j, k;
-  const bool ok = box_index(box, blockIdx.x * (long long)blockDim.x + threadIdx.x, i, j, k);
+  const bool ok = run && box_index(box, blockIdx.x * (long long)blockDim.x + threadIdx.x, i, j, k);
   double w = 0.0;
   int hits = 0, bad = 0;
   // axes along which this slot's patch is the last one of an outflow axis
@@ -172,10 +209,21 @@ __global__ void k_final(StageArgs A) {
   for (int d = 0; d < 3; ++d)
     if (((A.ohi_bc >> d) & 1) && pc[d] == A.np[d] - 1) ohi |= 1 << d;
   if (ok) w = wbu::final_update(A.v, blockIdx.y * A.slot_q, blockIdx.y * A.slot_w, dt, A.phys, i, j, k,
-                                ohi, &hits, &bad);
+                                wbu::neighbours(g, i, j, k, A.closed), ohi, &hits, &bad);
   if (hits) atomicAdd((unsigned long long*)&A.v.scal->floor_hits, (unsigned long long)hits);
   if (bad) atomicAdd((unsigned long long*)&A.v.scal->unphysical, (unsigned long long)bad);
-  block_max_atomic(w, &A.v.scal->wmax_next);
+  if (run) block_max_atomic(w, &A.v.scal->wmax_next);
+  if (c.chain) {
+    __syncthreads();  // the block's atomics precede thread 0's fence and count
+    if (threadIdx.x == 0) {
+      __threadfence();
+      if (atomicAdd(&A.v.scal->blocks_done, 1u) == gridDim.x * gridDim.y - 1) {
+        A.v.scal->blocks_done = 0u;
+        __threadfence();
+        dt_step(A.v.scal, c);
+      }
+    }
+  }
 }
 
 // Ghost fill of every patch: zone (i,j,k) outside the interior copies the
@@ -237,40 +285,7 @@ __global__ void k_dt_init(StageArgs A, long long npatch) {
   block_max_atomic(w, &A.v.scal->wmax_next);
 }
 
-// dt of the next step from the signal rate of its start state (reading R3),
-// or with lag from the rate of the previous step's start state (the paper
-// delays the dt reduction by one step to overlap it with work; the first two
-// steps both use the loaded state's rate)
-__global__ void k_dt_step(WbScalars* s, double cfl, double t_end, int lag) {
-  const double w_now = __longlong_as_double((long long)s->wmax_next);
-  double w = w_now;
-  if (lag) {
-    const double wl = __longlong_as_double((long long)s->wmax_lag);
-    if (wl > 0.0) w = wl;
-  }
-  double dt = cfl / w;
-  bool ok = (w > 0.0) && isfinite(w) && isfinite(dt) && dt > 0.0 && (w_now > 0.0) && isfinite(w_now);
-  bool last = false;
-  if (t_end > 0.0) {
-    double rem = t_end - s->t;
-    if (!(rem > 0.0)) { s->dt = 0.0; return; }  // past t_end: skip, keep the rate
-    // the step that reaches t_end lands on it exactly and leaves no sliver
-    // below 1e-10 of a step (a near-zero dt still carries the eps_k
-    // dissipation of Q_k and dx/(2 dt) overflows the flux scale)
-    if (ok && dt >= rem * (1.0 - 1e-10)) { dt = rem; last = true; }
-  }
-  if (!ok) {
-    s->dt = 0.0;
-    s->unphysical += 1;
-    return;
-  }
-  s->dt = dt;
-  s->t = last ? t_end : s->t + dt;
-  if (lag) s->wmax_lag = s->wmax_next;
-  s->steps += 1;
-  s->wmax_next = 0ULL;
-  s->rate_screen = 0u;
-}
+__global__ void k_dt_step(WbScalars* s, StepControl c) { dt_step(s, c); }
 
 __global__ void k_ccb(StageArgs A, long long npatch) {
   const WbGeo& g = A.v.geo;
@@ -282,9 +297,9 @@ __global__ void k_ccb(StageArgs A, long long npatch) {
   int j = (int)((r / g.n[0]) % g.n[1]);
   int k = (int)(r / ((long long)g.n[0] * g.n[1]));
   long long o = p * g.V + wb_at(g, i, j, k);
-  const long long s[3] = {1, g.sy, g.sz};
+  const wbu::Nbr nb = wbu::neighbours(g, i, j, k, A.closed);
 #pragma unroll
-  for (int e = 0; e < 3; ++e) A.v.q[F_BX + e][o] = 0.5 * (A.v.b[e][o] + A.v.b[e][o + s[e]]);
+  for (int e = 0; e < 3; ++e) A.v.q[F_BX + e][o] = 0.5 * (A.v.b[e][o] + A.v.b[e][o + nb.up[e]]);
 }
 
 // primitive (rho, v, P) in fields 0..4 -> conserved, with the zone field (Eq. totenergy)
@@ -319,6 +334,10 @@ __global__ void k_move(const double* src, double* dst, int comp, WbGeo g, GridMa
   G[0] = (int)(t % ext[0]);
   G[1] = (int)((t / ext[0]) % ext[1]);
   G[2] = (int)(t / ((long long)ext[0] * ext[1]));
+  // a read takes the high boundary face from the owned face it is an image of
+  // (periodic: the first, outflow: the last), not from a ghost
+  if (!SCATTER && comp >= 5 && G[comp - 5] == m.N[comp - 5])
+    G[comp - 5] = m.bc[comp - 5] == 0 ? 0 : m.N[comp - 5] - 1;
   long long patch = 0, mul = 1;
   int loc[3];
 #pragma unroll
@@ -350,8 +369,9 @@ __global__ void k_divb(StageArgs A, long long npatch, unsigned long long* out) {
     int j = (int)((r / g.n[0]) % g.n[1]);
     int k = (int)(r / ((long long)g.n[0] * g.n[1]));
     long long o = p * g.V + wb_at(g, i, j, k);
-    double dv = (A.v.b[0][o + 1] - A.v.b[0][o]) * g.idx[0] + (A.v.b[1][o + g.sy] - A.v.b[1][o]) * g.idx[1] +
-                (A.v.b[2][o + g.sz] - A.v.b[2][o]) * g.idx[2];
+    const wbu::Nbr nb = wbu::neighbours(g, i, j, k, A.closed);
+    double dv = (A.v.b[0][o + nb.up[0]] - A.v.b[0][o]) * g.idx[0] + (A.v.b[1][o + nb.up[1]] - A.v.b[1][o]) * g.idx[1] +
+                (A.v.b[2][o + nb.up[2]] - A.v.b[2][o]) * g.idx[2];
     w = fabs(dv);
   }
   block_max_atomic(w, out);
@@ -468,10 +488,6 @@ Boxes3 boxes3(const WbBox b[3]) {
 
 }  // namespace
 
-void wb_launch_eref(const StageArgs& a, const WbBox& box, cudaStream_t s) {
-  k_eref<<<grid_for(box_count(box), a.nslots, 256), 256, 0, s>>>(a, box);
-}
-
 void wb_launch_edges(const StageArgs& a, bool corr, const WbBox box[3], cudaStream_t s) {
   Boxes3 B = boxes3(box);
   k_edges<<<grid_for(box_count(B.u), a.nslots, 256), 256, 0, s>>>(a, corr, B);
@@ -491,9 +507,9 @@ void wb_launch_eref_half(const StageArgs& a, const WbBox& box, cudaStream_t s) {
   k_eref_half<<<grid_for(box_count(box), a.nslots, 256), 256, 0, s>>>(a, box);
 }
 
-void wb_launch_final(const StageArgs& a, cudaStream_t s) {
+void wb_launch_final(const StageArgs& a, const StepControl& c, cudaStream_t s) {
   long long n = (long long)a.v.geo.n[0] * a.v.geo.n[1] * a.v.geo.n[2];
-  k_final<<<grid_for(n, a.nslots, 256), 256, 0, s>>>(a);
+  k_final<<<grid_for(n, a.nslots, 256), 256, 0, s>>>(a, c);
 }
 
 void wb_launch_halo(double* const q[8], double* const b[3], const WbGeo& geo, const GridMap& m,
@@ -518,13 +534,14 @@ void wb_launch_dt_init(double* const q[8], const WbGeo& geo, long long npatch, c
   k_dt_init<<<grid_for(n, 1, 256), 256, 0, s>>>(a, npatch);
 }
 
-void wb_launch_dt_step(WbScalars* scal, double cfl, double t_end, int lag, cudaStream_t s) {
-  k_dt_step<<<1, 1, 0, s>>>(scal, cfl, t_end, lag);
+void wb_launch_dt_step(WbScalars* scal, const StepControl& c, cudaStream_t s) {
+  k_dt_step<<<1, 1, 0, s>>>(scal, c);
 }
 
-void wb_launch_ccb(double* const q[8], double* const b[3], const WbGeo& geo, long long npatch,
+void wb_launch_ccb(double* const q[8], double* const b[3], const WbGeo& geo, long long npatch, int closed,
                    cudaStream_t s) {
   StageArgs a = mini_args(q, b, geo);
+  a.closed = closed;
   long long n = (long long)geo.n[0] * geo.n[1] * geo.n[2] * npatch;
   k_ccb<<<grid_for(n, 1, 256), 256, 0, s>>>(a, npatch);
 }
@@ -553,10 +570,11 @@ void wb_launch_gather(const double* src_field, double* dst, int comp, const WbGe
   k_move<false><<<grid_for(n, 1, 256), 256, 0, s>>>(src_field, dst, comp, geo, m);
 }
 
-void wb_launch_divb(double* const b[3], const WbGeo& geo, long long npatch,
+void wb_launch_divb(double* const b[3], const WbGeo& geo, long long npatch, int closed,
                     unsigned long long* out_bits, cudaStream_t s) {
   double* q[8] = {};
   StageArgs a = mini_args(q, b, geo);
+  a.closed = closed;
   long long n = (long long)geo.n[0] * geo.n[1] * geo.n[2] * npatch;
   k_divb<<<grid_for(n, 1, 256), 256, 0, s>>>(a, npatch, out_bits);
 }

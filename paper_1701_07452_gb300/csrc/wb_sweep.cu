@@ -3,7 +3,8 @@
 // for the predictor fluxes of Step 1 and the corrector fluxes of Steps 6-7 of
 // the 3D CTU+CT integrator (Sec. "MHD in Three Dimensions").
 //
-// One launch takes the three axes, one thread one face: it builds the
+// One launch takes the three axes (and the predictor's the reference EMF of
+// Step 2, whose short blocks fill the tail), one thread one face: it builds the
 // Roe-averaged interface state (a Cargo-Gallice type average, App. A), the
 // characteristic amplitudes alpha_k, nu_k = (dt/dx) a_k and g-tilde_k, trades
 // g-tilde and limited slopes with its neighbours along the pencil and emits the
@@ -40,9 +41,29 @@ __global__ void __launch_bounds__(wbu::kBlock, wbu::kSweepBlocks) k_sweep(SweepA
   const double dt = *A.dt;
   if (!wb_pos(dt)) return;
   const long long t = blockIdx.x;
+  if (t >= A.tile0[3]) {  // Step 2: zone-centred reference EMF from q^n, one zone a thread
+    const WbBox& e = A.ebox;
+    const int nx = e.hi[0] - e.lo[0] + 1, ny = e.hi[1] - e.lo[1] + 1, nz = e.hi[2] - e.lo[2] + 1;
+    const long long z = (t - A.tile0[3]) * wbu::kBlock + threadIdx.x, per = (long long)nx * ny * nz;
+    if (z >= per * A.nslots) return;
+    const long long slot = z / per, r = z - slot * per;
+    const long long at = wb_at(A.geo, e.lo[0] + (int)(r % nx), e.lo[1] + (int)(r / nx % ny), e.lo[2] + (int)(r / nx / ny));
+    const double* const* q = A.s[0].q;  // the x frame: rho, Mx, My, Mz, E, Bx, By, Bz
+    const long long o = slot * A.slot_in + at;
+    wbu::ErefIn in;
+    in.w = slot * A.slot_out + at;
+    in.rho = __ldg(q[0] + o);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      in.m[c] = __ldg(q[1 + c] + o);
+      in.B[c] = __ldg(q[5 + c] + o);
+    }
+    wbu::eref_finish(A.Eref, in);
+    return;
+  }
   const int d = t >= A.tile0[2] ? 2 : (t >= A.tile0[1] ? 1 : 0);
-  const int hll = wbu::sweep_tile<EZ, PROT, true>(A.geo, A.box[d], d, A.s[d], t - A.tile0[d], A.ring[d] != 0, A.nslots,
-                                                  A.slot_in, A.slot_out, dt, A.phys, X);
+  const int hll = wbu::sweep_tile<EZ, PROT, true>(A.geo, A.box[d], d, A.s[d], t - A.tile0[d], (A.closed >> d) & 1, A.ring[d] != 0,
+                                                  A.nslots, A.slot_in, A.slot_out, dt, A.phys, X);
   if (hll) atomicAdd((unsigned long long*)&A.scal->hll_faces, 1ULL);
 }
 
@@ -50,17 +71,23 @@ __global__ void __launch_bounds__(wbu::kBlock, wbu::kSweepBlocks) k_sweep(SweepA
 
 // Kernel variants: eps_k = 0 on the linearly degenerate waves (the default)
 // or general eps; protection floors off (the default) or on.
-void wb_launch_sweeps(SweepArgs a, int closed, cudaStream_t s) {
+void wb_launch_sweeps(SweepArgs a, cudaStream_t s) {
   a.tile0[0] = 0;
   for (int d = 0; d < 3; ++d) {
     const int U = d == 0 ? 1 : 0, W = d == 2 ? 1 : 2;
     const WbBox& b = a.box[d];
     const int len = b.hi[d] - b.lo[d] + 1;
-    a.ring[d] = wbu::sweep_ring(len, (closed >> d) & 1);
+    a.ring[d] = wbu::sweep_ring(len, (a.closed >> d) & 1);
     a.tile0[d + 1] = a.tile0[d] + wbu::sweep_tiles((long long)(b.hi[U] - b.lo[U] + 1) * (b.hi[W] - b.lo[W] + 1) * a.nslots,
                                                    len, a.ring[d] != 0);
   }
-  const dim3 grid((unsigned)a.tile0[3]);
+  long long tiles = a.tile0[3];
+  if (a.Eref[0]) {
+    long long z = a.nslots;
+    for (int d = 0; d < 3; ++d) z *= a.ebox.hi[d] - a.ebox.lo[d] + 1;
+    tiles += (z + wbu::kBlock - 1) / wbu::kBlock;
+  }
+  const dim3 grid((unsigned)tiles);
   const bool ez = (a.phys.eps_zero & kEpsZeroLD) == kEpsZeroLD;
   if (a.phys.prot) {
     if (ez) k_sweep<kEpsZeroLD, true><<<grid, wbu::kBlock, 0, s>>>(a);

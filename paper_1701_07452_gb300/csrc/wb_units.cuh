@@ -508,8 +508,8 @@ __host__ __device__ __forceinline__ long long sweep_tiles(long long npen, int le
 // 2 warps per scheduler; one face per thread needs 168, 3 warps.
 template <int EZ, bool PROT, bool NC>
 __device__ __forceinline__ int sweep_tile(const WbGeo& g, const WbBox& box, int d, const SweepFrame& s, long long tile,
-                                          bool ring, int nslots, long long slot_in, long long slot_out, double dt,
-                                          const WbPhys& P, LaneEdge& X) {
+                                          bool closed, bool ring, int nslots, long long slot_in, long long slot_out,
+                                          double dt, const WbPhys& P, LaneEdge& X) {
   const int U = d == 0 ? 1 : 0, W = d == 2 ? 1 : 2;
   const int nu = box.hi[U] - box.lo[U] + 1, nw = box.hi[W] - box.lo[W] + 1;
   const int len = box.hi[d] - box.lo[d] + 1;
@@ -539,6 +539,9 @@ __device__ __forceinline__ int sweep_tile(const WbGeo& g, const WbBox& box, int 
     emit = emit && idx >= 0 && idx < len && t >= 2 && t <= kBlock - 2;
     left = (lane + 31) % 32;
     right = (lane + 1) % 32;
+    // the zones past the ends of a closed pencil are those of its other end
+    // (an open layout is only taken for 3 zones or more, see sweep_ring)
+    if (closed) idx = idx < 0 ? idx + len : (idx >= len ? idx - len : idx);
   }
   const long long slot = pen / ((long long)nu * nw);
   const int r = (int)(pen - slot * nu * nw);
@@ -572,7 +575,8 @@ __device__ __forceinline__ int sweep_tile(const WbGeo& g, const WbBox& box, int 
   bool hll = false;
   if (code) {
     if (has_left) {
-      const long long st = d == 0 ? 1LL : (d == 1 ? g.sy : g.sz);
+      long long st = d == 0 ? 1LL : (d == 1 ? g.sy : g.sz);
+      if (closed && idx == 0) st *= 1 - len;
       hll_face(L, R, ld<NC>(s.q[5] + off - st), ld<NC>(s.q[5] + off), code == 1, P, f);
       hll = true;
     }
@@ -632,6 +636,25 @@ __device__ __forceinline__ bool in_box(const WbBox& b, int i, int j, int k) {
 // arithmetic is written with explicit rounding: an item gives the same bits
 // whichever inlined copy (first or second of a pair, or alone) handles it.
 
+// Offsets to the high and low neighbours of a zone along each axis.  closed:
+// bit d set when axis d is periodic and whole in this patch; the neighbour of
+// its last zone is then its first one, so no stage of such a box reads a ghost.
+struct Nbr {
+  long long up[3], dn[3];
+};
+__device__ __forceinline__ Nbr neighbours(const WbGeo& g, int i, int j, int k, int closed) {
+  const int x[3] = {i, j, k};
+  const long long s[3] = {1, g.sy, g.sz};
+  Nbr b;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const bool c = (closed >> d) & 1;
+    b.up[d] = c && x[d] == g.n[d] - 1 ? -(g.n[d] - 1) * s[d] : s[d];
+    b.dn[d] = c && x[d] == 0 ? (g.n[d] - 1) * s[d] : -s[d];
+  }
+  return b;
+}
+
 // Step 2: zone-centred reference EMF E = -v x B from q^n.
 struct ErefIn {
   long long w;
@@ -650,19 +673,19 @@ __device__ __forceinline__ void eref_load(const WbView& v, long long qo, long lo
   }
 }
 
-__device__ __forceinline__ void eref_finish(const WbView& v, const ErefIn& in) {
+__device__ __forceinline__ void eref_finish(double* const* E, const ErefIn& in) {
   const double ir = wb_rcp(in.rho);
   const double vx = __dmul_rn(in.m[0], ir), vy = __dmul_rn(in.m[1], ir), vz = __dmul_rn(in.m[2], ir);
   const double bx = in.B[0], by = in.B[1], bz = in.B[2];
-  v.Eref[0][in.w] = __fma_rn(vz, by, __dmul_rn(-vy, bz));
-  v.Eref[1][in.w] = __fma_rn(vx, bz, __dmul_rn(-vz, bx));
-  v.Eref[2][in.w] = __fma_rn(vy, bx, __dmul_rn(-vx, by));
+  E[0][in.w] = __fma_rn(vz, by, __dmul_rn(-vy, bz));
+  E[1][in.w] = __fma_rn(vx, bz, __dmul_rn(-vz, bx));
+  E[2][in.w] = __fma_rn(vy, bx, __dmul_rn(-vx, by));
 }
 
 __device__ __forceinline__ void eref(const WbView& v, long long qo, long long wo, int i, int j, int k) {
   ErefIn in;
   eref_load(v, qo, wo, i, j, k, in);
-  eref_finish(v, in);
+  eref_finish(v.Eref, in);
 }
 
 // The mean of the two one-sided differences, for a zero mass flux.  Not
@@ -701,13 +724,12 @@ struct EdgeIn {
 };
 
 template <int C>
-__device__ __forceinline__ void edge_load(const WbView& v, long long wo, bool corr, int i, int j, int k,
+__device__ __forceinline__ void edge_load(const WbView& v, long long wo, bool corr, int i, int j, int k, const Nbr& nb,
                                           EdgeIn& in) {
   constexpr int a = (C + 1) % 3, b = (C + 2) % 3;
   const WbGeo& g = v.geo;
   const long long o = wo + wb_at(g, i, j, k);
-  const long long sa = a == 0 ? 1 : (a == 1 ? g.sy : g.sz);
-  const long long sb = b == 0 ? 1 : (b == 1 ? g.sy : g.sz);
+  const long long sa = -nb.dn[a], sb = -nb.dn[b];
   WB_CHECK_ZONE(g, i - (a == 0) - (b == 0), j - (a == 1) - (b == 1), k - (a == 2) - (b == 2));
   double* const* Fa = corr ? v.Fc[a] : v.Fp[a];
   double* const* Fb = corr ? v.Fc[b] : v.Fp[b];
@@ -738,9 +760,9 @@ __device__ __forceinline__ void edge_finish(const WbView& v, bool corr, const Ed
 }
 
 template <int C>
-__device__ __forceinline__ void edge(const WbView& v, long long wo, bool corr, int i, int j, int k) {
+__device__ __forceinline__ void edge(const WbView& v, long long wo, bool corr, int i, int j, int k, const Nbr& nb) {
   EdgeIn in;
-  edge_load<C>(v, wo, corr, i, j, k, in);
+  edge_load<C>(v, wo, corr, i, j, k, nb, in);
   edge_finish<C>(v, corr, in);
 }
 
@@ -753,13 +775,12 @@ struct CtIn {
 
 template <int D>
 __device__ __forceinline__ void ct_load(const WbView& v, long long qo, long long wo, bool fin, int i, int j,
-                                        int k, CtIn& in) {
+                                        int k, const Nbr& nb, CtIn& in) {
   constexpr int a = (D + 1) % 3, b = (D + 2) % 3;
   const WbGeo& g = v.geo;
   in.w = wo + wb_at(g, i, j, k);
   in.q = qo + wb_at(g, i, j, k);
-  const long long sa = a == 0 ? 1 : (a == 1 ? g.sy : g.sz);
-  const long long sb = b == 0 ? 1 : (b == 1 ? g.sy : g.sz);
+  const long long sa = nb.up[a], sb = nb.up[b];
   WB_CHECK_ZONE(g, i + (a == 0), j + (a == 1), k + (a == 2));
   WB_CHECK_ZONE(g, i + (b == 0), j + (b == 1), k + (b == 2));
   const double* Eb = fin ? v.Eedgeh[b] : v.Eedge[b];
@@ -783,9 +804,9 @@ __device__ __forceinline__ void ct_finish(const WbView& v, bool fin, double dt, 
 
 template <int D>
 __device__ __forceinline__ void ct(const WbView& v, long long qo, long long wo, bool fin, double dt,
-                                   int i, int j, int k) {
+                                   int i, int j, int k, const Nbr& nb) {
   CtIn in;
-  ct_load<D>(v, qo, wo, fin, i, j, k, in);
+  ct_load<D>(v, qo, wo, fin, i, j, k, nb, in);
   ct_finish<D>(v, fin, dt, in);
 }
 
@@ -806,9 +827,9 @@ struct TransZone {
 };
 
 __device__ __forceinline__ void trans_zone(const WbView& v, long long q, long long w, double dt,
-                                           int need, TransZone& z) {
+                                           int need, const Nbr& nb, TransZone& z) {
   const WbGeo& g = v.geo;
-  const long long s[3] = {1, g.sy, g.sz};
+  const long long (&s)[3] = nb.up;
   const double hdt = wb_half(dt);
 #pragma unroll
   for (int cc = 0; cc < 8; ++cc) z.qn[cc] = v.q[cc][q];
@@ -834,9 +855,9 @@ __device__ __forceinline__ void trans_zone(const WbView& v, long long q, long lo
 // q^{n+1/2}_D of one zone from its shared quantities.  The t1 (t2) field
 // component is carried only by the t2 (t1) sweep; density has no source.
 template <int D>
-__device__ __forceinline__ void trans_dir(const WbView& v, long long w, const TransZone& z) {
+__device__ __forceinline__ void trans_dir(const WbView& v, long long w, const Nbr& nb, const TransZone& z) {
   constexpr int t1 = (D + 1) % 3, t2 = (D + 2) % 3;
-  const long long sD = D == 0 ? 1 : (D == 1 ? v.geo.sy : v.geo.sz);
+  const long long sD = nb.up[D];
   const double hm2 = wb_minmod(z.hdb[D], wb_flip(z.hdb[t1]));  // for the t2 field component
   const double hm1 = wb_minmod(z.hdb[D], wb_flip(z.hdb[t2]));  // for the t1 field component
   const double hSe = __fma_rn(z.Bv[t1], hm1, __dmul_rn(z.Bv[t2], hm2));
@@ -857,7 +878,7 @@ __device__ __forceinline__ void trans_dir(const WbView& v, long long w, const Tr
 // The directions in mask (bit d) at one zone, sharing the zone quantities and
 // each transverse flux difference between the two states that use it.
 __device__ __forceinline__ void transverse_set(const WbView& v, long long qo, long long wo, double dt,
-                                               int mask, int i, int j, int k) {
+                                               int mask, int i, int j, int k, const Nbr& nb) {
   const long long q = qo + wb_at(v.geo, i, j, k);
   const long long w = wo + wb_at(v.geo, i, j, k);
   WB_CHECK_ZONE(v.geo, i + 1, j + 1, k + 1);  // the high neighbours of every axis
@@ -867,10 +888,10 @@ __device__ __forceinline__ void transverse_set(const WbView& v, long long qo, lo
   for (int e = 0; e < 3; ++e)
     if (mask & ~(1 << e)) need |= 1 << e;
   TransZone z;
-  trans_zone(v, q, w, dt, need, z);
-  if (mask & 1) trans_dir<0>(v, w, z);
-  if (mask & 2) trans_dir<1>(v, w, z);
-  if (mask & 4) trans_dir<2>(v, w, z);
+  trans_zone(v, q, w, dt, need, nb, z);
+  if (mask & 1) trans_dir<0>(v, w, nb, z);
+  if (mask & 2) trans_dir<1>(v, w, nb, z);
+  if (mask & 4) trans_dir<2>(v, w, nb, z);
 }
 
 // Step 8: reference EMF at n+1/2 from v of q^n - dt/2 div F* and B = mean of
@@ -883,11 +904,11 @@ struct ErefHalfIn {
 };
 
 __device__ __forceinline__ void eref_half_load(const WbView& v, long long qo, long long wo, int i, int j,
-                                               int k, ErefHalfIn& in) {
+                                               int k, const Nbr& nb, ErefHalfIn& in) {
   const WbGeo& g = v.geo;
   const long long q = qo + wb_at(g, i, j, k);
   const long long w = wo + wb_at(g, i, j, k);
-  const long long s[3] = {1, g.sy, g.sz};
+  const long long (&s)[3] = nb.up;
   WB_CHECK_ZONE(g, i + 1, j + 1, k + 1);
   in.w = w;
 #pragma unroll
@@ -925,9 +946,9 @@ __device__ __forceinline__ void eref_half_finish(const WbView& v, double dt, con
 }
 
 __device__ __forceinline__ void eref_half(const WbView& v, long long qo, long long wo, double dt,
-                                          int i, int j, int k) {
+                                          int i, int j, int k, const Nbr& nb) {
   ErefHalfIn in;
-  eref_half_load(v, qo, wo, i, j, k, in);
+  eref_half_load(v, qo, wo, i, j, k, nb, in);
   eref_half_finish(v, dt, in);
 }
 
@@ -1061,20 +1082,20 @@ __device__ __forceinline__ double signal_rate(double rho, double mx, double my, 
 // zero-gradient rule); the last zone's field then averages that copy, so the
 // stored state is the one a load of the same faces gives.
 __device__ __forceinline__ double final_update(const WbView& v, long long qo, long long wo,
-                                               double dt, const WbPhys& P, int i, int j, int k,
+                                               double dt, const WbPhys& P, int i, int j, int k, const Nbr& nb,
                                                int ohi, int* hits, int* bad) {
   const WbGeo& g = v.geo;
   const long long q = qo + wb_at(g, i, j, k);
   const long long wi = wo + wb_at(g, i, j, k);
   WB_CHECK_ZONE(g, i + 1, j + 1, k + 1);
-  const long long s[3] = {1, g.sy, g.sz};
+  const long long (&s)[3] = nb.up;
   // explicit rounding: the same bits in every kernel this is inlined into
   const double cx = __dmul_rn(dt, g.idx[0]), cy = __dmul_rn(dt, g.idx[1]), cz = __dmul_rn(dt, g.idx[2]);
   double u[5];
 #pragma unroll
   for (int c = 0; c < 5; ++c) {
     double x = v.q[c][q];
-    x = __fma_rn(-cx, __dsub_rn(v.Fc[0][c][wi + 1], v.Fc[0][c][wi]), x);
+    x = __fma_rn(-cx, __dsub_rn(v.Fc[0][c][wi + s[0]], v.Fc[0][c][wi]), x);
     x = __fma_rn(-cy, __dsub_rn(v.Fc[1][c][wi + s[1]], v.Fc[1][c][wi]), x);
     x = __fma_rn(-cz, __dsub_rn(v.Fc[2][c][wi + s[2]], v.Fc[2][c][wi]), x);
     u[c] = x;
