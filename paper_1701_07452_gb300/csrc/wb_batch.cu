@@ -229,14 +229,14 @@ __device__ __forceinline__ void warp_max_atomic(double w, unsigned long long* ds
 
 // One tile of a sweep of one box (every thread of the block).
 template <int EZ, bool PROT>
-__device__ __forceinline__ int box_sweep_tile(const BoxInfo& bi, bool corr, int d, long long tile, double dt,
+__device__ __forceinline__ int box_sweep_tile(const BoxInfo& bi, bool corr, int d, long long tile,
                                               const WbPhys& P, wbu::LaneEdge& X) {
   const WbView& v = bi.v;
   const bool wrap = bi.wrap != 0;
   const WbBox b = stage_box(corr ? BS_CORR : BS_PRED, d, v.geo.n, wrap);
-  return wbu::sweep_tile<EZ, PROT, false>(v.geo, b, d, bi.sw[corr ? 1 : 0][d], tile, wrap,
+  return wbu::sweep_tile<EZ, PROT, true, false>(v.geo, b, d, bi.sw[corr ? 1 : 0][d], tile, wrap,
                                           wbu::sweep_ring(b.hi[d] - b.lo[d] + 1, wrap), 1, 0, 0,
-                                          dt, P, X);
+                                          v.scal, P, X);
 }
 
 __device__ __forceinline__ void unit_item(const BatchParams& B, int s, int d, const BoxInfo& bi, long long item,
@@ -256,13 +256,13 @@ __device__ __forceinline__ void unit_item(const BatchParams& B, int s, int d, co
   switch (s) {
     case BS_TRANS: {
       const int mask = trans_mask(n, i, j, k);
-      if (mask == 7) wbu::transverse_set(v, 0, 0, dt, 7, i, j, k, nb);  // constant mask: see k_transverse
-      else if (mask) wbu::transverse_set(v, 0, 0, dt, mask, i, j, k, nb);
+      if (mask == 7) wbu::transverse_set(v, 0, 0, 7, i, j, k, nb);  // constant mask: see k_transverse
+      else if (mask) wbu::transverse_set(v, 0, 0, mask, i, j, k, nb);
       break;
     }
     case BS_EREF_H: wbu::eref_half(v, 0, 0, dt, i, j, k, nb); break;
     case BS_FINAL: {
-      const double w = wbu::final_update(v, 0, 0, dt, B.phys, i, j, k, nb, outflow_mask(bi), hits, bad);
+      const double w = wbu::final_update(v, 0, 0, B.phys, i, j, k, nb, outflow_mask(bi), hits, bad);
       // running max of the rate keys: integer compares, and a NaN stays
       const unsigned long long kw = wb_rate_bits(w);
       if (kw > *wkey) *wkey = kw;
@@ -408,7 +408,7 @@ __device__ void box_dt(const BatchParams& B, int box) {
     B.steps_left[box] = 0;
     return;
   }
-  s->dt = dt;
+  wb_set_dt(s, dt, B.boxes[box].v.geo.dx, B.boxes[box].v.geo.idx);
   s->t += dt;
   s->steps += 1;
   if (B.dt_lag) s->wmax_lag = s->wmax_next;
@@ -507,7 +507,7 @@ __global__ void __launch_bounds__(kB, wbu::kSweepBlocks) k_batch(BatchParams B, 
           unsigned long long wkey = 0ULL;
           int hits = 0, bad = 0, hll = 0;
           if (stage_is_sweep(s)) {
-            hll = box_sweep_tile<EZ, PROT>(bi, s == BS_CORR, sub, i0, dt, B.phys, X);
+            hll = box_sweep_tile<EZ, PROT>(bi, s == BS_CORR, sub, i0, B.phys, X);
           } else if (stage_pairs(s)) {
             for (long long it = i0 + threadIdx.x; it < i1; it += 2 * kB)
               unit_pair(s, sub, bi, it, it + kB < i1 ? it + kB : -1, dt);
@@ -598,7 +598,7 @@ __global__ void __launch_bounds__(kB, wbu::kSweepBlocks) k_bstage_sweep(BatchPar
   drain_stage(B, grp, s, ctr, [&](int box, int d, long long cc) {
     const double dt = B.scal[box].dt;
     if (!wb_pos(dt)) return;
-    const int hll = box_sweep_tile<EZ, PROT>(B.boxes[box], s == BS_CORR, d, cc, dt, B.phys, X);
+    const int hll = box_sweep_tile<EZ, PROT>(B.boxes[box], s == BS_CORR, d, cc, B.phys, X);
     if (hll) atomicAdd((unsigned long long*)&B.scal[box].hll_faces, 1ULL);
   });
   stage_stamp(B, s, seq);
@@ -640,12 +640,12 @@ __global__ void __launch_bounds__(kNtZone, zone_min_blocks(CLS))
       const wbu::Nbr nb = wbu::neighbours(v.geo, i, j, k, bi.wrap ? 7 : 0);
       if (CLS == SC_TRANS) {
         const int mask = trans_mask(v.geo.n, i, j, k);
-        if (mask == 7) wbu::transverse_set(v, 0, 0, dt, 7, i, j, k, nb);  // constant mask: see k_transverse
-        else if (mask) wbu::transverse_set(v, 0, 0, dt, mask, i, j, k, nb);
+        if (mask == 7) wbu::transverse_set(v, 0, 0, 7, i, j, k, nb);  // constant mask: see k_transverse
+        else if (mask) wbu::transverse_set(v, 0, 0, mask, i, j, k, nb);
       } else if (CLS == SC_EREF_H) {
         wbu::eref_half(v, 0, 0, dt, i, j, k, nb);
       } else {
-        const double w = wbu::final_update(v, 0, 0, dt, B.phys, i, j, k, nb, outflow_mask(bi), &hits, &bad);
+        const double w = wbu::final_update(v, 0, 0, B.phys, i, j, k, nb, outflow_mask(bi), &hits, &bad);
         const unsigned long long kw = wb_rate_bits(w);
         if (kw > wkey) wkey = kw;
       }

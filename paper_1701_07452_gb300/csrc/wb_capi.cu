@@ -276,7 +276,6 @@ SweepArgs sweep_args(wb_grid* g, const StageArgs& s, bool corr, const WbBox (&bx
   a.slot_out = s.slot_w;
   a.geo = g->geo;
   for (int d = 0; d < 3; ++d) a.box[d] = bx[d];
-  a.dt = &g->scal->dt;
   a.phys = g->phys;
   a.scal = g->scal;
   a.nslots = nslots;
@@ -427,6 +426,15 @@ void set_interior(wb_grid* g) {
   const bool one_pass = d.batch_patches == 0 || d.batch_patches >= g->npatch;
   g->closed = periodic && g->npatch == 1 ? 7 : 0;
   g->wrap = periodic && g->npatch > 1 && one_pass && !flat_z(&d);
+}
+
+StepControl step_control(const wb_grid* g, double t_end) {
+  StepControl c = {g->d.cfl, t_end, g->d.dt_lag, 0, {}, {}};
+  for (int d = 0; d < 3; ++d) {
+    c.dx[d] = g->geo.dx[d];
+    c.idx[d] = g->geo.idx[d];
+  }
+  return c;
 }
 
 int sync(wb_grid* g, const char* where) {
@@ -660,7 +668,7 @@ int wb_advance(wb_grid* g, int nsteps, double t_end, double* t_out) {
     // the previous step's update has prepared this step's dt, unless the clock
     // was read between the two (it must not count a step that may not come)
     const bool check_next = t_end > 0.0 && (st + 1) % kStepsPerCheck == 0;
-    StepControl c = {g->d.cfl, t_end, g->d.dt_lag, 0};
+    StepControl c = step_control(g, t_end);
     if (!chained) wb_launch_dt_step(g->scal, c, s);
     chained = st + 1 < nsteps && !check_next;
     for (long long p0 = 0; p0 < g->npatch; p0 += g->S) {
@@ -982,7 +990,8 @@ int wb_step_noalloc(const wb_desc* d, const double* U, const double* bx, const d
   wb_launch_ccb(g.q, g.b, g.geo, 1, g.closed, s);
   if (!g.closed) wb_launch_halo(g.q, g.b, g.geo, g.map, s);
   wb_launch_dt_init(g.q, g.geo, 1, g.phys, g.scal, s);
-  const StepControl c = {one.cfl, 0.0, 0, 0};
+  StepControl c = step_control(&g, 0.0);
+  c.lag = 0;
   wb_launch_dt_step(g.scal, c, s);
   enqueue_pass(&g, 0, 1, c);
   double* outs[3] = {bx_out, by_out, bz_out};

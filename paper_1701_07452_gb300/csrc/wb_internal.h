@@ -5,6 +5,22 @@
 #include "wb_device.cuh"
 #include "wb_units.cuh"
 
+// Launch of a kernel that begins with wb_pdl_begin(): it may be set up before
+// the kernel ahead of it on the stream has finished.
+template <class... P, class... A>
+inline void wb_launch_dependent(void (*kernel)(P...), dim3 grid, int threads, cudaStream_t s, const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 struct wb_desc;
 // Physics constants of a descriptor (gamma, CFL, eps_k, limiter, floors).
 WbPhys wb_phys_of(const struct wb_desc* d);
@@ -15,7 +31,6 @@ struct SweepArgs {
   long long slot_in, slot_out;
   WbGeo geo;
   WbBox box[3];            // faces along the sweep axis, zones across it
-  const double* dt;
   WbPhys phys;
   WbScalars* scal;
   int nslots;
@@ -62,6 +77,7 @@ void wb_launch_eref_half(const StageArgs& a, const WbBox& box, cudaStream_t s);
 struct StepControl {
   double cfl, t_end;
   int lag, chain;
+  double dx[3], idx[3];
 };
 void wb_launch_final(const StageArgs& a, const StepControl& c, cudaStream_t s);
 

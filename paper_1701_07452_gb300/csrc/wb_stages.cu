@@ -27,6 +27,17 @@ inline dim3 grid_for(long long n, int nslots, int bs) {
   return dim3((unsigned)((n + bs - 1) / bs), (unsigned)nslots);
 }
 
+// Threads per block of a stage over n items: the largest block (up to most)
+// that still leaves 16 blocks for each of the 152 SMs.  The stages are FP64
+// bound, a warp instruction takes the FP64 pipe of an SM 19 cycles, so a stage
+// ends with the SM that holds the most warps: 16^3 zones are 16 blocks of 256
+// threads on 16 SMs or 128 of 32 on 128 (the update 13 against 7 us).
+inline int stage_threads(long long n, int nslots, int most) {
+  int bs = most;
+  while (bs > 32 && n * nslots < (long long)bs * 16 * 152) bs /= 2;
+  return bs;
+}
+
 inline WbBox box_union(const WbBox b[3]) {
   WbBox u = b[0];
   for (int n = 1; n < 3; ++n)
@@ -45,6 +56,7 @@ struct Boxes3 {
 // Steps 3 and 9: the three corner-EMF components, one thread per index of
 // the union of their boxes.
 __global__ void k_edges(StageArgs A, bool corr, Boxes3 B) {
+  wb_pdl_begin();
   if (!wb_pos(A.v.scal->dt)) return;
   int i, j, k;
   if (!box_index(B.u, blockIdx.x * (long long)blockDim.x + threadIdx.x, i, j, k)) return;
@@ -57,6 +69,7 @@ __global__ void k_edges(StageArgs A, bool corr, Boxes3 B) {
 
 // Steps 4 and 11: constrained transport of the three face components.
 __global__ void k_ct(StageArgs A, bool fin, Boxes3 B) {
+  wb_pdl_begin();
   const double dt = A.v.scal->dt;
   if (!wb_pos(dt)) return;
   int i, j, k;
@@ -71,8 +84,8 @@ __global__ void k_ct(StageArgs A, bool fin, Boxes3 B) {
 // Steps 5 and 7: the three transverse-flux preconditioned states, all
 // directions of a zone in one thread.
 __global__ void k_transverse(StageArgs A, Boxes3 B) {
-  const double dt = A.v.scal->dt;
-  if (!wb_pos(dt)) return;
+  wb_pdl_begin();
+  if (!wb_pos(A.v.scal->dt)) return;
   int i, j, k;
   if (!box_index(B.u, blockIdx.x * (long long)blockDim.x + threadIdx.x, i, j, k)) return;
   const int mask = (wbu::in_box(B.b[0], i, j, k) ? 1 : 0) | (wbu::in_box(B.b[1], i, j, k) ? 2 : 0) |
@@ -80,12 +93,13 @@ __global__ void k_transverse(StageArgs A, Boxes3 B) {
   // zones that need every direction take the mask as a constant: with a run-time
   // mask the compiler recomputes shared zone terms (13 FP64 instructions a zone)
   const wbu::Nbr nb = wbu::neighbours(A.v.geo, i, j, k, A.closed);
-  if (mask == 7) wbu::transverse_set(A.v, blockIdx.y * A.slot_q, blockIdx.y * A.slot_w, dt, 7, i, j, k, nb);
-  else if (mask) wbu::transverse_set(A.v, blockIdx.y * A.slot_q, blockIdx.y * A.slot_w, dt, mask, i, j, k, nb);
+  if (mask == 7) wbu::transverse_set(A.v, blockIdx.y * A.slot_q, blockIdx.y * A.slot_w, 7, i, j, k, nb);
+  else if (mask) wbu::transverse_set(A.v, blockIdx.y * A.slot_q, blockIdx.y * A.slot_w, mask, i, j, k, nb);
 }
 
 // Step 8: half-step reference EMF.
 __global__ void k_eref_half(StageArgs A, WbBox box) {
+  wb_pdl_begin();
   const double dt = A.v.scal->dt;
   if (!wb_pos(dt)) return;
   int i, j, k;
@@ -101,6 +115,7 @@ __global__ void k_eref_half(StageArgs A, WbBox box) {
 // (the same function of the same inputs, so the copy equals a recomputation
 // bit for bit).  One thread per shell point.
 __global__ void k_wrap(WrapList L, WbGeo g, int depth, long long n) {
+  wb_pdl_begin();
   const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (t >= n) return;
   long long dst, src;
@@ -113,6 +128,7 @@ __global__ void k_wrap(WrapList L, WbGeo g, int depth, long long n) {
 // neighbouring patch (periodic across the domain) holds at that global
 // position.
 __global__ void k_wrap_patches(WrapList L, WbGeo g, GridMap m, int depth, long long n) {
+  wb_pdl_begin();
   const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (t >= n) return;
   const long long p = blockIdx.y;
@@ -179,7 +195,7 @@ __device__ void dt_step(volatile WbScalars* s, const StepControl& c) {
     s->unphysical += 1;
     return;
   }
-  s->dt = dt;
+  wb_set_dt(s, dt, c.dx, c.idx);
   s->t = last ? t_end : s->t + dt;
   if (c.lag) s->wmax_lag = s->wmax_next;
   s->steps += 1;
@@ -192,8 +208,8 @@ __device__ void dt_step(volatile WbScalars* s, const StepControl& c) {
 // launch that has nothing to do (dt = 0) still does that, as a launch of
 // k_dt_step would.
 __global__ void k_final(StageArgs A, StepControl c) {
-  const double dt = A.v.scal->dt;
-  const bool run = wb_pos(dt);
+  wb_pdl_begin();
+  const bool run = wb_pos(A.v.scal->dt);
   if (!run && !c.chain) return;
   const WbGeo& g = A.v.geo;
   WbBox box = {{0, 0, 0}, {g.n[0] - 1, g.n[1] - 1, g.n[2] - 1}};
@@ -208,7 +224,7 @@ __global__ void k_final(StageArgs A, StepControl c) {
 #pragma unroll
   for (int d = 0; d < 3; ++d)
     if (((A.ohi_bc >> d) & 1) && pc[d] == A.np[d] - 1) ohi |= 1 << d;
-  if (ok) w = wbu::final_update(A.v, blockIdx.y * A.slot_q, blockIdx.y * A.slot_w, dt, A.phys, i, j, k,
+  if (ok) w = wbu::final_update(A.v, blockIdx.y * A.slot_q, blockIdx.y * A.slot_w, A.phys, i, j, k,
                                 wbu::neighbours(g, i, j, k, A.closed), ohi, &hits, &bad);
   if (hits) atomicAdd((unsigned long long*)&A.v.scal->floor_hits, (unsigned long long)hits);
   if (bad) atomicAdd((unsigned long long*)&A.v.scal->unphysical, (unsigned long long)bad);
@@ -230,6 +246,7 @@ __global__ void k_final(StageArgs A, StepControl c) {
 // zone of the same global position wrapped (periodic) or clamped (outflow)
 // into the domain; face arrays use the same rule on their face index.
 __global__ void k_halo(StageArgs A, GridMap m) {
+  wb_pdl_begin();
   const WbGeo& g = A.v.geo;
   long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (t >= g.V) return;
@@ -285,7 +302,9 @@ __global__ void k_dt_init(StageArgs A, long long npatch) {
   block_max_atomic(w, &A.v.scal->wmax_next);
 }
 
-__global__ void k_dt_step(WbScalars* s, StepControl c) { dt_step(s, c); }
+__global__ void k_dt_step(WbScalars* s, StepControl c) {
+  wb_pdl_begin();
+  dt_step(s, c); }
 
 __global__ void k_ccb(StageArgs A, long long npatch) {
   const WbGeo& g = A.v.geo;
@@ -490,39 +509,44 @@ Boxes3 boxes3(const WbBox b[3]) {
 
 void wb_launch_edges(const StageArgs& a, bool corr, const WbBox box[3], cudaStream_t s) {
   Boxes3 B = boxes3(box);
-  k_edges<<<grid_for(box_count(B.u), a.nslots, 256), 256, 0, s>>>(a, corr, B);
+  const int bs = stage_threads(box_count(B.u), a.nslots, 256);
+  wb_launch_dependent(k_edges, grid_for(box_count(B.u), a.nslots, bs), bs, s, a, corr, B);
 }
 
 void wb_launch_ct(const StageArgs& a, bool fin, const WbBox box[3], cudaStream_t s) {
   Boxes3 B = boxes3(box);
-  k_ct<<<grid_for(box_count(B.u), a.nslots, 256), 256, 0, s>>>(a, fin, B);
+  const int bs = stage_threads(box_count(B.u), a.nslots, 256);
+  wb_launch_dependent(k_ct, grid_for(box_count(B.u), a.nslots, bs), bs, s, a, fin, B);
 }
 
 void wb_launch_transverse(const StageArgs& a, const WbBox box[3], cudaStream_t s) {
   Boxes3 B = boxes3(box);
-  k_transverse<<<grid_for(box_count(B.u), a.nslots, 128), 128, 0, s>>>(a, B);
+  const int bs = stage_threads(box_count(B.u), a.nslots, 128);
+  wb_launch_dependent(k_transverse, grid_for(box_count(B.u), a.nslots, bs), bs, s, a, B);
 }
 
 void wb_launch_eref_half(const StageArgs& a, const WbBox& box, cudaStream_t s) {
-  k_eref_half<<<grid_for(box_count(box), a.nslots, 256), 256, 0, s>>>(a, box);
+  const int bs = stage_threads(box_count(box), a.nslots, 256);
+  wb_launch_dependent(k_eref_half, grid_for(box_count(box), a.nslots, bs), bs, s, a, box);
 }
 
 void wb_launch_final(const StageArgs& a, const StepControl& c, cudaStream_t s) {
   long long n = (long long)a.v.geo.n[0] * a.v.geo.n[1] * a.v.geo.n[2];
-  k_final<<<grid_for(n, a.nslots, 256), 256, 0, s>>>(a, c);
+  const int bs = stage_threads(n, a.nslots, 256);
+  wb_launch_dependent(k_final, grid_for(n, a.nslots, bs), bs, s, a, c);
 }
 
 void wb_launch_halo(double* const q[8], double* const b[3], const WbGeo& geo, const GridMap& m,
                     cudaStream_t s) {
   StageArgs a = mini_args(q, b, geo);
-  k_halo<<<grid_for(geo.V, (int)m.npatch, 256), 256, 0, s>>>(a, m);
+  wb_launch_dependent(k_halo, grid_for(geo.V, (int)m.npatch, 256), 256, s, a, m);
 }
 
 void wb_launch_wrap(const WrapList& L, const WbGeo& geo, const GridMap& m, int depth, cudaStream_t s) {
   if (L.n <= 0) return;
   const long long n = wbu::shell_count(geo, depth);
-  if (m.npatch == 1) k_wrap<<<grid_for(n, 1, 256), 256, 0, s>>>(L, geo, depth, n);
-  else k_wrap_patches<<<grid_for(n, (int)m.npatch, 256), 256, 0, s>>>(L, geo, m, depth, n);
+  if (m.npatch == 1) wb_launch_dependent(k_wrap, grid_for(n, 1, 256), 256, s, L, geo, depth, n);
+  else wb_launch_dependent(k_wrap_patches, grid_for(n, (int)m.npatch, 256), 256, s, L, geo, m, depth, n);
 }
 
 void wb_launch_dt_init(double* const q[8], const WbGeo& geo, long long npatch, const WbPhys& ph,
@@ -535,7 +559,7 @@ void wb_launch_dt_init(double* const q[8], const WbGeo& geo, long long npatch, c
 }
 
 void wb_launch_dt_step(WbScalars* scal, const StepControl& c, cudaStream_t s) {
-  k_dt_step<<<1, 1, 0, s>>>(scal, c);
+  wb_launch_dependent(k_dt_step, 1, 1, s, scal, c);
 }
 
 void wb_launch_ccb(double* const q[8], double* const b[3], const WbGeo& geo, long long npatch, int closed,

@@ -55,12 +55,19 @@ __device__ __forceinline__ double ld(const double* p) {
   return *p;
 }
 
+// A product of the sweeps: on the integer pipes (SOFT) or the FP64 pipe, the
+// same bits.
+template <bool SOFT>
+__device__ __forceinline__ double mul(double x, double y) {
+  return SOFT ? wb_smul(x, y) : __dmul_rn(x, y);
+}
+
 // Zone state of a sweep.  The arithmetic is written with explicit rounding
 // (no contraction left to the compiler): a zone is loaded both before and
 // inside the march over a segment, and the two inlined copies must round
 // identically, or a face's flux would depend on where a segment starts.
 // q: the fields in the sweep's frame (rho, Mn, Mt1, Mt2, E, Bn, Bt1, Bt2).
-template <bool NC>
+template <bool NC, bool SOFT>
 __device__ __forceinline__ void load_cell(const double* const (&q)[8], long long off, const WbPhys& P,
                                                 Cell& c) {
   c.rho = ld<NC>(q[0] + off);
@@ -74,12 +81,12 @@ __device__ __forceinline__ void load_cell(const double* const (&q)[8], long long
   const WbRoots rr = wb_roots(c.rho);
   c.sr = rr.sq;
   c.ir = rr.rcp;
-  c.vn = wb_smul(c.mn, c.ir);
-  c.vt1 = wb_smul(c.mt1, c.ir);
-  c.vt2 = wb_smul(c.mt2, c.ir);
-  const double hbn = wb_half(bn), bn2 = wb_smul(bn, bn);
-  const double ke = wb_half(__fma_rn(c.mt2, c.vt2, __fma_rn(c.mt1, c.vt1, wb_smul(c.mn, c.vn))));
-  const double bt2 = __fma_rn(c.bt2, c.bt2, wb_smul(c.bt1, c.bt1));
+  c.vn = mul<SOFT>(c.mn, c.ir);
+  c.vt1 = mul<SOFT>(c.mt1, c.ir);
+  c.vt2 = mul<SOFT>(c.mt2, c.ir);
+  const double hbn = wb_half(bn), bn2 = mul<SOFT>(bn, bn);
+  const double ke = wb_half(__fma_rn(c.mt2, c.vt2, __fma_rn(c.mt1, c.vt1, mul<SOFT>(c.mn, c.vn))));
+  const double bt2 = __fma_rn(c.bt2, c.bt2, mul<SOFT>(c.bt1, c.bt1));
   const double me = wb_half(__dadd_rn(bn2, bt2));
   const double p = __dmul_rn(P.gm1, __dsub_rn(__dsub_rn(e, ke), me));
   const double pstar = __dadd_rn(p, me);
@@ -91,11 +98,11 @@ __device__ __forceinline__ void load_cell(const double* const (&q)[8], long long
   const double hmn = wb_half(c.mn), hvn = wb_half(c.vn);
   c.F[0] = hmn;
   c.F[1] = __fma_rn(hmn, c.vn, wb_half(__dsub_rn(pstar, bn2)));
-  c.F[2] = __fma_rn(hmn, c.vt1, -wb_smul(c.bt1, hbn));
-  c.F[3] = __fma_rn(hmn, c.vt2, -wb_smul(c.bt2, hbn));
-  c.F[4] = __fma_rn(c.bt1, hvn, -wb_smul(c.vt1, hbn));
-  c.F[5] = __fma_rn(c.bt2, hvn, -wb_smul(c.vt2, hbn));
-  const double bv = __fma_rn(c.bt2, c.vt2, __fma_rn(c.bt1, c.vt1, wb_smul(bn, c.vn)));
+  c.F[2] = __fma_rn(hmn, c.vt1, -mul<SOFT>(c.bt1, hbn));
+  c.F[3] = __fma_rn(hmn, c.vt2, -mul<SOFT>(c.bt2, hbn));
+  c.F[4] = __fma_rn(c.bt1, hvn, -mul<SOFT>(c.vt1, hbn));
+  c.F[5] = __fma_rn(c.bt2, hvn, -mul<SOFT>(c.vt2, hbn));
+  const double bv = __fma_rn(c.bt2, c.vt2, __fma_rn(c.bt1, c.vt1, mul<SOFT>(bn, c.vn)));
   c.F[6] = __fma_rn(ep, hvn, __dmul_rn(-hbn, bv));
 }
 
@@ -127,14 +134,14 @@ struct RegRec {
 
 // Q_k(nu) - nu^2 for the g-tilde of App. A.  Waves in the compile-time mask
 // EZ have eps_k = 0, where Q is |nu|; the branch test runs on the integer pipe.
-template <int EZ>
+template <int EZ, bool SOFT>
 __device__ __forceinline__ double Qk_m_nu2(double nu, int k, const WbPhys& P) {
   if (EZ & (1 << k)) return WB_FMA(-nu, nu, wb_fabs(nu));
   // |nu| - nu^2, or for |nu| < 2 eps nu^2 / (4 eps) + eps - nu^2 = nu^2 (1/(4 eps) - 1) + eps:
   // one FMA of operands chosen on the integer pipe, FMA(x, nu, y) with (x, y) = (-nu, |nu|)
   // or (nu (1/(4 eps) - 1), eps), so that no warp issues both forms
   const bool band = wb_abs_less(nu, P.two_eps[k]);
-  const double x = band ? wb_smul(nu, P.inv4eps_m1[k]) : wb_flip(nu);
+  const double x = band ? mul<SOFT>(nu, P.inv4eps_m1[k]) : wb_flip(nu);
   return WB_FMA(x, nu, band ? P.eps[k] : wb_fabs(nu));
 }
 
@@ -218,29 +225,29 @@ __device__ __forceinline__ void hll_face(const Cell& L, const Cell& R, double bn
 // flux (the record holds the Roe state), 2 when the Roe state has no real
 // sound speed (HLL without Roe speeds).  The protection test is compiled in
 // only when PROT is set.
-template <int EZ, bool PROT, class Rc>
+template <int EZ, bool PROT, bool SOFT, class Rc>
 __device__ __forceinline__ int face_system(const Cell& L, const Cell& R, double b, double dtdx,
                                            const WbPhys& P, const Rc& f, double gt[7]) {
   const double iD = wb_rcp(WB_ADD(L.sr, R.sr));
-  const double wL = wb_smul(L.sr, iD), wR = wb_smul(R.sr, iD);
-  const double rho = wb_smul(L.sr, R.sr);
+  const double wL = mul<SOFT>(L.sr, iD), wR = mul<SOFT>(R.sr, iD);
+  const double rho = mul<SOFT>(L.sr, R.sr);
   const WbRoots rroe = wb_roots(rho);
   const double irho = rroe.rcp, isrho = rroe.rsq, srho = rroe.sq;
-  const double vn = WB_FMA(wL, L.vn, wb_smul(R.vn, wR));
-  const double vt1 = WB_FMA(wL, L.vt1, wb_smul(R.vt1, wR));
-  const double vt2 = WB_FMA(wL, L.vt2, wb_smul(R.vt2, wR));
-  const double bt1 = WB_FMA(wR, L.bt1, wb_smul(R.bt1, wL));
-  const double bt2 = WB_FMA(wR, L.bt2, wb_smul(R.bt2, wL));
-  const double b2 = wb_smul(b, b);
+  const double vn = WB_FMA(wL, L.vn, mul<SOFT>(R.vn, wR));
+  const double vt1 = WB_FMA(wL, L.vt1, mul<SOFT>(R.vt1, wR));
+  const double vt2 = WB_FMA(wL, L.vt2, mul<SOFT>(R.vt2, wR));
+  const double bt1 = WB_FMA(wR, L.bt1, mul<SOFT>(R.bt1, wL));
+  const double bt2 = WB_FMA(wR, L.bt2, mul<SOFT>(R.bt2, wL));
+  const double b2 = mul<SOFT>(b, b);
   // H = wL (h_L + b^2)/rho_L + wR (h_R + b^2)/rho_R, with wL/rho_L + wR/rho_R = 1/rho_
-  const double H = WB_FMA(b2, irho, WB_FMA(wL, L.hr, wb_smul(R.hr, wR)));
+  const double H = WB_FMA(b2, irho, WB_FMA(wL, L.hr, mul<SOFT>(R.hr, wR)));
   const double dbt1 = WB_SUB(R.bt1, L.bt1), dbt2 = WB_SUB(R.bt2, L.bt2);
-  const double gX = WB_MUL(P.hgm2, WB_MUL(WB_FMA(dbt1, dbt1, wb_smul(dbt2, dbt2)), wb_smul(iD, iD)));  // (gamma-2) X
-  const double hv2 = wb_half(WB_FMA(vn, vn, WB_FMA(vt1, vt1, wb_smul(vt2, vt2))));
-  const double bt2s = WB_FMA(bt1, bt1, wb_smul(bt2, bt2));
+  const double gX = WB_MUL(P.hgm2, WB_MUL(WB_FMA(dbt1, dbt1, mul<SOFT>(dbt2, dbt2)), mul<SOFT>(iD, iD)));  // (gamma-2) X
+  const double hv2 = wb_half(WB_FMA(vn, vn, WB_FMA(vt1, vt1, mul<SOFT>(vt2, vt2))));
+  const double bt2s = WB_FMA(bt1, bt1, mul<SOFT>(bt2, bt2));
   const double a2 = WB_FMA(P.gm1, WB_FMA(-WB_ADD(b2, bt2s), irho, WB_SUB(H, hv2)), -gX);
   if (!wb_normal_pos(a2)) return 2;
-  const double ca2 = wb_smul(b2, irho), ct2 = wb_smul(bt2s, irho);
+  const double ca2 = mul<SOFT>(b2, irho), ct2 = mul<SOFT>(bt2s, irho);
   const double dac = WB_SUB(a2, ca2);
   const double disc = WB_FMA(dac, dac, WB_MUL(ct2, WB_FMA(2.0, WB_ADD(a2, ca2), ct2)));
   const double sum = WB_ADD(WB_ADD(a2, ca2), ct2);
@@ -250,8 +257,8 @@ __device__ __forceinline__ int face_system(const Cell& L, const Cell& R, double 
   const WbRoots rcf = wb_roots(cf2), ra_ = wb_roots(a2);
   const double icf = rcf.rsq, ia = ra_.rsq, ia2 = ra_.rcp;
   const double cf = rcf.sq, a = ra_.sq;
-  const double ca = wb_smul(wb_fabs(b), isrho);
-  const double cs = wb_smul(wb_smul(a, ca), icf);  // c_f c_s = a c_a
+  const double ca = mul<SOFT>(wb_fabs(b), isrho);
+  const double cs = mul<SOFT>(mul<SOFT>(a, ca), icf);  // c_f c_s = a c_a
   // 1/|B_t| and c_t = |B_t| / sqrt(rho_); a transverse field whose square is
   // not a normal double (underflowing noise ahead of a front) counts as 0
   double ib = 0.0, btm = 0.0;  // btm = |B_t|
@@ -271,9 +278,9 @@ __device__ __forceinline__ int face_system(const Cell& L, const Cell& R, double 
   const double t1 = WB_ADD(WB_SUB(ca2, a2), ct2);
   const bool slow_major = !wb_neg(t1);
   const double m = WB_ADD(sd, slow_major ? t1 : wb_flip(t1));
-  const double r = wb_rsqrt(wb_twice(wb_smul(sd, m)));
-  const double major = wb_smul(m, r);
-  const double minor = WB_MUL(wb_smul(a, wb_smul(btm, isrho)), wb_twice(r));
+  const double r = wb_rsqrt(wb_twice(mul<SOFT>(sd, m)));
+  const double major = mul<SOFT>(m, r);
+  const double minor = WB_MUL(mul<SOFT>(a, mul<SOFT>(btm, isrho)), wb_twice(r));
   double af = slow_major ? minor : major;
   double as = slow_major ? major : minor;
   if (wb_hi_scaled(sd, 39) <= wb_hi32(sum) && wb_at_most(sd, 1e-12, sum)) {
@@ -281,8 +288,8 @@ __device__ __forceinline__ int face_system(const Cell& L, const Cell& R, double 
     af = fast ? 1.0 : 0.0;
     as = fast ? 0.0 : 1.0;
   }
-  const double ra2 = wb_smul(rho, a2);
-  double b1n = wb_smul(bt1, ib), b2n = wb_smul(bt2, ib);
+  const double ra2 = mul<SOFT>(rho, a2);
+  double b1n = mul<SOFT>(bt1, ib), b2n = mul<SOFT>(bt2, ib);
   if (wb_maybe_small(bt2s, ra2, b2) && wb_at_most(bt2s, 1e-24, WB_ADD(WB_ADD(ra2, b2), bt2s)))
     b1n = b2n = 0.70710678118654752440;
   const double S = wb_sgn(b);
@@ -294,27 +301,27 @@ __device__ __forceinline__ int face_system(const Cell& L, const Cell& R, double 
   const double dvn = WB_FMA(-vn, drho, dmn);
   const double dvt1 = WB_FMA(-vt1, drho, dmt1);
   const double dvt2 = WB_FMA(-vt2, drho, dmt2);
-  const double vdm = WB_FMA(vn, dmn, WB_FMA(vt1, dmt1, wb_smul(vt2, dmt2)));
-  const double bdb = WB_FMA(bt1, dbt1, wb_smul(bt2, dbt2));
+  const double vdm = WB_FMA(vn, dmn, WB_FMA(vt1, dmt1, mul<SOFT>(vt2, dmt2)));
+  const double bdb = WB_FMA(bt1, dbt1, mul<SOFT>(bt2, dbt2));
   const double dp = WB_FMA(-gX, drho, WB_MUL(P.gm1, WB_SUB(WB_FMA(hv2, drho, WB_SUB(de, vdm)), bdb)));
   // projections on the transverse field direction beta and its normal; S = sign(b)
-  const double dvbS = wb_xsgn(WB_FMA(b1n, dvt1, wb_smul(dvt2, b2n)), S);
-  const double dvp = WB_FMA(-b2n, dvt1, wb_smul(dvt2, b1n));
-  const double dbb = WB_FMA(b1n, dbt1, wb_smul(dbt2, b2n));
-  const double dbpS = wb_xsgn(WB_FMA(-b2n, dbt1, wb_smul(dbt2, b1n)), S);
+  const double dvbS = wb_xsgn(WB_FMA(b1n, dvt1, mul<SOFT>(dvt2, b2n)), S);
+  const double dvp = WB_FMA(-b2n, dvt1, mul<SOFT>(dvt2, b1n));
+  const double dbb = WB_FMA(b1n, dbt1, mul<SOFT>(dbt2, b2n));
+  const double dbpS = wb_xsgn(WB_FMA(-b2n, dbt1, mul<SOFT>(dbt2, b1n)), S);
   const double hir = wb_half(irho), hisr = wb_half(isrho);
-  const double i2ra = wb_smul(hisr, ia);   // 1 / (2 sqrt(rho) a)
-  const double ri2a2 = wb_smul(hir, ia2);  // 1 / (2 rho a^2)
-  const double dpr = wb_smul(dp, ri2a2);
-  const double afcf = wb_smul(af, cf), ascs = wb_smul(as, cs);
-  const double dbbi = wb_smul(dbb, i2ra);
+  const double i2ra = mul<SOFT>(hisr, ia);   // 1 / (2 sqrt(rho) a)
+  const double ri2a2 = mul<SOFT>(hir, ia2);  // 1 / (2 rho a^2)
+  const double dpr = mul<SOFT>(dp, ri2a2);
+  const double afcf = mul<SOFT>(af, cf), ascs = mul<SOFT>(as, cs);
+  const double dbbi = mul<SOFT>(dbb, i2ra);
   // alpha_{1,7} = Cf -+ Xf / (2 rho a^2), alpha_{3,5} = Cs -+ Xs / (2 rho a^2): the factor
   // goes into the FMAs that form them
-  const double Xf = WB_FMA(afcf, dvn, -wb_smul(dvbS, ascs));
-  const double Cf = WB_FMA(as, dbbi, wb_smul(af, dpr));
-  const double Xs = WB_FMA(ascs, dvn, wb_smul(dvbS, afcf));
-  const double Cs = WB_FMA(-af, dbbi, wb_smul(as, dpr));
-  const double hAa = wb_smul(hisr, dbpS);
+  const double Xf = WB_FMA(afcf, dvn, -mul<SOFT>(dvbS, ascs));
+  const double Cf = WB_FMA(as, dbbi, mul<SOFT>(af, dpr));
+  const double Xs = WB_FMA(ascs, dvn, mul<SOFT>(dvbS, afcf));
+  const double Cs = WB_FMA(-af, dbbi, mul<SOFT>(as, dpr));
+  const double hAa = mul<SOFT>(hisr, dbpS);
   double al[7];
   al[0] = WB_FMA(-ri2a2, Xf, Cf);
   al[6] = WB_FMA(ri2a2, Xf, Cf);
@@ -324,7 +331,7 @@ __device__ __forceinline__ int face_system(const Cell& L, const Cell& R, double 
   al[5] = WB_FMA(hir, dvp, -hAa);
   al[3] = WB_FMA(-dp, ia2, drho);
   // nu_k = (dt/dx) a_k for the eigenvalues a_1..a_7 (Sec. 3)
-  const double tvn = wb_smul(vn, dtdx);
+  const double tvn = mul<SOFT>(vn, dtdx);
   const double nuk[7] = {WB_FMA(-dtdx, cf, tvn), WB_FMA(-dtdx, ca, tvn), WB_FMA(-dtdx, cs, tvn), tvn,
                          WB_FMA(dtdx, cs, tvn),  WB_FMA(dtdx, ca, tvn),  WB_FMA(dtdx, cf, tvn)};
 #pragma unroll
@@ -332,9 +339,9 @@ __device__ __forceinline__ int face_system(const Cell& L, const Cell& R, double 
     const double nu = nuk[k];
     f[R_AL + k] = al[k];
     f[R_NU + k] = nu;
-    gt[k] = wb_smul(Qk_m_nu2<EZ>(nu, k, P), al[k]);  // 2 g-tilde
+    gt[k] = mul<SOFT>(Qk_m_nu2<EZ, SOFT>(nu, k, P), al[k]);  // 2 g-tilde
   }
-  f[R_RHO] = rho; f[R_SRHO] = wb_xsgn(srho, S); f[R_A] = a; f[R_PG] = wb_smul(ra2, P.inv_gm1); f[R_CF] = cf;
+  f[R_RHO] = rho; f[R_SRHO] = wb_xsgn(srho, S); f[R_A] = a; f[R_PG] = mul<SOFT>(ra2, P.inv_gm1); f[R_CF] = cf;
   f[R_ASCS] = ascs; f[R_AFCF] = afcf; f[R_AF] = af; f[R_AS] = as; f[R_B1] = b1n; f[R_B2] = b2n;
   f[R_VN] = vn; f[R_VT1] = vt1; f[R_VT2] = vt2; f[R_BTM] = btm;
   f[R_KX] = WB_FMA(gX, P.inv_gm1, -hv2);  // K - v^2 (the energy row of face_flux)
@@ -355,7 +362,7 @@ __device__ __forceinline__ int face_system(const Cell& L, const Cell& R, double 
 // 2 w = 2 nu alpha + G_{i+1} - G_i.  alpha = 0 needs no case of its own: this
 // face's g-tilde is then 0, the limiter makes G_i = G_{i+1} = 0 and either form
 // gives 0.
-template <int EZ>
+template <int EZ, bool SOFT>
 __device__ __forceinline__ double beta_k(double al, double nu, double Gi, double Gi1, int k,
                                          const WbPhys& P) {
   if (EZ & (1 << k)) {
@@ -363,7 +370,7 @@ __device__ __forceinline__ double beta_k(double al, double nu, double Gi, double
     return (wb_order_less(b1, b2) != wb_neg(al)) ? b2 : b1;
   }
   const double d = WB_FMA(wb_twice(nu), al, WB_SUB(Gi1, Gi));  // 2 w
-  if (!wb_abs_less(d, wb_smul(al, P.four_eps[k]))) {
+  if (!wb_abs_less(d, mul<SOFT>(al, P.four_eps[k]))) {
     const bool same = (__double_as_longlong(d) ^ __double_as_longlong(al)) >= 0;
     return WB_FMA(same ? nu : wb_flip(nu), al, -(same ? Gi : Gi1));
   }
@@ -374,12 +381,12 @@ __device__ __forceinline__ double beta_k(double al, double nu, double Gi, double
 }
 
 // u-bar = (F_L + F_R)/2 - (dx/(2 dt)) sum_k beta_k R_k  (App. A)
-template <int EZ, class Rc>
+template <int EZ, bool SOFT, class Rc>
 __device__ __forceinline__ void face_flux(const Rc& f, const double gi[7], const double gi1[7],
                                           double dx_2dt, const WbPhys& P, double out[7]) {
   double be[7];
 #pragma unroll
-  for (int k = 0; k < 7; ++k) be[k] = beta_k<EZ>(f[R_AL + k], f[R_NU + k], gi[k], gi1[k], k, P);
+  for (int k = 0; k < 7; ++k) be[k] = beta_k<EZ, SOFT>(f[R_AL + k], f[R_NU + k], gi[k], gi1[k], k, P);
   const double rho = f[R_RHO], af = f[R_AF], as = f[R_AS];
   const double S = f[R_SRHO], b1 = f[R_B1], b2 = f[R_B2];  // S: sign(b) sqrt(rho_)
   // sum_k beta_k r_k in w = (rho, vn, vt, Bt, p)
@@ -387,19 +394,19 @@ __device__ __forceinline__ void face_flux(const Rc& f, const double gi[7], const
   const double ss = WB_ADD(be[2], be[4]), ds = WB_SUB(be[4], be[2]);
   const double afcf = f[R_AFCF], ascs = f[R_ASCS], srho = wb_fabs(S);
   const double vp = WB_ADD(be[1], be[5]);                             // along beta-perp
-  const double tfs = WB_FMA(af, sf, wb_smul(ss, as));
+  const double tfs = WB_FMA(af, sf, mul<SOFT>(ss, as));
   const double wr = WB_FMA(rho, tfs, be[3]);
-  const double wvn = WB_FMA(afcf, df, wb_smul(ds, ascs));
-  const double vb = wb_xsgn(WB_FMA(afcf, ds, -wb_smul(df, ascs)), S);  // along beta
-  const double bb = wb_smul(WB_FMA(as, sf, -wb_smul(ss, af)), wb_smul(f[R_A], srho));
-  const double bp = wb_xsgn(wb_smul(WB_SUB(be[1], be[5]), srho), S);
-  const double wvt1 = WB_FMA(b1, vb, -wb_smul(vp, b2)), wvt2 = WB_FMA(b2, vb, wb_smul(vp, b1));
-  const double wbt1 = WB_FMA(b1, bb, -wb_smul(bp, b2)), wbt2 = WB_FMA(b2, bb, wb_smul(bp, b1));
+  const double wvn = WB_FMA(afcf, df, mul<SOFT>(ds, ascs));
+  const double vb = wb_xsgn(WB_FMA(afcf, ds, -mul<SOFT>(df, ascs)), S);  // along beta
+  const double bb = mul<SOFT>(WB_FMA(as, sf, -mul<SOFT>(ss, af)), mul<SOFT>(f[R_A], srho));
+  const double bp = wb_xsgn(mul<SOFT>(WB_SUB(be[1], be[5]), srho), S);
+  const double wvt1 = WB_FMA(b1, vb, -mul<SOFT>(vp, b2)), wvt2 = WB_FMA(b2, vb, mul<SOFT>(vp, b1));
+  const double wbt1 = WB_FMA(b1, bb, -mul<SOFT>(bp, b2)), wbt2 = WB_FMA(b2, bb, mul<SOFT>(bp, b1));
   // to conserved variables (the pressure row enters the energy as p/(gamma-1))
   const double vn = f[R_VN], vt1 = f[R_VT1], vt2 = f[R_VT2];
-  const double u1 = WB_FMA(vn, wr, wb_smul(wvn, rho));
-  const double u2 = WB_FMA(vt1, wr, wb_smul(wvt1, rho));
-  const double u3 = WB_FMA(vt2, wr, wb_smul(wvt2, rho));
+  const double u1 = WB_FMA(vn, wr, mul<SOFT>(wvn, rho));
+  const double u2 = WB_FMA(vt1, wr, mul<SOFT>(wvt1, rho));
+  const double u3 = WB_FMA(vt2, wr, mul<SOFT>(wvt2, rho));
   // energy: B_t . w_Bt + p/(gamma-1) row + K w_rho + rho v . w_v, with
   // rho v . w_v = v . u - v^2 w_rho and the record holding K - v^2, and
   // B_t . w_Bt = |B_t| w_beta: beta is B_t / |B_t|, so the beta-perpendicular
@@ -506,10 +513,10 @@ __host__ __device__ __forceinline__ long long sweep_tiles(long long npen, int le
 // A thread that marched along a pencil kept two zones, two slopes and a face
 // record in 226 to 255 registers and 40 KB of shared memory a block, which left
 // 2 warps per scheduler; one face per thread needs 168, 3 warps.
-template <int EZ, bool PROT, bool NC>
+template <int EZ, bool PROT, bool SOFT, bool NC>
 __device__ __forceinline__ int sweep_tile(const WbGeo& g, const WbBox& box, int d, const SweepFrame& s, long long tile,
                                           bool closed, bool ring, int nslots, long long slot_in, long long slot_out,
-                                          double dt, const WbPhys& P, LaneEdge& X) {
+                                          const WbScalars* scal, const WbPhys& P, LaneEdge& X) {
   const int U = d == 0 ? 1 : 0, W = d == 2 ? 1 : 2;
   const int nu = box.hi[U] - box.lo[U] + 1, nw = box.hi[W] - box.lo[W] + 1;
   const int len = box.hi[d] - box.lo[d] + 1;
@@ -552,7 +559,7 @@ __device__ __forceinline__ int sweep_tile(const WbGeo& g, const WbBox& box, int 
   const long long at = wb_at(g, pos[0], pos[1], pos[2]);
   const long long off = slot * slot_in + at;
   Cell R;
-  load_cell<NC>(s.q, off, P, R);
+  load_cell<NC, SOFT>(s.q, off, P, R);
   const double b = ld<NC>(s.bn + off);
   Cell L;
   L.ir = 0.0;  // not used across a face
@@ -571,7 +578,7 @@ __device__ __forceinline__ int sweep_tile(const WbGeo& g, const WbBox& box, int 
   }
   RegRec f;
   double gt[7];
-  const int code = face_system<EZ, PROT>(L, R, b, __dmul_rn(dt, g.idx[d]), P, f, gt);
+  const int code = face_system<EZ, PROT, SOFT>(L, R, b, scal->dtdx[d], P, f, gt);
   bool hll = false;
   if (code) {
     if (has_left) {
@@ -616,7 +623,7 @@ __device__ __forceinline__ int sweep_tile(const WbGeo& g, const WbBox& box, int 
 #pragma unroll
     for (int m = 0; m < 7; ++m) out[m] = f[R_FAVG + m];
   } else {
-    face_flux<EZ>(f, gl, gz, __dmul_rn(wb_half(g.dx[d]), wb_rcp(dt)), P, out);
+    face_flux<EZ, SOFT>(f, gl, gz, scal->dx_2dt[d], P, out);
   }
   const long long o = slot * slot_out + at;
 #pragma unroll
@@ -826,11 +833,9 @@ struct TransZone {
   double dF[3][8];
 };
 
-__device__ __forceinline__ void trans_zone(const WbView& v, long long q, long long w, double dt,
-                                           int need, const Nbr& nb, TransZone& z) {
-  const WbGeo& g = v.geo;
+__device__ __forceinline__ void trans_zone(const WbView& v, long long q, long long w, int need,
+                                           const Nbr& nb, TransZone& z) {
   const long long (&s)[3] = nb.up;
-  const double hdt = wb_half(dt);
 #pragma unroll
   for (int cc = 0; cc < 8; ++cc) z.qn[cc] = v.q[cc][q];
   const double ir = wb_rcp(z.qn[F_RHO]);
@@ -839,7 +844,7 @@ __device__ __forceinline__ void trans_zone(const WbView& v, long long q, long lo
     z.vv[e] = __dmul_rn(z.qn[F_MX + e], ir);
     z.B[e] = z.qn[F_BX + e];
     z.Bv[e] = __dmul_rn(z.B[e], z.vv[e]);
-    z.c[e] = __dmul_rn(hdt, g.idx[e]);
+    z.c[e] = v.scal->hdtdx[e];
     z.hdb[e] = __dmul_rn(__dsub_rn(v.b[e][q + s[e]], v.b[e][q]), z.c[e]);
   }
 #pragma unroll
@@ -877,8 +882,8 @@ __device__ __forceinline__ void trans_dir(const WbView& v, long long w, const Nb
 
 // The directions in mask (bit d) at one zone, sharing the zone quantities and
 // each transverse flux difference between the two states that use it.
-__device__ __forceinline__ void transverse_set(const WbView& v, long long qo, long long wo, double dt,
-                                               int mask, int i, int j, int k, const Nbr& nb) {
+__device__ __forceinline__ void transverse_set(const WbView& v, long long qo, long long wo, int mask,
+                                               int i, int j, int k, const Nbr& nb) {
   const long long q = qo + wb_at(v.geo, i, j, k);
   const long long w = wo + wb_at(v.geo, i, j, k);
   WB_CHECK_ZONE(v.geo, i + 1, j + 1, k + 1);  // the high neighbours of every axis
@@ -888,7 +893,7 @@ __device__ __forceinline__ void transverse_set(const WbView& v, long long qo, lo
   for (int e = 0; e < 3; ++e)
     if (mask & ~(1 << e)) need |= 1 << e;
   TransZone z;
-  trans_zone(v, q, w, dt, need, nb, z);
+  trans_zone(v, q, w, need, nb, z);
   if (mask & 1) trans_dir<0>(v, w, nb, z);
   if (mask & 2) trans_dir<1>(v, w, nb, z);
   if (mask & 4) trans_dir<2>(v, w, nb, z);
@@ -1082,7 +1087,7 @@ __device__ __forceinline__ double signal_rate(double rho, double mx, double my, 
 // zero-gradient rule); the last zone's field then averages that copy, so the
 // stored state is the one a load of the same faces gives.
 __device__ __forceinline__ double final_update(const WbView& v, long long qo, long long wo,
-                                               double dt, const WbPhys& P, int i, int j, int k, const Nbr& nb,
+                                               const WbPhys& P, int i, int j, int k, const Nbr& nb,
                                                int ohi, int* hits, int* bad) {
   const WbGeo& g = v.geo;
   const long long q = qo + wb_at(g, i, j, k);
@@ -1090,7 +1095,7 @@ __device__ __forceinline__ double final_update(const WbView& v, long long qo, lo
   WB_CHECK_ZONE(g, i + 1, j + 1, k + 1);
   const long long (&s)[3] = nb.up;
   // explicit rounding: the same bits in every kernel this is inlined into
-  const double cx = __dmul_rn(dt, g.idx[0]), cy = __dmul_rn(dt, g.idx[1]), cz = __dmul_rn(dt, g.idx[2]);
+  const double cx = v.scal->dtdx[0], cy = v.scal->dtdx[1], cz = v.scal->dtdx[2];
   double u[5];
 #pragma unroll
   for (int c = 0; c < 5; ++c) {
