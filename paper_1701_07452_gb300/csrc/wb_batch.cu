@@ -223,10 +223,6 @@ __device__ __forceinline__ void warp_max_key(unsigned long long bits, unsigned l
   if ((threadIdx.x & 31) == 0 && bits) atomicMax(dst, bits);
 }
 
-__device__ __forceinline__ void warp_max_atomic(double w, unsigned long long* dst) {
-  warp_max_key(wb_rate_bits(w), dst);
-}
-
 // One tile of a sweep of one box (every thread of the block).
 template <int EZ, bool PROT>
 __device__ __forceinline__ int box_sweep_tile(const BoxInfo& bi, bool corr, int d, long long tile,
@@ -239,6 +235,14 @@ __device__ __forceinline__ int box_sweep_tile(const BoxInfo& bi, bool corr, int 
                                           v.scal, P, X);
 }
 
+__device__ __forceinline__ void item_ijk(const WbBox& b, long long item, int* i, int* j, int* k) {
+  const unsigned nx = b.hi[0] - b.lo[0] + 1, ny = b.hi[1] - b.lo[1] + 1;
+  const unsigned t = (unsigned)item, r = t / nx, z = r / ny;  // a box's items fit 32 bits
+  *i = b.lo[0] + (int)(t - r * nx);
+  *j = b.lo[1] + (int)(r - z * ny);
+  *k = b.lo[2] + (int)z;
+}
+
 __device__ __forceinline__ void unit_item(const BatchParams& B, int s, int d, const BoxInfo& bi, long long item,
                                           double dt, unsigned long long* wkey, int* hits, int* bad) {
   const WbView& v = bi.v;
@@ -247,11 +251,8 @@ __device__ __forceinline__ void unit_item(const BatchParams& B, int s, int d, co
   // the remaining stages (transverse states, half-step EMF, update); the
   // cheap ones go through unit_pair
   const WbBox b = stage_box(s, d, n, wrap);
-  const int nx = b.hi[0] - b.lo[0] + 1, ny = b.hi[1] - b.lo[1] + 1;
-  const int i = b.lo[0] + (int)(item % nx);
-  const long long r = item / nx;
-  const int j = b.lo[1] + (int)(r % ny);
-  const int k = b.lo[2] + (int)(r / ny);
+  int i, j, k;
+  item_ijk(b, item, &i, &j, &k);
   const wbu::Nbr nb = wbu::neighbours(v.geo, i, j, k, wrap ? 7 : 0);
   switch (s) {
     case BS_TRANS: {
@@ -278,14 +279,6 @@ __device__ __forceinline__ void unit_item(const BatchParams& B, int s, int d, co
 __host__ __device__ inline bool stage_pairs(int s) {
   return s == BS_EREF || s == BS_EDGE_P || s == BS_EDGE_C || s == BS_CT_H || s == BS_CT_F ||
          s == BS_HALO;
-}
-
-__device__ __forceinline__ void item_ijk(const WbBox& b, long long item, int* i, int* j, int* k) {
-  const int nx = b.hi[0] - b.lo[0] + 1, ny = b.hi[1] - b.lo[1] + 1;
-  *i = b.lo[0] + (int)(item % nx);
-  const long long r = item / nx;
-  *j = b.lo[1] + (int)(r % ny);
-  *k = b.lo[2] + (int)(r / ny);
 }
 
 // Copy of one array for two shell points: both loads issue before either
@@ -657,24 +650,6 @@ __global__ void __launch_bounds__(kNtZone, zone_min_blocks(CLS))
     }
   });
   stage_stamp(B, s, seq);
-}
-
-// initial signal rate of one box (the view is passed by value: the device box
-// table is only uploaded before the next launch of k_batch)
-__global__ void k_box_rate(WbView v, WbScalars* scal, WbPhys P) {
-  const WbGeo& g = v.geo;
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  const long long nint = (long long)g.n[0] * g.n[1] * g.n[2];
-  double w = 0.0;
-  if (t < nint) {
-    const int i = (int)(t % g.n[0]);
-    const int j = (int)((t / g.n[0]) % g.n[1]);
-    const int k = (int)(t / ((long long)g.n[0] * g.n[1]));
-    const long long o = wb_at(g, i, j, k);
-    w = wbu::signal_rate(v.q[0][o], v.q[1][o], v.q[2][o], v.q[3][o], v.q[4][o], v.q[5][o], v.q[6][o],
-                         v.q[7][o], P, g, scal);
-  }
-  warp_max_atomic(w, &scal->wmax_next);
 }
 
 const int kWorkB = 3 * 7 + 3 + 3 + 3 + 3 * 8;  // 54: corrector fluxes, half-step EMFs alias
@@ -1336,6 +1311,7 @@ int wb_batch_load(wb_batch* b, int box, const double* U, const double* bx, const
   cudaStream_t s = b->stream;
   const long long nc = (long long)d.n[0] * d.n[1] * d.n[2];
   const double* faces[3] = {bx, by, bz};
+  MoveList all = {};
   for (int comp = 0; comp < 8; ++comp) {
     long long ext[3] = {d.n[0], d.n[1], d.n[2]};
     const double* src;
@@ -1349,8 +1325,10 @@ int wb_batch_load(wb_batch* b, int box, const double* U, const double* bx, const
       dsrc = b->staging;
     }
     double* dst = comp < 5 ? bi.v.q[comp] : bi.v.b[comp - 5];
-    wb_launch_scatter(dsrc, dst, comp, g, m, s);
+    wb_add_move(all, dsrc, dst, comp);
     if (!on_device) {
+      wb_launch_scatter(all, g, m, s);
+      all.n = 0;
       cudaError_t e = cudaStreamSynchronize(s);
       if (e != cudaSuccess) return bcuda(b, e, "batch load");
     }
@@ -1359,14 +1337,12 @@ int wb_batch_load(wb_batch* b, int box, const double* U, const double* bx, const
   double* bb[3];
   for (int c = 0; c < 8; ++c) q[c] = bi.v.q[c];
   for (int c = 0; c < 3; ++c) bb[c] = bi.v.b[c];
-  wb_launch_halo(q, bb, g, m, s);
-  wb_launch_ccb(q, bb, g, 1, 0, s);
-  if (primitive) wb_launch_prim_to_cons(q, g, 1, b->phys, s);
-  wb_launch_halo(q, bb, g, m, s);
+  wb_launch_scatter(all, g, m, s);
   cudaError_t e = cudaMemsetAsync(b->d_scal + box, 0, sizeof(WbScalars), s);
   if (e != cudaSuccess) return bcuda(b, e, "batch load");
-  const long long nint = (long long)g.n[0] * g.n[1] * g.n[2];
-  k_box_rate<<<(unsigned)((nint + 255) / 256), 256, 0, s>>>(bi.v, b->d_scal + box, b->phys);
+  if (!bi.wrap) wb_launch_halo(q, bb, g, m, s);
+  wb_launch_init(q, bb, g, 1, bi.wrap ? 7 : 0, b->phys, primitive != 0, b->d_scal + box, s);
+  if (!bi.wrap) wb_launch_halo(q, bb, g, m, s);
   e = cudaStreamSynchronize(s);
   if (e == cudaSuccess) e = cudaGetLastError();
   return bcuda(b, e, "batch load");
@@ -1443,6 +1419,7 @@ int wb_batch_read(wb_batch* b, int box, double* U, double* bx, double* by, doubl
   cudaStream_t s = b->stream;
   const long long nc = (long long)d.n[0] * d.n[1] * d.n[2];
   double* faces[3] = {bx, by, bz};
+  MoveList all = {};
   for (int comp = 0; comp < 11; ++comp) {
     double* dst;
     const double* src;
@@ -1457,14 +1434,17 @@ int wb_batch_read(wb_batch* b, int box, double* U, double* bx, double* by, doubl
       dst = B + (comp - 8) * nc; src = bi.v.q[F_BX + comp - 8]; mcomp = 0;
     }
     double* ddst = on_device ? dst : b->staging;
-    wb_launch_gather(src, ddst, mcomp, g, m, s);
+    wb_add_move(all, src, ddst, mcomp);
     if (!on_device) {
+      wb_launch_gather(all, g, m, s);
+      all.n = 0;
       cudaError_t e = cudaMemcpyAsync(dst, b->staging, sizeof(double) * ext[0] * ext[1] * ext[2],
                                       cudaMemcpyDeviceToHost, s);
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);
       if (e != cudaSuccess) return bcuda(b, e, "batch read");
     }
   }
+  wb_launch_gather(all, g, m, s);
   return bcuda(b, cudaGetLastError(), "batch read");
 }
 

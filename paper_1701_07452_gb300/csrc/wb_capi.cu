@@ -465,6 +465,7 @@ int load_common(wb_grid* g, const double* U, const double* bx, const double* by,
   cudaStream_t s = g->stream;
   const long long nc = (long long)g->d.n[0] * g->d.n[1] * g->d.n[2];
   const double* faces[3] = {bx, by, bz};
+  MoveList direct = {};  // arrays a kernel can read where they are: one launch
   for (int comp = 0; comp < 8; ++comp) {
     long long ext[3] = {g->d.n[0], g->d.n[1], g->d.n[2]};
     const double* src;
@@ -481,22 +482,22 @@ int load_common(wb_grid* g, const double* U, const double* bx, const double* by,
       dsrc = g->staging;
     }
     double* dst = comp < 5 ? g->q[comp] : g->b[comp - 5];
-    wb_launch_scatter(dsrc, dst, comp, g->geo, g->map, s);
+    if (!staged) wb_add_move(direct, dsrc, dst, comp);
     if (staged) {
+      MoveList one = {};
+      wb_add_move(one, dsrc, dst, comp);
+      wb_launch_scatter(one, g->geo, g->map, s);
       // staging is reused by the next component
       int rc = sync(g, "load");
       if (rc) return rc;
     }
   }
-  if (!g->closed) wb_launch_halo(g->q, g->b, g->geo, g->map, s);
-  wb_launch_ccb(g->q, g->b, g->geo, g->npatch, g->closed, s);
-  if (primitive) wb_launch_prim_to_cons(g->q, g->geo, g->npatch, g->phys, s);
-  if (!g->closed) wb_launch_halo(g->q, g->b, g->geo, g->map, s);
-  WbScalars z;
-  std::memset(&z, 0, sizeof(z));
-  cudaError_t e = cudaMemcpyAsync(g->scal, &z, sizeof(z), cudaMemcpyHostToDevice, s);
+  wb_launch_scatter(direct, g->geo, g->map, s);
+  cudaError_t e = cudaMemsetAsync(g->scal, 0, sizeof(WbScalars), s);
   if (e != cudaSuccess) return check_cuda(g, e, "load scalars");
-  wb_launch_dt_init(g->q, g->geo, g->npatch, g->phys, g->scal, s);
+  if (!g->closed) wb_launch_halo(g->q, g->b, g->geo, g->map, s);
+  wb_launch_init(g->q, g->b, g->geo, g->npatch, g->closed, g->phys, primitive, g->scal, s);
+  if (!g->closed) wb_launch_halo(g->q, g->b, g->geo, g->map, s);
   int rc = sync(g, "load");
   if (rc) return rc;
   g->loaded = true;
@@ -698,6 +699,7 @@ int wb_read_state(wb_grid* g, double* U, double* bx, double* by, double* bz, dou
   cudaStream_t s = g->stream;
   const long long nc = (long long)g->d.n[0] * g->d.n[1] * g->d.n[2];
   double* faces[3] = {bx, by, bz};
+  MoveList direct = {};  // arrays a kernel can write where they are: one launch
   for (int comp = 0; comp < 11; ++comp) {
     double* dst;
     int mcomp = comp;
@@ -715,13 +717,17 @@ int wb_read_state(wb_grid* g, double* U, double* bx, double* by, double* bz, dou
     const void* mapped = on_device ? nullptr : host_mapped(dst, n);
     const bool staged = !on_device && !mapped;
     double* ddst = on_device ? dst : (mapped ? static_cast<double*>(const_cast<void*>(mapped)) : g->staging);
-    wb_launch_gather(src, ddst, mcomp, g->geo, g->map, s);
+    if (!staged) wb_add_move(direct, src, ddst, mcomp);
     if (staged) {
+      MoveList one = {};
+      wb_add_move(one, src, ddst, mcomp);
+      wb_launch_gather(one, g->geo, g->map, s);
       cudaError_t e = cudaMemcpyAsync(dst, g->staging, sizeof(double) * n, cudaMemcpyDeviceToHost, s);
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);
       if (e != cudaSuccess) return check_cuda(g, e, "read");
     }
   }
+  wb_launch_gather(direct, g->geo, g->map, s);
   // host arrays written in place by the kernels are complete once the stream is
   if (!on_device) {
     cudaError_t e = cudaStreamSynchronize(s);
@@ -980,26 +986,23 @@ int wb_step_noalloc(const wb_desc* d, const double* U, const double* bx, const d
   if (e != cudaSuccess) return noalloc_fail(WB_ERR_CUDA, std::string("memset: ") + cudaGetErrorString(e));
   const double* faces[3] = {bx, by, bz};
   const long long nc = (long long)one.n[0] * one.n[1] * one.n[2];
-  for (int comp = 0; comp < 8; ++comp) {
-    const double* src = comp < 5 ? U + comp * nc : faces[comp - 5];
-    double* dst = comp < 5 ? g.q[comp] : g.b[comp - 5];
-    wb_launch_scatter(src, dst, comp, g.geo, g.map, s);
-  }
+  MoveList in = {};
+  for (int comp = 0; comp < 8; ++comp)
+    wb_add_move(in, comp < 5 ? U + comp * nc : faces[comp - 5], comp < 5 ? g.q[comp] : g.b[comp - 5], comp);
+  wb_launch_scatter(in, g.geo, g.map, s);
   set_interior(&g);
   if (!g.closed) wb_launch_halo(g.q, g.b, g.geo, g.map, s);
-  wb_launch_ccb(g.q, g.b, g.geo, 1, g.closed, s);
+  wb_launch_init(g.q, g.b, g.geo, 1, g.closed, g.phys, false, g.scal, s);
   if (!g.closed) wb_launch_halo(g.q, g.b, g.geo, g.map, s);
-  wb_launch_dt_init(g.q, g.geo, 1, g.phys, g.scal, s);
   StepControl c = step_control(&g, 0.0);
   c.lag = 0;
   wb_launch_dt_step(g.scal, c, s);
   enqueue_pass(&g, 0, 1, c);
   double* outs[3] = {bx_out, by_out, bz_out};
-  for (int comp = 0; comp < 8; ++comp) {
-    const double* src = comp < 5 ? g.q[comp] : g.b[comp - 5];
-    double* dst = comp < 5 ? U_out + comp * nc : outs[comp - 5];
-    wb_launch_gather(src, dst, comp, g.geo, g.map, s);
-  }
+  MoveList out = {};
+  for (int comp = 0; comp < 8; ++comp)
+    wb_add_move(out, comp < 5 ? g.q[comp] : g.b[comp - 5], comp < 5 ? U_out + comp * nc : outs[comp - 5], comp);
+  wb_launch_gather(out, g.geo, g.map, s);
   if (dt_out) {
     e = cudaMemcpyAsync(dt_out, &g.scal->dt, sizeof(double), cudaMemcpyDeviceToDevice, s);
     if (e != cudaSuccess) return noalloc_fail(WB_ERR_CUDA, std::string("dt copy: ") + cudaGetErrorString(e));

@@ -93,18 +93,26 @@ struct WrapList {
 // Periodic images on every axis: one patch (the box's own interior) or all
 // patches of a grid resident in one pass (slot = patch, neighbour patches).
 void wb_launch_wrap(const WrapList& L, const WbGeo& geo, const GridMap& m, int depth, cudaStream_t s);
-void wb_launch_dt_init(double* const q[8], const WbGeo& geo, long long npatch, const WbPhys& ph,
-                       WbScalars* scal, cudaStream_t s);
+// The zone field, conserved state (from a primitive one) and first signal rate
+// of a loaded state.
+void wb_launch_init(double* const q[8], double* const b[3], const WbGeo& geo, long long npatch, int closed,
+                    const WbPhys& ph, bool primitive, WbScalars* scal, cudaStream_t s);
 void wb_launch_dt_step(WbScalars* scal, const StepControl& c, cudaStream_t s);
-void wb_launch_ccb(double* const q[8], double* const b[3], const WbGeo& geo, long long npatch, int closed,
-                   cudaStream_t s);
-void wb_launch_prim_to_cons(double* const q[8], const WbGeo& geo, long long npatch,
-                            const WbPhys& ph, cudaStream_t s);
-// global <-> patch copies; comp: 0..4 zone field, 5..7 face field of axis comp-5
-void wb_launch_scatter(const double* src, double* dst_field, int comp, const WbGeo& geo,
-                       const GridMap& m, cudaStream_t s);
-void wb_launch_gather(const double* src_field, double* dst, int comp, const WbGeo& geo,
-                      const GridMap& m, cudaStream_t s);
+// global <-> patch copies of up to 11 arrays; comp: 0..4 zone field, 5..7 face
+// field of axis comp-5
+struct MoveList {
+  const double* src[11];
+  double* dst[11];
+  int comp[11];
+  int n;
+};
+inline void wb_add_move(MoveList& L, const double* src, double* dst, int comp) {
+  L.src[L.n] = src;
+  L.dst[L.n] = dst;
+  L.comp[L.n++] = comp;
+}
+void wb_launch_scatter(const MoveList& L, const WbGeo& geo, const GridMap& m, cudaStream_t s);
+void wb_launch_gather(const MoveList& L, const WbGeo& geo, const GridMap& m, cudaStream_t s);
 // Conserved totals: nblocks partial pairs in part (16 doubles each), the 8
 // totals x vol in out (device memory).
 void wb_launch_totals(double* const q[8], double* const b[3], const WbGeo& geo, long long npatch, double vol,

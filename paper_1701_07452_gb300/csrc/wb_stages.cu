@@ -9,13 +9,16 @@
 
 namespace {
 
-__device__ __forceinline__ bool box_index(const WbBox& b, long long t, int& i, int& j, int& k) {
-  const int nx = b.hi[0] - b.lo[0] + 1, ny = b.hi[1] - b.lo[1] + 1, nz = b.hi[2] - b.lo[2] + 1;
-  if (t >= (long long)nx * ny * nz) return false;
-  i = b.lo[0] + (int)(t % nx);
-  long long r = t / nx;
-  j = b.lo[1] + (int)(r % ny);
-  k = b.lo[2] + (int)(r / ny);
+// Item t of an index box.  The item counts of a patch fit 32 bits (the padded
+// arrays of 2^32 zones would not fit any device), and 64-bit divisions cost a
+// thread some hundred instructions.
+__device__ __forceinline__ bool box_index(const WbBox& b, unsigned t, int& i, int& j, int& k) {
+  const unsigned nx = b.hi[0] - b.lo[0] + 1, ny = b.hi[1] - b.lo[1] + 1, nz = b.hi[2] - b.lo[2] + 1;
+  if (t >= nx * ny * nz) return false;
+  const unsigned r = t / nx, z = r / ny;
+  i = b.lo[0] + (int)(t - r * nx);
+  j = b.lo[1] + (int)(r - z * ny);
+  k = b.lo[2] + (int)z;
   return true;
 }
 
@@ -59,7 +62,7 @@ __global__ void k_edges(StageArgs A, bool corr, Boxes3 B) {
   wb_pdl_begin();
   if (!wb_pos(A.v.scal->dt)) return;
   int i, j, k;
-  if (!box_index(B.u, blockIdx.x * (long long)blockDim.x + threadIdx.x, i, j, k)) return;
+  if (!box_index(B.u, blockIdx.x * blockDim.x + threadIdx.x, i, j, k)) return;
   const long long wo = blockIdx.y * A.slot_w;
   const wbu::Nbr nb = wbu::neighbours(A.v.geo, i, j, k, A.closed);
   if (wbu::in_box(B.b[0], i, j, k)) wbu::edge<0>(A.v, wo, corr, i, j, k, nb);
@@ -73,7 +76,7 @@ __global__ void k_ct(StageArgs A, bool fin, Boxes3 B) {
   const double dt = A.v.scal->dt;
   if (!wb_pos(dt)) return;
   int i, j, k;
-  if (!box_index(B.u, blockIdx.x * (long long)blockDim.x + threadIdx.x, i, j, k)) return;
+  if (!box_index(B.u, blockIdx.x * blockDim.x + threadIdx.x, i, j, k)) return;
   const long long qo = blockIdx.y * A.slot_q, wo = blockIdx.y * A.slot_w;
   const wbu::Nbr nb = wbu::neighbours(A.v.geo, i, j, k, A.closed);
   if (wbu::in_box(B.b[0], i, j, k)) wbu::ct<0>(A.v, qo, wo, fin, dt, i, j, k, nb);
@@ -87,7 +90,7 @@ __global__ void k_transverse(StageArgs A, Boxes3 B) {
   wb_pdl_begin();
   if (!wb_pos(A.v.scal->dt)) return;
   int i, j, k;
-  if (!box_index(B.u, blockIdx.x * (long long)blockDim.x + threadIdx.x, i, j, k)) return;
+  if (!box_index(B.u, blockIdx.x * blockDim.x + threadIdx.x, i, j, k)) return;
   const int mask = (wbu::in_box(B.b[0], i, j, k) ? 1 : 0) | (wbu::in_box(B.b[1], i, j, k) ? 2 : 0) |
                    (wbu::in_box(B.b[2], i, j, k) ? 4 : 0);
   // zones that need every direction take the mask as a constant: with a run-time
@@ -103,7 +106,7 @@ __global__ void k_eref_half(StageArgs A, WbBox box) {
   const double dt = A.v.scal->dt;
   if (!wb_pos(dt)) return;
   int i, j, k;
-  if (!box_index(box, blockIdx.x * (long long)blockDim.x + threadIdx.x, i, j, k)) return;
+  if (!box_index(box, blockIdx.x * blockDim.x + threadIdx.x, i, j, k)) return;
   wbu::eref_half(A.v, blockIdx.y * A.slot_q, blockIdx.y * A.slot_w, dt, i, j, k,
                  wbu::neighbours(A.v.geo, i, j, k, A.closed));
 }
@@ -214,7 +217,7 @@ __global__ void k_final(StageArgs A, StepControl c) {
   const WbGeo& g = A.v.geo;
   WbBox box = {{0, 0, 0}, {g.n[0] - 1, g.n[1] - 1, g.n[2] - 1}};
   int i, j, k;
-  const bool ok = run && box_index(box, blockIdx.x * (long long)blockDim.x + threadIdx.x, i, j, k);
+  const bool ok = run && box_index(box, blockIdx.x * blockDim.x + threadIdx.x, i, j, k);
   double w = 0.0;
   int hits = 0, bad = 0;
   // axes along which this slot's patch is the last one of an outflow axis
@@ -284,75 +287,58 @@ __global__ void k_halo(StageArgs A, GridMap m) {
   for (int c = 0; c < 3; ++c) A.v.b[c][dst] = A.v.b[c][src];
 }
 
-__global__ void k_dt_init(StageArgs A, long long npatch) {
+__global__ void k_dt_step(WbScalars* s, StepControl c) {
+  wb_pdl_begin();
+  dt_step(s, c); }
+
+// The rest of a load, after the fields and owned faces (and, where the patch
+// is not its own neighbour, the face ghosts) are in place: the zone field as
+// the mean of the faces, primitive (rho, v, P) in fields 0..4 -> conserved (Eq.
+// totenergy), and the signal rate of the first step.
+__global__ void k_init(StageArgs A, int primitive) {
+  wb_pdl_begin();
   const WbGeo& g = A.v.geo;
-  long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  long long nint = (long long)g.n[0] * g.n[1] * g.n[2];
+  const WbBox box = {{0, 0, 0}, {g.n[0] - 1, g.n[1] - 1, g.n[2] - 1}};
+  int i, j, k;
   double w = 0.0;
-  if (t < nint * npatch) {
-    long long p = t / nint, r = t % nint;
-    int i = (int)(r % g.n[0]);
-    int j = (int)((r / g.n[0]) % g.n[1]);
-    int k = (int)(r / ((long long)g.n[0] * g.n[1]));
-    long long o = p * g.V + wb_at(g, i, j, k);
-    w = wbu::signal_rate(A.v.q[0][o], A.v.q[1][o], A.v.q[2][o], A.v.q[3][o], A.v.q[4][o], A.v.q[5][o], A.v.q[6][o],
-                    A.v.q[7][o], A.phys, g, A.v.scal);
+  if (box_index(box, blockIdx.x * blockDim.x + threadIdx.x, i, j, k)) {
+    const long long o = blockIdx.y * g.V + wb_at(g, i, j, k);
+    const wbu::Nbr nb = wbu::neighbours(g, i, j, k, A.closed);
+    double u[5], B[3];
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+      B[e] = 0.5 * (A.v.b[e][o] + A.v.b[e][o + nb.up[e]]);
+      A.v.q[F_BX + e][o] = B[e];
+    }
+#pragma unroll
+    for (int c = 0; c < 5; ++c) u[c] = A.v.q[c][o];
+    if (primitive) {
+      const double rho = u[0], vx = u[1], vy = u[2], vz = u[3], pr = u[4];
+      const double bx = B[0], by = B[1], bz = B[2];
+      u[1] = rho * vx;
+      u[2] = rho * vy;
+      u[3] = rho * vz;
+      u[4] = pr * A.phys.inv_gm1 + 0.5 * rho * (vx * vx + vy * vy + vz * vz) + 0.5 * (bx * bx + by * by + bz * bz);
+#pragma unroll
+      for (int c = 1; c < 5; ++c) A.v.q[c][o] = u[c];
+    }
+    w = wbu::signal_rate(u[0], u[1], u[2], u[3], u[4], B[0], B[1], B[2], A.phys, g, A.v.scal);
     if (!(w >= 0.0)) w = __longlong_as_double(0x7ff8000000000000LL);
   }
   block_max_atomic(w, &A.v.scal->wmax_next);
 }
 
-__global__ void k_dt_step(WbScalars* s, StepControl c) {
-  wb_pdl_begin();
-  dt_step(s, c); }
-
-__global__ void k_ccb(StageArgs A, long long npatch) {
-  const WbGeo& g = A.v.geo;
-  long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  long long nint = (long long)g.n[0] * g.n[1] * g.n[2];
-  if (t >= nint * npatch) return;
-  long long p = t / nint, r = t % nint;
-  int i = (int)(r % g.n[0]);
-  int j = (int)((r / g.n[0]) % g.n[1]);
-  int k = (int)(r / ((long long)g.n[0] * g.n[1]));
-  long long o = p * g.V + wb_at(g, i, j, k);
-  const wbu::Nbr nb = wbu::neighbours(g, i, j, k, A.closed);
-#pragma unroll
-  for (int e = 0; e < 3; ++e) A.v.q[F_BX + e][o] = 0.5 * (A.v.b[e][o] + A.v.b[e][o + nb.up[e]]);
-}
-
-// primitive (rho, v, P) in fields 0..4 -> conserved, with the zone field (Eq. totenergy)
-__global__ void k_prim_to_cons(StageArgs A, long long npatch) {
-  const WbGeo& g = A.v.geo;
-  long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  long long nint = (long long)g.n[0] * g.n[1] * g.n[2];
-  if (t >= nint * npatch) return;
-  long long p = t / nint, r = t % nint;
-  int i = (int)(r % g.n[0]);
-  int j = (int)((r / g.n[0]) % g.n[1]);
-  int k = (int)(r / ((long long)g.n[0] * g.n[1]));
-  long long o = p * g.V + wb_at(g, i, j, k);
-  double rho = A.v.q[0][o], vx = A.v.q[1][o], vy = A.v.q[2][o], vz = A.v.q[3][o], pr = A.v.q[4][o];
-  double bx = A.v.q[5][o], by = A.v.q[6][o], bz = A.v.q[7][o];
-  A.v.q[1][o] = rho * vx;
-  A.v.q[2][o] = rho * vy;
-  A.v.q[3][o] = rho * vz;
-  A.v.q[4][o] = pr * A.phys.inv_gm1 + 0.5 * rho * (vx * vx + vy * vy + vz * vz) +
-              0.5 * (bx * bx + by * by + bz * bz);
-}
-
-// global array (host layout) <-> patch interiors
+// global arrays (host layout) <-> patch interiors, one array per blockIdx.y
 template <bool SCATTER>
-__global__ void k_move(const double* src, double* dst, int comp, WbGeo g, GridMap m) {
-  int ext[3] = {m.N[0], m.N[1], m.N[2]};
+__global__ void k_move(MoveList L, WbGeo g, GridMap m) {
+  wb_pdl_begin();
+  const int comp = L.comp[blockIdx.y];
+  unsigned ext[3] = {(unsigned)m.N[0], (unsigned)m.N[1], (unsigned)m.N[2]};
   if (comp >= 5) ext[comp - 5] += 1;
-  long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  long long tot = (long long)ext[0] * ext[1] * ext[2];
-  if (t >= tot) return;
-  int G[3];
-  G[0] = (int)(t % ext[0]);
-  G[1] = (int)((t / ext[0]) % ext[1]);
-  G[2] = (int)(t / ((long long)ext[0] * ext[1]));
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= ext[0] * ext[1] * ext[2]) return;
+  const unsigned row = t / ext[0], z = row / ext[1];
+  int G[3] = {(int)(t - row * ext[0]), (int)(row - z * ext[1]), (int)z};
   // a read takes the high boundary face from the owned face it is an image of
   // (periodic: the first, outflow: the last), not from a ghost
   if (!SCATTER && comp >= 5 && G[comp - 5] == m.N[comp - 5])
@@ -361,19 +347,22 @@ __global__ void k_move(const double* src, double* dst, int comp, WbGeo g, GridMa
   int loc[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    int pc = G[d] / g.n[d];
-    if (pc >= m.np[d]) pc = m.np[d] - 1;  // the high boundary face of the last patch
-    loc[d] = G[d] - pc * g.n[d];
-    patch += pc * mul;
-    mul *= m.np[d];
+    loc[d] = G[d];
+    if (m.np[d] > 1) {
+      int pc = G[d] / g.n[d];
+      if (pc >= m.np[d]) pc = m.np[d] - 1;  // the high boundary face of the last patch
+      loc[d] = G[d] - pc * g.n[d];
+      patch += pc * mul;
+      mul *= m.np[d];
+    }
   }
-  long long o = patch * g.V + wb_at(g, loc[0], loc[1], loc[2]);
+  const long long o = patch * g.V + wb_at(g, loc[0], loc[1], loc[2]);
   if (SCATTER) {
     // faces at the high boundary are ghosts: filled by the halo fill instead
     if (comp >= 5 && loc[comp - 5] >= g.n[comp - 5]) return;
-    dst[o] = src[t];
+    L.dst[blockIdx.y][o] = L.src[blockIdx.y][t];
   } else {
-    dst[t] = src[o];
+    L.dst[blockIdx.y][t] = L.src[blockIdx.y][o];
   }
 }
 
@@ -549,49 +538,41 @@ void wb_launch_wrap(const WrapList& L, const WbGeo& geo, const GridMap& m, int d
   else wb_launch_dependent(k_wrap_patches, grid_for(n, (int)m.npatch, 256), 256, s, L, geo, m, depth, n);
 }
 
-void wb_launch_dt_init(double* const q[8], const WbGeo& geo, long long npatch, const WbPhys& ph,
-                       WbScalars* scal, cudaStream_t s) {
-  StageArgs a = mini_args(q, nullptr, geo);
+void wb_launch_init(double* const q[8], double* const b[3], const WbGeo& geo, long long npatch, int closed,
+                    const WbPhys& ph, bool primitive, WbScalars* scal, cudaStream_t s) {
+  StageArgs a = mini_args(q, b, geo);
+  a.closed = closed;
   a.phys = ph;
   a.v.scal = scal;
-  long long n = (long long)geo.n[0] * geo.n[1] * geo.n[2] * npatch;
-  k_dt_init<<<grid_for(n, 1, 256), 256, 0, s>>>(a, npatch);
+  const long long n = (long long)geo.n[0] * geo.n[1] * geo.n[2];
+  const int bs = stage_threads(n, (int)npatch, 256);
+  wb_launch_dependent(k_init, grid_for(n, (int)npatch, bs), bs, s, a, primitive ? 1 : 0);
 }
 
 void wb_launch_dt_step(WbScalars* scal, const StepControl& c, cudaStream_t s) {
   wb_launch_dependent(k_dt_step, 1, 1, s, scal, c);
 }
 
-void wb_launch_ccb(double* const q[8], double* const b[3], const WbGeo& geo, long long npatch, int closed,
-                   cudaStream_t s) {
-  StageArgs a = mini_args(q, b, geo);
-  a.closed = closed;
-  long long n = (long long)geo.n[0] * geo.n[1] * geo.n[2] * npatch;
-  k_ccb<<<grid_for(n, 1, 256), 256, 0, s>>>(a, npatch);
+namespace {
+template <bool SCATTER>
+void launch_move(const MoveList& L, const WbGeo& geo, const GridMap& m, cudaStream_t s) {
+  if (L.n <= 0) return;
+  long long most = 0;
+  for (int a = 0; a < L.n; ++a) {
+    long long ext[3] = {m.N[0], m.N[1], m.N[2]};
+    if (L.comp[a] >= 5) ext[L.comp[a] - 5] += 1;
+    most = ext[0] * ext[1] * ext[2] > most ? ext[0] * ext[1] * ext[2] : most;
+  }
+  wb_launch_dependent(k_move<SCATTER>, grid_for(most, L.n, 256), 256, s, L, geo, m);
+}
+}  // namespace
+
+void wb_launch_scatter(const MoveList& L, const WbGeo& geo, const GridMap& m, cudaStream_t s) {
+  launch_move<true>(L, geo, m, s);
 }
 
-void wb_launch_prim_to_cons(double* const q[8], const WbGeo& geo, long long npatch,
-                            const WbPhys& ph, cudaStream_t s) {
-  StageArgs a = mini_args(q, nullptr, geo);
-  a.phys = ph;
-  long long n = (long long)geo.n[0] * geo.n[1] * geo.n[2] * npatch;
-  k_prim_to_cons<<<grid_for(n, 1, 256), 256, 0, s>>>(a, npatch);
-}
-
-void wb_launch_scatter(const double* src, double* dst_field, int comp, const WbGeo& geo,
-                       const GridMap& m, cudaStream_t s) {
-  long long ext[3] = {m.N[0], m.N[1], m.N[2]};
-  if (comp >= 5) ext[comp - 5] += 1;
-  long long n = ext[0] * ext[1] * ext[2];
-  k_move<true><<<grid_for(n, 1, 256), 256, 0, s>>>(src, dst_field, comp, geo, m);
-}
-
-void wb_launch_gather(const double* src_field, double* dst, int comp, const WbGeo& geo,
-                      const GridMap& m, cudaStream_t s) {
-  long long ext[3] = {m.N[0], m.N[1], m.N[2]};
-  if (comp >= 5) ext[comp - 5] += 1;
-  long long n = ext[0] * ext[1] * ext[2];
-  k_move<false><<<grid_for(n, 1, 256), 256, 0, s>>>(src_field, dst, comp, geo, m);
+void wb_launch_gather(const MoveList& L, const WbGeo& geo, const GridMap& m, cudaStream_t s) {
+  launch_move<false>(L, geo, m, s);
 }
 
 void wb_launch_divb(double* const b[3], const WbGeo& geo, long long npatch, int closed,

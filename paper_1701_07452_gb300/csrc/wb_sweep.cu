@@ -43,11 +43,11 @@ __global__ void __launch_bounds__(wbu::kBlock, wbu::kSweepBlocks) k_sweep(SweepA
   const long long t = blockIdx.x;
   if (t >= A.tile0[3]) {  // Step 2: zone-centred reference EMF from q^n, one zone a thread
     const WbBox& e = A.ebox;
-    const int nx = e.hi[0] - e.lo[0] + 1, ny = e.hi[1] - e.lo[1] + 1, nz = e.hi[2] - e.lo[2] + 1;
-    const long long z = (t - A.tile0[3]) * wbu::kBlock + threadIdx.x, per = (long long)nx * ny * nz;
-    if (z >= per * A.nslots) return;
-    const long long slot = z / per, r = z - slot * per;
-    const long long at = wb_at(A.geo, e.lo[0] + (int)(r % nx), e.lo[1] + (int)(r / nx % ny), e.lo[2] + (int)(r / nx / ny));
+    const unsigned nx = e.hi[0] - e.lo[0] + 1, ny = e.hi[1] - e.lo[1] + 1, nz = e.hi[2] - e.lo[2] + 1;
+    const unsigned z = (unsigned)(t - A.tile0[3]) * wbu::kBlock + threadIdx.x, per = nx * ny * nz;
+    if (z >= per * (unsigned)A.nslots) return;
+    const unsigned slot = z / per, r = z - slot * per, row = r / nx, k = row / ny;
+    const long long at = wb_at(A.geo, e.lo[0] + (int)(r - row * nx), e.lo[1] + (int)(row - k * ny), e.lo[2] + (int)k);
     const double* const* q = A.s[0].q;  // the x frame: rho, Mx, My, Mz, E, Bx, By, Bz
     const long long o = slot * A.slot_in + at;
     wbu::ErefIn in;

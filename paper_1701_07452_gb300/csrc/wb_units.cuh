@@ -520,15 +520,16 @@ __device__ __forceinline__ int sweep_tile(const WbGeo& g, const WbBox& box, int 
   const int U = d == 0 ? 1 : 0, W = d == 2 ? 1 : 2;
   const int nu = box.hi[U] - box.lo[U] + 1, nw = box.hi[W] - box.lo[W] + 1;
   const int len = box.hi[d] - box.lo[d] + 1;
-  const long long npen = (long long)nu * nw * nslots;
+  // pencils and zones of a launch fit 32 bits (64-bit divisions cost hundreds of instructions)
+  const unsigned npen = (unsigned)(nu * nw) * (unsigned)nslots;
   const int t = threadIdx.x, lane = t % 32, wp = t / 32;
-  long long pen;
+  unsigned pen;
   int idx, left, right;  // zone along the pencil; neighbour lanes
   bool has_left, emit;
   if (ring) {
     const int per = 32 / len, seg = lane / len;
     idx = lane - seg * len;
-    pen = (tile * kWarps + wp) * per + seg;
+    pen = ((unsigned)tile * kWarps + wp) * per + seg;
     emit = seg < per && pen < npen;
     if (pen >= npen) pen = npen - 1;
     has_left = true;
@@ -536,12 +537,12 @@ __device__ __forceinline__ int sweep_tile(const WbGeo& g, const WbBox& box, int 
     right = idx < len - 1 ? lane + 1 : lane - len + 1;
     if (seg >= per) left = right = lane;
   } else {
-    const long long total = npen * (len + 3);
-    long long z = tile * kTile + t;
+    const unsigned total = npen * (unsigned)(len + 3);
+    unsigned z = (unsigned)tile * kTile + t;
     emit = z < total;
     if (z >= total) z = total - 1;
-    pen = z / (len + 3);
-    idx = (int)(z - pen * (len + 3)) - 2;
+    pen = z / (unsigned)(len + 3);
+    idx = (int)(z - pen * (unsigned)(len + 3)) - 2;
     has_left = idx > -2 && t > 0;
     emit = emit && idx >= 0 && idx < len && t >= 2 && t <= kBlock - 2;
     left = (lane + 31) % 32;
@@ -550,8 +551,8 @@ __device__ __forceinline__ int sweep_tile(const WbGeo& g, const WbBox& box, int 
     // (an open layout is only taken for 3 zones or more, see sweep_ring)
     if (closed) idx = idx < 0 ? idx + len : (idx >= len ? idx - len : idx);
   }
-  const long long slot = pen / ((long long)nu * nw);
-  const int r = (int)(pen - slot * nu * nw);
+  const long long slot = pen / (unsigned)(nu * nw);
+  const int r = (int)(pen - (unsigned)slot * (unsigned)(nu * nw));
   int pos[3];
   pos[U] = box.lo[U] + r % nu;
   pos[W] = box.lo[W] + r / nu;
