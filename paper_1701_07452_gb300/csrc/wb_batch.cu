@@ -230,7 +230,7 @@ __device__ __forceinline__ int box_sweep_tile(const BoxInfo& bi, bool corr, int 
   const WbView& v = bi.v;
   const bool wrap = bi.wrap != 0;
   const WbBox b = stage_box(corr ? BS_CORR : BS_PRED, d, v.geo.n, wrap);
-  return wbu::sweep_tile<EZ, PROT, true, false>(v.geo, b, d, bi.sw[corr ? 1 : 0][d], tile, wrap,
+  return wbu::sweep_tile<EZ, PROT, true, false, wbu::kAnyLayout>(v.geo, b, d, bi.sw[corr ? 1 : 0][d], tile, wrap,
                                           wbu::sweep_ring(b.hi[d] - b.lo[d] + 1, wrap), 1, 0, 0,
                                           v.scal, P, X);
 }

@@ -35,7 +35,7 @@ namespace {
 
 using wbu::kEpsZeroLD;
 
-template <int EZ, bool PROT, bool SOFT>
+template <int EZ, bool PROT, bool SOFT, int LAYOUT>
 __global__ void __launch_bounds__(wbu::kBlock, wbu::kSweepBlocks) k_sweep(SweepArgs A) {
   __shared__ wbu::LaneEdge X;
   wb_pdl_begin();
@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(wbu::kBlock, wbu::kSweepBlocks) k_sweep(SweepA
     return;
   }
   const int d = t >= A.tile0[2] ? 2 : (t >= A.tile0[1] ? 1 : 0);
-  const int hll = wbu::sweep_tile<EZ, PROT, SOFT, true>(A.geo, A.box[d], d, A.s[d], t - A.tile0[d], (A.closed >> d) & 1, A.ring[d] != 0,
+  const int hll = wbu::sweep_tile<EZ, PROT, SOFT, true, LAYOUT>(A.geo, A.box[d], d, A.s[d], t - A.tile0[d], (A.closed >> d) & 1, A.ring[d] != 0,
                                                   A.nslots, A.slot_in, A.slot_out, A.scal, A.phys, X);
   if (hll) atomicAdd((unsigned long long*)&A.scal->hll_faces, 1ULL);
 }
@@ -72,36 +72,51 @@ __global__ void __launch_bounds__(wbu::kBlock, wbu::kSweepBlocks) k_sweep(SweepA
 // Kernel variants: eps_k = 0 on the linearly degenerate waves (the default)
 // or general eps; protection floors off (the default) or on.
 void wb_launch_sweeps(SweepArgs a, cudaStream_t s) {
-  a.tile0[0] = 0;
-  for (int d = 0; d < 3; ++d) {
+  const bool ez = (a.phys.eps_zero & kEpsZeroLD) == kEpsZeroLD;
+  auto axis = [&](int d) {  // faces of a pencil
+    return a.box[d].hi[d] - a.box[d].lo[d] + 1;
+  };
+  int rings = 0;
+  for (int d = 0; d < 3; ++d) rings += a.ring[d] = wbu::sweep_ring(axis(d), (a.closed >> d) & 1);
+  auto tiles_of = [&](int d) {
     const int U = d == 0 ? 1 : 0, W = d == 2 ? 1 : 2;
     const WbBox& b = a.box[d];
-    const int len = b.hi[d] - b.lo[d] + 1;
-    a.ring[d] = wbu::sweep_ring(len, (a.closed >> d) & 1);
-    a.tile0[d + 1] = a.tile0[d] + wbu::sweep_tiles((long long)(b.hi[U] - b.lo[U] + 1) * (b.hi[W] - b.lo[W] + 1) * a.nslots,
-                                                   len, a.ring[d] != 0);
-  }
-  long long tiles = a.tile0[3];
+    return wbu::sweep_tiles((long long)(b.hi[U] - b.lo[U] + 1) * (b.hi[W] - b.lo[W] + 1) * a.nslots, axis(d), a.ring[d] != 0);
+  };
+  long long e = 0;  // tiles of the reference EMF
   if (a.Eref[0]) {
-    long long z = a.nslots;
-    for (int d = 0; d < 3; ++d) z *= a.ebox.hi[d] - a.ebox.lo[d] + 1;
-    tiles += (z + wbu::kBlock - 1) / wbu::kBlock;
+    e = a.nslots;
+    for (int d = 0; d < 3; ++d) e *= a.ebox.hi[d] - a.ebox.lo[d] + 1;
+    e = (e + wbu::kBlock - 1) / wbu::kBlock;
   }
-  const dim3 grid((unsigned)tiles);
-  const bool ez = (a.phys.eps_zero & kEpsZeroLD) == kEpsZeroLD;
   // With a block or less for each SM a scheduler has one warp: nothing hides the
   // integer products' latency, and the FP64 pipe has room for them (16^3: 18.7
   // against 22.4 us a launch; 24^3, 500 blocks: 35.1 against 28.9)
-  const bool soft = tiles > 152;
+  const bool soft = tiles_of(0) + tiles_of(1) + tiles_of(2) + e > 152;
+  // The default variant's large launches are compiled for each layout; when the
+  // axes differ, all take the open one (a thin axis only as a ring)
+  const bool fixed = ez && !a.phys.prot && soft && !(rings > 0 && rings < 3 && (axis(0) < 3 || axis(1) < 3 || axis(2) < 3));
+  if (fixed && rings < 3)
+    for (int d = 0; d < 3; ++d) a.ring[d] = 0;
+  a.tile0[0] = 0;
+  for (int d = 0; d < 3; ++d) a.tile0[d + 1] = a.tile0[d] + tiles_of(d);
+  const dim3 grid((unsigned)(a.tile0[3] + e));
+#define WB_SWEEP(...) wb_launch_dependent(k_sweep<__VA_ARGS__>, grid, wbu::kBlock, s, a)
   if (a.phys.prot) {
-    if (ez) wb_launch_dependent(k_sweep<kEpsZeroLD, true, true>, grid, wbu::kBlock, s, a);
-    else wb_launch_dependent(k_sweep<0, true, true>, grid, wbu::kBlock, s, a);
-  } else if (ez) {
-    if (soft) wb_launch_dependent(k_sweep<kEpsZeroLD, false, true>, grid, wbu::kBlock, s, a);
-    else wb_launch_dependent(k_sweep<kEpsZeroLD, false, false>, grid, wbu::kBlock, s, a);
+    if (ez) WB_SWEEP(kEpsZeroLD, true, true, wbu::kAnyLayout);
+    else WB_SWEEP(0, true, true, wbu::kAnyLayout);
+  } else if (!ez) {
+    WB_SWEEP(0, false, true, wbu::kAnyLayout);
+  } else if (!soft) {
+    WB_SWEEP(kEpsZeroLD, false, false, wbu::kAnyLayout);
+  } else if (!fixed) {
+    WB_SWEEP(kEpsZeroLD, false, true, wbu::kAnyLayout);
+  } else if (rings == 3) {
+    WB_SWEEP(kEpsZeroLD, false, true, wbu::kRing);
   } else {
-    wb_launch_dependent(k_sweep<0, false, true>, grid, wbu::kBlock, s, a);
+    WB_SWEEP(kEpsZeroLD, false, true, wbu::kOpen);
   }
+#undef WB_SWEEP
 }
 
 // Self-test of the FP64 reciprocal helpers against the library division and

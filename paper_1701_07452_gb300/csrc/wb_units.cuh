@@ -444,10 +444,13 @@ __device__ __forceinline__ double& cell_word(Cell& c, int i) {
   }
 }
 
-// The words that cross from one warp of a block to the next.
+// The words that cross from one warp of a block to another.  Of a warp's
+// threads at most two have a right neighbour in another warp, lane 31 (slot 0)
+// and the end of a ring that began in an earlier warp (slot 1), and two a left
+// one, lane 0 and the start of a ring that ends in a later warp.
 struct LaneEdge {
-  double cell[kWarps][kCellWords];                // zone of lane 31
-  double gt0[kWarps][7], gz31[kWarps][7];         // g-tilde of lane 0, limited slope of lane 31
+  double cell[kWarps][2][kCellWords];             // zone, to the right neighbour
+  double gt[kWarps][2][7], gz[kWarps][2][7];      // g-tilde to the left, limited slope to the right neighbour
 };
 
 // A sweep along one axis: fields in the sweep's frame (q: rho, Mn, Mt1, Mt2,
@@ -486,15 +489,18 @@ __host__ __device__ __forceinline__ void sweep_frame(const double* const* q, con
 // block takes kBlock zones of them, emits the faces that find both neighbours'
 // slopes in the block and advances by kTile: kTile / kBlock x len / (len + 3)
 // of the threads emit a face.  A closed pencil (periodic, its first and last
-// zone neighbours) of at most 32 zones can sit in a warp as a ring instead:
-// floor(32 / len) len of the 32 lanes emit.  The better of the two is taken
-// (16 and 32 zones: all lanes against 82 and 89 %; 24: 75 against 87 %).
+// zone neighbours) of at most kBlock zones can sit in a block as a ring
+// instead: floor(kBlock / len) len of its threads emit.  The better of the two
+// is taken: a ring at 16, 32, 64, 128 zones (all threads against 82, 89, 93,
+// 95 %), at 40 (94 against 91), not at 48 or 96 (75 against 92 and 95).
 __host__ __device__ __forceinline__ bool sweep_ring(int len, bool closed) {
-  return closed && len <= 32 && (32 / len) * len * (len + 3) * kBlock >= 32 * len * kTile;
+  return closed && len <= kBlock && (kBlock / len) * (len + 3) >= kTile;
 }
+// Kernels compiled for one layout, or for either at run time (2 % slower).
+enum { kOpen = 0, kRing = 1, kAnyLayout = 2 };
 // tiles (blocks' worth of work) of npen pencils
 __host__ __device__ __forceinline__ long long sweep_tiles(long long npen, int len, bool ring) {
-  const long long per = ring ? (long long)(32 / len) * kWarps : kTile;
+  const long long per = ring ? kBlock / len : kTile;
   const long long n = ring ? npen : npen * (len + 3) - 3;
   return (n + per - 1) / per;
 }
@@ -513,10 +519,11 @@ __host__ __device__ __forceinline__ long long sweep_tiles(long long npen, int le
 // A thread that marched along a pencil kept two zones, two slopes and a face
 // record in 226 to 255 registers and 40 KB of shared memory a block, which left
 // 2 warps per scheduler; one face per thread needs 168, 3 warps.
-template <int EZ, bool PROT, bool SOFT, bool NC>
+template <int EZ, bool PROT, bool SOFT, bool NC, int LAYOUT>
 __device__ __forceinline__ int sweep_tile(const WbGeo& g, const WbBox& box, int d, const SweepFrame& s, long long tile,
-                                          bool closed, bool ring, int nslots, long long slot_in, long long slot_out,
+                                          bool closed, bool ring_, int nslots, long long slot_in, long long slot_out,
                                           const WbScalars* scal, const WbPhys& P, LaneEdge& X) {
+  const bool ring = LAYOUT == kAnyLayout ? ring_ : LAYOUT == kRing;
   const int U = d == 0 ? 1 : 0, W = d == 2 ? 1 : 2;
   const int nu = box.hi[U] - box.lo[U] + 1, nw = box.hi[W] - box.lo[W] + 1;
   const int len = box.hi[d] - box.lo[d] + 1;
@@ -524,18 +531,18 @@ __device__ __forceinline__ int sweep_tile(const WbGeo& g, const WbBox& box, int 
   const unsigned npen = (unsigned)(nu * nw) * (unsigned)nslots;
   const int t = threadIdx.x, lane = t % 32, wp = t / 32;
   unsigned pen;
-  int idx, left, right;  // zone along the pencil; neighbour lanes
+  int idx, lt, rt;  // zone along the pencil; threads of the neighbours
   bool has_left, emit;
   if (ring) {
-    const int per = 32 / len, seg = lane / len;
-    idx = lane - seg * len;
-    pen = ((unsigned)tile * kWarps + wp) * per + seg;
+    const int per = kBlock / len, seg = t / len;
+    idx = t - seg * len;
+    pen = (unsigned)tile * per + seg;
     emit = seg < per && pen < npen;
     if (pen >= npen) pen = npen - 1;
     has_left = true;
-    left = idx > 0 ? lane - 1 : lane + len - 1;
-    right = idx < len - 1 ? lane + 1 : lane - len + 1;
-    if (seg >= per) left = right = lane;
+    lt = idx > 0 ? t - 1 : t + len - 1;
+    rt = idx < len - 1 ? t + 1 : t - len + 1;
+    if (seg >= per) lt = rt = t;
   } else {
     const unsigned total = npen * (unsigned)(len + 3);
     unsigned z = (unsigned)tile * kTile + t;
@@ -545,8 +552,8 @@ __device__ __forceinline__ int sweep_tile(const WbGeo& g, const WbBox& box, int 
     idx = (int)(z - pen * (unsigned)(len + 3)) - 2;
     has_left = idx > -2 && t > 0;
     emit = emit && idx >= 0 && idx < len && t >= 2 && t <= kBlock - 2;
-    left = (lane + 31) % 32;
-    right = (lane + 1) % 32;
+    lt = t > 0 ? t - 1 : t;
+    rt = t < kBlock - 1 ? t + 1 : t;
     // the zones past the ends of a closed pencil are those of its other end
     // (an open layout is only taken for 3 zones or more, see sweep_ring)
     if (closed) idx = idx < 0 ? idx + len : (idx >= len ? idx - len : idx);
@@ -564,18 +571,22 @@ __device__ __forceinline__ int sweep_tile(const WbGeo& g, const WbBox& box, int 
   const double b = ld<NC>(s.bn + off);
   Cell L;
   L.ir = 0.0;  // not used across a face
-  if (!ring) {
-    if (lane == 31) {
+  // neighbours in other warps go through X, unless every ring sits in a warp
+  const bool cross = !(ring && 32 % len == 0);
+  const int wl = lt / 32, wr = rt / 32, sl = lt % 32 == 31 ? 0 : 1, sr = rt % 32 == 0 ? 0 : 1;
+  const int mine_r = lane == 31 ? 0 : 1, mine_l = lane == 0 ? 0 : 1;
+  if (cross) {
+    if (wr != wp) {
 #pragma unroll
-      for (int i = 0; i < kCellWords; ++i) X.cell[wp][i] = cell_word(R, i);
+      for (int i = 0; i < kCellWords; ++i) X.cell[wp][mine_r][i] = cell_word(R, i);
     }
     __syncthreads();
   }
 #pragma unroll
-  for (int i = 0; i < kCellWords; ++i) cell_word(L, i) = __shfl_sync(0xffffffffu, cell_word(R, i), left);
-  if (!ring && lane == 0 && wp > 0) {
+  for (int i = 0; i < kCellWords; ++i) cell_word(L, i) = __shfl_sync(0xffffffffu, cell_word(R, i), lt % 32);
+  if (cross && wl != wp) {
 #pragma unroll
-    for (int i = 0; i < kCellWords; ++i) cell_word(L, i) = X.cell[wp - 1][i];
+    for (int i = 0; i < kCellWords; ++i) cell_word(L, i) = X.cell[wl][sl][i];
   }
   RegRec f;
   double gt[7];
@@ -592,31 +603,31 @@ __device__ __forceinline__ int sweep_tile(const WbGeo& g, const WbBox& box, int 
     for (int k = 0; k < 7; ++k) gt[k] = 0.0;
   }
   __syncwarp();
-  if (!ring) {
-    if (lane == 0) {
+  if (cross) {
+    if (wl != wp) {
 #pragma unroll
-      for (int k = 0; k < 7; ++k) X.gt0[wp][k] = gt[k];
+      for (int k = 0; k < 7; ++k) X.gt[wp][mine_l][k] = gt[k];
     }
     __syncthreads();
   }
   double gz[7], gl[7];  // 2 g of this zone, of the left zone
 #pragma unroll
   for (int k = 0; k < 7; ++k) {
-    double gr = __shfl_sync(0xffffffffu, gt[k], right);
-    if (!ring && lane == 31 && wp < kWarps - 1) gr = X.gt0[wp + 1][k];
+    double gr = __shfl_sync(0xffffffffu, gt[k], rt % 32);
+    if (cross && wr != wp) gr = X.gt[wr][sr][k];
     gz[k] = wb_sweby(gr, gt[k], P.sweby, P.minmod);
   }
-  if (!ring) {
-    if (lane == 31) {
+  if (cross) {
+    if (wr != wp) {
 #pragma unroll
-      for (int k = 0; k < 7; ++k) X.gz31[wp][k] = gz[k];
+      for (int k = 0; k < 7; ++k) X.gz[wp][mine_r][k] = gz[k];
     }
     __syncthreads();
   }
 #pragma unroll
   for (int k = 0; k < 7; ++k) {
-    gl[k] = __shfl_sync(0xffffffffu, gz[k], left);
-    if (!ring && lane == 0 && wp > 0) gl[k] = X.gz31[wp - 1][k];
+    gl[k] = __shfl_sync(0xffffffffu, gz[k], lt % 32);
+    if (cross && wl != wp) gl[k] = X.gz[wl][sl][k];
   }
   if (!emit) return 0;
   double out[7];

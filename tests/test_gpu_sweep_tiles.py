@@ -1,5 +1,6 @@
 """The sweeps' thread layouts (wbu::sweep_tile) at the sizes where they change:
-rings of periodic pencils of up to 32 zones, the open layout's block edges
+rings of periodic pencils of up to 128 zones (inside a warp, straddling two,
+spanning a block), the open layout's block edges
 (125 faces emitted from 128 zones, 3 zones between pencils), pencils shorter
 than the stencil, and outflow boxes, whose pencils are never closed.  One step
 against the oracle."""
@@ -22,7 +23,7 @@ def wb():
 
 @pytest.mark.parametrize("n,bc", [
     ((16, 8, 4), (0, 0, 0)), ((32, 24, 5), (0, 0, 0)), ((30, 17, 33), (0, 0, 0)), ((122, 3, 2), (0, 0, 0)),
-    ((125, 31, 1), (0, 0, 0)), ((2, 126, 6), (0, 0, 0)), ((1, 5, 40), (0, 0, 0)),
+    ((125, 31, 1), (0, 0, 0)), ((2, 126, 6), (0, 0, 0)), ((1, 5, 40), (0, 0, 0)), ((20, 64, 42), (0, 0, 0)), ((128, 3, 21), (0, 0, 0)), ((127, 60, 3), (0, 0, 0)),
     ((16, 32, 8), (1, 1, 1)), ((59, 4, 61), (1, 0, 0)), ((119, 2, 3), (0, 0, 1)), ((1, 1, 7), (1, 1, 1)),
 ])
 def test_one_step_matches_the_oracle(wb, oracle_mod, n, bc):
