@@ -56,10 +56,32 @@ __device__ __forceinline__ double ld(const double* p) {
 }
 
 // A product of the sweeps: on the integer pipes (SOFT) or the FP64 pipe, the
-// same bits.
-template <bool SOFT>
+// same bits.  The integer form neither looks for infinities and NaN nor for
+// overflow: a sweep takes it where every zone field and face field is below
+// 2^50 in magnitude, the density above 2^-50 (field_wild) and the Roe state's
+// a^2 above 2^-100 (face_system).  No product then leaves the range: with
+// dt/dx < 2^50 too, |v| < 2^100, a^2 < 2^204, every alpha_k < 2^356, |nu_k| <
+// 2^155, g-tilde < 2^668, the sum of beta_k R_k below 2^920.
+// KNOWN: what follows from those bounds for the factors (wb_smul_finite).
+template <bool SOFT, int KNOWN = 0>
 __device__ __forceinline__ double mul(double x, double y) {
-  return SOFT ? wb_smul(x, y) : __dmul_rn(x, y);
+  return SOFT ? wb_smul_finite<KNOWN>(x, y) : __dmul_rn(x, y);
+}
+// Reciprocals and roots of values those bounds keep normal (the FP64 form of a
+// sweep, which meets everything else, looks at its inputs).
+template <bool SOFT>
+__device__ __forceinline__ double recip(double x) {
+  return SOFT ? wb_rcp_sure(x) : wb_rcp(x);
+}
+template <bool SOFT>
+__device__ __forceinline__ WbRoots roots(double x) {
+  return SOFT ? wb_roots_sure(x) : wb_roots(x);
+}
+
+// |x| or dt/dx in units of the test above: the high word without its sign, twice
+__device__ __forceinline__ unsigned field_size(double x) { return wb_hi32(x) << 1; }
+__device__ __forceinline__ bool field_wild(unsigned size, double rho) {
+  return size >= ((1023u + 50u) << 21) || wb_hi32(rho) - ((1023u - 50u) << 20) >= (100u << 20);
 }
 
 // Zone state of a sweep.  The arithmetic is written with explicit rounding
@@ -67,9 +89,9 @@ __device__ __forceinline__ double mul(double x, double y) {
 // inside the march over a segment, and the two inlined copies must round
 // identically, or a face's flux would depend on where a segment starts.
 // q: the fields in the sweep's frame (rho, Mn, Mt1, Mt2, E, Bn, Bt1, Bt2).
+// Returns the largest field_size of its fields.
 template <bool NC, bool SOFT>
-__device__ __forceinline__ void load_cell(const double* const (&q)[8], long long off, const WbPhys& P,
-                                                Cell& c) {
+__device__ __forceinline__ unsigned load_cell(const double* const (&q)[8], long long off, const WbPhys& P, Cell& c) {
   c.rho = ld<NC>(q[0] + off);
   c.mn = ld<NC>(q[1] + off);
   c.mt1 = ld<NC>(q[2] + off);
@@ -78,12 +100,14 @@ __device__ __forceinline__ void load_cell(const double* const (&q)[8], long long
   const double bn = ld<NC>(q[5] + off);
   c.bt1 = ld<NC>(q[6] + off);
   c.bt2 = ld<NC>(q[7] + off);
-  const WbRoots rr = wb_roots(c.rho);
+  const unsigned size = max(max(max(field_size(c.mn), field_size(c.mt1)), max(field_size(c.mt2), field_size(e))),
+                            max(max(field_size(bn), field_size(c.bt1)), field_size(c.bt2)));
+  const WbRoots rr = roots<SOFT>(c.rho);
   c.sr = rr.sq;
   c.ir = rr.rcp;
-  c.vn = mul<SOFT>(c.mn, c.ir);
-  c.vt1 = mul<SOFT>(c.mt1, c.ir);
-  c.vt2 = mul<SOFT>(c.mt2, c.ir);
+  c.vn = mul<SOFT, 2>(c.mn, c.ir);
+  c.vt1 = mul<SOFT, 2>(c.mt1, c.ir);
+  c.vt2 = mul<SOFT, 2>(c.mt2, c.ir);
   const double hbn = wb_half(bn), bn2 = mul<SOFT>(bn, bn);
   const double ke = wb_half(__fma_rn(c.mt2, c.vt2, __fma_rn(c.mt1, c.vt1, mul<SOFT>(c.mn, c.vn))));
   const double bt2 = __fma_rn(c.bt2, c.bt2, mul<SOFT>(c.bt1, c.bt1));
@@ -104,6 +128,7 @@ __device__ __forceinline__ void load_cell(const double* const (&q)[8], long long
   c.F[5] = __fma_rn(c.bt2, hvn, -mul<SOFT>(c.vt2, hbn));
   const double bv = __fma_rn(c.bt2, c.vt2, __fma_rn(c.bt1, c.vt1, mul<SOFT>(bn, c.vn)));
   c.F[6] = __fma_rn(ep, hvn, __dmul_rn(-hbn, bv));
+  return size;
 }
 
 // Per-face record.
@@ -220,6 +245,14 @@ __device__ __forceinline__ void hll_face(const Cell& L, const Cell& R, double bn
   f[R_RHO] = kHllFace;
 }
 
+// Bit of face_system's result: the interface's numbers may be beyond the range of
+// the integer products, its flux takes FP64 ones too.
+constexpr int kFp64Face = 4;
+
+template <int EZ, bool PROT>
+__device__ __noinline__ int face_system_fp64(const Cell& L, const Cell& R, double b, double dtdx, const WbPhys& P, const RegRec& f,
+                                double gt[7]);
+
 // Roe state, eigen-system, alpha_k, nu_k and g-tilde_k (doubled) of one interface.
 // Returns 0 for an MHDTVD face, 1 when the protection floor asks for the HLL
 // flux (the record holds the Roe state), 2 when the Roe state has no real
@@ -228,42 +261,53 @@ __device__ __forceinline__ void hll_face(const Cell& L, const Cell& R, double bn
 template <int EZ, bool PROT, bool SOFT, class Rc>
 __device__ __forceinline__ int face_system(const Cell& L, const Cell& R, double b, double dtdx,
                                            const WbPhys& P, const Rc& f, double gt[7]) {
-  const double iD = wb_rcp(WB_ADD(L.sr, R.sr));
-  const double wL = mul<SOFT>(L.sr, iD), wR = mul<SOFT>(R.sr, iD);
-  const double rho = mul<SOFT>(L.sr, R.sr);
-  const WbRoots rroe = wb_roots(rho);
+  const double iD = recip<SOFT>(WB_ADD(L.sr, R.sr));
+  const double wL = mul<SOFT, 7>(L.sr, iD), wR = mul<SOFT, 7>(R.sr, iD);
+  const double rho = mul<SOFT, 7>(L.sr, R.sr);
+  const WbRoots rroe = roots<SOFT>(rho);
   const double irho = rroe.rcp, isrho = rroe.rsq, srho = rroe.sq;
-  const double vn = WB_FMA(wL, L.vn, mul<SOFT>(R.vn, wR));
-  const double vt1 = WB_FMA(wL, L.vt1, mul<SOFT>(R.vt1, wR));
-  const double vt2 = WB_FMA(wL, L.vt2, mul<SOFT>(R.vt2, wR));
-  const double bt1 = WB_FMA(wR, L.bt1, mul<SOFT>(R.bt1, wL));
-  const double bt2 = WB_FMA(wR, L.bt2, mul<SOFT>(R.bt2, wL));
+  const double vn = WB_FMA(wL, L.vn, mul<SOFT, 2>(R.vn, wR));
+  const double vt1 = WB_FMA(wL, L.vt1, mul<SOFT, 2>(R.vt1, wR));
+  const double vt2 = WB_FMA(wL, L.vt2, mul<SOFT, 2>(R.vt2, wR));
+  const double bt1 = WB_FMA(wR, L.bt1, mul<SOFT, 2>(R.bt1, wL));
+  const double bt2 = WB_FMA(wR, L.bt2, mul<SOFT, 2>(R.bt2, wL));
   const double b2 = mul<SOFT>(b, b);
   // H = wL (h_L + b^2)/rho_L + wR (h_R + b^2)/rho_R, with wL/rho_L + wR/rho_R = 1/rho_
-  const double H = WB_FMA(b2, irho, WB_FMA(wL, L.hr, mul<SOFT>(R.hr, wR)));
+  const double H = WB_FMA(b2, irho, WB_FMA(wL, L.hr, mul<SOFT, 2>(R.hr, wR)));
   const double dbt1 = WB_SUB(R.bt1, L.bt1), dbt2 = WB_SUB(R.bt2, L.bt2);
-  const double gX = WB_MUL(P.hgm2, WB_MUL(WB_FMA(dbt1, dbt1, mul<SOFT>(dbt2, dbt2)), mul<SOFT>(iD, iD)));  // (gamma-2) X
+  const double gX = WB_MUL(P.hgm2, WB_MUL(WB_FMA(dbt1, dbt1, mul<SOFT>(dbt2, dbt2)), mul<SOFT, 7>(iD, iD)));  // (gamma-2) X
   const double hv2 = wb_half(WB_FMA(vn, vn, WB_FMA(vt1, vt1, mul<SOFT>(vt2, vt2))));
   const double bt2s = WB_FMA(bt1, bt1, mul<SOFT>(bt2, bt2));
   const double a2 = WB_FMA(P.gm1, WB_FMA(-WB_ADD(b2, bt2s), irho, WB_SUB(H, hv2)), -gX);
   if (!wb_normal_pos(a2)) return 2;
-  const double ca2 = mul<SOFT>(b2, irho), ct2 = mul<SOFT>(bt2s, irho);
+  if (SOFT && wb_hi32(a2) < ((1023u - 100u) << 20)) {  // 1/a^2 may carry products out of the range
+    Cell l = L, r = R;
+    RegRec f2;
+    double g2[7];
+    const int code = face_system_fp64<EZ, PROT>(l, r, b, dtdx, P, f2, g2);
+#pragma unroll
+    for (int i = 0; i < R_WORDS; ++i) f[i] = f2[i];
+#pragma unroll
+    for (int k = 0; k < 7; ++k) gt[k] = g2[k];
+    return code | kFp64Face;
+  }
+  const double ca2 = mul<SOFT, 2>(b2, irho), ct2 = mul<SOFT, 2>(bt2s, irho);
   const double dac = WB_SUB(a2, ca2);
   const double disc = WB_FMA(dac, dac, WB_MUL(ct2, WB_FMA(2.0, WB_ADD(a2, ca2), ct2)));
   const double sum = WB_ADD(WB_ADD(a2, ca2), ct2);
   // a subnormal discriminant is degenerate (sd ~ 0)
-  const double sd = wb_normal_pos(disc) ? wb_sqrt(disc) : 0.0;
+  const double sd = wb_normal_pos(disc) ? roots<SOFT>(disc).sq : 0.0;
   const double cf2 = wb_half(WB_ADD(sum, sd));
-  const WbRoots rcf = wb_roots(cf2), ra_ = wb_roots(a2);
+  const WbRoots rcf = roots<SOFT>(cf2), ra_ = roots<SOFT>(a2);
   const double icf = rcf.rsq, ia = ra_.rsq, ia2 = ra_.rcp;
   const double cf = rcf.sq, a = ra_.sq;
-  const double ca = mul<SOFT>(wb_fabs(b), isrho);
-  const double cs = mul<SOFT>(mul<SOFT>(a, ca), icf);  // c_f c_s = a c_a
+  const double ca = mul<SOFT, 2>(wb_fabs(b), isrho);
+  const double cs = mul<SOFT, 2>(mul<SOFT, 1>(a, ca), icf);  // c_f c_s = a c_a
   // 1/|B_t| and c_t = |B_t| / sqrt(rho_); a transverse field whose square is
   // not a normal double (underflowing noise ahead of a front) counts as 0
   double ib = 0.0, btm = 0.0;  // btm = |B_t|
   if (wb_normal_pos(bt2s)) {
-    const WbRoots rb = wb_roots(bt2s);
+    const WbRoots rb = roots<SOFT>(bt2s);
     ib = rb.rsq;
     btm = rb.sq;
   }
@@ -278,9 +322,9 @@ __device__ __forceinline__ int face_system(const Cell& L, const Cell& R, double 
   const double t1 = WB_ADD(WB_SUB(ca2, a2), ct2);
   const bool slow_major = !wb_neg(t1);
   const double m = WB_ADD(sd, slow_major ? t1 : wb_flip(t1));
-  const double r = wb_rsqrt(wb_twice(mul<SOFT>(sd, m)));
+  const double r = roots<SOFT>(wb_twice(mul<SOFT>(sd, m))).rsq;
   const double major = mul<SOFT>(m, r);
-  const double minor = WB_MUL(mul<SOFT>(a, mul<SOFT>(btm, isrho)), wb_twice(r));
+  const double minor = WB_MUL(mul<SOFT, 1>(a, mul<SOFT, 2>(btm, isrho)), wb_twice(r));
   double af = slow_major ? minor : major;
   double as = slow_major ? major : minor;
   if (wb_hi_scaled(sd, 39) <= wb_hi32(sum) && wb_at_most(sd, 1e-12, sum)) {
@@ -288,7 +332,7 @@ __device__ __forceinline__ int face_system(const Cell& L, const Cell& R, double 
     af = fast ? 1.0 : 0.0;
     as = fast ? 0.0 : 1.0;
   }
-  const double ra2 = mul<SOFT>(rho, a2);
+  const double ra2 = mul<SOFT, 7>(rho, a2);
   double b1n = mul<SOFT>(bt1, ib), b2n = mul<SOFT>(bt2, ib);
   if (wb_maybe_small(bt2s, ra2, b2) && wb_at_most(bt2s, 1e-24, WB_ADD(WB_ADD(ra2, b2), bt2s)))
     b1n = b2n = 0.70710678118654752440;
@@ -310,18 +354,18 @@ __device__ __forceinline__ int face_system(const Cell& L, const Cell& R, double 
   const double dbb = WB_FMA(b1n, dbt1, mul<SOFT>(dbt2, b2n));
   const double dbpS = wb_xsgn(WB_FMA(-b2n, dbt1, mul<SOFT>(dbt2, b1n)), S);
   const double hir = wb_half(irho), hisr = wb_half(isrho);
-  const double i2ra = mul<SOFT>(hisr, ia);   // 1 / (2 sqrt(rho) a)
-  const double ri2a2 = mul<SOFT>(hir, ia2);  // 1 / (2 rho a^2)
-  const double dpr = mul<SOFT>(dp, ri2a2);
-  const double afcf = mul<SOFT>(af, cf), ascs = mul<SOFT>(as, cs);
-  const double dbbi = mul<SOFT>(dbb, i2ra);
+  const double i2ra = mul<SOFT, 7>(hisr, ia);   // 1 / (2 sqrt(rho) a)
+  const double ri2a2 = mul<SOFT, 7>(hir, ia2);  // 1 / (2 rho a^2)
+  const double dpr = mul<SOFT, 2>(dp, ri2a2);
+  const double afcf = mul<SOFT, 2>(af, cf), ascs = mul<SOFT>(as, cs);
+  const double dbbi = mul<SOFT, 2>(dbb, i2ra);
   // alpha_{1,7} = Cf -+ Xf / (2 rho a^2), alpha_{3,5} = Cs -+ Xs / (2 rho a^2): the factor
   // goes into the FMAs that form them
   const double Xf = WB_FMA(afcf, dvn, -mul<SOFT>(dvbS, ascs));
   const double Cf = WB_FMA(as, dbbi, mul<SOFT>(af, dpr));
   const double Xs = WB_FMA(ascs, dvn, mul<SOFT>(dvbS, afcf));
   const double Cs = WB_FMA(-af, dbbi, mul<SOFT>(as, dpr));
-  const double hAa = mul<SOFT>(hisr, dbpS);
+  const double hAa = mul<SOFT, 1>(hisr, dbpS);
   double al[7];
   al[0] = WB_FMA(-ri2a2, Xf, Cf);
   al[6] = WB_FMA(ri2a2, Xf, Cf);
@@ -331,7 +375,7 @@ __device__ __forceinline__ int face_system(const Cell& L, const Cell& R, double 
   al[5] = WB_FMA(hir, dvp, -hAa);
   al[3] = WB_FMA(-dp, ia2, drho);
   // nu_k = (dt/dx) a_k for the eigenvalues a_1..a_7 (Sec. 3)
-  const double tvn = mul<SOFT>(vn, dtdx);
+  const double tvn = mul<SOFT, 2>(vn, dtdx);
   const double nuk[7] = {WB_FMA(-dtdx, cf, tvn), WB_FMA(-dtdx, ca, tvn), WB_FMA(-dtdx, cs, tvn), tvn,
                          WB_FMA(dtdx, cs, tvn),  WB_FMA(dtdx, ca, tvn),  WB_FMA(dtdx, cf, tvn)};
 #pragma unroll
@@ -341,7 +385,7 @@ __device__ __forceinline__ int face_system(const Cell& L, const Cell& R, double 
     f[R_NU + k] = nu;
     gt[k] = mul<SOFT>(Qk_m_nu2<EZ, SOFT>(nu, k, P), al[k]);  // 2 g-tilde
   }
-  f[R_RHO] = rho; f[R_SRHO] = wb_xsgn(srho, S); f[R_A] = a; f[R_PG] = mul<SOFT>(ra2, P.inv_gm1); f[R_CF] = cf;
+  f[R_RHO] = rho; f[R_SRHO] = wb_xsgn(srho, S); f[R_A] = a; f[R_PG] = mul<SOFT, 7>(ra2, P.inv_gm1); f[R_CF] = cf;
   f[R_ASCS] = ascs; f[R_AFCF] = afcf; f[R_AF] = af; f[R_AS] = as; f[R_B1] = b1n; f[R_B2] = b2n;
   f[R_VN] = vn; f[R_VT1] = vt1; f[R_VT2] = vt2; f[R_BTM] = btm;
   f[R_KX] = WB_FMA(gX, P.inv_gm1, -hv2);  // K - v^2 (the energy row of face_flux)
@@ -349,6 +393,13 @@ __device__ __forceinline__ int face_system(const Cell& L, const Cell& R, double 
   for (int m = 0; m < 7; ++m) f[R_FAVG + m] = WB_ADD(L.F[m], R.F[m]);
   if (PROT && P.prot && protection_hit(L, R, rho, ra2, af, as, al, P)) return 1;
   return 0;
+}
+
+// The same with FP64 products, for the rare interface (not inlined).
+template <int EZ, bool PROT>
+__device__ int face_system_fp64(const Cell& L, const Cell& R, double b, double dtdx, const WbPhys& P,
+                                             const RegRec& f, double gt[7]) {
+  return face_system<EZ, PROT, false>(L, R, b, dtdx, P, f, gt);
 }
 
 // beta_k of App. A from the limited slopes carried doubled, G = 2 g (the
@@ -377,7 +428,7 @@ __device__ __forceinline__ double beta_k(double al, double nu, double Gi, double
   // |nu + gamma| < 2 eps: beta = (2 w)^2 / (16 eps alpha) + eps alpha - (g_i + g_{i+1})
   const double t = WB_FMA(P.eps[k], al, -wb_half(WB_ADD(Gi, Gi1)));
   if (wb_abs_less(al, 1e-290)) return t;  // (2 w)^2 / (16 eps alpha) < eps |alpha|
-  return WB_FMA(WB_MUL(WB_MUL(d, d), P.inv16eps[k]), wb_rcp(al), t);
+  return WB_FMA(WB_MUL(WB_MUL(d, d), P.inv16eps[k]), recip<SOFT>(al), t);
 }
 
 // u-bar = (F_L + F_R)/2 - (dx/(2 dt)) sum_k beta_k R_k  (App. A)
@@ -398,15 +449,15 @@ __device__ __forceinline__ void face_flux(const Rc& f, const double gi[7], const
   const double wr = WB_FMA(rho, tfs, be[3]);
   const double wvn = WB_FMA(afcf, df, mul<SOFT>(ds, ascs));
   const double vb = wb_xsgn(WB_FMA(afcf, ds, -mul<SOFT>(df, ascs)), S);  // along beta
-  const double bb = mul<SOFT>(WB_FMA(as, sf, -mul<SOFT>(ss, af)), mul<SOFT>(f[R_A], srho));
-  const double bp = wb_xsgn(mul<SOFT>(WB_SUB(be[1], be[5]), srho), S);
+  const double bb = mul<SOFT>(WB_FMA(as, sf, -mul<SOFT>(ss, af)), mul<SOFT, 7>(f[R_A], srho));
+  const double bp = wb_xsgn(mul<SOFT, 2>(WB_SUB(be[1], be[5]), srho), S);
   const double wvt1 = WB_FMA(b1, vb, -mul<SOFT>(vp, b2)), wvt2 = WB_FMA(b2, vb, mul<SOFT>(vp, b1));
   const double wbt1 = WB_FMA(b1, bb, -mul<SOFT>(bp, b2)), wbt2 = WB_FMA(b2, bb, mul<SOFT>(bp, b1));
   // to conserved variables (the pressure row enters the energy as p/(gamma-1))
   const double vn = f[R_VN], vt1 = f[R_VT1], vt2 = f[R_VT2];
-  const double u1 = WB_FMA(vn, wr, mul<SOFT>(wvn, rho));
-  const double u2 = WB_FMA(vt1, wr, mul<SOFT>(wvt1, rho));
-  const double u3 = WB_FMA(vt2, wr, mul<SOFT>(wvt2, rho));
+  const double u1 = WB_FMA(vn, wr, mul<SOFT, 2>(wvn, rho));
+  const double u2 = WB_FMA(vt1, wr, mul<SOFT, 2>(wvt1, rho));
+  const double u3 = WB_FMA(vt2, wr, mul<SOFT, 2>(wvt2, rho));
   // energy: B_t . w_Bt + p/(gamma-1) row + K w_rho + rho v . w_v, with
   // rho v . w_v = v . u - v^2 w_rho and the record holding K - v^2, and
   // B_t . w_Bt = |B_t| w_beta: beta is B_t / |B_t|, so the beta-perpendicular
@@ -422,6 +473,13 @@ __device__ __forceinline__ void face_flux(const Rc& f, const double gi[7], const
   out[4] = WB_FMA(-dx_2dt, wbt1, f[R_FAVG + 4]);
   out[5] = WB_FMA(-dx_2dt, wbt2, f[R_FAVG + 5]);
   out[6] = WB_FMA(-dx_2dt, u6, f[R_FAVG + 6]);
+}
+
+// The same with FP64 products, for the rare interface (not inlined).
+template <int EZ>
+__device__ __noinline__ void face_flux_fp64(const RegRec& f, const double gi[7], const double gi1[7], double dx_2dt,
+                                            const WbPhys& P, double out[7]) {
+  face_flux<EZ, false>(f, gi, gi1, dx_2dt, P, out);
 }
 
 // What a face needs of its left zone, word by word.
@@ -505,6 +563,11 @@ __host__ __device__ __forceinline__ long long sweep_tiles(long long npen, int le
   return (n + per - 1) / per;
 }
 
+template <int EZ, bool PROT, bool NC>
+__device__ __noinline__ int sweep_tile_fp64(const WbGeo& g, const WbBox& box, int d, const SweepFrame& s, long long tile, bool closed,
+                               bool ring, int nslots, long long slot_in, long long slot_out, const WbScalars* scal,
+                               const WbPhys& P, LaneEdge& X);
+
 // One tile of a sweep, one face per thread: the thread holds a zone and its low
 // face; its neighbours along the pencil hand over zone state, g-tilde and
 // limited slopes by shuffles and, at the ends of a warp, through shared memory
@@ -567,8 +630,9 @@ __device__ __forceinline__ int sweep_tile(const WbGeo& g, const WbBox& box, int 
   const long long at = wb_at(g, pos[0], pos[1], pos[2]);
   const long long off = slot * slot_in + at;
   Cell R;
-  load_cell<NC, SOFT>(s.q, off, P, R);
-  const double b = ld<NC>(s.bn + off);
+  const unsigned size = load_cell<NC, SOFT>(s.q, off, P, R);
+  const double b = ld<NC>(s.bn + off), dtdx = scal->dtdx[d];
+  const bool wild = SOFT && field_wild(max(size, max(field_size(b), field_size(dtdx))), R.rho);
   Cell L;
   L.ir = 0.0;  // not used across a face
   // neighbours in other warps go through X, unless every ring sits in a warp
@@ -580,6 +644,13 @@ __device__ __forceinline__ int sweep_tile(const WbGeo& g, const WbBox& box, int 
 #pragma unroll
       for (int i = 0; i < kCellWords; ++i) X.cell[wp][mine_r][i] = cell_word(R, i);
     }
+  }
+  // a block (a warp of its own rings) that meets a field beyond the integer
+  // products' range starts over with FP64 products
+  if (SOFT) {
+    if (cross ? __syncthreads_or(wild) : __any_sync(0xffffffffu, wild))
+      return sweep_tile_fp64<EZ, PROT, NC>(g, box, d, s, tile, closed, ring, nslots, slot_in, slot_out, scal, P, X);
+  } else if (cross) {
     __syncthreads();
   }
 #pragma unroll
@@ -590,7 +661,9 @@ __device__ __forceinline__ int sweep_tile(const WbGeo& g, const WbBox& box, int 
   }
   RegRec f;
   double gt[7];
-  const int code = face_system<EZ, PROT, SOFT>(L, R, b, scal->dtdx[d], P, f, gt);
+  int code = face_system<EZ, PROT, SOFT>(L, R, b, dtdx, P, f, gt);
+  const bool fp64 = SOFT && (code & kFp64Face);
+  code &= ~kFp64Face;
   bool hll = false;
   if (code) {
     if (has_left) {
@@ -634,6 +707,17 @@ __device__ __forceinline__ int sweep_tile(const WbGeo& g, const WbBox& box, int 
   if (hll) {
 #pragma unroll
     for (int m = 0; m < 7; ++m) out[m] = f[R_FAVG + m];
+  } else if (fp64) {
+    RegRec f2 = f;
+    double a[7], c[7], o2[7];
+#pragma unroll
+    for (int k = 0; k < 7; ++k) {
+      a[k] = gl[k];
+      c[k] = gz[k];
+    }
+    face_flux_fp64<EZ>(f2, a, c, scal->dx_2dt[d], P, o2);
+#pragma unroll
+    for (int m = 0; m < 7; ++m) out[m] = o2[m];
   } else {
     face_flux<EZ, SOFT>(f, gl, gz, scal->dx_2dt[d], P, out);
   }
@@ -641,6 +725,14 @@ __device__ __forceinline__ int sweep_tile(const WbGeo& g, const WbBox& box, int 
 #pragma unroll
   for (int m = 0; m < 7; ++m) s.F[m][o] = out[m];
   return hll && pos[0] >= 0 && pos[0] < g.n[0] && pos[1] >= 0 && pos[1] < g.n[1] && pos[2] >= 0 && pos[2] < g.n[2];
+}
+
+template <int EZ, bool PROT, bool NC>
+__device__ int sweep_tile_fp64(const WbGeo& g, const WbBox& box, int d, const SweepFrame& s, long long tile,
+                                            bool closed, bool ring, int nslots, long long slot_in, long long slot_out,
+                                            const WbScalars* scal, const WbPhys& P, LaneEdge& X) {
+  return sweep_tile<EZ, PROT, false, NC, kAnyLayout>(g, box, d, s, tile, closed, ring, nslots, slot_in, slot_out, scal, P,
+                                                     X);
 }
 
 // ---------------------------------------------------------------- stages ---
