@@ -28,9 +28,10 @@ namespace wbu {
 constexpr int kWarps = 4;             // warps of a sweep block
 constexpr int kBlock = 32 * kWarps;
 constexpr int kTile = kBlock - 3;     // faces a block emits from its kBlock zones
-// resident blocks per SM the sweep kernels are compiled for: 168 registers a
-// thread, 12 warps per SM
-constexpr int kSweepBlocks = 3;
+// resident blocks per SM the sweep kernels are compiled for: 128 registers a
+// thread, 16 warps per SM (3 blocks, 168 registers and fewer spills: 17.8
+// against 17.4 ms a launch of a 256^3 box, 2.21 against 2.07 of a 128^3)
+constexpr int kSweepBlocks = 4;
 
 // waves 2, 4, 6 (Alfven, entropy, Alfven) have eps = 0 (the default eps_k):
 // the mask of the sweep specialisation that drops their Q-branch arithmetic
@@ -208,24 +209,28 @@ __device__ __forceinline__ double zone_fast_speed(const Cell& c, double bn, cons
   return sqrt(wb_half(WB_ADD(s, sqrt(disc))));
 }
 
-// Marker of a face record that holds a finished HLL flux (a Roe density is > 0)
-constexpr double kHllFace = -1.0;
-
-// HLL flux of App. A into the record of one face:
+// HLL flux of App. A of one face:
 //   b+ = max(a_max, vR + cfR, 0), b- = min(a_min, vL - cfL, 0),
 //   u = (b+ F_L - b- F_R + b+ b- (q_R - q_L)) / (b+ - b-),
 // with a_max, a_min = vn_ +- cf_ of the Roe state when it exists (roe), the
 // Einfeldt sign of the F_R term (the printed +b- F_R is not consistent), and
 // bounds +-max(|v| + c_f) if both speeds vanish.  Rare path.
-template <class Rc>
-__device__ __forceinline__ void hll_face(const Cell& L, const Cell& R, double bnL, double bnR, bool roe,
-                                      const WbPhys& P, const Rc& f) {
-  const double cfL = zone_fast_speed(L, bnL, P), cfR = zone_fast_speed(R, bnR, P);
+//
+// The zones are loaded again: this path is rare, and its use of both zone states
+// would keep 40 doubles of every thread in registers through face_system.  vn,
+// cf: of the Roe state (roe).  The interface's flux in out.
+template <bool NC>
+__device__ __noinline__ void hll_face(const double* const (&q)[8], long long offL, long long offR, bool roe, double vn,
+                                      double cf, const WbPhys& P, double* out) {
+  Cell L, R;
+  load_cell<NC, false>(q, offL, P, L);
+  load_cell<NC, false>(q, offR, P, R);
+  const double cfL = zone_fast_speed(L, ld<NC>(q[5] + offL), P), cfR = zone_fast_speed(R, ld<NC>(q[5] + offR), P);
   double bp = fmax(WB_ADD(R.vn, cfR), 0.0);
   double bm = fmin(WB_SUB(L.vn, cfL), 0.0);
   if (roe) {
-    bp = fmax(bp, WB_ADD(f[R_VN], f[R_CF]));
-    bm = fmin(bm, WB_SUB(f[R_VN], f[R_CF]));
+    bp = fmax(bp, WB_ADD(vn, cf));
+    bm = fmin(bm, WB_SUB(vn, cf));
   }
   if (!(WB_SUB(bp, bm) > 0.0)) {
     const double sp = fmax(WB_ADD(fabs(L.vn), cfL), WB_ADD(fabs(R.vn), cfR));
@@ -240,9 +245,8 @@ __device__ __forceinline__ void hll_face(const Cell& L, const Cell& R, double bn
   for (int m = 0; m < 7; ++m) {
     // the zone fluxes hold F/2
     const double FL = WB_MUL(2.0, L.F[m]), FR = WB_MUL(2.0, R.F[m]);
-    f[R_FAVG + m] = WB_MUL(WB_FMA(bpm, dq[m], WB_FMA(bp, FL, -WB_MUL(bm, FR))), inv);
+    out[m] = WB_MUL(WB_FMA(bpm, dq[m], WB_FMA(bp, FL, -WB_MUL(bm, FR))), inv);
   }
-  f[R_RHO] = kHllFace;
 }
 
 // Bit of face_system's result: the interface's numbers may be beyond the range of
@@ -428,7 +432,7 @@ __device__ __forceinline__ double beta_k(double al, double nu, double Gi, double
   // |nu + gamma| < 2 eps: beta = (2 w)^2 / (16 eps alpha) + eps alpha - (g_i + g_{i+1})
   const double t = WB_FMA(P.eps[k], al, -wb_half(WB_ADD(Gi, Gi1)));
   if (wb_abs_less(al, 1e-290)) return t;  // (2 w)^2 / (16 eps alpha) < eps |alpha|
-  return WB_FMA(WB_MUL(WB_MUL(d, d), P.inv16eps[k]), recip<SOFT>(al), t);
+  return WB_FMA(mul<SOFT>(mul<SOFT>(d, d), P.inv16eps[k]), recip<SOFT>(al), t);
 }
 
 // u-bar = (F_L + F_R)/2 - (dx/(2 dt)) sum_k beta_k R_k  (App. A)
@@ -581,7 +585,9 @@ __device__ __noinline__ int sweep_tile_fp64(const WbGeo& g, const WbBox& box, in
 // beside it the latency of the integer work that takes FP64 work over (wb_soft).
 // A thread that marched along a pencil kept two zones, two slopes and a face
 // record in 226 to 255 registers and 40 KB of shared memory a block, which left
-// 2 warps per scheduler; one face per thread needs 168, 3 warps.
+// 2 warps per scheduler; one face per thread runs with 128 registers, 4 warps
+// (some 200 bytes of spills).  (F_L + F_R)/2 in shared memory rather than in the
+// spills was no faster (17.5 against 17.4 ms a 256^3 launch).
 template <int EZ, bool PROT, bool SOFT, bool NC, int LAYOUT>
 __device__ __forceinline__ int sweep_tile(const WbGeo& g, const WbBox& box, int d, const SweepFrame& s, long long tile,
                                           bool closed, bool ring_, int nslots, long long slot_in, long long slot_out,
@@ -669,7 +675,10 @@ __device__ __forceinline__ int sweep_tile(const WbGeo& g, const WbBox& box, int 
     if (has_left) {
       long long st = d == 0 ? 1LL : (d == 1 ? g.sy : g.sz);
       if (closed && idx == 0) st *= 1 - len;
-      hll_face(L, R, ld<NC>(s.q[5] + off - st), ld<NC>(s.q[5] + off), code == 1, P, f);
+      double h[7];
+      hll_face<NC>(s.q, off - st, off, code == 1, code == 1 ? f[R_VN] : 0.0, code == 1 ? f[R_CF] : 0.0, P, h);
+#pragma unroll
+      for (int m = 0; m < 7; ++m) f[R_FAVG + m] = h[m];
       hll = true;
     }
 #pragma unroll
