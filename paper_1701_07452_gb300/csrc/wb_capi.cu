@@ -265,7 +265,9 @@ StageArgs stage_args(wb_grid* g, long long p0, int nslots) {
 }
 
 // ebox: the zones of the reference EMF (Step 2) that the predictor's launch takes along
-SweepArgs sweep_args(wb_grid* g, const StageArgs& s, bool corr, const WbBox (&bx)[3], int nslots, const WbBox& ebox) {
+// one_patch: the sweeps cover an outflow box's faces once (enqueue_pass)
+SweepArgs sweep_args(wb_grid* g, const StageArgs& s, bool corr, const WbBox (&bx)[3], int nslots, const WbBox& ebox,
+                     bool one_patch = false) {
   SweepArgs a;
   std::memset(&a, 0, sizeof(a));
   const WbView& v = s.v;
@@ -280,7 +282,7 @@ SweepArgs sweep_args(wb_grid* g, const StageArgs& s, bool corr, const WbBox (&bx
   a.scal = g->scal;
   a.nslots = nslots;
   for (int d = 0; d < 3; ++d)  // whole periodic pencils: one patch along the axis
-    if ((g->closed || g->wrap) && g->map.np[d] == 1) a.closed |= 1 << d;
+    if ((g->closed || g->wrap || (one_patch && g->map.bc[d] == WB_BC_PERIODIC)) && g->map.np[d] == 1) a.closed |= 1 << d;
   if (!corr) {
     for (int d = 0; d < 3; ++d) a.Eref[d] = v.Eref[d];
     a.ebox = ebox;
@@ -374,7 +376,30 @@ void enqueue_pass(wb_grid* g, long long p0, int nslots, const StepControl& c) {
     return flat ? ::box(l0, h0, l1, h1, 0, 0) : ::box(l0, h0, l1, h1, l2, h2);
   };
   // Step 1: predictor fluxes from q^n; Step 2: reference EMF
-  {
+  if (g->npatch == 1) {
+    // The rows of ghost zones repeat the boundary rows (or are periodic images),
+    // and so do the predictor's fluxes and reference EMF there: computed once on
+    // the box and copied, where recomputing the rings 4 deep cost 60 % more
+    // predictor faces on 45 x 38 x 51 zones: five steps of that box 2012 us before,
+    // 1798 us now.  (From here on the stages take one-sided differences of the face
+    // field, which a ghost row does not repeat.)
+    int hi[3];  // the high boundary face of an outflow axis is computed, a periodic one is face 0
+    for (int d = 0; d < 3; ++d) hi[d] = g->geo.n[d] - 1 + (g->map.bc[d] == WB_BC_OUTFLOW ? 1 : 0);
+    const WbBox pb[3] = {box(0, hi[0], 0, N1 - 1, 0, N2 - 1), box(0, N0 - 1, 0, hi[1], 0, N2 - 1),
+                         box(0, N0 - 1, 0, N1 - 1, 0, hi[2])};
+    sweeps(g, sweep_args(g, A, false, pb, nslots, box(0, N0 - 1, 0, N1 - 1, 0, N2 - 1), true));
+    ImageList L = {};
+    for (int d = 0; d < 3; ++d) {
+      for (int c = 0; c < 8; ++c)
+        if (c != F_BX + d) {
+          L.face[L.n] = d;
+          L.a[L.n++] = g->Fp[d][c];
+        }
+      L.face[L.n] = -1;
+      L.a[L.n++] = g->Eref[d];
+    }
+    wb_launch_images(L, g->geo, g->map, 4, s);
+  } else {
     const WbBox pb[3] = {box(-3, N0 + 3, -4, N1 + 3, -4, N2 + 3), box(-4, N0 + 3, -3, N1 + 3, -4, N2 + 3),
                          box(-4, N0 + 3, -4, N1 + 3, -3, N2 + 3)};
     sweeps(g, sweep_args(g, A, false, pb, nslots, box(-4, N0 + 3, -4, N1 + 3, -4, N2 + 3)));

@@ -97,6 +97,17 @@ void wb_launch_wrap(const WrapList& L, const WbGeo& geo, const GridMap& m, int d
 // of a loaded state.
 void wb_launch_init(double* const q[8], double* const b[3], const WbGeo& geo, long long npatch, int closed,
                     const WbPhys& ph, bool primitive, WbScalars* scal, cudaStream_t s);
+// Ghost points of the predictor's arrays (fluxes and reference EMF) of a grid of
+// one patch, `depth` zones deep: a ghost row of an outflow axis holds the data of
+// the boundary row and a periodic one that of its image, so the values there are
+// those of the interior, copied.  face[a]: the axis along which array a lives on
+// faces (computed up to the high boundary face of an outflow axis), or -1.
+struct ImageList {
+  double* a[24];
+  int face[24];
+  int n;
+};
+void wb_launch_images(const ImageList& L, const WbGeo& geo, const GridMap& m, int depth, cudaStream_t s);
 void wb_launch_dt_step(WbScalars* scal, const StepControl& c, cudaStream_t s);
 // global <-> patch copies of up to 11 arrays; comp: 0..4 zone field, 5..7 face
 // field of axis comp-5

@@ -126,6 +126,26 @@ __global__ void k_wrap(WrapList L, WbGeo g, int depth, long long n) {
   for (int a = 0; a < L.n; ++a) L.a[a][dst] = L.a[a][src];
 }
 
+// Ghost points of the predictor's arrays of a single patch with an outflow axis
+// (wb_launch_images): one thread per shell point, blockIdx.y the array.
+__global__ void k_images(ImageList L, WbGeo g, GridMap m, int depth, unsigned first, unsigned n) {
+  wb_pdl_begin();
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= n) return;
+  int x[3], src[3];
+  wbu::shell_point(g, depth, (long long)first + t, &x[0], &x[1], &x[2]);
+  const int face = L.face[blockIdx.y];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const int N = m.N[d];
+    if (m.bc[d] == 0) src[d] = ((x[d] % N) + N) % N;
+    else src[d] = min(max(x[d], 0), face == d ? N : N - 1);
+  }
+  if (src[0] == x[0] && src[1] == x[1] && src[2] == x[2]) return;  // the high boundary face itself
+  double* a = L.a[blockIdx.y];
+  a[wb_at(g, x[0], x[1], x[2])] = a[wb_at(g, src[0], src[1], src[2])];
+}
+
 // The same for a grid of patches periodic on every axis, all patches resident
 // (slot = patch): a ghost point of patch blockIdx.y takes the value the
 // neighbouring patch (periodic across the domain) holds at that global
@@ -564,6 +584,13 @@ void wb_launch_init(double* const q[8], double* const b[3], const WbGeo& geo, lo
   const long long n = (long long)geo.n[0] * geo.n[1] * geo.n[2];
   const int bs = stage_threads(n, (int)npatch, 256);
   wb_launch_dependent(k_init, grid_for(n, (int)npatch, bs), bs, s, a, primitive ? 1 : 0);
+}
+
+void wb_launch_images(const ImageList& L, const WbGeo& geo, const GridMap& m, int depth, cudaStream_t s) {
+  // one-plane storage: every layer is the plane, only its x and y ghosts are copied
+  const long long first = geo.sz == 0 ? (long long)(geo.n[0] + 2 * depth) * (geo.n[1] + 2 * depth) * 2 * depth : 0;
+  const long long n = wbu::shell_count(geo, depth) - first;
+  wb_launch_dependent(k_images, grid_for(n, L.n, 256), 256, s, L, geo, m, depth, (unsigned)first, (unsigned)n);
 }
 
 void wb_launch_dt_step(WbScalars* scal, const StepControl& c, cudaStream_t s) {
