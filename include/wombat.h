@@ -272,8 +272,9 @@ const char* wb_noalloc_last_error(void);
  * above.  WB_BATCH_STAGED: one ordinary launch per stage of each step over
  * all boxes of a workspace group (the same work lists and results bit for
  * bit), each stage class compiled into its own kernel so that the zone
- * stages run with their own occupancy; no grid barrier, so no
- * WB_ERR_TIMEOUT.  With the stage timer on, the staged form times every
+ * stages run with their own occupancy, one block per piece of work (the
+ * number of blocks per SM applies to the persistent form); no grid barrier,
+ * so no WB_ERR_TIMEOUT.  With the stage timer on, the staged form times every
  * stage but dt.  Drops a captured graph.  wb_batch_autotune tries both forms
  * and keeps the faster; wb_batch_get_form reports the current one. */
 #define WB_BATCH_PERSISTENT 0

@@ -16,8 +16,8 @@
 //
 // The staged form runs the same stages as one ordinary launch each (the
 // sweeps in a kernel that holds only the sweep, the zone stages in kernels
-// compiled per stage class with their own occupancy), all captured in one
-// CUDA graph; the stage arithmetic is explicitly rounded, so both forms (and
+// compiled per stage class with their own occupancy), one block per chunk, all
+// captured in one CUDA graph; the stage arithmetic is explicitly rounded, so both forms (and
 // the single-grid path) give the same bits.
 #include <cuda_runtime.h>
 
@@ -224,13 +224,13 @@ __device__ __forceinline__ void warp_max_key(unsigned long long bits, unsigned l
 }
 
 // One tile of a sweep of one box (every thread of the block).
-template <int EZ, bool PROT>
+template <int EZ, bool PROT, int LAYOUT>
 __device__ __forceinline__ int box_sweep_tile(const BoxInfo& bi, bool corr, int d, long long tile,
                                               const WbPhys& P, wbu::LaneEdge& X) {
   const WbView& v = bi.v;
   const bool wrap = bi.wrap != 0;
   const WbBox b = stage_box(corr ? BS_CORR : BS_PRED, d, v.geo.n, wrap);
-  return wbu::sweep_tile<EZ, PROT, true, false, wbu::kAnyLayout>(v.geo, b, d, bi.sw[corr ? 1 : 0][d], tile, wrap,
+  return wbu::sweep_tile<EZ, PROT, true, false, LAYOUT>(v.geo, b, d, bi.sw[corr ? 1 : 0][d], tile, wrap,
                                           wbu::sweep_ring(b.hi[d] - b.lo[d] + 1, wrap), 1, 0, 0,
                                           v.scal, P, X);
 }
@@ -416,27 +416,16 @@ __device__ __forceinline__ unsigned long long global_ns() {
   return t;
 }
 
-// EZ: compile-time mask of waves with eps_k = 0 (their Q-branch arithmetic is
-// dropped); PROT: the protection-floor test is compiled in.  The launch picks
-// the variant from the physics, as the grid path's sweep launches do.
-// Launch seq of a sequence uses chunk counter seq & 1 (and done counter
-// 5 + (seq & 1) when timing); its block 0 clears the other pair, which the
-// launch before it (complete by stream order) used.
-__device__ __forceinline__ unsigned* stage_counter(const BatchParams& B, unsigned seq) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    atomicExch(B.sync + 3 + ((seq + 1) & 1u), 0u);
-    atomicExch(B.sync + 5 + ((seq + 1) & 1u), 0u);
-  }
-  return B.sync + 3 + (seq & 1u);
-}
-
 // Stage timer of the staged form: the last block to finish a launch adds the
 // time since the previous launch's end to the stage (the dt launch only sets
-// the mark, so time between advances is not counted).
+// the mark, so time between advances is not counted).  Launch seq of a sequence
+// counts its blocks at 5 + (seq & 1); its block 0 clears the other word, which
+// the launch before it (complete by then) used.
 __device__ __forceinline__ void stage_stamp(const BatchParams& B, int s, unsigned seq) {
   if (!B.prof) return;
   __syncthreads();
   if (threadIdx.x == 0) {
+    if (blockIdx.x == 0) atomicExch(B.sync + 5 + ((seq + 1) & 1u), 0u);
     __threadfence();
     const unsigned done = atomicAdd(B.sync + 5 + (seq & 1u), 1u);
     if (done == gridDim.x - 1) {
@@ -448,10 +437,29 @@ __device__ __forceinline__ void stage_stamp(const BatchParams& B, int s, unsigne
   }
 }
 
+// The (box, sub) entry holding chunk c: the last of n prefix sums (the first is
+// 0) that is not above it.  Every warp searches for itself, 32 sums a round (all
+// its lanes call).
+__device__ __forceinline__ int chunk_entry(const long long* pre, int n, long long c) {
+  const int lane = threadIdx.x & 31;
+  int lo = 0;
+  while (n > 1) {
+    const int step = (n + 31) >> 5;
+    const int at = lane * step;
+    const int before = __popc(__ballot_sync(0xffffffffu, at < n && pre[lo + at] <= c)) - 1;
+    lo += before * step;
+    n = min(step, n - before * step);
+  }
+  return lo;
+}
+
+// EZ: compile-time mask of waves with eps_k = 0 (their Q-branch arithmetic is
+// dropped); PROT: the protection-floor test is compiled in.  The launch picks
+// the variant from the physics, as the grid path's sweep launches do.
 template <int EZ, bool PROT>
 __global__ void __launch_bounds__(kB, wbu::kSweepBlocks) k_batch(BatchParams B, int nsteps) {
   __shared__ wbu::LaneEdge X;
-  __shared__ long long s_chunk;
+  __shared__ unsigned s_chunk[2];
   const unsigned nblocks = gridDim.x;
   unsigned stage_seq = 0;
   // stage timer: block 0 stamps the end of every stage (after its barrier)
@@ -472,46 +480,44 @@ __global__ void __launch_bounds__(kB, wbu::kSweepBlocks) k_batch(BatchParams B, 
         if (blockIdx.x == 0 && threadIdx.x == 0) atomicExch(B.sync + 3 + ((stage_seq + 1) & 1u), 0u);
         ++stage_seq;
         const int ipc = items_per_chunk(s);
-        for (;;) {
-          if (threadIdx.x == 0) s_chunk = (long long)atomicAdd(ctr, 1u);
-          __syncthreads();
-          const long long c = s_chunk;
-          __syncthreads();
-          if (c >= nchunks) break;
-          // (box, sub) entry holding chunk c
-          int lo = 0, hi = nent - 1;
-          while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (pre[mid] <= c) lo = mid; else hi = mid - 1;
-          }
+        // A block's first chunk is its index; the next one is claimed before the
+        // work on this one and read after it.
+        unsigned c = blockIdx.x;
+        for (int turn = 0; c < nchunks; turn ^= 1) {
+          unsigned next = 0;
+          if (threadIdx.x == 0) next = nblocks + atomicAdd(ctr, 1u);
+          const int lo = chunk_entry(pre, nent, c);
           const int box = B.gbox[gb0 + lo / nsub];
           const int sub = lo % nsub;
+          const double dt = *(volatile const double*)&B.scal[box].dt;
           if (s == BS_DT) {
             if (threadIdx.x == 0) box_dt(B, box);
-            continue;
+          } else if (wb_pos(dt)) {
+            const BoxInfo& bi = B.boxes[box];
+            unsigned long long wkey = 0ULL;
+            int hits = 0, bad = 0, hll = 0;
+            if (stage_is_sweep(s)) {
+              hll = box_sweep_tile<EZ, PROT, wbu::kAnyLayout>(bi, s == BS_CORR, sub, c - pre[lo], B.phys, X);
+            } else {
+              const long long nitems = stage_items(s, sub, bi.v.geo, bi.wrap != 0);
+              const long long i0 = (c - pre[lo]) * ipc;
+              const long long i1 = i0 + ipc < nitems ? i0 + ipc : nitems;
+              if (stage_pairs(s)) {
+                for (long long it = i0 + threadIdx.x; it < i1; it += 2 * kB)
+                  unit_pair(s, sub, bi, it, it + kB < i1 ? it + kB : -1, dt);
+              } else {
+                for (long long it = i0 + threadIdx.x; it < i1; it += kB)
+                  unit_item(B, s, sub, bi, it, dt, &wkey, &hits, &bad);
+              }
+            }
+            if (s == BS_FINAL) warp_max_key(wkey, &B.scal[box].wmax_next);
+            if (hits) atomicAdd((unsigned long long*)&B.scal[box].floor_hits, (unsigned long long)hits);
+            if (bad) atomicAdd((unsigned long long*)&B.scal[box].unphysical, (unsigned long long)bad);
+            if (hll) atomicAdd((unsigned long long*)&B.scal[box].hll_faces, (unsigned long long)hll);
           }
-          const double dt = *(volatile const double*)&B.scal[box].dt;
-          if (!wb_pos(dt)) continue;
-          const BoxInfo& bi = B.boxes[box];
-          const long long nitems = stage_items(s, sub, bi.v.geo, bi.wrap != 0);
-          const long long i0 = (c - pre[lo]) * ipc;
-          long long i1 = i0 + ipc;
-          if (i1 > nitems) i1 = nitems;
-          unsigned long long wkey = 0ULL;
-          int hits = 0, bad = 0, hll = 0;
-          if (stage_is_sweep(s)) {
-            hll = box_sweep_tile<EZ, PROT>(bi, s == BS_CORR, sub, i0, B.phys, X);
-          } else if (stage_pairs(s)) {
-            for (long long it = i0 + threadIdx.x; it < i1; it += 2 * kB)
-              unit_pair(s, sub, bi, it, it + kB < i1 ? it + kB : -1, dt);
-          } else {
-            for (long long it = i0 + threadIdx.x; it < i1; it += kB)
-              unit_item(B, s, sub, bi, it, dt, &wkey, &hits, &bad);
-          }
-          if (s == BS_FINAL) warp_max_key(wkey, &B.scal[box].wmax_next);
-          if (hits) atomicAdd((unsigned long long*)&B.scal[box].floor_hits, (unsigned long long)hits);
-          if (bad) atomicAdd((unsigned long long*)&B.scal[box].unphysical, (unsigned long long)bad);
-          if (hll) atomicAdd((unsigned long long*)&B.scal[box].hll_faces, (unsigned long long)hll);
+          if (threadIdx.x == 0) s_chunk[turn] = next;
+          __syncthreads();
+          c = s_chunk[turn];
         }
         if (!grid_barrier(B, nblocks)) return;
         if (timer) {
@@ -525,14 +531,17 @@ __global__ void __launch_bounds__(kB, wbu::kSweepBlocks) k_batch(BatchParams B, 
 }
 
 // ------------------------------------------------------------ staged form
-// The same stages as separate launches, one per stage and workspace group: a
-// kernel boundary takes the place of each grid barrier, and blocks drain the
-// same chunk lists from the stage's counter.  The sweeps run in a kernel that
-// holds only the sweep; the zone stages run in kernels compiled per stage
-// class, with as many resident warps as their own registers allow (inside the
-// persistent kernel every stage keeps the sweep's 4 blocks of 64 threads per
-// SM).  All stage arithmetic is written with explicit rounding, so both forms
-// compute the same bits.
+// The same stages as separate launches, one per stage and workspace group, with
+// one block per chunk: a kernel boundary takes the place of each grid barrier
+// and the hardware's block scheduler that of the chunk counter.  (Resident
+// blocks that drained the counter left the FP64 pipe idle between two chunks,
+// through an atomic, two block barriers and a serial search.)  The sweeps run in
+// a kernel that holds only the sweep, compiled for one thread layout where a
+// group's boxes agree on it: both together took four steps of ten boxes of edges
+// 16..96 from 18.1 to 16.2 ms; the persistent form, with the next chunk claimed
+// ahead, takes 19.0.  The zone stages run in kernels compiled per stage class,
+// with as many resident warps as their own registers allow.  All stage arithmetic
+// is written with explicit rounding, so both forms compute the same bits.
 enum { SC_SWEEP = 0, SC_COPY, SC_EMF, SC_TRANS, SC_EREF_H, SC_FINAL, SC_DT, SC_COUNT };
 
 __host__ __device__ inline int stage_class(int s) {
@@ -553,102 +562,91 @@ __host__ __device__ constexpr int zone_min_blocks(int cls) {
   return cls == SC_TRANS ? 2 : ((cls == SC_EREF_H || cls == SC_FINAL) ? 3 : 4);
 }
 
-// Chunks of stage s for the boxes of group grp, claimed by whole blocks:
-// body(box, sub, chunk index within the (box, sub) entry).
-template <class Body>
-__device__ __forceinline__ void drain_stage(const BatchParams& B, int grp, int s, unsigned* ctr,
-                                            Body&& body) {
-  __shared__ long long s_chunk;
-  const int gb0 = B.gfirst[grp];
-  const int nbox = B.gfirst[grp + 1] - gb0;
+// Chunk blockIdx.x of stage s of group grp: its box, its sub-stage (axis) and
+// the chunk's index within that (box, sub) entry.
+struct Job {
+  int box, sub;
+  long long chunk;
+};
+__device__ __forceinline__ Job stage_job(const BatchParams& B, int grp, int s) {
+  const int gb0 = B.gfirst[grp], nsub = stage_nsub(s);
   const long long* pre = B.pre + B.pre_off[grp * BS_COUNT + s];
-  const int nsub = stage_nsub(s);
-  const int nent = nbox * nsub;
-  const long long nchunks = pre[nent];
-  for (;;) {
-    if (threadIdx.x == 0) s_chunk = (long long)atomicAdd(ctr, 1u);
-    __syncthreads();
-    const long long c = s_chunk;
-    __syncthreads();
-    if (c >= nchunks) break;
-    int lo = 0, hi = nent - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (pre[mid] <= c) lo = mid; else hi = mid - 1;
-    }
-    body(B.gbox[gb0 + lo / nsub], lo % nsub, c - pre[lo]);
-  }
+  const int e = chunk_entry(pre, (B.gfirst[grp + 1] - gb0) * nsub, blockIdx.x);
+  return {B.gbox[gb0 + e / nsub], e % nsub, blockIdx.x - pre[e]};
 }
 
 // The sweep stages of the staged form: the same chunks and per-item code as
 // the persistent kernel's sweep stage, in a kernel that holds nothing else
 // (the flux arithmetic is explicitly rounded, so the bits do not depend on
 // which kernel runs it).
-template <int EZ, bool PROT>
+template <int EZ, bool PROT, int LAYOUT>
 __global__ void __launch_bounds__(kB, wbu::kSweepBlocks) k_bstage_sweep(BatchParams B, int grp, int s, unsigned seq) {
   __shared__ wbu::LaneEdge X;
-  unsigned* ctr = stage_counter(B, seq);
-  drain_stage(B, grp, s, ctr, [&](int box, int d, long long cc) {
-    const double dt = B.scal[box].dt;
-    if (!wb_pos(dt)) return;
-    const int hll = box_sweep_tile<EZ, PROT>(B.boxes[box], s == BS_CORR, d, cc, B.phys, X);
-    if (hll) atomicAdd((unsigned long long*)&B.scal[box].hll_faces, 1ULL);
-  });
+  wb_pdl_begin();
+  const Job j = stage_job(B, grp, s);
+  if (wb_pos(B.scal[j.box].dt)) {
+    const int hll = box_sweep_tile<EZ, PROT, LAYOUT>(B.boxes[j.box], s == BS_CORR, j.sub, j.chunk, B.phys, X);
+    if (hll) atomicAdd((unsigned long long*)&B.scal[j.box].hll_faces, 1ULL);
+  }
   stage_stamp(B, s, seq);
+}
+
+template <int CLS>
+__device__ __forceinline__ void zone_job(const BatchParams& B, int s, const Job& job) {
+  constexpr int NT = kNtZone;
+  if (CLS == SC_DT) {
+    if (threadIdx.x == 0) box_dt(B, job.box);
+    return;
+  }
+  const double dt = B.scal[job.box].dt;
+  if (!wb_pos(dt)) return;
+  const BoxInfo& bi = B.boxes[job.box];
+  const int d = job.sub, ipc = items_per_chunk(s);
+  const long long nitems = stage_items(s, d, bi.v.geo, bi.wrap != 0);
+  const long long i0 = job.chunk * ipc;
+  const long long i1 = i0 + ipc < nitems ? i0 + ipc : nitems;
+  if (CLS == SC_COPY) {
+    for (long long it = i0 + threadIdx.x; it < i1; it += 2 * NT)
+      unit_pair_halo(bi, it, it + NT < i1 ? it + NT : -1);
+    return;
+  }
+  if (CLS == SC_EMF) {
+    for (long long it = i0 + threadIdx.x; it < i1; it += NT) unit_emf(s, d, bi, it, dt);
+    return;
+  }
+  const WbView& v = bi.v;
+  const WbBox b = stage_box(s, d, v.geo.n, bi.wrap != 0);
+  unsigned long long wkey = 0ULL;
+  int hits = 0, bad = 0;
+  for (long long it = i0 + threadIdx.x; it < i1; it += NT) {
+    int i, j, k;
+    item_ijk(b, it, &i, &j, &k);
+    const wbu::Nbr nb = wbu::neighbours(v.geo, i, j, k, bi.wrap ? 7 : 0);
+    if (CLS == SC_TRANS) {
+      const int mask = trans_mask(v.geo.n, i, j, k);
+      if (mask == 7) wbu::transverse_set(v, 0, 0, 7, i, j, k, nb);  // constant mask: see k_transverse
+      else if (mask) wbu::transverse_set(v, 0, 0, mask, i, j, k, nb);
+    } else if (CLS == SC_EREF_H) {
+      wbu::eref_half(v, 0, 0, dt, i, j, k, nb);
+    } else {
+      const double w = wbu::final_update(v, 0, 0, B.phys, i, j, k, nb, outflow_mask(bi), &hits, &bad);
+      const unsigned long long kw = wb_rate_bits(w);
+      if (kw > wkey) wkey = kw;
+    }
+  }
+  if (CLS == SC_FINAL) {
+    WbScalars& sc = B.scal[job.box];
+    warp_max_key(wkey, &sc.wmax_next);
+    if (hits) atomicAdd((unsigned long long*)&sc.floor_hits, (unsigned long long)hits);
+    if (bad) atomicAdd((unsigned long long*)&sc.unphysical, (unsigned long long)bad);
+  }
 }
 
 template <int CLS>
 __global__ void __launch_bounds__(kNtZone, zone_min_blocks(CLS))
     k_bstage_zone(BatchParams B, int grp, int s, unsigned seq) {
-  constexpr int NT = kNtZone;
-  unsigned* ctr = stage_counter(B, seq);
-  const int ipc = items_per_chunk(s);
-  drain_stage(B, grp, s, ctr, [&](int box, int d, long long cc) {
-    if (CLS == SC_DT) {
-      if (threadIdx.x == 0) box_dt(B, box);
-      return;
-    }
-    const double dt = B.scal[box].dt;
-    if (!wb_pos(dt)) return;
-    const BoxInfo& bi = B.boxes[box];
-    const long long nitems = stage_items(s, d, bi.v.geo, bi.wrap != 0);
-    const long long i0 = cc * ipc;
-    const long long i1 = i0 + ipc < nitems ? i0 + ipc : nitems;
-    if (CLS == SC_COPY) {
-      for (long long it = i0 + threadIdx.x; it < i1; it += 2 * NT)
-        unit_pair_halo(bi, it, it + NT < i1 ? it + NT : -1);
-      return;
-    }
-    if (CLS == SC_EMF) {
-      for (long long it = i0 + threadIdx.x; it < i1; it += NT) unit_emf(s, d, bi, it, dt);
-      return;
-    }
-    const WbView& v = bi.v;
-    const WbBox b = stage_box(s, d, v.geo.n, bi.wrap != 0);
-    unsigned long long wkey = 0ULL;
-    int hits = 0, bad = 0;
-    for (long long it = i0 + threadIdx.x; it < i1; it += NT) {
-      int i, j, k;
-      item_ijk(b, it, &i, &j, &k);
-      const wbu::Nbr nb = wbu::neighbours(v.geo, i, j, k, bi.wrap ? 7 : 0);
-      if (CLS == SC_TRANS) {
-        const int mask = trans_mask(v.geo.n, i, j, k);
-        if (mask == 7) wbu::transverse_set(v, 0, 0, 7, i, j, k, nb);  // constant mask: see k_transverse
-        else if (mask) wbu::transverse_set(v, 0, 0, mask, i, j, k, nb);
-      } else if (CLS == SC_EREF_H) {
-        wbu::eref_half(v, 0, 0, dt, i, j, k, nb);
-      } else {
-        const double w = wbu::final_update(v, 0, 0, B.phys, i, j, k, nb, outflow_mask(bi), &hits, &bad);
-        const unsigned long long kw = wb_rate_bits(w);
-        if (kw > wkey) wkey = kw;
-      }
-    }
-    if (CLS == SC_FINAL) {
-      warp_max_key(wkey, &B.scal[box].wmax_next);
-      if (hits) atomicAdd((unsigned long long*)&B.scal[box].floor_hits, (unsigned long long)hits);
-      if (bad) atomicAdd((unsigned long long*)&B.scal[box].unphysical, (unsigned long long)bad);
-    }
-  });
+  wb_pdl_begin();
+  zone_job<CLS>(B, s, stage_job(B, grp, s));
   stage_stamp(B, s, seq);
 }
 
@@ -712,8 +710,6 @@ struct wb_batch {
   size_t pre_cap;
   // launch configuration
   int form = WB_BATCH_PERSISTENT;
-  int zone_blocks[SC_COUNT];  // resident blocks per SM of each zone-stage kernel (staged form)
-  int sweep_blocks = 1;       // resident blocks per SM of the staged form's sweep kernel
   int seg_len;  // accepted and reported for callers; the sweeps have no segments
   int blocks_per_sm;
   int max_blocks_per_sm;
@@ -942,21 +938,44 @@ const void* batch_kernel(const WbPhys& ph) {
   return (const void*)k_batch<0, true>;
 }
 
-const void* bstage_sweep_kernel(const WbPhys& ph) {
+typedef void (*StageKernel)(BatchParams, int, int, unsigned);
+
+template <int LAYOUT>
+StageKernel bstage_sweep_of(const WbPhys& ph) {
   const bool ez = (ph.eps_zero & wbu::kEpsZeroLD) == wbu::kEpsZeroLD;
-  if (ez && !ph.prot) return (const void*)k_bstage_sweep<wbu::kEpsZeroLD, false>;
-  return (const void*)k_bstage_sweep<0, true>;
+  if (ez && !ph.prot) return k_bstage_sweep<wbu::kEpsZeroLD, false, LAYOUT>;
+  return k_bstage_sweep<0, true, LAYOUT>;
 }
 
-const void* bstage_zone_kernel(int cls) {
+StageKernel bstage_sweep_kernel(const WbPhys& ph, int layout) {
+  if (layout == wbu::kRing) return bstage_sweep_of<wbu::kRing>(ph);
+  if (layout == wbu::kOpen) return bstage_sweep_of<wbu::kOpen>(ph);
+  return bstage_sweep_of<wbu::kAnyLayout>(ph);
+}
+
+StageKernel bstage_zone_kernel(int cls) {
   switch (cls) {
-    case SC_COPY: return (const void*)k_bstage_zone<SC_COPY>;
-    case SC_EMF: return (const void*)k_bstage_zone<SC_EMF>;
-    case SC_TRANS: return (const void*)k_bstage_zone<SC_TRANS>;
-    case SC_EREF_H: return (const void*)k_bstage_zone<SC_EREF_H>;
-    case SC_FINAL: return (const void*)k_bstage_zone<SC_FINAL>;
-    default: return (const void*)k_bstage_zone<SC_DT>;
+    case SC_COPY: return k_bstage_zone<SC_COPY>;
+    case SC_EMF: return k_bstage_zone<SC_EMF>;
+    case SC_TRANS: return k_bstage_zone<SC_TRANS>;
+    case SC_EREF_H: return k_bstage_zone<SC_EREF_H>;
+    case SC_FINAL: return k_bstage_zone<SC_FINAL>;
+    default: return k_bstage_zone<SC_DT>;
   }
+}
+
+// The thread layout of sweep stage s for the boxes of group grp, where they agree.
+int group_layout(const wb_batch* b, int grp, int s) {
+  int rings = 0, open = 0;
+  for (int e = b->gfirst[grp]; e < b->gfirst[grp + 1]; ++e) {
+    const int box = b->gbox[e];
+    const bool wrap = b->info[box].wrap != 0;
+    for (int d = 0; d < 3; ++d) {
+      const WbBox r = stage_box(s, d, b->geo[box].n, wrap);
+      if (wbu::sweep_ring(r.hi[d] - r.lo[d] + 1, wrap)) rings = 1; else open = 1;
+    }
+  }
+  return rings && open ? wbu::kAnyLayout : (rings ? wbu::kRing : wbu::kOpen);
 }
 
 // enqueue the staged form of nsteps steps: one launch per (step, group,
@@ -969,21 +988,19 @@ cudaError_t enqueue_staged(wb_batch* b, int nsteps) {
   for (int step = 0; step < nsteps; ++step)
     for (int grp = 0; grp < p.ngroups; ++grp)
       for (int s = 0; s < BS_COUNT; ++s) {
-        if (!b->stage_chunks[(size_t)grp * BS_COUNT + s]) continue;
-        const int cls = stage_class(s);
-        const void* fn;
-        unsigned nt, nblocks;
-        if (cls == SC_SWEEP) {
-          fn = bstage_sweep_kernel(b->phys);
-          nt = kB;
-          nblocks = (unsigned)(std::min(b->blocks_per_sm, b->sweep_blocks) * b->sms);
+        // one block per chunk: a box holds more than 64 KB, so the count fits a grid
+        const unsigned nblocks = (unsigned)b->stage_chunks[(size_t)grp * BS_COUNT + s];
+        if (!nblocks) continue;
+        const bool sweep = stage_class(s) == SC_SWEEP;
+        const StageKernel fn =
+            sweep ? bstage_sweep_kernel(b->phys, group_layout(b, grp, s)) : bstage_zone_kernel(stage_class(s));
+        const int nt = sweep ? kB : kNtZone;
+        if (seq == 0) {  // follows the copy above, not a kernel
+          fn<<<nblocks, nt, 0, b->stream>>>(p, grp, s, seq);
         } else {
-          fn = bstage_zone_kernel(cls);
-          nt = kNtZone;
-          nblocks = (unsigned)((cls == SC_DT ? 1 : b->zone_blocks[cls]) * b->sms);
+          wb_launch_dependent(fn, nblocks, nt, b->stream, p, grp, s, seq);
         }
-        void* args[] = {&p, &grp, &s, &seq};
-        e = cudaLaunchKernel(fn, dim3(nblocks), dim3(nt), args, 0, b->stream);
+        e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         ++seq;
       }
@@ -1116,14 +1133,6 @@ int wb_pool_create(const wb_desc* physics, size_t state_bytes, size_t work_bytes
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, batch_kernel(b->phys), kB, 0);
   b->max_blocks_per_sm = nb > 0 ? nb : 1;
   b->blocks_per_sm = b->max_blocks_per_sm;
-  nb = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, bstage_sweep_kernel(b->phys), kB, 0);
-  b->sweep_blocks = nb > 0 ? nb : 1;
-  for (int c = 0; c < SC_COUNT; ++c) {
-    nb = 0;
-    if (c != SC_SWEEP) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, bstage_zone_kernel(c), kNtZone, 0);
-    b->zone_blocks[c] = nb > 0 ? nb : 1;
-  }
   b->seg_len = 32;
   int clk_khz = 0;
   cudaDeviceGetAttribute(&clk_khz, cudaDevAttrClockRate, dev);
