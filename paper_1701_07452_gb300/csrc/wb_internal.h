@@ -84,30 +84,32 @@ void wb_launch_final(const StageArgs& a, const StepControl& c, cudaStream_t s);
 void wb_launch_halo(double* const q[8], double* const b[3], const WbGeo& geo, const GridMap& m,
                     cudaStream_t s);
 
-// Arrays whose ghost points a periodic wrap fills (null entries skipped by
-// the caller that builds the list).
+// Arrays whose ghost points a periodic wrap fills, and the sides of the patch on
+// which a later stage reads them: bit 2 d the low side of axis d, 2 d + 1 the high one.
 struct WrapList {
   double* a[24];
+  unsigned char sides[24];
   int n;
 };
-// Periodic images on every axis: one patch (the box's own interior) or all
-// patches of a grid resident in one pass (slot = patch, neighbour patches).
-void wb_launch_wrap(const WrapList& L, const WbGeo& geo, const GridMap& m, int depth, cudaStream_t s);
+// Periodic images of the shell sh of the patches p0 .. p0 + nslots (slot = patch
+// - p0); along the axes that sh has a depth for, every patch of a row is among them.
+void wb_launch_wrap(const WrapList& L, const WbGeo& geo, const GridMap& m, const wbu::Shell& sh, long long p0,
+                    int nslots, cudaStream_t s);
 // The zone field, conserved state (from a primitive one) and first signal rate
 // of a loaded state.
 void wb_launch_init(double* const q[8], double* const b[3], const WbGeo& geo, long long npatch, int closed,
                     const WbPhys& ph, bool primitive, WbScalars* scal, cudaStream_t s);
-// Ghost points of the predictor's arrays (fluxes and reference EMF) of a grid of
-// one patch, `depth` zones deep: a ghost row of an outflow axis holds the data of
-// the boundary row and a periodic one that of its image, so the values there are
-// those of the interior, copied.  face[a]: the axis along which array a lives on
-// faces (computed up to the high boundary face of an outflow axis), or -1.
+// Ghost points sh of the predictor's arrays (fluxes and reference EMF) of a grid
+// of one patch: a ghost row of an outflow axis holds the data of the boundary
+// row, so the values there are those of the interior, copied.  face[a]: the axis
+// along which array a lives on faces (computed up to the high boundary face of an
+// outflow axis), or -1.
 struct ImageList {
   double* a[24];
   int face[24];
   int n;
 };
-void wb_launch_images(const ImageList& L, const WbGeo& geo, const GridMap& m, int depth, cudaStream_t s);
+void wb_launch_images(const ImageList& L, const WbGeo& geo, const wbu::Shell& sh, cudaStream_t s);
 void wb_launch_dt_step(WbScalars* scal, const StepControl& c, cudaStream_t s);
 // global <-> patch copies of up to 11 arrays; comp: 0..4 zone field, 5..7 face
 // field of axis comp-5

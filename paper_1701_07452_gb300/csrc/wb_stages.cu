@@ -111,70 +111,56 @@ __global__ void k_eref_half(StageArgs A, WbBox box) {
                  wbu::neighbours(A.v.geo, i, j, k, A.closed));
 }
 
-// Periodic images of intermediate arrays of a single-patch box that is
-// periodic on every axis (its stages read across the ends themselves; stage
-// dumps want the high boundary faces): each ghost point within `depth` zones of the
-// interior takes the value computed at the interior point it is an image of
-// (the same function of the same inputs, so the copy equals a recomputation
-// bit for bit).  One thread per shell point.
-__global__ void k_wrap(WrapList L, WbGeo g, int depth, long long n) {
-  wb_pdl_begin();
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (t >= n) return;
-  long long dst, src;
-  wbu::wrap_shell_point(g, depth, t, &dst, &src);
-  for (int a = 0; a < L.n; ++a) L.a[a][dst] = L.a[a][src];
-}
-
 // Ghost points of the predictor's arrays of a single patch with an outflow axis
 // (wb_launch_images): one thread per shell point, blockIdx.y the array.
-__global__ void k_images(ImageList L, WbGeo g, GridMap m, int depth, unsigned first, unsigned n) {
+__global__ void k_images(ImageList L, WbGeo g, wbu::Shell sh, unsigned n) {
   wb_pdl_begin();
   const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n) return;
   int x[3], src[3];
-  wbu::shell_point(g, depth, (long long)first + t, &x[0], &x[1], &x[2]);
+  wbu::shell_point(sh, t, x);
   const int face = L.face[blockIdx.y];
 #pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    const int N = m.N[d];
-    if (m.bc[d] == 0) src[d] = ((x[d] % N) + N) % N;
-    else src[d] = min(max(x[d], 0), face == d ? N : N - 1);
-  }
+  for (int d = 0; d < 3; ++d) src[d] = sh.dep[d] ? min(max(x[d], 0), face == d ? g.n[d] : g.n[d] - 1) : x[d];
   if (src[0] == x[0] && src[1] == x[1] && src[2] == x[2]) return;  // the high boundary face itself
   double* a = L.a[blockIdx.y];
   a[wb_at(g, x[0], x[1], x[2])] = a[wb_at(g, src[0], src[1], src[2])];
 }
 
-// The same for a grid of patches periodic on every axis, all patches resident
-// (slot = patch): a ghost point of patch blockIdx.y takes the value the
-// neighbouring patch (periodic across the domain) holds at that global
-// position.
-__global__ void k_wrap_patches(WrapList L, WbGeo g, GridMap m, int depth, long long n) {
+// Periodic images of intermediate arrays (wb_launch_wrap): a ghost point of the
+// patch in slot blockIdx.y takes the value the slot of the neighbouring patch
+// (periodic across the domain) holds at that global position, the same function
+// of the same inputs.  One thread per shell point; an array takes part where the
+// point lies outside on no other side than L.sides says.
+__global__ void k_wrap(WrapList L, WbGeo g, GridMap m, wbu::Shell sh, long long p0, unsigned n) {
   wb_pdl_begin();
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n) return;
-  const long long p = blockIdx.y;
   int loc[3];
-  wbu::shell_point(g, depth, t, &loc[0], &loc[1], &loc[2]);
-  long long pc[3];
-  pc[0] = p % m.np[0];
-  pc[1] = (p / m.np[0]) % m.np[1];
-  pc[2] = p / ((long long)m.np[0] * m.np[1]);
-  long long sp = 0, mul = 1;
+  wbu::shell_point(sh, t, loc);
+  const unsigned p = (unsigned)p0 + blockIdx.y;
+  const int pc[3] = {(int)(p % m.np[0]), (int)(p / m.np[0] % m.np[1]), (int)(p / m.np[0] / m.np[1])};
+  int sp = 0, mul = 1, out = 0;
   int sl[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    long long G = pc[d] * g.n[d] + loc[d];
-    G = ((G % m.N[d]) + m.N[d]) % m.N[d];
-    const long long q = G / g.n[d];
-    sl[d] = (int)(G - q * g.n[d]);
+    int q = pc[d];
+    sl[d] = loc[d];
+    if (sh.dep[d]) {
+      if (loc[d] < 0) out |= 1 << (2 * d);
+      if (loc[d] >= g.n[d]) out |= 2 << (2 * d);
+      int G = (pc[d] * g.n[d] + loc[d]) % m.N[d];
+      if (G < 0) G += m.N[d];
+      q = G / g.n[d];
+      sl[d] = G - q * g.n[d];
+    }
     sp += q * mul;
     mul *= m.np[d];
   }
-  const long long dst = p * g.V + wb_at(g, loc[0], loc[1], loc[2]);
-  const long long src = sp * g.V + wb_at(g, sl[0], sl[1], sl[2]);
-  for (int a = 0; a < L.n; ++a) L.a[a][dst] = L.a[a][src];
+  const long long dst = blockIdx.y * g.V + wb_at(g, loc[0], loc[1], loc[2]);
+  const long long src = (sp - p0) * g.V + wb_at(g, sl[0], sl[1], sl[2]);
+  for (int a = 0; a < L.n; ++a)
+    if (!(out & ~L.sides[a])) L.a[a][dst] = L.a[a][src];
 }
 
 __device__ __forceinline__ void block_max_atomic(double w, unsigned long long* dst) {
@@ -568,11 +554,10 @@ void wb_launch_halo(double* const q[8], double* const b[3], const WbGeo& geo, co
   wb_launch_dependent(k_halo, grid_for(geo.V, (int)m.npatch, 256), 256, s, a, m);
 }
 
-void wb_launch_wrap(const WrapList& L, const WbGeo& geo, const GridMap& m, int depth, cudaStream_t s) {
-  if (L.n <= 0) return;
-  const long long n = wbu::shell_count(geo, depth);
-  if (m.npatch == 1) wb_launch_dependent(k_wrap, grid_for(n, 1, 256), 256, s, L, geo, depth, n);
-  else wb_launch_dependent(k_wrap_patches, grid_for(n, (int)m.npatch, 256), 256, s, L, geo, m, depth, n);
+void wb_launch_wrap(const WrapList& L, const WbGeo& geo, const GridMap& m, const wbu::Shell& sh, long long p0,
+                    int nslots, cudaStream_t s) {
+  const long long n = wbu::shell_count(sh);
+  if (L.n > 0 && n > 0) wb_launch_dependent(k_wrap, grid_for(n, nslots, 256), 256, s, L, geo, m, sh, p0, (unsigned)n);
 }
 
 void wb_launch_init(double* const q[8], double* const b[3], const WbGeo& geo, long long npatch, int closed,
@@ -586,11 +571,9 @@ void wb_launch_init(double* const q[8], double* const b[3], const WbGeo& geo, lo
   wb_launch_dependent(k_init, grid_for(n, (int)npatch, bs), bs, s, a, primitive ? 1 : 0);
 }
 
-void wb_launch_images(const ImageList& L, const WbGeo& geo, const GridMap& m, int depth, cudaStream_t s) {
-  // one-plane storage: every layer is the plane, only its x and y ghosts are copied
-  const long long first = geo.sz == 0 ? (long long)(geo.n[0] + 2 * depth) * (geo.n[1] + 2 * depth) * 2 * depth : 0;
-  const long long n = wbu::shell_count(geo, depth) - first;
-  wb_launch_dependent(k_images, grid_for(n, L.n, 256), 256, s, L, geo, m, depth, (unsigned)first, (unsigned)n);
+void wb_launch_images(const ImageList& L, const WbGeo& geo, const wbu::Shell& sh, cudaStream_t s) {
+  const long long n = wbu::shell_count(sh);
+  wb_launch_dependent(k_images, grid_for(n, L.n, 256), 256, s, L, geo, sh, (unsigned)n);
 }
 
 void wb_launch_dt_step(WbScalars* scal, const StepControl& c, cudaStream_t s) {

@@ -1252,62 +1252,52 @@ __device__ __forceinline__ double final_update(const WbView& v, long long qo, lo
   return screened_rate(ir, vv, p, B, P, g, v.scal);
 }
 
-// The shell of ghost points within `depth` zones of a box's interior,
-// enumerated as the two z slabs of the depth-padded box, then the two y slabs
-// and the two x slabs of its interior z (and y) range.  Used for the periodic
-// images of intermediates (interior-only stages of a box periodic on every
-// axis) and for the ghost fill of a box that is its own domain.
+// The shell of points outside a block of n[] zones from off[] on, dep[] zones
+// deep along each axis: enumerated as the two z slabs of the padded block, then
+// the two y slabs and the two x slabs of its own z (and y) range.
+struct Shell {
+  int off[3], n[3], dep[3];
+};
+__host__ __device__ __forceinline__ Shell shell_of(const WbGeo& g, int depth) {
+  return {{0, 0, 0}, {g.n[0], g.n[1], g.n[2]}, {depth, depth, depth}};
+}
+__host__ __device__ __forceinline__ long long shell_count(const Shell& s) {
+  const long long e0 = s.n[0] + 2 * s.dep[0], e1 = s.n[1] + 2 * s.dep[1];
+  return e0 * e1 * (2 * s.dep[2]) + e0 * (2 * s.dep[1]) * s.n[2] + (long long)(2 * s.dep[0]) * s.n[1] * s.n[2];
+}
 __host__ __device__ __forceinline__ long long shell_count(const WbGeo& g, int depth) {
-  const long long w = 2 * depth;
-  return (long long)(g.n[0] + w) * (g.n[1] + w) * w + (long long)(g.n[0] + w) * w * g.n[2] +
-         w * g.n[1] * (long long)g.n[2];
+  return shell_count(shell_of(g, depth));
 }
 
-// Shell point t (0 <= t < shell_count) -> its zone index (i, j, k).
-__device__ __forceinline__ void shell_point(const WbGeo& g, int depth, long long t, int* pi, int* pj,
-                                            int* pk) {
-  const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
-  const int w = 2 * depth;
-  const unsigned e0 = (unsigned)(n0 + w), e1 = (unsigned)(n1 + w);
-  const unsigned long long zs = (unsigned long long)e0 * e1 * w;
-  const unsigned long long ys = (unsigned long long)e0 * w * n2;
+// Shell point t (0 <= t < shell_count) -> its zone index.
+__device__ __forceinline__ void shell_point(const Shell& s, long long t, int x[3]) {
+  const unsigned e0 = s.n[0] + 2 * s.dep[0], e1 = s.n[1] + 2 * s.dep[1];
+  const unsigned wx = 2 * s.dep[0], wy = 2 * s.dep[1], wz = 2 * s.dep[2];
+  const unsigned long long zs = (unsigned long long)e0 * e1 * wz, ys = (unsigned long long)e0 * wy * s.n[2];
   unsigned long long u = (unsigned long long)t;
-  int i, j, k;
   if (u < zs) {
     const unsigned r = (unsigned)(u % ((unsigned long long)e0 * e1));
     const int dz = (int)(u / ((unsigned long long)e0 * e1));
-    i = (int)(r % e0) - depth;
-    j = (int)(r / e0) - depth;
-    k = dz < depth ? dz - depth : n2 + dz - depth;
+    x[0] = (int)(r % e0) - s.dep[0];
+    x[1] = (int)(r / e0) - s.dep[1];
+    x[2] = dz < s.dep[2] ? dz - s.dep[2] : s.n[2] + dz - s.dep[2];
   } else if ((u -= zs) < ys) {
-    const unsigned per = e0 * (unsigned)w;
-    k = (int)(u / per);
+    const unsigned per = e0 * wy;
+    x[2] = (int)(u / per);
     const unsigned r = (unsigned)(u % per);
     const int dy = (int)(r / e0);
-    i = (int)(r % e0) - depth;
-    j = dy < depth ? dy - depth : n1 + dy - depth;
+    x[0] = (int)(r % e0) - s.dep[0];
+    x[1] = dy < s.dep[1] ? dy - s.dep[1] : s.n[1] + dy - s.dep[1];
   } else {
     u -= ys;
-    const unsigned r = (unsigned)(u / (unsigned)w);
-    const int dx = (int)(u % (unsigned)w);
-    j = (int)(r % (unsigned)n1);
-    k = (int)(r / (unsigned)n1);
-    i = dx < depth ? dx - depth : n0 + dx - depth;
+    const unsigned r = (unsigned)(u / wx);
+    const int dx = (int)(u % wx);
+    x[1] = (int)(r % (unsigned)s.n[1]);
+    x[2] = (int)(r / (unsigned)s.n[1]);
+    x[0] = dx < s.dep[0] ? dx - s.dep[0] : s.n[0] + dx - s.dep[0];
   }
-  *pi = i;
-  *pj = j;
-  *pk = k;
-}
-
-// Shell point t -> its offset and the offset of the interior point it is a
-// periodic image of.
-__device__ __forceinline__ void wrap_shell_point(const WbGeo& g, int depth, long long t, long long* dst,
-                                                 long long* src) {
-  int i, j, k;
-  shell_point(g, depth, t, &i, &j, &k);
-  const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
-  *dst = wb_at(g, i, j, k);
-  *src = wb_at(g, ((i % n0) + n0) % n0, ((j % n1) + n1) % n1, ((k % n2) + n2) % n2);
+#pragma unroll
+  for (int d = 0; d < 3; ++d) x[d] += s.off[d];
 }
 
 // Ghost fill of a box that is its own periodic/outflow domain (no patches):
@@ -1317,7 +1307,7 @@ __device__ __forceinline__ void wrap_shell_point(const WbGeo& g, int depth, long
 __device__ __forceinline__ void halo_self_offsets(const WbGeo& g, const int bc[3], long long t, long long* dst,
                                                   long long* src_off) {
   int loc[3];
-  shell_point(g, WB_NG, t, &loc[0], &loc[1], &loc[2]);
+  shell_point(shell_of(g, WB_NG), t, loc);
   int src[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
