@@ -339,9 +339,13 @@ void enqueue_pass(wb_grid* g, long long p0, int nslots, const StepControl& c) {
     sh.off[d] = -ring;
     sh.n[d] = G.n[d] + 2 * ring;
   }
-  auto images = [&](const WrapList& L, int depth) {
+  auto images = [&](int depth, auto&& list) {
+    if (!g->imaged) return;
+    WrapList L;
+    L.n = 0;
+    list(L);
     for (int d = 0; d < 3; ++d) sh.dep[d] = (g->imaged >> d) & 1 ? depth : 0;
-    if (g->imaged) wb_launch_wrap(L, G, g->map, sh, p0, nslots, s);
+    wb_launch_wrap(L, G, g->map, sh, p0, nslots, s);
   };
   // transverse differences read the fluxes' high faces, corner EMFs their low rows
   auto flux_images = [&](double* (&F)[3][8], WrapList& L) {
@@ -379,19 +383,19 @@ void enqueue_pass(wb_grid* g, long long p0, int nslots, const StepControl& c) {
     const WbBox pb[3] = {box(-3, N0 + 3, -4, N1 + 3, -4, N2 + 3), box(-4, N0 + 3, -3, N1 + 3, -4, N2 + 3),
                          box(-4, N0 + 3, -4, N1 + 3, -3, N2 + 3)};
     sweeps(g, sweep_args(g, A, false, pb, nslots, box(-4, N0 + 3, -4, N1 + 3, -4, N2 + 3)));
-    WrapList L = {};
-    flux_images(g->Fp, L);
-    for (int e = 0; e < 3; ++e) add_wrap(L, g->Eref[e], low_across(e));
-    images(L, 1);
+    images(1, [&](WrapList& L) {
+      flux_images(g->Fp, L);
+      for (int e = 0; e < 3; ++e) add_wrap(L, g->Eref[e], low_across(e));
+    });
   }
   // Step 3: corner EMFs
   {
     const WbBox eb[3] = {box(-1, N0, -3, N1 + 3, -3, N2 + 3), box(-3, N0 + 3, -1, N1, -3, N2 + 3),
                          box(-3, N0 + 3, -3, N1 + 3, -1, N2)};
     wb_launch_edges(A, false, eb, s);
-    WrapList L = {};
-    for (int e = 0; e < 3; ++e) add_wrap(L, g->Eedge[e], high_across(e));
-    images(L, 1);
+    images(1, [&](WrapList& L) {
+      for (int e = 0; e < 3; ++e) add_wrap(L, g->Eedge[e], high_across(e));
+    });
   }
   // Step 4: b^{n+1/2}
   {
@@ -400,42 +404,38 @@ void enqueue_pass(wb_grid* g, long long p0, int nslots, const StepControl& c) {
     wb_launch_ct(A, false, bb, s);
     // 2 deep, as the states: a sweep's block takes every zone's face field in
     // (NaN from a ghost nobody filled would send it to the FP64 products)
-    WrapList L = {};
-    for (int d = 0; d < 3; ++d) add_wrap(L, g->bh[d], low_side(d) | high_side(d));
-    images(L, 2);
+    images(2, [&](WrapList& L) {
+      for (int d = 0; d < 3; ++d) add_wrap(L, g->bh[d], low_side(d) | high_side(d));
+    });
   }
   // Steps 5, 7: transverse-flux preconditioned states
   {
     const WbBox tb[3] = {box(-3, N0 + 2, -1, N1, -1, N2), box(-1, N0, -3, N1 + 2, -1, N2),
                          box(-1, N0, -1, N1, -3, N2 + 2)};
     wb_launch_transverse(A, tb, s);
-    WrapList L = {};
-    for (int d = 0; d < 3; ++d)
-      for (int cc = 0; cc < 8; ++cc) add_wrap(L, g->qh[d][cc], low_side(d) | high_side(d));
-    images(L, 2);
+    images(2, [&](WrapList& L) {
+      for (int d = 0; d < 3; ++d)
+        for (int cc = 0; cc < 8; ++cc) add_wrap(L, g->qh[d][cc], low_side(d) | high_side(d));
+    });
   }
   // Steps 6, 7: corrector fluxes
   {
     const WbBox cb[3] = {box(-1, N0 + 1, -1, N1, -1, N2), box(-1, N0, -1, N1 + 1, -1, N2),
                          box(-1, N0, -1, N1, -1, N2 + 1)};
     sweeps(g, sweep_args(g, A, true, cb, nslots, cb[0]));
-    WrapList L = {};
-    flux_images(g->Fc, L);
-    images(L, 1);
+    images(1, [&](WrapList& L) { flux_images(g->Fc, L); });
   }
   // Step 8: half-step reference EMF; Step 9: corner EMFs
-  {
-    wb_launch_eref_half(A, box(-1, N0, -1, N1, -1, N2), s);
-    WrapList L = {};
+  wb_launch_eref_half(A, box(-1, N0, -1, N1, -1, N2), s);
+  images(1, [&](WrapList& L) {
     for (int e = 0; e < 3; ++e) add_wrap(L, g->Erefh[e], low_across(e));
-    images(L, 1);
-  }
+  });
   {
     const WbBox eb[3] = {box(0, N0 - 1, 0, N1, 0, N2), box(0, N0, 0, N1 - 1, 0, N2), box(0, N0, 0, N1, 0, N2 - 1)};
     wb_launch_edges(A, true, eb, s);
-    WrapList L = {};
-    for (int e = 0; e < 3; ++e) add_wrap(L, g->Eedgeh[e], high_across(e));
-    images(L, 1);
+    images(1, [&](WrapList& L) {
+      for (int e = 0; e < 3; ++e) add_wrap(L, g->Eedgeh[e], high_across(e));
+    });
   }
   // Step 11 (faces; a closed axis's high boundary face is face 0), then Step 10 +
   // zone field + floors + next signal rate
