@@ -39,8 +39,8 @@ namespace {
 
 // Stages of a step.  Boxes periodic on every axis (wrap) run every stage on
 // their interior and read across their own ends, as a single-patch grid does
-// (enqueue_pass_interior): they need no ghost fill.  BS_W* (once the images of
-// their intermediates) have no work and are not launched; they keep their
+// (enqueue_pass): they need no ghost fill.  BS_W* (once the images of their
+// intermediates) have no work and are not launched; they keep their
 // places in the stage times.
 enum {
   BS_DT = 0, BS_PRED, BS_EREF, BS_W_FP, BS_EDGE_P, BS_W_EE, BS_CT_H, BS_W_BH, BS_TRANS, BS_W_QH,
@@ -1447,8 +1447,9 @@ int wb_batch_read(wb_batch* b, int box, double* U, double* bx, double* by, doubl
     if (!on_device) {
       wb_launch_gather(all, g, m, s);
       all.n = 0;
-      cudaError_t e = cudaMemcpyAsync(dst, b->staging, sizeof(double) * ext[0] * ext[1] * ext[2],
-                                      cudaMemcpyDeviceToHost, s);
+      const size_t len = sizeof(double) * ext[0] * ext[1] * ext[2];
+      wb_touch_pages(dst, len);
+      cudaError_t e = cudaMemcpyAsync(dst, b->staging, len, cudaMemcpyDeviceToHost, s);
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);
       if (e != cudaSuccess) return bcuda(b, e, "batch read");
     }

@@ -763,6 +763,7 @@ int wb_read_state(wb_grid* g, double* U, double* bx, double* by, double* bz, dou
       MoveList one = {};
       wb_add_move(one, src, ddst, mcomp);
       wb_launch_gather(one, g->geo, g->map, s);
+      wb_touch_pages(dst, sizeof(double) * n);
       cudaError_t e = cudaMemcpyAsync(dst, g->staging, sizeof(double) * n, cudaMemcpyDeviceToHost, s);
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);
       if (e != cudaSuccess) return check_cuda(g, e, "read");
