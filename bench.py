@@ -60,22 +60,22 @@ SEED = 2
 # faces plus every other stage of the step); profiles/oracle_flop_count.md.
 ALG_FLOPS_PER_FACE = 879.0
 ALG_FLOPS_PER_CELL_UPDATE = 5871.0
-# FP64 flops (DFMA = 2, DMUL = DADD = 1) the kernels execute, from the ncu
-# FP64 instruction counters of one step of the 96^3 box: per interface system
-# of k_sweep (the mean over a step), and per zone of the other stage
-# kernels of the step together (profiles/k_sweep_96cube_ncu_full.md,
-# profiles/stages_96cube_fp64_counts.md).  Counted per face of the box the
-# figure leaves out the ~2 % of overlap systems a 256^3 launch adds.
-EXEC_FLOPS_PER_FACE = 450.8
-EXEC_STAGE_FLOPS_PER_ZONE = 431.8
+# FP64 flops (DFMA = 2, DMUL = DADD = 1) the kernels execute on the FP64 pipe,
+# from the ncu FP64 instruction counters of one step of the 96^3 box: per face of
+# k_sweep (the mean of the two launches of a step, the reference EMF of the
+# first included), and per zone of the other stage kernels of the step together
+# (profiles/stages_96cube_fp64_counts.md).  Products, reciprocals and roots that
+# run on the integer pipes are not FP64 instructions and do not count here.
+EXEC_FLOPS_PER_FACE = 283.9
+EXEC_STAGE_FLOPS_PER_ZONE = 382.5
 # DRAM bytes (read + write) of one k_sweep launch at the 256^3 workload, the
-# mean of the launches of a step from one ncu capture
+# mean of the two launches of a step (three axes each) from one ncu capture
 # (profiles/k_sweep_256cube_dram.md), valid only for the kernel sources it was
 # taken on (their SHA-256 over csrc/wb_sweep.cu, wb_units.cuh, wb_soft.cuh,
 # wb_device.cuh);
 # the algorithmic figure is 128 B per face.
-SWEEP_DRAM_CAPTURE = {"n": 256, "bytes": 3.6763e9,
-                      "src_sha256": "68f8615198707e20999cb9332cdfca1bc16d4505845845c06e39a34523ecfa46"}
+SWEEP_DRAM_CAPTURE = {"n": 256, "bytes": 7.5590e9,
+                      "src_sha256": "d8ddff9e0f71794c51439ff03719b0def97420ff05fd4de7551c578234199db9"}
 SWEEP_BYTES_PER_FACE = 128.0
 # algorithmic state bytes per cell-update: 5 conserved fields and 3 face fields
 # read and written once (the step's HBM roofline)
@@ -122,18 +122,29 @@ def step_launches(desc):
     (2 sweeps of all axes, the first with the reference EMF, corner EMFs, half
     CT, transverse states, half-step reference EMF, corner EMFs, final CT and
     the update, which also prepares the next dt) and the ghost fill, which a
-    single patch periodic on every axis does without; several patches of such a
-    grid in one pass add the 7 image fills of its interior-only stages.  (The dt
-    kernel of a call's first step is not counted.)"""
-    npatch = desc.patches[0] * desc.patches[1] * desc.patches[2]
-    per_pass = desc.batch_patches if desc.batch_patches > 0 else npatch
+    single patch periodic on every axis does without.  7 image fills a pass where
+    a pass holds whole rows of patches along a periodic axis and enough zones for
+    them to pay (the rule of set_interior in wb_capi.cu); one copy of the
+    predictor's ghosts for a single patch with an outflow axis.  (The dt kernel
+    of a call's first step is not counted.)"""
+    np_ = [desc.patches[a] for a in range(3)]
+    npatch = np_[0] * np_[1] * np_[2]
+    per_pass = min(desc.batch_patches, npatch) if desc.batch_patches > 0 else npatch
     passes = -(-npatch // per_pass)
-    periodic = all(desc.bc[a] == 0 for a in range(3))
-    if periodic and npatch == 1:
+    closed, imaged, row, zones = 0, 0, 1, per_pass
+    for a in range(3):
+        zones *= desc.n[a] // np_[a]
+        if desc.bc[a] == 0:
+            if np_[a] == 1:
+                closed += 1
+            elif per_pass % (row * np_[a]) == 0:
+                imaged += 1
+        row *= np_[a]
+    if closed + imaged < 3 and zones < (1 << 13 if imaged > 1 else 1 << 16):
+        imaged = 0
+    if closed == 3:
         return 9
-    flat = desc.n[2] == 1 and desc.patches[2] == 1 and desc.bc[2] == 0
-    images = passes == 1 and not flat and periodic
-    return 1 + (16 if images else 9) * passes
+    return 1 + (9 + (7 if imaged else 0) + (1 if npatch == 1 else 0)) * passes
 
 
 def workload_name(n):
@@ -521,19 +532,20 @@ def run_mode(args):
             torch.cuda.empty_cache()
             return ms, out
         if args.mode == "patches":
-            # every patch resident: periodic images between stages
+            # every patch resident: images of the neighbours between stages
             ms_p, out_p = run(p, 0)
             how = "all patches resident, neighbour images between stages"
         else:
             ms_p, out_p = run(p, 152, read=False)
-            how = "152 patches per pipeline pass, ghost rings recomputed"
+            how = ("152 patches per pipeline pass, images along the rows a pass holds whole, "
+                   "ghost rings across them")
         line = {"metric": METRIC, "mode": args.mode, "value": n ** 3 * args.steps / (ms_p * 1e-3),
                 "unit": UNIT, "higher_is_better": True, "steps": args.steps, "dtype": "f64",
                 "ms_per_step": ms_p / args.steps, "data": "synthetic",
                 "config": {"workload": f"{n}^3 periodic turbulence box in {p}^3 patches of {n // p}^3, " + how}}
         if args.mode == "big":
-            # the same box as one resident grid with periodic images, when the
-            # device holds it (about 250 GB at 768^3 besides the initial data)
+            # the same box as one resident grid, when the device holds it (about
+            # 250 GB at 768^3 besides the initial data)
             del out_p
             torch.cuda.empty_cache()
             need = wb.grid_bytes(wb.make_desc((n, n, n), length=st["length"])) + (4 << 30)
@@ -541,7 +553,7 @@ def run_mode(args):
             if free > need:
                 ms_s, _ = run(1, 0, read=False)
                 line["single_grid_value"] = n ** 3 * args.steps / (ms_s * 1e-3)
-                line["single_grid_config"] = f"one {n}^3 grid, all resident, periodic images between stages"
+                line["single_grid_config"] = f"one {n}^3 grid, all resident, read across its own ends"
             else:
                 line["single_grid_value"] = None
                 line["single_grid_config"] = f"not run: {need / 2**30:.0f} GiB needed, {free / 2**30:.0f} GiB free"
@@ -549,7 +561,8 @@ def run_mode(args):
             ms_q, out_q = run(p, 152)
             ms_s, out_s = run(1, 0)
             line["pipelined_value"] = n ** 3 * args.steps / (ms_q * 1e-3)
-            line["pipelined_config"] = "152 patches per pipeline pass, ghost rings recomputed"
+            line["pipelined_config"] = ("152 patches per pipeline pass, images along the rows a pass holds "
+                                        "whole, ghost rings across them")
             line["single_grid_value"] = n ** 3 * args.steps / (ms_s * 1e-3)
             line["bit_exact_vs_single_grid"] = all(bool(torch.equal(a, b)) for a, b in zip(out_p, out_s))
             line["pipelined_bit_exact_vs_single_grid"] = all(bool(torch.equal(a, b))

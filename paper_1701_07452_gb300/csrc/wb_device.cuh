@@ -42,8 +42,7 @@ __host__ __device__ __forceinline__ bool wb_zone_ok(const WbGeo& g, int i, int j
          (g.sz == 0 || (k >= -WB_NG && k < g.pd[2] - WB_NG));
 }
 
-// The checked build (-DWB_CHECKED; a substitute for a memory checker, which
-// this GPU pool does not offer): every zone index a kernel forms is tested
+// The checked build (-DWB_CHECKED; in the place of a memory checker): every zone index a kernel forms is tested
 // against the padded storage; a bad one sets a bit in the translation unit's
 // check word (read through wb_check_flags) and wb_at redirects it to zone
 // (0, 0, 0), so the access stays inside the array.

@@ -1,6 +1,6 @@
 // Device "units" of the CTU+CT MHDTVD step (Sec. "MHD in Three Dimensions",
 // Steps 1-11 with the App. A flux): one function per stage, each working on
-// one index (zone, face, edge or pencil segment) of one box.  The per-stage
+// one index (zone, face, edge or sweep tile) of one box.  The per-stage
 // kernels of a grid (wb_stages.cu, wb_sweep.cu) and the persistent batch
 // kernel (wb_batch.cu) call the same functions.
 #pragma once
@@ -86,9 +86,9 @@ __device__ __forceinline__ bool field_wild(unsigned size, double rho) {
 }
 
 // Zone state of a sweep.  The arithmetic is written with explicit rounding
-// (no contraction left to the compiler): a zone is loaded both before and
-// inside the march over a segment, and the two inlined copies must round
-// identically, or a face's flux would depend on where a segment starts.
+// (no contraction left to the compiler): several kernels and both forms of
+// the products inline it, and all must round identically, or a face's flux would
+// depend on how a box is split and launched.
 // q: the fields in the sweep's frame (rho, Mn, Mt1, Mt2, E, Bn, Bt1, Bt2).
 // Returns the largest field_size of its fields.
 template <bool NC, bool SOFT>

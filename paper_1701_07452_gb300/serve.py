@@ -16,9 +16,8 @@ been admitted, released at the next tick boundary if it is resident.
 
 Each tick runs in the pool's staged form by default (one launch per stage;
 form="persistent" selects the one cooperative launch); results do not depend
-on the form.  seg_len sets the pool's sweep segment length (0 keeps the
-library's 32; longer segments measured no faster on the request stream of
-the bench, 136 about 5 % slower).
+on the form.  seg_len is handed to the pool's configuration, which reports it
+(the sweeps have no segments).
 
 Two tick policies.  "fair": every resident run advances up to tick_steps per
 tick (processor sharing).  "srpt": each tick grants up to tick_steps steps to
