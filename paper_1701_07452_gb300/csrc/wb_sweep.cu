@@ -109,8 +109,8 @@ void wb_launch_sweeps(SweepArgs a, cudaStream_t s) {
     WB_SWEEP(0, false, true, wbu::kAnyLayout);
   } else if (!soft) {
     WB_SWEEP(kEpsZeroLD, false, false, wbu::kAnyLayout);
-  } else if (!fixed) {
-    WB_SWEEP(kEpsZeroLD, false, true, wbu::kAnyLayout);
+  } else if (!fixed || (rings == 3 && (axis(0) == 1 || axis(1) == 1 || axis(2) == 1))) {
+    WB_SWEEP(kEpsZeroLD, false, true, wbu::kThin);
   } else if (rings == 3) {
     WB_SWEEP(kEpsZeroLD, false, true, wbu::kRing);
   } else {

@@ -26,6 +26,9 @@ def wb():
     ((125, 31, 1), (0, 0, 0)), ((2, 126, 6), (0, 0, 0)), ((1, 5, 40), (0, 0, 0)), ((20, 64, 42), (0, 0, 0)), ((128, 3, 21), (0, 0, 0)), ((127, 60, 3), (0, 0, 0)),
     ((16, 32, 8), (1, 1, 1)), ((59, 4, 61), (1, 0, 0)), ((119, 2, 3), (0, 0, 1)), ((1, 1, 7), (1, 1, 1)),
     ((40, 1, 3), (1, 1, 0)), ((3, 2, 1), (1, 1, 1)), ((20, 24, 1), (1, 0, 0)), ((4, 33, 18), (0, 1, 0)),
+    # one-zone closed axes in launches of more than 152 tiles
+    ((200, 120, 1), (0, 0, 0)), ((200, 120, 1), (1, 0, 0)), ((64, 1, 250), (0, 0, 0)), ((1, 150, 130), (0, 0, 0)),
+    ((1, 64, 128), (0, 0, 0)),
 ])
 def test_one_step_matches_the_oracle(wb, oracle_mod, n, bc):
     from paper_1701_07452_gb300.initial_conditions import random_box
