@@ -140,7 +140,7 @@ def step_launches(desc):
             elif per_pass % (row * np_[a]) == 0:
                 imaged += 1
         row *= np_[a]
-    if closed + imaged < 3 and zones < (1 << 13 if imaged > 1 else 1 << 16):
+    if closed + imaged < 3 and zones < (1 << 10 if imaged > 1 else 5 << 10):
         imaged = 0
     if closed == 3:
         return 9

@@ -318,8 +318,8 @@ constexpr int high_across(int e) { return high_side((e + 1) % 3) | high_side((e 
 // Along imaged axes the ghost points that a later stage reads (1 deep; 2 for what
 // the corrector sweeps read) are filled between the stages from the neighbouring
 // patch, only on the sides where they are read.  A step of 96^3 zones in 27 patches: in
-// passes of 9 (layers) 4.01 ms with the rings recomputed, 3.24 with images; in one
-// pass 3.41 ms with images on every side, 2.74 so.
+// passes of 9 (layers) 4.01 ms with the rings recomputed, 3.14 with images; in one
+// pass 3.41 ms with images on every side, 2.70 so.
 void enqueue_pass(wb_grid* g, long long p0, int nslots, const StepControl& c) {
   cudaStream_t s = g->stream;
   StageArgs A = stage_args(g, p0, nslots);
@@ -458,15 +458,15 @@ void set_interior(wb_grid* g) {
     }
     row *= np;
   }
-  // Nine more launches a pass: they pay from some zones a pass on.  Rows (one axis)
-  // of 28 000 zones +8 %, of 41 000 to 66 000 +1, of 98 000 and 128 000 -3 and -2 %
-  // of a step's time; layers (two) of 2 000 zones +20 %, of 7 000 +5, of 8 000 and 16 000 -18
-  // and -7 %.  With no ring left at all the images always did better (2 000
-  // zones: 142 us with all of them, 126 now; in passes with rings 184).
+  // Seven more launches a pass: they pay from some zones a pass on.  Rows (one axis)
+  // of 1 000, 2 000 and 3 500 zones +12, +8 and +4 % of a step's time, of 7 000,
+  // 8 000, 28 000 and 65 000 -4, -4, -2 and -7 %; layers (two) of 860 zones +8 %, of
+  // 1 000 to 3 500 -17 and -18 (thin patches) to 0, of 4 000 to 16 000 -6 to -18 %.
+  // With no ring left at all the images always did better.
   long long zones = g->S;
   for (int d = 0; d < 3; ++d) zones *= g->geo.n[d];
   const bool several = (g->imaged & (g->imaged - 1)) != 0;
-  if ((g->closed | g->imaged) != 7 && zones < (several ? 1 << 13 : 1 << 16)) g->imaged = 0;
+  if ((g->closed | g->imaged) != 7 && zones < (several ? 1 << 10 : 5 << 10)) g->imaged = 0;
 }
 
 StepControl step_control(const wb_grid* g, double t_end) {
