@@ -995,12 +995,12 @@ cudaError_t enqueue_staged(wb_batch* b, int nsteps) {
         const StageKernel fn =
             sweep ? bstage_sweep_kernel(b->phys, group_layout(b, grp, s)) : bstage_zone_kernel(stage_class(s));
         const int nt = sweep ? kB : kNtZone;
-        if (seq == 0) {  // follows the copy above, not a kernel
-          fn<<<nblocks, nt, 0, b->stream>>>(p, grp, s, seq);
+        if (seq == 0) {  // follows the memset above, not a kernel
+          void* args[] = {&p, &grp, &s, &seq};
+          e = cudaLaunchKernel((const void*)fn, dim3(nblocks), dim3(nt), args, 0, b->stream);
         } else {
-          wb_launch_dependent(fn, nblocks, nt, b->stream, p, grp, s, seq);
+          e = wb_launch_dependent(fn, nblocks, nt, b->stream, p, grp, s, seq);
         }
-        e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         ++seq;
       }

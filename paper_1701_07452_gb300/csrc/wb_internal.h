@@ -9,7 +9,7 @@
 // Launch of a kernel that begins with wb_pdl_begin(): it may be set up before
 // the kernel ahead of it on the stream has finished.
 template <class... P, class... A>
-inline void wb_launch_dependent(void (*kernel)(P...), dim3 grid, int threads, cudaStream_t s, const A&... args) {
+inline cudaError_t wb_launch_dependent(void (*kernel)(P...), dim3 grid, int threads, cudaStream_t s, const A&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3((unsigned)threads);
@@ -19,7 +19,7 @@ inline void wb_launch_dependent(void (*kernel)(P...), dim3 grid, int threads, cu
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
 // Brings in the pages of a host buffer that a copy from the device is about to
