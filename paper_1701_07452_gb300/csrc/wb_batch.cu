@@ -1429,6 +1429,7 @@ int wb_batch_read(wb_batch* b, int box, double* U, double* bx, double* by, doubl
   const long long nc = (long long)d.n[0] * d.n[1] * d.n[2];
   double* faces[3] = {bx, by, bz};
   MoveList all = {};
+  bool idle = false;  // the caller's earlier work on the stream is done
   for (int comp = 0; comp < 11; ++comp) {
     double* dst;
     const double* src;
@@ -1448,8 +1449,8 @@ int wb_batch_read(wb_batch* b, int box, double* U, double* bx, double* by, doubl
       wb_launch_gather(all, g, m, s);
       all.n = 0;
       const size_t len = sizeof(double) * ext[0] * ext[1] * ext[2];
-      wb_touch_pages(dst, len);
-      cudaError_t e = cudaMemcpyAsync(dst, b->staging, len, cudaMemcpyDeviceToHost, s);
+      cudaError_t e = wb_touch_in_order(dst, len, s, &idle);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(dst, b->staging, len, cudaMemcpyDeviceToHost, s);
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);
       if (e != cudaSuccess) return bcuda(b, e, "batch read");
     }

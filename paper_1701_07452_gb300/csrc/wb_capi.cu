@@ -741,6 +741,7 @@ int wb_read_state(wb_grid* g, double* U, double* bx, double* by, double* bz, dou
   const long long nc = (long long)g->d.n[0] * g->d.n[1] * g->d.n[2];
   double* faces[3] = {bx, by, bz};
   MoveList direct = {};  // arrays a kernel can write where they are: one launch
+  bool idle = false;     // the caller's earlier work on the stream is done
   for (int comp = 0; comp < 11; ++comp) {
     double* dst;
     int mcomp = comp;
@@ -763,8 +764,8 @@ int wb_read_state(wb_grid* g, double* U, double* bx, double* by, double* bz, dou
       MoveList one = {};
       wb_add_move(one, src, ddst, mcomp);
       wb_launch_gather(one, g->geo, g->map, s);
-      wb_touch_pages(dst, sizeof(double) * n);
-      cudaError_t e = cudaMemcpyAsync(dst, g->staging, sizeof(double) * n, cudaMemcpyDeviceToHost, s);
+      cudaError_t e = wb_touch_in_order(dst, sizeof(double) * n, s, &idle);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(dst, g->staging, sizeof(double) * n, cudaMemcpyDeviceToHost, s);
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);
       if (e != cudaSuccess) return check_cuda(g, e, "read");
     }

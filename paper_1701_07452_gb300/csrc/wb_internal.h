@@ -36,6 +36,20 @@ inline void wb_touch_pages(void* p, size_t bytes) {
   c[bytes - 1] = 0;
 }
 
+// The same ahead of a copy on stream s, in the stream's order: work enqueued
+// earlier may still read the buffer (a copy out of it, a host function), so the
+// stream is waited for first.  *idle: already waited for in this call (what the
+// call itself enqueues afterwards uses no other of the caller's arrays).
+inline cudaError_t wb_touch_in_order(void* p, size_t bytes, cudaStream_t s, bool* idle) {
+  if (!*idle) {
+    const cudaError_t e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) return e;
+    *idle = true;
+  }
+  wb_touch_pages(p, bytes);
+  return cudaSuccess;
+}
+
 struct wb_desc;
 // Physics constants of a descriptor (gamma, CFL, eps_k, limiter, floors).
 WbPhys wb_phys_of(const struct wb_desc* d);
