@@ -1448,8 +1448,9 @@ int wb_batch_read(wb_batch* b, int box, double* U, double* bx, double* by, doubl
     if (!on_device) {
       wb_launch_gather(all, g, m, s);
       all.n = 0;
-      const size_t len = sizeof(double) * ext[0] * ext[1] * ext[2];
-      cudaError_t e = wb_touch_in_order(dst, len, s, &idle);
+      const long long n = ext[0] * ext[1] * ext[2];
+      const size_t len = sizeof(double) * n;
+      cudaError_t e = wb_host_array(dst, n).plain ? wb_touch_in_order(dst, len, s, &idle) : cudaSuccess;
       if (e == cudaSuccess) e = cudaMemcpyAsync(dst, b->staging, len, cudaMemcpyDeviceToHost, s);
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);
       if (e != cudaSuccess) return bcuda(b, e, "batch read");

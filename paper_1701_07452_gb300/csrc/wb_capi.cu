@@ -482,24 +482,6 @@ int sync(wb_grid* g, const char* where) {
   return check_cuda(g, cudaStreamSynchronize(g->stream), where);
 }
 
-// Device address of a host array of n doubles that lives in page-locked host
-// memory the GPU can address (cudaHostAlloc / cudaHostRegister), or null.
-// Kernels then read or write it in place over the CPU-GPU link instead of
-// going through a staging copy; both ends of the array are checked.
-const void* host_mapped(const void* p, long long n) {
-  if (!p || n <= 0) return nullptr;
-  cudaPointerAttributes a0, a1;
-  if (cudaPointerGetAttributes(&a0, p) != cudaSuccess) { cudaGetLastError(); return nullptr; }
-  const char* last = static_cast<const char*>(p) + sizeof(double) * (size_t)(n - 1);
-  if (cudaPointerGetAttributes(&a1, last) != cudaSuccess) { cudaGetLastError(); return nullptr; }
-  if (a0.type != cudaMemoryTypeHost || a1.type != cudaMemoryTypeHost) return nullptr;
-  if (!a0.devicePointer || !a1.devicePointer) return nullptr;
-  const char* d0 = static_cast<const char*>(a0.devicePointer);
-  const char* d1 = static_cast<const char*>(a1.devicePointer);
-  if (d1 - d0 != last - static_cast<const char*>(p)) return nullptr;
-  return a0.devicePointer;
-}
-
 int load_common(wb_grid* g, const double* U, const double* bx, const double* by,
                 const double* bz, int on_device, bool primitive) {
   if (!g || !U || !bx || !by || !bz) return fail(g, WB_ERR_INVALID, "null argument");
@@ -514,7 +496,7 @@ int load_common(wb_grid* g, const double* U, const double* bx, const double* by,
     else { ext[comp - 5] += 1; src = faces[comp - 5]; }
     long long n = ext[0] * ext[1] * ext[2];
     const double* dsrc = src;
-    const void* mapped = on_device ? nullptr : host_mapped(src, n);
+    void* mapped = on_device ? nullptr : wb_host_array(src, n).mapped;
     const bool staged = !on_device && !mapped;
     if (mapped) dsrc = static_cast<const double*>(mapped);
     if (staged) {
@@ -756,15 +738,15 @@ int wb_read_state(wb_grid* g, double* U, double* bx, double* by, double* bz, dou
       dst = B + (comp - 8) * nc; src = g->q[F_BX + comp - 8]; mcomp = 0;
     }
     long long n = ext[0] * ext[1] * ext[2];
-    const void* mapped = on_device ? nullptr : host_mapped(dst, n);
-    const bool staged = !on_device && !mapped;
-    double* ddst = on_device ? dst : (mapped ? static_cast<double*>(const_cast<void*>(mapped)) : g->staging);
+    const WbHostArray host = on_device ? WbHostArray{nullptr, false} : wb_host_array(dst, n);
+    const bool staged = !on_device && !host.mapped;
+    double* ddst = on_device ? dst : (host.mapped ? static_cast<double*>(host.mapped) : g->staging);
     if (!staged) wb_add_move(direct, src, ddst, mcomp);
     if (staged) {
       MoveList one = {};
       wb_add_move(one, src, ddst, mcomp);
       wb_launch_gather(one, g->geo, g->map, s);
-      cudaError_t e = wb_touch_in_order(dst, sizeof(double) * n, s, &idle);
+      cudaError_t e = host.plain ? wb_touch_in_order(dst, sizeof(double) * n, s, &idle) : cudaSuccess;
       if (e == cudaSuccess) e = cudaMemcpyAsync(dst, g->staging, sizeof(double) * n, cudaMemcpyDeviceToHost, s);
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);
       if (e != cudaSuccess) return check_cuda(g, e, "read");

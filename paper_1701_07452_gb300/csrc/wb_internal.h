@@ -1,9 +1,9 @@
 // Host-side declarations of the kernel launchers (internal to the library).
 #pragma once
 #include <cuda_runtime.h>
-#include <unistd.h>
 
 #include "wb_device.cuh"
+#include "wb_pages.h"
 #include "wb_units.cuh"
 
 // Launch of a kernel that begins with wb_pdl_begin(): it may be set up before
@@ -20,34 +20,6 @@ inline cudaError_t wb_launch_dependent(void (*kernel)(P...), dim3 grid, int thre
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
-}
-
-// Brings in the pages of a host buffer that a copy from the device is about to
-// fill.  The copy writes pageable memory in place over the CPU-GPU link, and a
-// page nobody has written yet then costs a fault taken from the GPU: 129 MB into
-// fresh arrays took 37 to 49 ms (64 KB pages), into written ones 3.1; writing
-// to each page here costs 3.9.  (Reading a page first maps the zero page, and the
-// write after it is as slow as the GPU's fault.)
-inline void wb_touch_pages(void* p, size_t bytes) {
-  const long page = sysconf(_SC_PAGESIZE);
-  if (page <= 0 || !bytes) return;
-  volatile char* c = static_cast<volatile char*>(p);
-  for (size_t at = 0; at < bytes; at += (size_t)page) c[at] = 0;
-  c[bytes - 1] = 0;
-}
-
-// The same ahead of a copy on stream s, in the stream's order: work enqueued
-// earlier may still read the buffer (a copy out of it, a host function), so the
-// stream is waited for first.  *idle: already waited for in this call (what the
-// call itself enqueues afterwards uses no other of the caller's arrays).
-inline cudaError_t wb_touch_in_order(void* p, size_t bytes, cudaStream_t s, bool* idle) {
-  if (!*idle) {
-    const cudaError_t e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return e;
-    *idle = true;
-  }
-  wb_touch_pages(p, bytes);
-  return cudaSuccess;
 }
 
 struct wb_desc;
