@@ -57,13 +57,17 @@ __device__ __forceinline__ double ld(const double* p) {
 }
 
 // A product of the sweeps: on the integer pipes (SOFT) or the FP64 pipe, the
-// same bits.  The integer form neither looks for infinities and NaN nor for
-// overflow: a sweep takes it where every zone field and face field is below
-// 2^50 in magnitude, the density above 2^-50 (field_wild) and the Roe state's
-// a^2 above 2^-100 (face_system).  No product then leaves the range: with
-// dt/dx < 2^50 too, |v| < 2^100, a^2 < 2^204, every alpha_k < 2^356, |nu_k| <
-// 2^155, g-tilde < 2^668, the sum of beta_k R_k below 2^920.
-// KNOWN: what follows from those bounds for the factors (wb_smul_finite).
+// same bits wherever the product is zero or of magnitude 2^-1021 and up (below,
+// the integer form gives zero).  The integer form neither looks for infinities and
+// NaN nor for overflow: a sweep takes it where every zone field and face field is zero
+// or of magnitude between 2^-100 and 2^50, the density between 2^-50 and 2^50, dt/dx
+// between 2^-100 and 2^50 (FieldRange) and the Roe state's a^2 above 2^-100
+// (face_system).  No product then leaves the range upwards: with |v| < 2^100, a^2 <
+// 2^204, every alpha_k < 2^356, |nu_k| < 2^155, g-tilde < 2^668, the sum of beta_k R_k
+// below 2^920.  Downwards, a difference of two fields is zero or 2^-152 and up, and
+// the longest product, w^2 in the band of beta_k, has dt/dx, a speed, a field and a
+// difference twice each, 2^-904 for unit density: one below 2^-1021 takes rounding
+// residues as factors several times over.
 template <bool SOFT, int KNOWN = 0>
 __device__ __forceinline__ double mul(double x, double y) {
   return SOFT ? wb_smul_finite<KNOWN>(x, y) : __dmul_rn(x, y);
@@ -79,20 +83,32 @@ __device__ __forceinline__ WbRoots roots(double x) {
   return SOFT ? wb_roots_sure(x) : wb_roots(x);
 }
 
-// |x| or dt/dx in units of the test above: the high word without its sign, twice
-__device__ __forceinline__ unsigned field_size(double x) { return wb_hi32(x) << 1; }
-__device__ __forceinline__ bool field_wild(unsigned size, double rho) {
-  return size >= ((1023u + 50u) << 21) || wb_hi32(rho) - ((1023u - 50u) << 20) >= (100u << 20);
-}
+// The range of the fields a thread takes in (magnitudes, by twice their high words;
+// zero counts as none; a bit below says that the low word is not zero, so that the
+// smallest subnormals do not pass for it).
+struct FieldRange {
+  unsigned most = 0, least = 0xffffffffu;
+  __device__ __forceinline__ void add(double x) {
+    const unsigned u = (wb_hi32(x) << 1) + min(wb_lo32(x), 1u);
+    most = max(most, u);
+    least = min(least, u - 1u);
+  }
+  // Fields of other magnitudes go to the FP64 products (NaN and infinities too).
+  // Nonzero fields below 2^-100 did not before; their products' flush to zero then
+  // gave a grid of 32^3 zones with a tail of 2^-1000 other bits than its patches.
+  __device__ __forceinline__ bool wild(double rho) const {
+    return most >= ((1023u + 50u) << 21) || least < ((1023u - 100u) << 21) - 1u ||
+           wb_hi32(rho) - ((1023u - 50u) << 20) >= (100u << 20);
+  }
+};
 
 // Zone state of a sweep.  The arithmetic is written with explicit rounding
 // (no contraction left to the compiler): several kernels and both forms of
 // the products inline it, and all must round identically, or a face's flux would
 // depend on how a box is split and launched.
 // q: the fields in the sweep's frame (rho, Mn, Mt1, Mt2, E, Bn, Bt1, Bt2).
-// Returns the largest field_size of its fields.
 template <bool NC, bool SOFT>
-__device__ __forceinline__ unsigned load_cell(const double* const (&q)[8], long long off, const WbPhys& P, Cell& c) {
+__device__ __forceinline__ FieldRange load_cell(const double* const (&q)[8], long long off, const WbPhys& P, Cell& c) {
   c.rho = ld<NC>(q[0] + off);
   c.mn = ld<NC>(q[1] + off);
   c.mt1 = ld<NC>(q[2] + off);
@@ -101,8 +117,14 @@ __device__ __forceinline__ unsigned load_cell(const double* const (&q)[8], long 
   const double bn = ld<NC>(q[5] + off);
   c.bt1 = ld<NC>(q[6] + off);
   c.bt2 = ld<NC>(q[7] + off);
-  const unsigned size = max(max(max(field_size(c.mn), field_size(c.mt1)), max(field_size(c.mt2), field_size(e))),
-                            max(max(field_size(bn), field_size(c.bt1)), field_size(c.bt2)));
+  FieldRange range;
+  range.add(c.mn);
+  range.add(c.mt1);
+  range.add(c.mt2);
+  range.add(e);
+  range.add(bn);
+  range.add(c.bt1);
+  range.add(c.bt2);
   const WbRoots rr = roots<SOFT>(c.rho);
   c.sr = rr.sq;
   c.ir = rr.rcp;
@@ -129,7 +151,7 @@ __device__ __forceinline__ unsigned load_cell(const double* const (&q)[8], long 
   c.F[5] = __fma_rn(c.bt2, hvn, -mul<SOFT>(c.vt2, hbn));
   const double bv = __fma_rn(c.bt2, c.vt2, __fma_rn(c.bt1, c.vt1, mul<SOFT>(bn, c.vn)));
   c.F[6] = __fma_rn(ep, hvn, __dmul_rn(-hbn, bv));
-  return size;
+  return range;
 }
 
 // Per-face record.
@@ -674,9 +696,11 @@ __device__ __forceinline__ int sweep_tile(const WbGeo& g, const WbBox& box, int 
     for (int m = 0; m < 7; ++m) s.F[m][o] = out[m];
     return hll && pos[0] >= 0 && pos[0] < g.n[0] && pos[1] >= 0 && pos[1] < g.n[1] && pos[2] >= 0 && pos[2] < g.n[2];
   }
-  const unsigned size = load_cell<NC, SOFT>(s.q, off, P, R);
+  FieldRange range = load_cell<NC, SOFT>(s.q, off, P, R);
   const double b = ld<NC>(s.bn + off), dtdx = scal->dtdx[d];
-  const bool wild = SOFT && field_wild(max(size, max(field_size(b), field_size(dtdx))), R.rho);
+  range.add(b);
+  range.add(dtdx);
+  const bool wild = SOFT && range.wild(R.rho);
   Cell L;
   L.ir = 0.0;  // not used across a face
   // neighbours in other warps go through X, unless every ring sits in a warp
