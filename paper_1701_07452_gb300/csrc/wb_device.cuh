@@ -196,12 +196,17 @@ __device__ __forceinline__ bool wb_zero(double x) {
 __device__ __forceinline__ bool wb_le_nonneg(double a, double b) {
   return __double_as_longlong(a) <= __double_as_longlong(b);
 }
-// x 2^n in the order of high words (x >= 0): a quick comparison by magnitude
-__device__ __forceinline__ unsigned wb_hi_scaled(double x, int n) { return wb_hi32(x) + ((unsigned)n << 20); }
+// x <= 2^-n s is possible (x, s >= 0, 1 <= n < 1023): a quick comparison by high
+// words ahead of an exact one.  True for every x below the normal range, whose
+// exponent does not grow with 2^n: s itself may be near its end (x = 0 beside s =
+// 2^-990 was ruled out once, and a cold gas at rest divided by a zero root).
+__device__ __forceinline__ bool wb_maybe_below(double x, int n, unsigned s_hi) {
+  return wb_hi32(x) + ((unsigned)n << 20) <= max(s_hi, ((unsigned)(n + 1) << 20) - 1u);
+}
 // x <= 2^-77 max(a, b) is possible (x, a, b >= 0): a cheap test ahead of
 // x <= 1e-24 (a + b + x), whose right side is below 2^-78 max(a, b) (1 + 2^-20)
 __device__ __forceinline__ bool wb_maybe_small(double x, double a, double b) {
-  return wb_hi_scaled(x, 77) <= max(wb_hi32(a), wb_hi32(b));
+  return wb_maybe_below(x, 77, max(wb_hi32(a), wb_hi32(b)));
 }
 // x <= f s for x, s >= 0.  Not inlined: the multiply would be issued by every
 // warp, its lanes predicated off, where a quick test has ruled the case out.

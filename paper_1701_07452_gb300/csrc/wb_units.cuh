@@ -370,7 +370,7 @@ __device__ __forceinline__ int face_system(const Cell& L, const Cell& R, double 
   const double minor = WB_MUL(mul<SOFT, 1>(a, mul<SOFT, 2>(btm, isrho)), wb_twice(r));
   double af = slow_major ? minor : major;
   double as = slow_major ? major : minor;
-  if (wb_hi_scaled(sd, 39) <= wb_hi32(sum) && wb_at_most(sd, 1e-12, sum)) {
+  if (wb_maybe_below(sd, 39, wb_hi32(sum)) && wb_at_most(sd, 1e-12, sum)) {
     const bool fast = wb_le_nonneg(ca2, a2);
     af = fast ? 1.0 : 0.0;
     as = fast ? 0.0 : 1.0;
