@@ -995,12 +995,7 @@ cudaError_t enqueue_staged(wb_batch* b, int nsteps) {
         const StageKernel fn =
             sweep ? bstage_sweep_kernel(b->phys, group_layout(b, grp, s)) : bstage_zone_kernel(stage_class(s));
         const int nt = sweep ? kB : kNtZone;
-        if (seq == 0) {  // follows the memset above, not a kernel
-          void* args[] = {&p, &grp, &s, &seq};
-          e = cudaLaunchKernel((const void*)fn, dim3(nblocks), dim3(nt), args, 0, b->stream);
-        } else {
-          e = wb_launch_dependent(fn, nblocks, nt, b->stream, p, grp, s, seq);
-        }
+        e = wb_launch(seq > 0, fn, nblocks, nt, b->stream, p, grp, s, seq);  // (the first follows the memset)
         if (e != cudaSuccess) return e;
         ++seq;
       }
@@ -1320,6 +1315,8 @@ int wb_batch_load(wb_batch* b, int box, const double* U, const double* bx, const
   cudaStream_t s = b->stream;
   const long long nc = (long long)d.n[0] * d.n[1] * d.n[2];
   const double* faces[3] = {bx, by, bz};
+  cudaError_t e = cudaMemsetAsync(b->d_scal + box, 0, sizeof(WbScalars), s);
+  if (e != cudaSuccess) return bcuda(b, e, "batch load");
   MoveList all = {};
   for (int comp = 0; comp < 8; ++comp) {
     long long ext[3] = {d.n[0], d.n[1], d.n[2]};
@@ -1328,8 +1325,7 @@ int wb_batch_load(wb_batch* b, int box, const double* U, const double* bx, const
     else { ext[comp - 5] += 1; src = faces[comp - 5]; }
     const double* dsrc = src;
     if (!on_device) {
-      cudaError_t e = cudaMemcpyAsync(b->staging, src, sizeof(double) * ext[0] * ext[1] * ext[2],
-                                      cudaMemcpyHostToDevice, s);
+      e = cudaMemcpyAsync(b->staging, src, sizeof(double) * ext[0] * ext[1] * ext[2], cudaMemcpyHostToDevice, s);
       if (e != cudaSuccess) return bcuda(b, e, "batch load");
       dsrc = b->staging;
     }
@@ -1338,7 +1334,7 @@ int wb_batch_load(wb_batch* b, int box, const double* U, const double* bx, const
     if (!on_device) {
       wb_launch_scatter(all, g, m, s);
       all.n = 0;
-      cudaError_t e = cudaStreamSynchronize(s);
+      e = cudaStreamSynchronize(s);
       if (e != cudaSuccess) return bcuda(b, e, "batch load");
     }
   }
@@ -1347,8 +1343,6 @@ int wb_batch_load(wb_batch* b, int box, const double* U, const double* bx, const
   for (int c = 0; c < 8; ++c) q[c] = bi.v.q[c];
   for (int c = 0; c < 3; ++c) bb[c] = bi.v.b[c];
   wb_launch_scatter(all, g, m, s);
-  cudaError_t e = cudaMemsetAsync(b->d_scal + box, 0, sizeof(WbScalars), s);
-  if (e != cudaSuccess) return bcuda(b, e, "batch load");
   if (!bi.wrap) wb_launch_halo(q, bb, g, m, s);
   wb_launch_init(q, bb, g, 1, bi.wrap ? 7 : 0, b->phys, primitive != 0, b->d_scal + box, s);
   if (!bi.wrap) wb_launch_halo(q, bb, g, m, s);

@@ -488,6 +488,8 @@ int load_common(wb_grid* g, const double* U, const double* bx, const double* by,
   cudaStream_t s = g->stream;
   const long long nc = (long long)g->d.n[0] * g->d.n[1] * g->d.n[2];
   const double* faces[3] = {bx, by, bz};
+  cudaError_t e = cudaMemsetAsync(g->scal, 0, sizeof(WbScalars), s);
+  if (e != cudaSuccess) return check_cuda(g, e, "load scalars");
   MoveList direct = {};  // arrays a kernel can read where they are: one launch
   for (int comp = 0; comp < 8; ++comp) {
     long long ext[3] = {g->d.n[0], g->d.n[1], g->d.n[2]};
@@ -500,7 +502,7 @@ int load_common(wb_grid* g, const double* U, const double* bx, const double* by,
     const bool staged = !on_device && !mapped;
     if (mapped) dsrc = static_cast<const double*>(mapped);
     if (staged) {
-      cudaError_t e = cudaMemcpyAsync(g->staging, src, sizeof(double) * n, cudaMemcpyHostToDevice, s);
+      e = cudaMemcpyAsync(g->staging, src, sizeof(double) * n, cudaMemcpyHostToDevice, s);
       if (e != cudaSuccess) return check_cuda(g, e, "load copy");
       dsrc = g->staging;
     }
@@ -516,8 +518,6 @@ int load_common(wb_grid* g, const double* U, const double* bx, const double* by,
     }
   }
   wb_launch_scatter(direct, g->geo, g->map, s);
-  cudaError_t e = cudaMemsetAsync(g->scal, 0, sizeof(WbScalars), s);
-  if (e != cudaSuccess) return check_cuda(g, e, "load scalars");
   if (g->closed != 7) wb_launch_halo(g->q, g->b, g->geo, g->map, s);
   wb_launch_init(g->q, g->b, g->geo, g->npatch, g->closed, g->phys, primitive, g->scal, s);
   if (g->closed != 7) wb_launch_halo(g->q, g->b, g->geo, g->map, s);
@@ -1008,29 +1008,28 @@ int wb_step_noalloc(const wb_desc* d, const double* U, const double* bx, const d
   g.prof = false;
   g.ev_used = 0;
   cudaStream_t s = g.stream;
-  // the array keeps the previous call's contents: the scalars (time, dt,
-  // signal-rate accumulator, counters) must start at zero
-  cudaError_t e = cudaMemsetAsync(g.scal, 0, L.scalars, s);
-  if (e != cudaSuccess) return noalloc_fail(WB_ERR_CUDA, std::string("memset: ") + cudaGetErrorString(e));
   const double* faces[3] = {bx, by, bz};
   const long long nc = (long long)one.n[0] * one.n[1] * one.n[2];
   MoveList in = {};
   for (int comp = 0; comp < 8; ++comp)
     wb_add_move(in, comp < 5 ? U + comp * nc : faces[comp - 5], comp < 5 ? g.q[comp] : g.b[comp - 5], comp);
-  wb_launch_scatter(in, g.geo, g.map, s);
+  // the array keeps the previous call's contents: the scalars (time, dt,
+  // signal-rate accumulator, counters) must start at zero
+  wb_launch_scatter(in, g.geo, g.map, s, g.scal);
   set_interior(&g);
   if (g.closed != 7) wb_launch_halo(g.q, g.b, g.geo, g.map, s);
   wb_launch_init(g.q, g.b, g.geo, 1, g.closed, g.phys, false, g.scal, s);
   if (g.closed != 7) wb_launch_halo(g.q, g.b, g.geo, g.map, s);
   StepControl c = step_control(&g, 0.0);
   c.lag = 0;
-  wb_launch_dt_step(g.scal, c, s);
+  wb_launch_dt_step(g.scal, c, s, true);
   enqueue_pass(&g, 0, 1, c);
   double* outs[3] = {bx_out, by_out, bz_out};
   MoveList out = {};
   for (int comp = 0; comp < 8; ++comp)
     wb_add_move(out, comp < 5 ? g.q[comp] : g.b[comp - 5], comp < 5 ? U_out + comp * nc : outs[comp - 5], comp);
-  wb_launch_gather(out, g.geo, g.map, s);
+  wb_launch_gather(out, g.geo, g.map, s, true);
+  cudaError_t e;
   if (dt_out) {
     e = cudaMemcpyAsync(dt_out, &g.scal->dt, sizeof(double), cudaMemcpyDeviceToDevice, s);
     if (e != cudaSuccess) return noalloc_fail(WB_ERR_CUDA, std::string("dt copy: ") + cudaGetErrorString(e));

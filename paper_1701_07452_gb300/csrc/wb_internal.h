@@ -6,10 +6,14 @@
 #include "wb_pages.h"
 #include "wb_units.cuh"
 
-// Launch of a kernel that begins with wb_pdl_begin(): it may be set up before
-// the kernel ahead of it on the stream has finished.
+// Launch of a kernel that begins with wb_pdl_begin().  Dependent: it may be set up
+// before the kernel ahead of it on the stream has finished.  Under stream capture
+// that becomes a programmatic edge, whose source has to be a kernel; a launch that
+// may follow anything else (a memset or copy, whatever the caller captured before
+// the call) is a plain one.
 template <class... P, class... A>
-inline cudaError_t wb_launch_dependent(void (*kernel)(P...), dim3 grid, int threads, cudaStream_t s, const A&... args) {
+inline cudaError_t wb_launch(bool dependent, void (*kernel)(P...), dim3 grid, int threads, cudaStream_t s,
+                             const A&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3((unsigned)threads);
@@ -18,8 +22,12 @@ inline cudaError_t wb_launch_dependent(void (*kernel)(P...), dim3 grid, int thre
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = dependent ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+template <class... P, class... A>
+inline cudaError_t wb_launch_dependent(void (*kernel)(P...), dim3 grid, int threads, cudaStream_t s, const A&... args) {
+  return wb_launch(true, kernel, grid, threads, s, args...);
 }
 
 struct wb_desc;
@@ -111,7 +119,8 @@ struct ImageList {
   int n;
 };
 void wb_launch_images(const ImageList& L, const WbGeo& geo, const wbu::Shell& sh, cudaStream_t s);
-void wb_launch_dt_step(WbScalars* scal, const StepControl& c, cudaStream_t s);
+// (dependent: right behind a kernel of the same call, not the first of an advance)
+void wb_launch_dt_step(WbScalars* scal, const StepControl& c, cudaStream_t s, bool dependent = false);
 // global <-> patch copies of up to 11 arrays; comp: 0..4 zone field, 5..7 face
 // field of axis comp-5
 struct MoveList {
@@ -125,8 +134,11 @@ inline void wb_add_move(MoveList& L, const double* src, double* dst, int comp) {
   L.dst[L.n] = dst;
   L.comp[L.n++] = comp;
 }
-void wb_launch_scatter(const MoveList& L, const WbGeo& geo, const GridMap& m, cudaStream_t s);
-void wb_launch_gather(const MoveList& L, const WbGeo& geo, const GridMap& m, cudaStream_t s);
+// (plain launches, but for a gather right behind a kernel of the same call; fresh:
+// the scalars of the loaded state, set to zero by the scatter)
+void wb_launch_scatter(const MoveList& L, const WbGeo& geo, const GridMap& m, cudaStream_t s,
+                       WbScalars* fresh = nullptr);
+void wb_launch_gather(const MoveList& L, const WbGeo& geo, const GridMap& m, cudaStream_t s, bool dependent = false);
 // Conserved totals: nblocks partial pairs in part (16 doubles each), the 8
 // totals x vol in out (device memory).
 void wb_launch_totals(double* const q[8], double* const b[3], const WbGeo& geo, long long npatch, double vol,

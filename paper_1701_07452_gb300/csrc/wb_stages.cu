@@ -375,11 +375,17 @@ __device__ __forceinline__ long long patch_offset(unsigned t, const unsigned ext
 // global arrays (host layout) <-> patch interiors, one array per blockIdx.y.
 // A thread moves kMove elements a block width apart, all loaded before any is
 // stored: one element a thread kept too little memory in flight (192^3, 8
-// arrays: 0.83 ms, 1.1 TB/s of reads and writes).
+// arrays: 0.83 ms, 1.1 TB/s of reads and writes).  The first block sets fresh (if
+// given) to zero: behind a memset the scatter would have to be a plain launch that
+// waits for it (a one-step call on 16^3 zones 83.5 us, 80.5 so).
 constexpr int kMove = 4;
 template <bool SCATTER>
-__global__ void k_move(MoveList L, WbGeo g, GridMap m) {
+__global__ void k_move(MoveList L, WbGeo g, GridMap m, WbScalars* fresh) {
   wb_pdl_begin();
+  constexpr unsigned kScalarWords = sizeof(WbScalars) / sizeof(unsigned long long);
+  static_assert(sizeof(WbScalars) % sizeof(unsigned long long) == 0 && kScalarWords <= 256, "one word a thread");
+  if (fresh && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < kScalarWords)
+    reinterpret_cast<unsigned long long*>(fresh)[threadIdx.x] = 0ULL;
   const int comp = L.comp[blockIdx.y];
   unsigned ext[3] = {(unsigned)m.N[0], (unsigned)m.N[1], (unsigned)m.N[2]};
   if (comp >= 5) ext[comp - 5] += 1;
@@ -589,13 +595,14 @@ void wb_launch_images(const ImageList& L, const WbGeo& geo, const wbu::Shell& sh
   wb_launch_dependent(k_images, grid_for(n, L.n, 256), 256, s, L, geo, sh, (unsigned)n);
 }
 
-void wb_launch_dt_step(WbScalars* scal, const StepControl& c, cudaStream_t s) {
-  wb_launch_dependent(k_dt_step, 1, 1, s, scal, c);
+void wb_launch_dt_step(WbScalars* scal, const StepControl& c, cudaStream_t s, bool dependent) {
+  wb_launch(dependent, k_dt_step, 1, 1, s, scal, c);
 }
 
 namespace {
 template <bool SCATTER>
-void launch_move(const MoveList& L, const WbGeo& geo, const GridMap& m, cudaStream_t s) {
+void launch_move(const MoveList& L, const WbGeo& geo, const GridMap& m, cudaStream_t s, bool dependent,
+                 WbScalars* fresh) {
   if (L.n <= 0) return;
   long long most = 0;
   for (int a = 0; a < L.n; ++a) {
@@ -603,16 +610,16 @@ void launch_move(const MoveList& L, const WbGeo& geo, const GridMap& m, cudaStre
     if (L.comp[a] >= 5) ext[L.comp[a] - 5] += 1;
     most = ext[0] * ext[1] * ext[2] > most ? ext[0] * ext[1] * ext[2] : most;
   }
-  wb_launch_dependent(k_move<SCATTER>, grid_for((most + kMove - 1) / kMove, L.n, 256), 256, s, L, geo, m);
+  wb_launch(dependent, k_move<SCATTER>, grid_for((most + kMove - 1) / kMove, L.n, 256), 256, s, L, geo, m, fresh);
 }
 }  // namespace
 
-void wb_launch_scatter(const MoveList& L, const WbGeo& geo, const GridMap& m, cudaStream_t s) {
-  launch_move<true>(L, geo, m, s);
+void wb_launch_scatter(const MoveList& L, const WbGeo& geo, const GridMap& m, cudaStream_t s, WbScalars* fresh) {
+  launch_move<true>(L, geo, m, s, false, fresh);
 }
 
-void wb_launch_gather(const MoveList& L, const WbGeo& geo, const GridMap& m, cudaStream_t s) {
-  launch_move<false>(L, geo, m, s);
+void wb_launch_gather(const MoveList& L, const WbGeo& geo, const GridMap& m, cudaStream_t s, bool dependent) {
+  launch_move<false>(L, geo, m, s, dependent, nullptr);
 }
 
 void wb_launch_divb(double* const b[3], const WbGeo& geo, long long npatch, int closed,
