@@ -249,9 +249,11 @@ const char* wb_noalloc_last_error(void);
  * wb_batch_advance: one persistent launch of nsteps steps; use_graph != 0
  * replays it from a captured CUDA graph (captured on first use per nsteps).
  * Synchronises the stream; returns WB_ERR_TIMEOUT if a barrier wait ran out.
- * wb_batch_autotune: times trial_steps real steps per candidate number of
- * blocks per SM in each form (below), keeps the fastest (cached per box-size
- * mix).
+ * wb_batch_autotune: times trial_steps real steps of the persistent form (forms:
+ * below) for each number of blocks per SM and of the staged form, and keeps the
+ * fastest (cached per box-size mix).  It ends early, with what it has timed, when
+ * the steps left no longer allow another trial of the same work; best_ms is 0, and
+ * the configuration as it was, when no box had steps left.
  * wb_batch_config: set them explicitly (0 = keep; seg_len is accepted and
  * reported, but the sweeps have no segments); barrier_budget_cycles is
  * the per-barrier wait limit in SM clock cycles (default 20 s worth).

@@ -978,6 +978,12 @@ int group_layout(const wb_batch* b, int grp, int s) {
   return rings && open ? wbu::kAnyLayout : (rings ? wbu::kRing : wbu::kOpen);
 }
 
+// the staged form's kernel for stage s of group grp
+StageKernel stage_kernel(const wb_batch* b, int grp, int s) {
+  return stage_class(s) == SC_SWEEP ? bstage_sweep_kernel(b->phys, group_layout(b, grp, s))
+                                    : bstage_zone_kernel(stage_class(s));
+}
+
 // enqueue the staged form of nsteps steps: one launch per (step, group,
 // stage), no synchronisation
 cudaError_t enqueue_staged(wb_batch* b, int nsteps) {
@@ -991,11 +997,9 @@ cudaError_t enqueue_staged(wb_batch* b, int nsteps) {
         // one block per chunk: a box holds more than 64 KB, so the count fits a grid
         const unsigned nblocks = (unsigned)b->stage_chunks[(size_t)grp * BS_COUNT + s];
         if (!nblocks) continue;
-        const bool sweep = stage_class(s) == SC_SWEEP;
-        const StageKernel fn =
-            sweep ? bstage_sweep_kernel(b->phys, group_layout(b, grp, s)) : bstage_zone_kernel(stage_class(s));
-        const int nt = sweep ? kB : kNtZone;
-        e = wb_launch(seq > 0, fn, nblocks, nt, b->stream, p, grp, s, seq);  // (the first follows the memset)
+        const int nt = stage_class(s) == SC_SWEEP ? kB : kNtZone;
+        // (the first launch follows the memset)
+        e = wb_launch(seq > 0, stage_kernel(b, grp, s), nblocks, nt, b->stream, p, grp, s, seq);
         if (e != cudaSuccess) return e;
         ++seq;
       }
@@ -1528,55 +1532,87 @@ int wb_batch_get_config(wb_batch* b, int* seg_len, int* blocks_per_sm, int* grou
   return WB_OK;
 }
 
-// Online autotuner: time trial_steps steps of each form under each block count,
-// keep the fastest.  The candidates change only the work decomposition, so the
-// trial steps are ordinary steps of the simulation (results do not depend on
-// the configuration).
+// Online autotuner: time trial_steps steps of each configuration that differs in what
+// runs (the persistent form under each block count, the staged form, which has
+// none, once) and keep the fastest.  The trial steps are ordinary steps of the
+// simulation (results do not depend on the configuration).  Trials are compared only
+// over the same work: once the boxes' steps left no longer allow what the first
+// trial took, tuning ends with what was timed so far (the configuration stays as it
+// was if that is nothing), and only a comparison of all configurations goes into the
+// cache.
 int wb_batch_autotune(wb_batch* b, int trial_steps, double* best_ms) {
   if (!b || trial_steps < 1) return bfail(b, WB_ERR_INVALID, "bad argument");
   int brc = ensure_built(b);
   if (brc) return brc;
+  if (best_ms) *best_ms = 0.0;
+  // steps of each box in a trial now; the first trial's
+  std::vector<int> work(b->cap), first;
+  auto same_work = [&](bool* same) -> int {
+    const int rc = wb_batch_steps_left(b, work.data());
+    if (rc) return rc;
+    bool any = false;
+    for (int& w : work) any = (w = std::min(w, trial_steps)) > 0 || any;
+    if (first.empty()) first = work;
+    *same = any && work == first;
+    return WB_OK;
+  };
+  struct Config {
+    int form, blocks;
+  };
+  std::vector<Config> configs;
+  for (int bps = b->max_blocks_per_sm; bps >= 1; --bps) configs.push_back({WB_BATCH_PERSISTENT, bps});
+  configs.push_back({WB_BATCH_STAGED, b->max_blocks_per_sm});
+  Config best = {b->form, b->blocks_per_sm};
+  // kernels are loaded at their first use: not inside a form's only trial
+  cudaFuncAttributes loaded;
+  cudaFuncGetAttributes(&loaded, batch_kernel(b->phys));
+  for (int grp = 0; grp + 1 < (int)b->gfirst.size(); ++grp)
+    for (int s = 0; s < BS_COUNT; ++s) cudaFuncGetAttributes(&loaded, (const void*)stage_kernel(b, grp, s));
+  float best_time = 1e30f;
+  size_t timed = 0;
+  int rc = WB_OK;
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
-  auto trial = [&](int bps, float* ms) -> int {
-    int rc = wb_batch_config(b, 0, bps, 0);
-    if (rc) return rc;
+  for (const Config& c : configs) {
+    bool same = false;
+    rc = same_work(&same);
+    if (rc || !same) break;
+    b->form = c.form;
+    rc = wb_batch_config(b, 0, c.blocks, 0);
+    if (rc) break;
     cudaEventRecord(e0, b->stream);
-    cudaError_t e = enqueue_advance(b, trial_steps);
-    if (e != cudaSuccess) return bcuda(b, e, "autotune");
+    const cudaError_t e = enqueue_advance(b, trial_steps);
+    if (e != cudaSuccess) {
+      rc = bcuda(b, e, "autotune");
+      break;
+    }
     cudaEventRecord(e1, b->stream);
     rc = read_sync_error(b);
-    if (rc) return rc;
-    cudaEventElapsedTime(ms, e0, e1);
-    return WB_OK;
-  };
-  int best_b = b->max_blocks_per_sm, best_form = b->form;
-  float best = 1e30f, ms = 0.f;
-  int rc = WB_OK;
-  for (int form = WB_BATCH_PERSISTENT; rc == WB_OK && form <= WB_BATCH_STAGED; ++form) {
-    b->form = form;
-    for (int bps = b->max_blocks_per_sm; bps >= 1; --bps) {
-      rc = trial(bps, &ms);
-      if (rc) break;
-      if (ms < best) { best = ms; best_b = bps; best_form = form; }
+    if (rc) break;
+    float ms = 0.f;
+    cudaEventElapsedTime(&ms, e0, e1);
+    ++timed;
+    if (ms < best_time) {
+      best_time = ms;
+      best = c;
     }
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  b->form = best_form;
+  b->form = best.form;
   if (rc) return rc;
-  rc = wb_batch_config(b, 0, best_b, 0);
+  rc = wb_batch_config(b, 0, best.blocks, 0);
   if (rc) return rc;
-  {
+  if (timed == configs.size()) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     TuneKey key;
     for (int i = 0; i < b->cap; ++i)
       if (b->alive[i]) key.sizes.push_back(b->d[i].n[0] * 1000000 + b->d[i].n[1] * 1000 + b->d[i].n[2]);
     std::sort(key.sizes.begin(), key.sizes.end());
-    g_tune_cache[key] = {best_b, best_form};
+    g_tune_cache[key] = {best.blocks, best.form};
   }
-  if (best_ms) *best_ms = best;
+  if (best_ms && timed) *best_ms = best_time;
   return WB_OK;
 }
 
