@@ -1,5 +1,8 @@
-// FP64 arithmetic on the integer pipes (host and device: the same integer
-// operations give the same bits on the CPU, where the tests check them).
+// FP64 arithmetic on the integer pipes.  Reciprocals and roots are the same integer
+// operations on host and device (the FP32 seeds differ by an ulp or two, which the
+// fixed-point step absorbs); the product's device form is PTX of its own (carry
+// chains, funnel shifts).  The tests hold the host forms against exact integers
+// and the device forms against the FP64 multiply and exact integers.
 #pragma once
 #include <cuda_runtime.h>
 #include <string.h>
@@ -241,7 +244,7 @@ WB_HD double wb_smul_t(double x, double y) {
   return wb_make64(hi, lo);
 }
 WB_HD double wb_smul(double x, double y) { return wb_smul_t<false, 0>(x, y); }
-// The same for finite factors whose product is known to stay below the top of
+// The form the sweeps take: the same for finite factors whose product is known to stay below the top of
 // the range (4 of the 40 instructions less, 6 % of a sweep).  KNOWN: 1, 2: x, y
 // normal; 7: both, and the product above 2^-1021 (1 to 5 instructions less).
 template <int KNOWN>
