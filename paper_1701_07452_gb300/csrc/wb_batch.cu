@@ -39,18 +39,15 @@ namespace {
 
 // Stages of a step.  Boxes periodic on every axis (wrap) run every stage on
 // their interior and read across their own ends, as a single-patch grid does
-// (enqueue_pass): they need no ghost fill.  BS_W* (once the images of their
-// intermediates) have no work and are not launched; they keep their
-// places in the stage times.
+// (enqueue_pass): they need no ghost fill.
 enum {
-  BS_DT = 0, BS_PRED, BS_EREF, BS_W_FP, BS_EDGE_P, BS_W_EE, BS_CT_H, BS_W_BH, BS_TRANS, BS_W_QH,
-  BS_CORR, BS_W_FC, BS_EREF_H, BS_W_ERH, BS_EDGE_C, BS_W_EEH, BS_CT_F, BS_FINAL, BS_HALO, BS_COUNT
+  BS_DT = 0, BS_PRED, BS_EREF, BS_EDGE_P, BS_CT_H, BS_TRANS, BS_CORR, BS_EREF_H, BS_EDGE_C, BS_CT_F, BS_FINAL, BS_HALO,
+  BS_COUNT
 };
-
-__host__ __device__ inline bool stage_is_wrap(int s) {
-  return s == BS_W_FP || s == BS_W_EE || s == BS_W_BH || s == BS_W_QH || s == BS_W_FC ||
-         s == BS_W_ERH || s == BS_W_EEH;
-}
+// Places of the stages in wb_batch_stage_times, whose other entries (images of
+// intermediates, which no box needs) read 0.
+constexpr int kReported = 19;
+constexpr int kReportAt[BS_COUNT] = {0, 1, 2, 4, 6, 8, 10, 12, 14, 16, 17, 18};
 
 constexpr int kB = wbu::kBlock;        // threads per block
 constexpr int kItemsPerThread = 8;     // items per thread in a chunk of a cheap stage
@@ -133,7 +130,6 @@ __host__ __device__ inline long long sweep_pencils(const WbBox& b, int d) {
 
 __host__ __device__ inline long long stage_items(int s, int d, const WbGeo& g, bool wrap) {
   if (s == BS_DT) return 1;
-  if (stage_is_wrap(s)) return 0;
   if (s == BS_HALO) return wrap ? 0 : wbu::shell_count(g, WB_NG);
   WbBox b = stage_box(s, d, g.n, wrap);
   if (stage_is_sweep(s)) {
@@ -1496,12 +1492,14 @@ int wb_batch_stage_timer(wb_batch* b, int on) {
 
 int wb_batch_stage_times(wb_batch* b, double* ms, int n, int* count) {
   if (!b || (!ms && n > 0)) return WB_ERR_INVALID;
-  if (count) *count = BS_COUNT;
+  if (count) *count = kReported;
   unsigned long long ns[BS_COUNT];
   cudaError_t e = cudaMemcpyAsync(ns, b->d_prof, sizeof(ns), cudaMemcpyDeviceToHost, b->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) return bcuda(b, e, "stage times");
-  for (int i = 0; i < n && i < BS_COUNT; ++i) ms[i] = 1e-6 * (double)ns[i];
+  for (int i = 0; i < n && i < kReported; ++i) ms[i] = 0.0;
+  for (int s = 0; s < BS_COUNT; ++s)
+    if (kReportAt[s] < n) ms[kReportAt[s]] = 1e-6 * (double)ns[s];
   return WB_OK;
 }
 

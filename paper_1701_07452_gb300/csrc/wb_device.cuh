@@ -83,11 +83,6 @@ __host__ __device__ __forceinline__ long long wb_at(const WbGeo& g, int i, int j
   return (long long)(k + WB_NG) * g.sz + (long long)(j + WB_NG) * g.sy + (i + WB_NG);
 }
 
-template <int D>
-__host__ __device__ __forceinline__ long long wb_stride(const WbGeo& g) {
-  return D == 0 ? 1LL : (D == 1 ? g.sy : g.sz);
-}
-
 // Inclusive index box relative to the patch interior.
 struct WbBox {
   int lo[3], hi[3];
@@ -230,13 +225,6 @@ __device__ __forceinline__ bool wb_order_less(double a, double b) {
   kb ^= (kb >> 63) & 0x7fffffffffffffffLL;
   return ka < kb;
 }
-// min(max(x, 0), 1)
-__device__ __forceinline__ double wb_clamp01(double x) {
-  const long long b = __double_as_longlong(x);
-  if (b <= 0) return 0.0;                                 // negative or zero
-  return b > 0x3ff0000000000000LL ? 1.0 : x;              // above 1 (or NaN -> 1)
-}
-
 // x / 2^s for s = 1, 2 on the integer pipe: the exponent field is lowered by
 // s, which is exact for every normal x whose quotient is normal.  Inputs
 // below 2^(s-1022) in magnitude (zero, subnormals, the lowest binades) give a
@@ -280,13 +268,6 @@ __device__ __forceinline__ double wb_xsgn(double x, double s) {
   return __longlong_as_double(__double_as_longlong(x) ^ sg);
 }
 
-// |x| with the sign of s (integer pipe)
-__device__ __forceinline__ double wb_copysign_abs(double mag, double s) {
-  long long m = __double_as_longlong(mag) & 0x7fffffffffffffffLL;
-  long long sg = __double_as_longlong(s) & (long long)0x8000000000000000ULL;
-  return __longlong_as_double(m | sg);
-}
-
 // Key of a signal rate w for an unsigned atomicMax: the bits of w > 0, 0 for
 // w <= 0, the canonical NaN for any NaN (so that a NaN rate poisons the max),
 // from the bit pattern alone: the FP64 compares (w >= 0, w != w) would each
@@ -297,12 +278,6 @@ __device__ __forceinline__ unsigned long long wb_rate_bits(double w) {
   asm("and.b32 %0, %1, 0x7fffffff;" : "=r"(mh) : "r"(__double2hiint(w)));
   const bool nan = mh > 0x7ff00000 || (mh == 0x7ff00000 && __double2loint(w) != 0);
   return nan ? 0x7ff8000000000000ULL : (b > 0 ? (unsigned long long)b : 0ULL);
-}
-
-// atomic max of a non-negative double through its bit pattern (exact, order independent)
-__device__ __forceinline__ void wb_atomic_max_pos(unsigned long long* addr, double v) {
-  if (v >= 0.0) atomicMax(addr, (unsigned long long)__double_as_longlong(v));
-  else if (!(v >= 0.0) && v != v) atomicMax(addr, 0x7ff8000000000000ULL);  // NaN poisons
 }
 
 // Sets the step's dt and what follows from it.

@@ -6,6 +6,8 @@
 #include "wb_pages.h"
 #include "wb_units.cuh"
 
+constexpr int kSMs = 152;  // streaming multiprocessors of the GPU this is written for
+
 // Launch of a kernel that begins with wb_pdl_begin().  Dependent: it may be set up
 // before the kernel ahead of it on the stream has finished.  Under stream capture
 // that becomes a programmatic edge, whose source has to be a kernel; a launch that

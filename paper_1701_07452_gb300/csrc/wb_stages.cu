@@ -37,7 +37,7 @@ inline dim3 grid_for(long long n, int nslots, int bs) {
 // threads on 16 SMs or 128 of 32 on 128 (the update 13 against 7 us).
 inline int stage_threads(long long n, int nslots, int most) {
   int bs = most;
-  while (bs > 32 && n * nslots < (long long)bs * 16 * 152) bs /= 2;
+  while (bs > 32 && n * nslots < (long long)bs * 16 * kSMs) bs /= 2;
   return bs;
 }
 

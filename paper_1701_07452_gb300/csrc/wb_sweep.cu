@@ -92,7 +92,7 @@ void wb_launch_sweeps(SweepArgs a, cudaStream_t s) {
   // With a block or less for each SM a scheduler has one warp: nothing hides the
   // integer products' latency, and the FP64 pipe has room for them (16^3: 18.7
   // against 22.4 us a launch; 24^3, 500 blocks: 35.1 against 28.9)
-  const bool soft = tiles_of(0) + tiles_of(1) + tiles_of(2) + e > 152;
+  const bool soft = tiles_of(0) + tiles_of(1) + tiles_of(2) + e > kSMs;
   // The default variant's large launches are compiled for each layout; when the
   // axes differ, all take the open one (a thin axis only as a ring)
   const bool fixed = ez && !a.phys.prot && soft && !(rings > 0 && rings < 3 && (axis(0) < 3 || axis(1) < 3 || axis(2) < 3));

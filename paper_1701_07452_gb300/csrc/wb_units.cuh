@@ -1384,15 +1384,4 @@ __device__ __forceinline__ void halo_self_offsets(const WbGeo& g, const int bc[3
   *src_off = wb_at(g, src[0], src[1], src[2]);
 }
 
-__device__ __forceinline__ void halo_self(const WbView& v, long long qo, const int bc[3], long long t) {
-  long long dst, so;
-  halo_self_offsets(v.geo, bc, t, &dst, &so);
-  dst += qo;
-  so += qo;
-#pragma unroll
-  for (int c = 0; c < 8; ++c) v.q[c][dst] = v.q[c][so];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) v.b[c][dst] = v.b[c][so];
-}
-
 }  // namespace wbu
