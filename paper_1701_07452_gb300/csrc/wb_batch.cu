@@ -1423,7 +1423,8 @@ int wb_batch_read(wb_batch* b, int box, double* U, double* bx, double* by, doubl
   const long long nc = (long long)d.n[0] * d.n[1] * d.n[2];
   double* faces[3] = {bx, by, bz};
   MoveList all = {};
-  bool idle = false;  // the caller's earlier work on the stream is done
+  bool idle = !on_device && wb_stream_idle(s);
+  bool plain = false;  // of the caller's array that holds the component
   for (int comp = 0; comp < 11; ++comp) {
     double* dst;
     const double* src;
@@ -1444,7 +1445,8 @@ int wb_batch_read(wb_batch* b, int box, double* U, double* bx, double* by, doubl
       all.n = 0;
       const long long n = ext[0] * ext[1] * ext[2];
       const size_t len = sizeof(double) * n;
-      cudaError_t e = wb_host_array(dst, n).plain ? wb_touch_in_order(dst, len, s, &idle) : cudaSuccess;
+      if (comp == 0 || (comp >= 5 && comp <= 8)) plain = wb_host_array(dst, comp == 0 ? 5 * n : (comp == 8 ? 3 * n : n)).plain;
+      cudaError_t e = plain ? wb_touch_in_order(dst, len, s, &idle) : cudaSuccess;
       if (e == cudaSuccess) e = cudaMemcpyAsync(dst, b->staging, len, cudaMemcpyDeviceToHost, s);
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);
       if (e != cudaSuccess) return bcuda(b, e, "batch read");

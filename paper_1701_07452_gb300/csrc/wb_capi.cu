@@ -723,7 +723,7 @@ int wb_read_state(wb_grid* g, double* U, double* bx, double* by, double* bz, dou
   const long long nc = (long long)g->d.n[0] * g->d.n[1] * g->d.n[2];
   double* faces[3] = {bx, by, bz};
   MoveList direct = {};  // arrays a kernel can write where they are: one launch
-  bool idle = false;     // the caller's earlier work on the stream is done
+  bool idle = !on_device && wb_stream_idle(s);
   for (int comp = 0; comp < 11; ++comp) {
     double* dst;
     int mcomp = comp;

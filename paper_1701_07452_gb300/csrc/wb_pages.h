@@ -52,10 +52,18 @@ inline void wb_touch_pages(void* p, size_t bytes) {
   c[bytes - 1] = 0;
 }
 
+// Whether everything enqueued on s so far is done (false: unknown).
+inline bool wb_stream_idle(cudaStream_t s) {
+  if (cudaPeekAtLastError() != cudaSuccess) return false;  // an earlier error is the caller's to see
+  const cudaError_t e = cudaStreamQuery(s);
+  if (e == cudaErrorNotReady) cudaGetLastError();
+  return e == cudaSuccess;
+}
+
 // The same ahead of a copy on stream s, in the stream's order: work enqueued
-// earlier may still read the buffer (a copy out of it, a host function), so the
-// stream is waited for first.  *idle: already waited for in this call (what the
-// call itself enqueues afterwards uses no other of the caller's arrays).
+// earlier may still read the buffer (a copy out of it, a host function), so unless
+// the stream was idle before this call enqueued anything (*idle; what the call
+// enqueues uses no other of the caller's arrays) it is waited for first.
 inline cudaError_t wb_touch_in_order(void* p, size_t bytes, cudaStream_t s, bool* idle) {
   if (!*idle) {
     const cudaError_t e = cudaStreamSynchronize(s);
